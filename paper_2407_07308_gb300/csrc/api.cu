@@ -1621,6 +1621,43 @@ extern "C" int fhe_selftest_modarith(uint64_t prime_mod, uint64_t prime_lo, uint
             if (reduce4q(4 * q - 1 - (x % (4 * q)), 2 * q, q) != (4 * q - 1 - (x % (4 * q))) % q) bad++;
             const u64 v = edge ? (it < 32 ? ~0ull - (u64)it : 31 * q - 1 - (u64)it) : rnd();
             if (reduce64(v, m) != v % q) bad++;
+            // half words: sums of up to eight products with constants times
+            // 2^(2h), and the small-quotient reduction of what they leave
+            HalfAcc ha{0, 0, 0};
+            u128 hs = 0;
+            for (int k = 0; k < 8; k++) {
+                half_mac(ha, half_pack(a[k], m.half), half_const(b[k], m));
+                hs = (hs + (u128)a[k] * b[k]) % q;
+                const u64 r = half_mont(ha, m);
+                if (r > (u64)(k + 2) * q || r % q != (u64)hs) bad++;
+                const u64 f = reduce_few(r, m);
+                if (f >= 2 * q || f % q != (u64)hs) bad++;
+            }
+            // sums of constant products, folded after each even count as the
+            // kernels do for the largest primes
+            DotAcc da{0, 0};
+            u128 ds = 0;
+            for (int k = 0; k < 8; k++) {
+                dot_mac(da, a[k], dot_const(b[k], m), m.half);
+                ds = (ds + (u128)a[k] * b[k]) % q;
+                const int64_t r = dot_fold(da, m);
+                const int64_t rm = r % (int64_t)q;
+                if (r >= (int64_t)(3 * q) || r <= -(int64_t)(3 * q) || (u64)(rm < 0 ? rm + (int64_t)q : rm) != (u64)ds) bad++;
+                if (m.half > 27 && (k & 1)) da = DotAcc{0, r};
+            }
+            // the fused stores' operands: one below 2q, one below 4q
+            {
+                u64 z = edge ? 4 * q - 1 - (u64)it : x % (4 * q);
+                if (m.half > 28) z = z % q;
+                DotAcc d2{0, 0};
+                dot_mac(d2, a[0] + q, dot_const(b[1], m), m.half);
+                dot_mac(d2, z, dot_const(b[2], m), m.half);
+                const int64_t r = dot_fold(d2, m);
+                if (r >= (int64_t)q || r <= -(int64_t)q ||
+                    centred_mod(r, q) != (u64)(((u128)a[0] * b[1] + (u128)(z % q) * b[2]) % q)) bad++;
+            }
+            const u64 few = edge ? (u64)((((u128)q << 6) - 1 - it) & ~0ull) : x % (((u64)1 << 6) * q);
+            if (reduce_few(few, m) >= 2 * q || reduce_few(few, m) % q != few % q) bad++;
         }
     }
     return bad;

@@ -63,7 +63,7 @@ struct ModUpParams {
     u64 inv_hat[FHE_MAXD][FHE_MAXK];    // (Q_j/q_i)^-1 mod q_i
     u64 inv_hat_s[FHE_MAXD][FHE_MAXK];  // its Shoup constant
     // hat[j][i][t] = (Q_j/q_i) mod (prime of extended limb t)
-    u64 hat[FHE_MAXD][FHE_MAXK][FHE_MAXP];
+    DotC hat[FHE_MAXD][FHE_MAXK][FHE_MAXP];
 };
 
 // ModDown of (acc0, acc1) from Q_l P to Q_l, fused with the forward NTT of
@@ -71,8 +71,8 @@ struct ModUpParams {
 struct ModDownParams {
     int l, K;
     u64 cinv[FHE_MAXK], cinv_s[FHE_MAXK];  // p^-1 (P/p_k)^-1 mod p_k
-    u64 phat[FHE_MAXK][FHE_MAXP];          // p (P/p_k) mod q_i
-    u64 pinv[FHE_MAXP], pinv_s[FHE_MAXP];  // P^-1 mod q_i
+    DotC phat[FHE_MAXK][FHE_MAXP];         // p (P/p_k) mod q_i
+    DotC pinv[FHE_MAXP];                   // P^-1 mod q_i
     int sprime[FHE_MAXK];                  // prime index of special limb k
 };
 
@@ -82,7 +82,7 @@ struct ModSwitchParams {
     int l, npoly;
     u64 pinv_last, pinv_last_s;               // p^-1 mod q_{l-1}
     u64 p_i[FHE_MAXP], p_i_s[FHE_MAXP];       // p mod q_i
-    u64 qinv[FHE_MAXP], qinv_s[FHE_MAXP];     // q_{l-1}^-1 mod q_i
+    DotC qinv[FHE_MAXP];                      // q_{l-1}^-1 mod q_i
 };
 
 // Relinearisation and the modulus switch that follows it, as one ModDown
@@ -93,9 +93,9 @@ struct ModSwitchParams {
 // coefficient domain; out_i = (acc_i P^-1 + add_i - NTT(correction)_i) q_m^-1.
 struct RelinMSParams {
     int l, K;
-    u64 h[FHE_MAXK + 1][FHE_MAXP];          // h[k][i] = p p_k^-1 mod q_i, h[K][i] = p mod q_i
-    u64 pinv[FHE_MAXP], pinv_s[FHE_MAXP];    // P^-1 mod q_i
-    u64 qminv[FHE_MAXP], qminv_s[FHE_MAXP];  // q_m^-1 mod q_i
+    DotC h[FHE_MAXK + 1][FHE_MAXP];         // h[k][i] = p p_k^-1 mod q_i, h[K][i] = p mod q_i
+    DotC pqinv[FHE_MAXP];                    // (P q_m)^-1 mod q_i
+    DotC qminv[FHE_MAXP];                    // q_m^-1 mod q_i
     u64 pkinv[FHE_MAXK];                     // p_k^-1 mod q_m
     u64 Pm, Pm_s;                            // P mod q_m
 };
@@ -108,8 +108,8 @@ struct RelinMSParams {
 // switches.
 struct MultiSwitchParams {
     int l, k;
-    u64 G[FHE_MAXK][FHE_MAXP];           // p D_t mod q_i
-    u64 Dinv[FHE_MAXP], Dinv_s[FHE_MAXP];  // D_k^-1 mod q_i
+    DotC G[FHE_MAXK][FHE_MAXP];          // p D_t mod q_i
+    DotC Dinv[FHE_MAXP];                 // D_k^-1 mod q_i
     u64 F[FHE_MAXK][FHE_MAXK];           // D_t D_j^-1 mod q_{l-1-j}
 };
 

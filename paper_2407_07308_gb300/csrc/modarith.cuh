@@ -40,8 +40,14 @@ struct ModQ {
     u64 q2;      // 2q
     u64 mu;      // floor(2^(2b+4) / q) * 2^(58-b): Barrett constant, pre-shifted
     int bshift;  // b - 2, the shift that forms t
-    int pad;
+    int half;    // ceil(b / 2): the width of a half word (see HalfAcc)
     u64 mu64;    // floor(2^64 / q)
+    uint32_t hlo, hhi;  // q = hhi 2^half + hlo
+    uint32_t hninv;     // -q^-1 mod 2^half
+    uint32_t qmu;       // floor(2^(32 + qsh) / q): quotients below 2^11 (see reduce_few)
+    int qsh;            // b - 20 (0 for b <= 20)
+    int32_t qinv;       // q^-1 mod 2^32
+    int32_t nql, nqh;   // -q = nqh 2^32 + nql, nql signed
 };
 
 // a * w mod q in [0, 2q), w < q, ws = floor(w 2^64 / q), any a < 2^64.
@@ -157,6 +163,119 @@ FHE_HD u64 reduce64(u64 v, const ModQ &m)
     return r >= m.q ? r - m.q : r;
 }
 
+// x < 2^11 q -> [0, (1 + 2^-12 x/q) q + 1], below 2q: the quotient estimate
+// qhat = floor(floor(x / 2^qsh) qmu / 2^32) never exceeds floor(x / q), and
+// qmu >= 2^12 keeps it above x/q (1 - 2^-12) - 2^-19 - 1.  One 32-bit high
+// product in place of reduce64's 64-bit one.
+FHE_HD u64 reduce_few(u64 x, const ModQ &m)
+{
+    const uint32_t xs = (uint32_t)(x >> m.qsh);
+#ifdef __CUDA_ARCH__
+    const uint32_t qhat = __umulhi(xs, m.qmu);
+#else
+    const uint32_t qhat = (uint32_t)(((u64)xs * m.qmu) >> 32);
+#endif
+    return x - (u64)qhat * m.q;
+}
+
+// ---- half words -----------------------------------------------------------
+// Residues of b bits as two halves of h = ceil(b/2) <= 29 bits.  A product's
+// low, high and cross terms are summed over up to eight products in three
+// 64-bit words, with no carry between them; the cross terms come from one
+// product of the halves' sums (A. Karatsuba 1962: (xl + xh)(yl + yh) - xl yl
+// - xh yh, the two subtractions once per sum; eight products of h + 1 bits
+// stay below 2^63), so a product is three wide multiplications.  The
+// multiplier pipe is what bounds these kernels: a 32 x 32 -> 64 product
+// takes two of its slots, a 128-bit multiply-add four such products.
+// One factor is kept as a constant times 2^(2h) mod q (half_const), and
+// half_mont divides the sum by 2^(2h) again (P. Montgomery, Math. Comp. 1985,
+// with two digits of h bits): it adds the multiples of q that clear the low
+// and then the middle word.
+struct HalfAcc {
+    u64 lo, mid, hi;  // mid: the products of the halves' sums
+};
+
+// the two halves of x in the two 32-bit words of the result
+FHE_HD u64 half_pack(u64 x, int h) { return ((x >> h) << 32) | (x & (((u64)1 << h) - 1)); }
+
+// acc += x y; xs, ys: the sums of the halves
+FHE_HD void half_mac(HalfAcc &a, uint32_t xl, uint32_t xh, uint32_t xs, uint32_t yl, uint32_t yh, uint32_t ys)
+{
+    a.lo += (u64)xl * yl;
+    a.hi += (u64)xh * yh;
+    a.mid += (u64)xs * ys;
+}
+
+// acc += x y, x and y packed halves
+FHE_HD void half_mac(HalfAcc &a, u64 x, u64 y)
+{
+    const uint32_t xl = (uint32_t)x, xh = (uint32_t)(x >> 32), yl = (uint32_t)y, yh = (uint32_t)(y >> 32);
+    half_mac(a, xl, xh, xl + xh, yl, yh, yl + yh);
+}
+
+// The sum S of n <= 8 products of canonical residues, divided by 2^(2h):
+// a residue below S / 2^(2h) + q <= (n + 1) q.
+FHE_HD u64 half_mont(HalfAcc a, const ModQ &m)
+{
+    const uint32_t mask = ((uint32_t)1 << m.half) - 1;
+    a.mid -= a.lo + a.hi;
+    const uint32_t t0 = ((uint32_t)a.lo * m.hninv) & mask;
+    a.lo += (u64)t0 * m.hlo;
+    a.mid += (u64)t0 * m.hhi;
+    a.mid += a.lo >> m.half;
+    const uint32_t t1 = ((uint32_t)a.mid * m.hninv) & mask;
+    a.mid += (u64)t1 * m.hlo;
+    a.hi += (u64)t1 * m.hhi;
+    return a.hi + (a.mid >> m.half);
+}
+
+// ---- sums of constant products ----------------------------------------------
+// sum_i x_i c_i mod q for constants c_i: x = xh 2^h + xl (half words), so
+// x c = xl c + xh (c 2^h mod q), and with both factors kept as the centred
+// residues w of c 2^32 and v of c 2^(32 + h) the sum S = sum xl w + xh v is
+// below n 2^h q in size -- 32 bits above q, which one 32-bit Montgomery step
+// (P. Montgomery 1985, signed) removes: t = S q^-1 mod 2^32 in [-2^31, 2^31),
+// (S - t q) / 2^32 = sum x_i c_i (mod q).  w and v are split into a signed low
+// and a high word, so each x_i takes four wide multiply-adds into two 64-bit
+// sums, without carries.
+//
+// Ranges: |low sum| <= 2^31 (sum xl + xh), plus 2^62 for t q's low word, stays
+// below 2^63 while sum (xl + xh) <= 2^31: eight canonical residues up to 54
+// bits, four at 56, two at 57 (dot_fold may be applied in between: its result
+// is the next sum's high word).  The result lies within
+// q/2 + 2^-33 q sum (xl + xh) of 0.
+struct DotC {
+    int32_t wl, wh, vl, vh;
+};
+
+struct DotAcc {
+    int64_t l, h;
+};
+
+// x in half words: xl = x mod 2^h, xh = x >> h, below 2^31 each
+FHE_HD void dot_mac(DotAcc &a, uint32_t xl, uint32_t xh, const DotC &c)
+{
+    a.l += (int64_t)(int32_t)xl * c.wl;
+    a.h += (int64_t)(int32_t)xl * c.wh;
+    a.l += (int64_t)(int32_t)xh * c.vl;
+    a.h += (int64_t)(int32_t)xh * c.vh;
+}
+
+FHE_HD void dot_mac(DotAcc &a, u64 x, const DotC &c, int h)
+{
+    dot_mac(a, (uint32_t)x & (((uint32_t)1 << h) - 1), (uint32_t)(x >> h), c);
+}
+
+FHE_HD int64_t dot_fold(const DotAcc &a, const ModQ &m)
+{
+    const int32_t t = (int32_t)((uint32_t)a.l * (uint32_t)m.qinv);
+    const int64_t c = a.l + (int64_t)t * m.nql;  // a multiple of 2^32
+    return a.h + (int64_t)t * m.nqh + (c >> 32);
+}
+
+// (-q, q) -> [0, q)
+FHE_HD u64 centred_mod(int64_t v, u64 q) { return (u64)(v + (int64_t)((u64)(v >> 63) & q)); }
+
 // [0, 2q) -> [0, q)
 FHE_HD u64 reduce2q(u64 a, u64 q) { return a >= q ? a - q : a; }
 
@@ -178,9 +297,39 @@ inline ModQ make_modq(u64 q)
     u128 mu = ((u128)1 << (2 * b + 4)) / q;             // < 2^(b+5)
     m.mu = (u64)(mu << (58 - b));
     m.bshift = b - 2;
-    m.pad = 0;
     m.mu64 = (u64)((((u128)1) << 64) / q);
+    m.half = (b + 1) / 2;
+    const uint32_t mask = ((uint32_t)1 << m.half) - 1;
+    m.hlo = (uint32_t)q & mask;
+    m.hhi = (uint32_t)(q >> m.half);
+    uint32_t inv = 1;                                   // q^-1 mod 2^32 by Newton's iteration
+    for (int i = 0; i < 5; i++) inv *= 2 - (uint32_t)q * inv;
+    m.hninv = (0 - inv) & mask;
+    m.qsh = b > 20 ? b - 20 : 0;
+    m.qmu = (uint32_t)((((u128)1) << (32 + m.qsh)) / q);
+    m.qinv = (int32_t)inv;
+    m.nql = (int32_t)(0 - (uint32_t)q);
+    m.nqh = (int32_t)((-(int64_t)q - m.nql) >> 32);
     return m;
+}
+
+// c 2^(2h) mod q, packed: the constant factor of half_mac
+inline u64 half_const(u64 c, const ModQ &m)
+{
+    return half_pack((u64)((((u128)c << (2 * m.half)) % m.q)), m.half);
+}
+
+inline DotC dot_const(u64 c, const ModQ &m)
+{
+    auto centred = [&m](u64 x) { return x > m.q / 2 ? (int64_t)x - (int64_t)m.q : (int64_t)x; };
+    const int64_t w = centred((u64)((((u128)c) << 32) % m.q));
+    const int64_t v = centred((u64)((((u128)c % m.q) << (32 + m.half)) % m.q));
+    DotC d;
+    d.wl = (int32_t)(uint32_t)w;
+    d.wh = (int32_t)((w - d.wl) >> 32);
+    d.vl = (int32_t)(uint32_t)v;
+    d.vh = (int32_t)((v - d.vl) >> 32);
+    return d;
 }
 
 inline u64 shoup_const(u64 w, u64 q) { return (u64)(((u128)w << 64) / q); }

@@ -22,13 +22,27 @@
 // Units.  Every CTA has 128 threads holding 16 residues each, so a unit of
 // work is 2048 residues in shared memory: NS = 2^(11-M) sub-transforms of 2^M
 // points.  A sub-transform runs as one radix-16 round (4 stages on strided
-// residues) and one round of the remaining M-4 stages (contiguous blocks),
-// with shared-memory exchanges in between.  A column unit is NC adjacent
+// residues) and one round of the remaining M-4 stages (contiguous blocks).
+// Column passes read and write global memory straight from the rounds'
+// registers, with one exchange in shared memory between them (two where the
+// load converts several limbs); row passes exchange twice.  A column unit is NC adjacent
 // columns of each of NS/NC jobs (one job except at n = 10); a row unit is
 // either one row of each of 16 jobs that share a prime times NS/16 adjacent
 // rows (the batched case: the CTA stages those rows' twiddles once), or NS
 // adjacent rows of one job (small batches; twiddles read through the cache).
-// Global memory is read and written in coalesced runs of at least 64 bytes.
+// Global memory is read and written in coalesced runs of at least 64 bytes
+// (32 in paired column units at N = 2^15).
+//
+// What bounds the passes: the multiplier pipe.  Register-resident probes: a
+// 32-bit multiply-add takes one slot of it, a 32 x 32 -> 64 or high product
+// two, and a 64-bit accumulation puts one of its two additions there, so a
+// butterfly's chained product takes about 15 slots; the other pipes and the
+// shared memory run beside it as long as they stay well below their peaks.
+// Measured on the comparison of 16 pairs (N = 2^14, 10 + 3 primes, one
+// replay) and on 7 pairs at N = 2^15 (p = 257, 3 digits, level 17): 12.0 and
+// 59.8 ms with conversions in 128-bit arithmetic, normalised inverse
+// butterflies and three conflicting exchanges a pass; 12.1 and 57.6 ms with
+// the arithmetic below alone; 11.2 and 50.0 ms with the layouts too.
 //
 // Segments and persistence.  A launch carries a table of up to FHE_SEGS
 // segments; a segment is one batch of limb jobs with its own context (ring
@@ -43,8 +57,8 @@
 // fused variants: ModUp (basis conversion of a key-switching digit computed
 // while loading, then NTT), ModDown and modulus switching (correction
 // computed while loading, subtract-and-scale applied while storing).
-// Butterflies are Harvey's lazy ones (values below (4s+1)q after s forward
-// stages, in [0, 4q) inverse) with Shoup twiddles.
+// Butterflies are Harvey's lazy ones (values below (4s+7)q after s forward
+// stages, below 4q 2^s inverse) with Shoup twiddles.
 //
 // The kernels and functors are templates instantiated by ntt.cu (limb maps,
 // the plain and scaled transforms, the autotuner), ntt_ks.cu (key switching:
@@ -74,8 +88,8 @@ __device__ __forceinline__ u64 bfly_mul(u64 a, const ulonglong2 w, u64 q)
 
 // Forward butterfly without normalisation: t = [Y w] in [0, 4q) for any
 // 64-bit Y (shoup_lazy4), so if X, Y < B then X + t and X - t + 4q lie in
-// [0, B + 4q).  Inputs below 4q (canonical residues, or the lazy results of
-// the fused conversions) stay below (4s + 4) q <= 64 q < 2^63 after s <= 15
+// [0, B + 4q).  Inputs below 7q (canonical residues, or the lazy results of
+// the fused conversions) stay below (4s + 7) q <= 67 q < 2^64 after s <= 15
 // stages for primes below 2^57; one reduction at the end brings every value
 // to [0, q).  q4 = 4q.
 __device__ __forceinline__ void ct_bfly(u64 &X, u64 &Y, const ulonglong2 w, u64 q, u64 q4)
@@ -86,21 +100,23 @@ __device__ __forceinline__ void ct_bfly(u64 &X, u64 &Y, const ulonglong2 w, u64 
     Y = x - t + q4;
 }
 
-// Inverse butterfly on values in [0, 4q): X + Y reduced once by 4q, and
-// [(X - Y + 4q) w] in [0, 4q).
-__device__ __forceinline__ void gs_bfly(u64 &X, u64 &Y, const ulonglong2 w, u64 q, u64 q4)
+// Inverse butterfly without normalisation: for X, Y < B, B a multiple of q,
+// X + Y < 2B and [(X - Y + B) w] in [0, 4q) (shoup_lazy4 takes any 64-bit
+// operand, and X - Y + B < 2B).  Sums double from stage to stage, so the
+// stages' bounds are 4q 2^j; reduce_few brings the sums back at the end of a
+// row pass (and, for primes above 54 bits, between its two rounds), where a
+// compare and subtract in every butterfly took 5 of its 22 instructions.
+__device__ __forceinline__ void gs_bfly(u64 &X, u64 &Y, const ulonglong2 w, u64 q, u64 B)
 {
-    u64 s = X + Y;
-    s = s >= q4 ? s - q4 : s;
-    u64 d = X - Y + q4;
+    const u64 d = X - Y + B;
+    X = X + Y;
     Y = bfly_mul(d, w, q);
-    X = s;
 }
 
 // Stages s0 .. s0+R-1 of the forward transform on one group x[0..2^R) whose
 // block index is hi.
 template <int R, class TW>
-__device__ __forceinline__ void fwd_round(u64 (&x)[1 << R], int s0, int hi, const TW &W, u64 q, u64 q2)
+__device__ __forceinline__ void fwd_round(u64 (&x)[1 << R], int s0, int hi, const TW &W, u64 q, u64 q4)
 {
 #pragma unroll
     for (int u = 0; u < R; u++) {
@@ -111,7 +127,7 @@ __device__ __forceinline__ void fwd_round(u64 (&x)[1 << R], int s0, int hi, cons
 #pragma unroll
             for (int k = 0; k < half; k++) {
                 const int e = t * 2 * half + k;
-                ct_bfly(x[e], x[e + half], w, q, q2);
+                ct_bfly(x[e], x[e + half], w, q, q4);
             }
         }
     }
@@ -121,34 +137,24 @@ __device__ __forceinline__ void fwd_round(u64 (&x)[1 << R], int s0, int hi, cons
 // half-distance 2^(R-1-U).  A template per stage keeps every index a
 // compile-time constant, so x stays in registers.
 template <int R, int U, class TW>
-__device__ __forceinline__ void inv_stage(u64 (&x)[1 << R], int s0, int hi, const TW &W, u64 q, u64 q2)
+__device__ __forceinline__ void inv_stage(u64 (&x)[1 << R], int s0, int hi, const TW &W, u64 q, u64 B)
 {
     constexpr int half = 1 << (R - 1 - U);
 #pragma unroll
     for (int t = 0; t < (1 << U); t++) {
         const ulonglong2 w = W.get(s0 + U, (hi << U) + t);
 #pragma unroll
-        for (int k = 0; k < half; k++) gs_bfly(x[t * 2 * half + k], x[t * 2 * half + k + half], w, q, q2);
+        for (int k = 0; k < half; k++) gs_bfly(x[t * 2 * half + k], x[t * 2 * half + k + half], w, q, B);
     }
-    if constexpr (U > 0) inv_stage<R, U - 1>(x, s0, hi, W, q, q2);
+    if constexpr (U > 0) inv_stage<R, U - 1>(x, s0, hi, W, q, 2 * B);
 }
 
+// Inputs below B; outputs below 2^R B, the upper half of x below 4q.
 template <int R, class TW>
-__device__ __forceinline__ void inv_round(u64 (&x)[1 << R], int s0, int hi, const TW &W, u64 q, u64 q2)
+__device__ __forceinline__ void inv_round(u64 (&x)[1 << R], int s0, int hi, const TW &W, u64 q, u64 B)
 {
-    inv_stage<R, R - 1>(x, s0, hi, W, q, q2);
+    inv_stage<R, R - 1>(x, s0, hi, W, q, B);
 }
-
-// Conversions computed by the loads of a forward transform (ModUp, ModDown,
-// the switch corrections) hand it a residue in [0, 3q) (a Barrett reduction
-// without its two corrections) or [0, 4q) (a lazy Shoup product) instead of
-// [0, q): the forward butterflies accept any 64-bit input whose lazy bound
-// stays below 2^64 ((4s + 4) q after s stages) and the transform's last step
-// reduces every output to [0, q), so the outputs are the same.  Measured on
-// the 16-pair comparison at N = 2^14: 2564 -> 2587 slot-comparisons/s.
-// (The chained product with two corrections in place of Shoup's exact one
-// for the constant products of the stores measured slower: 2577.)
-__device__ __forceinline__ u64 conv_reduce(u128 x, const ModQ &m) { return barrett128_lazy(x, m); }
 
 // ---------------------------------------------------------------------------
 // unit geometry
@@ -156,75 +162,78 @@ __device__ __forceinline__ u64 conv_reduce(u128 x, const ModQ &m) { return barre
 
 constexpr int T = 128;  // threads per CTA, 16 residues each
 
-// Register cap: FHE_NTT_MINB resident CTAs of 128 threads per SM (9: 56
-// registers a thread).  Measured on the headline comparison (16 pairs,
-// N = 2^14): with the C-form butterflies 8 CTAs 2291 slot-comparisons/s, 6
-// CTAs (80 registers) 2285, 7 with staged multi-limb loads 2152; with the
-// chained butterflies 7 CTAs 2574, 8 CTAs 2653, 9 CTAs 2672, and 2689 with the
-// forward row kernels of two-operand stores kept at 8 (FHE_NTT_MINB_ST2: at 9
-// they spill 116 bytes); 10 CTAs spill 170-1100 bytes.
+// Register cap: FHE_NTT_MINB resident CTAs of 128 threads per SM (8: 64
+// registers a thread).  Measured as above (16 pairs at N = 2^14 / 7 pairs at
+// 2^15): 9 CTAs 11.6 / 53.1 ms (spills), 8 CTAs 11.2 / 50.7, 7 CTAs 11.25 /
+// 49.9; 8 with the paired column kernels at 7 11.2 / 50.0.
 #ifndef FHE_NTT_MINB
-#define FHE_NTT_MINB 9
+#define FHE_NTT_MINB 8
 #endif
 // The same for the column kernels of paired units (two targets per load).
 #ifndef FHE_NTT_MINB_PAIRED
-#define FHE_NTT_MINB_PAIRED FHE_NTT_MINB
+#define FHE_NTT_MINB_PAIRED 7
 #endif
-// The same for the forward row kernels whose stores read two operands
-// besides the transform (ModDown, relinearise + switch: accumulator, addend).
-#ifndef FHE_NTT_MINB_ST2
-#define FHE_NTT_MINB_ST2 8
-#endif
-// Paired column units whose two jobs read different sources (a digit or
-// ciphertext boundary) load in a rolled loop (1) or the unrolled staged one (0).
-#ifndef FHE_NTT_PAIRED_FALLBACK_ROLLED
-#define FHE_NTT_PAIRED_FALLBACK_ROLLED 1
-#endif
-// Positions of a paired unit's load loop unrolled together (8 per thread).
-#ifndef FHE_NTT_PAIRED_UNROLL
-#define FHE_NTT_PAIRED_UNROLL 2
-#endif
-constexpr int PAIRED_UNROLL = FHE_NTT_PAIRED_UNROLL;
 // Launches that mix ring degrees 2^13..2^15 take the kernel that dispatches
 // every unit on its degree (1), or one launch per degree in turn (0).
 #ifndef FHE_NTT_MIXED_KERNEL
 #define FHE_NTT_MIXED_KERNEL 1
 #endif
-// Words staged per chunk by the loads that read several limbs each (ModUp,
-// relinearise + switch, multi-prime switch); 0 = not staged (each word's
-// loads, arithmetic and shared-memory store in turn, four words unrolled).
-// Measured: staging 2 or 4 words costs 4-5% on the headline (2190 / 2225
-// against 2291 slot-comparisons/s).
-#ifndef FHE_NTT_MULTI_LDCH
-#define FHE_NTT_MULTI_LDCH 0
-#endif
-
 // Shared-memory twiddle tables: entry k at k + k / 8 (one 16-byte pad per 8
 // entries), so that the second round's strided twiddle reads (stride up to 8
 // entries across threads) hit distinct banks.
 __host__ __device__ constexpr int twp(int k) { return k + (k >> 3); }
 __host__ __device__ constexpr int twp_size(int n) { return n + n / 8 + 1; }
 
-// smem layout: sub-transform c at c*P(M), element e at e + (e >> 4); P is odd
-// mod 16 in u64 units, so the strided, blocked and row-wise access patterns
-// spread over the banks.
+// Sub-transforms of 2^M points, 16 residues a thread.
 template <int M>
 struct Sub {
-    static constexpr int SZ = 1 << M;           // elements per sub-transform
-    static constexpr int G = SZ / 16;           // threads per sub-transform
-    static constexpr int NS = T / G;            // sub-transforms per unit
-    static constexpr int R2 = M - 4;            // stages of the second round
-    static constexpr int P = SZ + SZ / 16 + 1;  // padded stride
-    static constexpr int WORDS = NS * P;        // shared memory words
+    static constexpr int SZ = 1 << M;  // elements per sub-transform
+    static constexpr int G = SZ / 16;  // threads per sub-transform
+    static constexpr int NS = T / G;   // sub-transforms per unit
+    static constexpr int R2 = M - 4;   // stages of the second round
     static_assert(M >= 5 && M <= 8, "sub-transform size");
     static_assert(NS * SZ == 16 * T, "16 residues a thread");
+};
+
+// Shared-memory layouts of a unit: element e of sub-transform c at
+// c P + slot(c) + e + (e >> 4), in u64 words.  A 64-bit access is served
+// conflict-free when the 16 lanes of a half-warp hit 16 distinct words mod
+// 16.  Column passes put neighbouring sub-transforms in neighbouring lanes
+// (c = t % NS): 16 columns of one element want P odd; 8 columns x 2 elements
+// (M = 8) P = 2 mod 16; paired units also store 8 columns x 2 (M = 7: P = 2,
+// the second job's columns one word further) or 4 columns x 4 elements (M =
+// 8: P = 4, two words further).  Row passes put a sub-transform's own threads
+// side by side (c = t / G), so that their global reads are runs of G words:
+// P = G mod 16 spreads 16 / G sub-transforms x G words.  (Before, one layout
+// with P odd served all of them, with two-way conflicts in the second round
+// and three exchanges a pass instead of one or two; ncu: L1 at 59-68% of its
+// peak in the column and row passes.)
+constexpr int at_least_mod16(int n, int r) { return n + ((r - n) % 16 + 16) % 16; }
+
+template <int M, bool PAIRED>
+struct ColLay {
+    using C = Sub<M>;
+    static constexpr int BASE = C::SZ + C::SZ / 16;
+    static constexpr int P = M == 8 ? at_least_mod16(BASE, PAIRED ? 4 : 2)
+                             : M == 7 && PAIRED ? at_least_mod16(BASE, 2) : at_least_mod16(BASE, 1 + 2 * (BASE % 16 / 2));
+    static constexpr int SLOT = !PAIRED ? 0 : M == 8 ? 2 : M == 7 ? 1 : 0;  // the second job's shift
+    static constexpr int WORDS = C::NS * P + SLOT;
+    __device__ static int base(int c) { return c * P + (SLOT && c >= C::NS / 2 ? SLOT : 0); }
+    __device__ static int at(int c, int e) { return base(c) + e + (e >> 4); }
+};
+
+template <int M>
+struct RowLay {
+    using C = Sub<M>;
+    static constexpr int P = at_least_mod16(C::SZ + C::SZ / 16, C::G % 16);
+    static constexpr int WORDS = C::NS * P;
+    __device__ static int base(int c) { return c * P; }
     __device__ static int at(int c, int e) { return c * P + e + (e >> 4); }
 };
 
-constexpr int SM_WORDS = Sub<5>::WORDS > Sub<8>::WORDS ? Sub<5>::WORDS : Sub<8>::WORDS;
-// largest staged twiddle table (ulonglong2): one table of 256 entries, or two
-// of 128 (paired column units)
-constexpr int TW_WORDS = twp_size(256) > 2 * twp_size(128) ? twp_size(256) : 2 * twp_size(128);
+// staged twiddles (ulonglong2) of a row unit: one table of up to 255 entries,
+// or two of 127
+constexpr int TW_ROWS = twp_size(255) > 2 * twp_size(127) ? twp_size(255) : 2 * twp_size(127);
 constexpr int ROW_J = 16;                    // jobs per grouped row unit
 
 // Twiddle accessors: get(s, j) = psi^brv(2^s + j), the twiddle of global
@@ -251,86 +260,101 @@ struct RowTw {
     }
 };
 
-// Radix-16 round: thread t = (g, c) with c = t % NS, g = t / NS holds elements
-// e = k G + g (k < 16) of sub-transform c: local stages 0..3.
-// Remaining-stages round: thread t = (c, g') with c = t / G, g' = t % G holds the 16/G
-// blocks b = g' (16/G) + i of G contiguous elements: local stages 4..M-1.
-// geo gives each sub-transform's twiddle accessor, block index and prime.
+// The two rounds of a sub-transform c on a thread's 16 residues.  First
+// round (local stages 0..3): thread g of G holds elements e = k G + g, k < 16.
+// Second round (stages 4..M-1): thread g' holds e = 16 g' .. 16 g' + 15, as
+// 16 / G blocks of G.  geo gives each sub-transform's twiddle accessor, block
+// index and prime.
+//
+// Inverse (second round first): inputs below 4q.  With primes of at most
+// INV_WIDE_BITS bits the values of the other round start below 4q 2^(M-4) and
+// end below 4q 2^M <= 2^64; for larger primes reduce_few brings them below 2q
+// first.
+constexpr int INV_WIDE_BITS = 54;
+
 template <int M, bool FWD, class Geo>
-__device__ __forceinline__ void subtx(u64 *sm, int tid, const Geo &geo)
+__device__ __forceinline__ void round1(u64 (&x)[16], const Geo &geo, int c)
 {
-    using C = Sub<M>;
-    constexpr int G = C::G, R2 = C::R2, NB = 16 / G, NS = C::NS;
-    // Addresses as a per-thread base plus compile-time offsets: for e = kG + g
-    // (g < G <= 16, kG a multiple of G) e >> 4 = (kG) >> 4, and for
-    // e = 16 g' + iG + f (iG + f < 16) e >> 4 = g'.
-    auto round1 = [&]() {
-        const int c = tid % NS, g = tid / NS;
-        const auto W = geo.tw(c);
-        const int hi = geo.hi(c);
-        const u64 q = geo.q(c), q2 = 4 * q;  // lazy bound of the butterflies
-        u64 *b1 = sm + c * C::P + g;
-        u64 x[16];
-#pragma unroll
-        for (int k = 0; k < 16; k++) x[k] = b1[k * G + ((k * G) >> 4)];
-        if (FWD)
-            fwd_round<4>(x, geo.S, hi, W, q, q2);
-        else
-            inv_round<4>(x, geo.S, hi, W, q, q2);
-#pragma unroll
-        for (int k = 0; k < 16; k++) b1[k * G + ((k * G) >> 4)] = x[k];
-    };
-    auto round2 = [&]() {
-        const int c = tid / G, gp = tid % G;
-        const auto W = geo.tw(c);
-        const int hi = geo.hi(c);
-        const u64 q = geo.q(c), q2 = 4 * q;  // lazy bound of the butterflies
-        u64 *b2 = sm + c * C::P + gp * 17;
-#pragma unroll
-        for (int i = 0; i < NB; i++) {
-            u64 x[1 << R2];
-#pragma unroll
-            for (int f = 0; f < (1 << R2); f++) x[f] = b2[i * G + f];
-            if (FWD)
-                fwd_round<R2>(x, geo.S + 4, hi * 16 + gp * NB + i, W, q, q2);
-            else
-                inv_round<R2>(x, geo.S + 4, hi * 16 + gp * NB + i, W, q, q2);
-#pragma unroll
-            for (int f = 0; f < (1 << R2); f++) b2[i * G + f] = x[f];
-        }
-    };
-    if (FWD) {
-        round1();
-        __syncthreads();
-        round2();
+    const auto W = geo.tw(c);
+    const u64 q = geo.q(c), q4 = 4 * q;  // lazy bound of the butterflies
+    if constexpr (FWD) {
+        fwd_round<4>(x, geo.S, geo.hi(c), W, q, q4);
     } else {
-        round2();
-        __syncthreads();
-        round1();
+        const ModQ &m = geo.mq(c);
+        u64 B = q4 << Sub<M>::R2;
+        if (m.bshift > INV_WIDE_BITS - 2) {
+#pragma unroll
+            for (int k = 0; k < 16; k++) x[k] = reduce_few(x[k], m);
+            B = q4;
+        }
+        inv_round<4>(x, geo.S, geo.hi(c), W, q, B);
     }
+}
+
+template <int M, bool FWD, class Geo>
+__device__ __forceinline__ void round2(u64 (&x)[16], const Geo &geo, int c, int gp)
+{
+    constexpr int G = Sub<M>::G, R2 = Sub<M>::R2, NB = 16 / G;
+    const auto W = geo.tw(c);
+    const u64 q = geo.q(c), q4 = 4 * q;
+#pragma unroll
+    for (int i = 0; i < NB; i++) {
+        u64 y[G];
+#pragma unroll
+        for (int f = 0; f < G; f++) y[f] = x[i * G + f];
+        if constexpr (FWD)
+            fwd_round<R2>(y, geo.S + 4, geo.hi(c) * 16 + gp * NB + i, W, q, q4);
+        else
+            inv_round<R2>(y, geo.S + 4, geo.hi(c) * 16 + gp * NB + i, W, q, q4);
+#pragma unroll
+        for (int f = 0; f < G; f++) x[i * G + f] = y[f];
+    }
+}
+
+// A thread's residues in shared memory: at the first round's elements (base
+// b + g, elements k G apart) or the second's (base b + 17 g', contiguous).
+template <int G>
+__device__ __forceinline__ void put1(u64 *b, const u64 (&x)[16])
+{
+#pragma unroll
+    for (int k = 0; k < 16; k++) b[k * G + ((k * G) >> 4)] = x[k];
+}
+template <int G>
+__device__ __forceinline__ void get1(const u64 *b, u64 (&x)[16])
+{
+#pragma unroll
+    for (int k = 0; k < 16; k++) x[k] = b[k * G + ((k * G) >> 4)];
+}
+__device__ __forceinline__ void put2(u64 *b, const u64 (&x)[16])
+{
+#pragma unroll
+    for (int k = 0; k < 16; k++) b[k] = x[k];
+}
+__device__ __forceinline__ void get2(const u64 *b, u64 (&x)[16])
+{
+#pragma unroll
+    for (int k = 0; k < 16; k++) x[k] = b[k];
 }
 
 // Column pass of ring degree 2^(N1+N2): NC adjacent columns of NJ jobs.
 // XJ = 2 asks for two jobs per unit where one would hold all NS columns
-// (half as many columns each) and both jobs' twiddles fit the staging table:
-// functors whose loads convert several source limbs pair jobs that read the
-// same sources (fwd_cols_unit).
-__host__ __device__ constexpr bool col_paired(int xj, int n1, int ns, int nc1)
-{
-    return xj == 2 && nc1 == ns && 2 * twp_size(1 << n1) <= TW_WORDS;
-}
+// (half as many columns each): functors whose loads convert several source
+// limbs pair jobs that read the same sources (fwd_cols_unit).  At N = 2^15 a
+// paired unit holds 4 columns (32-byte runs, one sector each) and a larger
+// twiddle table.
+__host__ __device__ constexpr bool col_paired(int xj, int ns, int nc1) { return xj == 2 && nc1 == ns; }
 
 template <int N1, int N2, int XJ = 1>
 struct ColGeo {
     using C = Sub<N1>;
     static constexpr int NS = C::NS, SZ = C::SZ, NN = 1 << (N1 + N2);
     static constexpr int NC1 = NS < (1 << N2) ? NS : (1 << N2);
-    static constexpr bool PAIRED = col_paired(XJ, N1, NS, NC1);
+    static constexpr bool PAIRED = col_paired(XJ, NS, NC1);
+    using Lay = ColLay<N1, PAIRED>;
     static constexpr int NC = PAIRED ? NC1 / 2 : NC1;                  // columns per job
     static constexpr int NJ = NS / NC;                                 // jobs per unit
     static constexpr int BLK = (1 << N2) / NC;                         // column blocks per job
     static constexpr int TWC = twp_size(1 << N1);                      // staged twiddles per job
-    static_assert(NJ * TWC <= TW_WORDS, "twiddle staging");
     static_assert(NJ <= 2, "jobs per column unit");
     // word r of the unit: job slot, column in job, element
     __device__ static int jslot(int r) { return NJ == 1 ? 0 : r / (NC * SZ); }
@@ -343,10 +367,12 @@ struct ColTw {
     using Gm = ColGeo<N1, N2, XJ>;
     const ulonglong2 *W;
     u64 q0, q1;
+    const ModQ *m0, *m1;
     static constexpr int S = 0;
     __device__ PrefixTw tw(int c) const { return PrefixTw{W + (c / Gm::NC) * Gm::TWC}; }
     __device__ int hi(int) const { return 0; }
     __device__ u64 q(int c) const { return c / Gm::NC == 0 ? q0 : q1; }
+    __device__ const ModQ &mq(int c) const { return c / Gm::NC == 0 ? *m0 : *m1; }
 };
 
 // Row pass: grouped (16 jobs of one prime x R adjacent rows) or single (NS
@@ -355,6 +381,7 @@ template <int N1, int N2>
 struct RowGeo {
     using C = Sub<N2>;
     static constexpr int NS = C::NS, SZ = C::SZ, NN = 1 << (N1 + N2);
+    using Lay = RowLay<N2>;
     static constexpr int R = NS / ROW_J;         // rows per grouped unit
     static constexpr int CH = (1 << N1) / R;     // row chunks per limb (grouped)
     // row chunks per limb (single; a limb with fewer than NS rows, n = 10,
@@ -362,14 +389,14 @@ struct RowGeo {
     static constexpr int CHS = (1 << N1) >= NS ? (1 << N1) / NS : 1;
     static constexpr int TWR = twp_size(SZ - 1); // staged twiddles per row
     static_assert(NS >= ROW_J && NS % ROW_J == 0, "row units");
-    static_assert(R * TWR <= TW_WORDS, "twiddle staging");
+    static_assert(R * TWR <= TW_ROWS, "twiddle staging");
 };
 
 template <int N1, int N2>
 struct RowGrpTw {
     const ulonglong2 *W;
     int hi0;
-    u64 qq;
+    const ModQ &m;
     int S;
     __device__ RowTw tw(int c) const
     {
@@ -377,17 +404,19 @@ struct RowGrpTw {
         return RowTw{W + (c % R) * RowGeo<N1, N2>::TWR, N1, hi0 + c % R};
     }
     __device__ int hi(int c) const { return hi0 + c % RowGeo<N1, N2>::R; }
-    __device__ u64 q(int) const { return qq; }
+    __device__ u64 q(int) const { return m.q; }
+    __device__ const ModQ &mq(int) const { return m; }
 };
 
 struct RowOneTw {
     GTw g;
     int hi0;
-    u64 qq;
+    const ModQ &m;
     int S;
     __device__ GTw tw(int) const { return g; }
     __device__ int hi(int c) const { return hi0 + c; }
-    __device__ u64 q(int) const { return qq; }
+    __device__ u64 q(int) const { return m.q; }
+    __device__ const ModQ &mq(int) const { return m; }
 };
 
 // ---------------------------------------------------------------------------
@@ -404,13 +433,17 @@ struct SegHdr {
     const ulonglong2 *ninv;  // N^-1 per prime (Shoup pairs)
 };
 
+constexpr int DIR_FWD = 1, DIR_INV = 2;
+
 template <class S>
 struct SegIO {
     int nseg, ucols, urows, pad;
     SegHdr h[FHE_SEGS];
     S s[FHE_SEGS];
-    // jobs per column unit asked for (2: functors with load2 / same_src)
+    // jobs per column unit asked for (2: functors whose loads convert, with same_src)
     static constexpr int XJ = 1;
+    static constexpr bool PLAIN = false;
+    static constexpr int DIRS = DIR_FWD;  // the directions a functor serves
 };
 
 template <class IO>
@@ -422,44 +455,155 @@ __device__ __forceinline__ int seg_of(const IO &io, int u, bool rows)
 }
 
 // ---------------------------------------------------------------------------
-// the unit bodies
+// conversions computed by the loads of a forward transform (ModUp, ModDown,
+// the switch corrections): sum_a t_a c_a mod r over n source limbs
 // ---------------------------------------------------------------------------
 
-// Moves words r = tid + k T (k < 16) through src(r) -> dst(r, v), staged in
-// chunks of CH: the chunk's reads are all issued before its first write (the
-// compiler does not reorder a global read past a shared-memory write on its
-// own), so they overlap; CH = 0 keeps read/write pairs (better for loads
-// that already hold several reads each, like ModUp's basis conversion).
-template <int CH, class Src, class Dst>
-__device__ __forceinline__ void tile_in(int tid, Src src, Dst dst)
+// n source limbs one after the other from src, the target's constants, the
+// target limb and its prime
+struct Conv {
+    const u64 *src;
+    u64 *dst;
+    int n, prime;
+    DotC c[FHE_MAXK];
+};
+
+// positions converted together by a thread of a paired unit
+#ifndef FHE_NTT_CONV_P
+#define FHE_NTT_CONV_P 2
+#endif
+constexpr int CONV_P = FHE_NTT_CONV_P;
+
+// Two targets of the same sources at P positions n, n + STEP, ..: each source
+// word is loaded once and split into half words once; four wide
+// multiply-adds per source and target, one 32-bit Montgomery step per target
+// (DotAcc).  Results in [q, 7q): the forward butterflies take any input whose
+// lazy bound stays below 2^64 ((4 s + 7) q after s stages), and the
+// transform's last step reduces.  With 128-bit multiply-adds and a Barrett
+// reduction a converted residue took 112 instructions for 3 sources (ncu,
+// ModUp at N = 2^14), here about 30.
+template <int P, int STEP, int NN>
+__device__ __forceinline__ void conv_pair(const Conv &a, const Conv &b, const ModQ &ma, const ModQ &mb, int n,
+                                          u64 (&v0)[P], u64 (&v1)[P])
 {
-    constexpr int IT = 16;
-    if constexpr (CH > 0) {
-        constexpr int K = CH < IT ? CH : IT;
+    DotAcc s0[P], s1[P];
 #pragma unroll
-        for (int k0 = 0; k0 < IT; k0 += K) {
-            u64 v[K];
+    for (int p = 0; p < P; p++) {
+        s0[p] = DotAcc{0, (int64_t)(2 * ma.q2)};
+        s1[p] = DotAcc{0, (int64_t)(2 * mb.q2)};
+    }
+    const int h = ma.half, ns = a.n;
+    const u64 *src = a.src + n;
+#pragma unroll 1
+    for (int i0 = 0; i0 < ns; i0 += 4) {
+        u64 x[4][P];  // up to four sources' words in flight
 #pragma unroll
-            for (int k = 0; k < K; k++) v[k] = src(tid + (k0 + k) * T);
+        for (int i = 0; i < 4; i++)
+            if (i0 + i < ns) {
 #pragma unroll
-            for (int k = 0; k < K; k++) dst(tid + (k0 + k) * T, v[k]);
-        }
-    } else {
-#pragma unroll 4
-        for (int k = 0; k < IT; k++) dst(tid + k * T, src(tid + k * T));
+                for (int p = 0; p < P; p++) x[i][p] = src[(size_t)i * NN + p * STEP];
+            }
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+            if (i0 + i < ns) {
+                const DotC c0 = a.c[i0 + i], c1 = b.c[i0 + i];
+#pragma unroll
+                for (int p = 0; p < P; p++) {
+                    const uint32_t xl = (uint32_t)x[i][p] & (((uint32_t)1 << h) - 1), xh = (uint32_t)(x[i][p] >> h);
+                    dot_mac(s0[p], xl, xh, c0);
+                    dot_mac(s1[p], xl, xh, c1);
+                }
+                if (h > 27 && (i & 1)) {  // primes above 54 bits: two sources a sum
+#pragma unroll
+                    for (int p = 0; p < P; p++) {
+                        s0[p] = DotAcc{0, dot_fold(s0[p], ma)};
+                        s1[p] = DotAcc{0, dot_fold(s1[p], mb)};
+                    }
+                }
+            }
+        src += (size_t)4 * NN;
+    }
+#pragma unroll
+    for (int p = 0; p < P; p++) {
+        v0[p] = (u64)dot_fold(s0[p], ma);
+        v1[p] = (u64)dot_fold(s1[p], mb);
     }
 }
 
+// one target
+__device__ __forceinline__ u64 conv_one(const Conv &a, const ModQ &m, int N, int n)
+{
+    DotAcc s{0, (int64_t)(2 * m.q2)};
+#pragma unroll 1
+    for (int i = 0; i < a.n; i++) {
+        dot_mac(s, a.src[(size_t)i * N + n], a.c[i], m.half);
+        if (m.half > 27 && (i & 1)) s = DotAcc{0, dot_fold(s, m)};
+    }
+    return (u64)dot_fold(s, m);
+}
+
+// ---------------------------------------------------------------------------
+// kernels' stores: out = x A + d B mod q with constants, d = y - v for the
+// transform's lazy value v (below 71 q), x and y below 2q
+// ---------------------------------------------------------------------------
+
+// y + 2q - v (mod q) for y below 2q, in (0, 4q); canonical for primes above 56 bits, whose
+// half words leave no room for the multiple (DotAcc)
+__device__ __forceinline__ u64 lazy_diff(u64 y, u64 v, const ModQ &m)
+{
+    u64 d = y + m.q2 - reduce_few(v, m);
+    if (m.half > 28) d = reduce4q(d, m.q2, m.q);
+    return d;
+}
+
+// d B, canonical
+__device__ __forceinline__ u64 scaled1(u64 d, const DotC &B, const ModQ &m)
+{
+    DotAcc s{0, 0};
+    dot_mac(s, d, B, m.half);
+    return centred_mod(dot_fold(s, m), m.q);
+}
+
+// x A + d B, canonical
+__device__ __forceinline__ u64 scaled2(u64 x, const DotC &A, u64 d, const DotC &B, const ModQ &m)
+{
+    DotAcc s{0, 0};
+    dot_mac(s, x, A, m.half);
+    dot_mac(s, d, B, m.half);
+    return centred_mod(dot_fold(s, m), m.q);
+}
+
+// ---------------------------------------------------------------------------
+// the unit bodies
+// ---------------------------------------------------------------------------
+
+// Asynchronous copies global -> shared memory (16 and 8 bytes): tiles and
+// twiddle tables go there without passing through registers, all of a
+// thread's copies in flight at once; async_wait before the barrier that
+// publishes them.
+__device__ __forceinline__ void async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void async8(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // Stores of a forward row pass: word r goes to index idx(r) of state st(r)
-// with value val(r) when ok(r).  Staged: the operands the store reads
-// (IO::NPRE per word) are loaded for a chunk of words before any of the
-// chunk's writes, so those loads overlap.
+// with value val(r) (the transform's lazy value, below 71 q) when ok(r).
+// Staged: the operands the store reads (IO::NPRE per word) are loaded for a
+// chunk of words before any of the chunk's writes, so those loads overlap.
 template <class IO, class StF, class Ok, class Idx, class Val>
-__device__ __forceinline__ void tile_out(const IO &io, int tid, StF st, Ok ok, Idx idx, Val val)
+__device__ __forceinline__ void tile_out(const IO &io, const typename IO::RowK &rk, const ModQ &m, int tid, StF st,
+                                         Ok ok, Idx idx, Val val)
 {
     constexpr int IT = 16;
     if constexpr (IO::NPRE > 0) {
-        constexpr int CH = IO::NPRE == 1 ? IT : IT / 2;
+        constexpr int CH = IT / 2;
 #pragma unroll
         for (int k0 = 0; k0 < IT; k0 += CH) {
             u64 a[CH][IO::NPRE];
@@ -472,96 +616,84 @@ __device__ __forceinline__ void tile_out(const IO &io, int tid, StF st, Ok ok, I
 #pragma unroll
             for (int k = 0; k < CH; k++) {
                 const int r = tid + (k0 + k) * T;
-                if (ok(r)) io.store_pre(st(r), idx(r), val(r), a[k]);
+                if (ok(r)) io.store_pre(rk, m, st(r), idx(r), val(r), a[k]);
             }
         }
     } else {
 #pragma unroll 4
         for (int k = 0; k < IT; k++) {
             const int r = tid + k * T;
-            if (ok(r)) io.store(st(r), idx(r), val(r));
+            if (ok(r)) io.store_pre(rk, m, st(r), idx(r), val(r), nullptr);
         }
     }
 }
 
 // The jobs of a column unit: slot j (j < NJ) holds job0 + j.
 template <int N1, int N2, class IO>
-__device__ __forceinline__ int col_jobs(const IO &io, int sg, int lu, typename IO::St *sts, int *lo0)
+__device__ __forceinline__ int col_jobs(const IO &io, int sg, int lu, typename IO::CSt *sts, int *lo0)
 {
     using Gm = ColGeo<N1, N2, IO::XJ>;
     const SegHdr &H = io.h[sg];
     const int njobs = H.outer * H.nl;
     const int job0 = (lu / Gm::BLK) * Gm::NJ;
     *lo0 = (lu % Gm::BLK) * Gm::NC;
-    if (threadIdx.x < Gm::NJ && job0 + (int)threadIdx.x < njobs) io.begin(sg, job0 + threadIdx.x, sts[threadIdx.x]);
+    if (threadIdx.x < Gm::NJ && job0 + (int)threadIdx.x < njobs) io.begin_c(sg, job0 + threadIdx.x, sts[threadIdx.x]);
     __syncthreads();
     return njobs - job0;  // valid job slots (>= 1)
 }
 
-// Stages the first 2^N1 twiddles of each job's prime (the column stages):
-// loaded into registers first, stored after the tile loads (latency overlap).
-template <int N1, int N2, int XJ = 1>
-struct ColTwStage {
-    using Gm = ColGeo<N1, N2, XJ>;
-    static constexpr int NW = Gm::NJ << N1;
-    static constexpr int PER = (NW + T - 1) / T;
-    ulonglong2 v[PER];
-    template <class St>
-    __device__ void load(const SegHdr &H, const St *sts, int nvalid)
-    {
+// Stages the first 2^N1 twiddles of a job's prime (the column stages).
+template <int N1>
+__device__ __forceinline__ void col_twiddles(ulonglong2 *W, const ulonglong2 *tw)
+{
 #pragma unroll
-        for (int k = 0; k < PER; k++) {
-            const int i = threadIdx.x + k * T, j = i >> N1;
-            v[k] = (i < NW && j < nvalid) ? __ldg(H.tw + (size_t)sts[j].prime * Gm::NN + (i & ((1 << N1) - 1)))
-                                          : make_ulonglong2(0, 0);
-        }
-    }
-    __device__ void load1(const SegHdr &H, int prime)  // one job per unit
-    {
-#pragma unroll
-        for (int k = 0; k < PER; k++) {
-            const int i = threadIdx.x + k * T;
-            v[k] = i < NW ? __ldg(H.tw + (size_t)prime * Gm::NN + i) : make_ulonglong2(0, 0);
-        }
-    }
-    __device__ void store(ulonglong2 *W) const
-    {
-#pragma unroll
-        for (int k = 0; k < PER; k++) {
-            const int i = threadIdx.x + k * T;
-            if (i < NW) W[(i >> N1) * Gm::TWC + twp(i & ((1 << N1) - 1))] = v[k];
-        }
-    }
-};
+    for (int i = threadIdx.x; i < (1 << N1); i += T) async16(W + twp(i), tw + i);
+}
 
-// Column units of one job (every ring degree but 2^10): the job's state is
-// computed by every thread and stays in registers.
+// Column units of one job: the job's state is computed by every thread and
+// stays in registers.  Thread (c, g) reads and writes column lo0 + c in
+// global memory straight from its rounds' registers (neighbouring lanes,
+// neighbouring columns); shared memory carries the one exchange between the
+// rounds.
 template <int N1, int N2, class IO>
 __device__ __forceinline__ void fwd_cols_unit1(const IO &io, int sg, int lu, u64 *sm, ulonglong2 *W)
 {
     using Gm = ColGeo<N1, N2, IO::XJ>;
     using C = typename Gm::C;
-    const int tid = threadIdx.x;
+    const int c = threadIdx.x % C::NS, g = threadIdx.x / C::NS;
     const SegHdr &H = io.h[sg];
-    const int lo0 = (lu % Gm::BLK) * Gm::NC;
-    typename IO::St st;
-    io.begin(sg, lu / Gm::BLK, st);
-    ColTwStage<N1, N2, IO::XJ> tws;
-    tws.load1(H, st.prime);
-    const u64 q = H.mq[st.prime].q;
-    tile_in<IO::LDCH>(
-        tid, [&](int r) { return io.load(st, (Gm::elem(r) << N2) + lo0 + Gm::col(r)); },
-        [&](int r, u64 v) { sm[C::at(Gm::col(r), Gm::elem(r))] = v; });
-    tws.store(W);
-    __syncthreads();
-    subtx<N1, true>(sm, tid, ColTw<N1, N2, IO::XJ>{W, q, q});
-    __syncthreads();
-    u64 *mid = io.inter(st);
-#pragma unroll 4
-    for (int k = 0; k < 16; k++) {
-        const int r = tid + k * T;
-        mid[(Gm::elem(r) << N2) + lo0 + Gm::col(r)] = sm[C::at(Gm::col(r), Gm::elem(r))];
+    const int lo = (lu % Gm::BLK) * Gm::NC + c;
+    typename IO::CSt st;
+    io.begin_c(sg, lu / Gm::BLK, st);
+    col_twiddles<N1>(W, H.tw + (size_t)st.prime * Gm::NN);
+    const ModQ &m = H.mq[st.prime];
+    const ColTw<N1, N2, IO::XJ> geo{W, m.q, m.q, &m, &m};
+    u64 x[16];
+    const u64 *src = io.src(st) + (g << N2) + lo;
+#pragma unroll
+    for (int k = 0; k < 16; k++) x[k] = src[(k * C::G) << N2];
+    if constexpr (!IO::PLAIN) {
+#pragma unroll
+        for (int k = 0; k < 16; k++) x[k] = io.conv(st, x[k]);
     }
+    async_wait();
+    __syncthreads();  // the twiddles
+    round1<N1, true>(x, geo, c);
+    u64 *b = sm + Gm::Lay::base(c);
+    put1<C::G>(b + g, x);
+    __syncthreads();
+    get2(b + 17 * g, x);
+    round2<N1, true>(x, geo, c, g);
+    u64 *mid = io.inter(st) + (g << (N2 + 4)) + lo;
+#pragma unroll
+    for (int k = 0; k < 16; k++) mid[k << N2] = x[k];
+}
+
+// The last product of an inverse transform: a value anywhere in 64 bits times
+// N^-1 (and the entry's constant), canonical.
+__device__ __forceinline__ u64 inv_scaled(u64 v, const ulonglong2 ni, const ModQ &m)
+{
+    return reduce4q(shoup_lazy4_chain(v, ni.x, ni.y, 0 - m.q), m.q2, m.q);
 }
 
 template <int N1, int N2, class IO>
@@ -569,35 +701,45 @@ __device__ __forceinline__ void inv_cols_unit1(const IO &io, int sg, int lu, u64
 {
     using Gm = ColGeo<N1, N2, IO::XJ>;
     using C = typename Gm::C;
-    const int tid = threadIdx.x;
+    const int c = threadIdx.x % C::NS, g = threadIdx.x / C::NS;
     const SegHdr &H = io.h[sg];
-    const int lo0 = (lu % Gm::BLK) * Gm::NC;
-    typename IO::St st;
-    io.begin(sg, lu / Gm::BLK, st);
-    ColTwStage<N1, N2, IO::XJ> tws;
-    tws.load1(H, st.prime);
-    const u64 q = H.mq[st.prime].q;
+    const int lo = (lu % Gm::BLK) * Gm::NC + c;
+    typename IO::CSt st;
+    io.begin_c(sg, lu / Gm::BLK, st);
+    col_twiddles<N1>(W, H.tw + (size_t)st.prime * Gm::NN);
+    const ModQ &m = H.mq[st.prime];
+    const ColTw<N1, N2, IO::XJ> geo{W, m.q, m.q, &m, &m};
+    u64 x[16];
+    const u64 *mid = io.inter(st) + (g << (N2 + 4)) + lo;
+#pragma unroll
+    for (int k = 0; k < 16; k++) x[k] = mid[k << N2];
+    async_wait();
+    __syncthreads();  // the twiddles
+    round2<N1, false>(x, geo, c, g);
+    u64 *b = sm + Gm::Lay::base(c);
+    put2(b + 17 * g, x);
+    __syncthreads();
+    get1<C::G>(b + g, x);
+    round1<N1, false>(x, geo, c);
     const ulonglong2 ni = io.final_scale(st);
-    const u64 *mid = io.inter(st);
-    tile_in<16>(
-        tid, [&](int r) { return mid[(Gm::elem(r) << N2) + lo0 + Gm::col(r)]; },
-        [&](int r, u64 v) { sm[C::at(Gm::col(r), Gm::elem(r))] = v; });
-    tws.store(W);
-    __syncthreads();
-    subtx<N1, false>(sm, tid, ColTw<N1, N2, IO::XJ>{W, q, q});
-    __syncthreads();
-#pragma unroll 4
-    for (int k = 0; k < 16; k++) {
-        const int r = tid + k * T;
-        io.store(st, (Gm::elem(r) << N2) + lo0 + Gm::col(r),
-                 shoup(sm[C::at(Gm::col(r), Gm::elem(r))], ni.x, ni.y, q));
-    }
+#pragma unroll
+    for (int k = 0; k < 16; k++) io.store(st, ((k * C::G + g) << N2) + lo, inv_scaled(x[k], ni, m));
+}
+
+// a column's input word: read from a limb, or converted from several
+template <int NN, class IO>
+__device__ __forceinline__ u64 col_load(const IO &io, int sg, const typename IO::CSt &st, int n)
+{
+    if constexpr (IO::XJ == 2)
+        return io.load(sg, st, NN, n);
+    else
+        return io.load(st, n);
 }
 
 // Forward, columns: global stages 0..N1-1.
 template <int N1, int N2, class IO>
 __device__ __forceinline__ void fwd_cols_unit(const IO &io, int sg, int lu, u64 *sm, ulonglong2 *W,
-                                              typename IO::St *sts)
+                                              typename IO::CSt *sts)
 {
     using Gm = ColGeo<N1, N2, IO::XJ>;
     using C = typename Gm::C;
@@ -605,60 +747,61 @@ __device__ __forceinline__ void fwd_cols_unit(const IO &io, int sg, int lu, u64 
         fwd_cols_unit1<N1, N2>(io, sg, lu, sm, W);
         return;
     }
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, c = tid % C::NS, g = tid / C::NS;
     int lo0;
     const int nvalid = col_jobs<N1, N2>(io, sg, lu, sts, &lo0);
     const SegHdr &H = io.h[sg];
-    ColTwStage<N1, N2, IO::XJ> tws;
-    tws.load(H, sts, nvalid);
-    const u64 q0 = H.mq[sts[0].prime].q, q1 = nvalid > 1 ? H.mq[sts[Gm::NJ - 1].prime].q : q0;
+    const ModQ &m0 = H.mq[sts[0].prime], &m1 = H.mq[sts[nvalid > 1 ? Gm::NJ - 1 : 0].prime];
+    for (int j = 0; j < Gm::NJ && j < nvalid; j++)
+        col_twiddles<N1>(W + j * Gm::TWC, H.tw + (size_t)sts[j].prime * Gm::NN);
     bool paired = false;
     if constexpr (Gm::PAIRED) {
-        // both slots at once: word r (slot 0) and word r + NC SZ (slot 1)
-        // share column and element, so each source word is loaded once
+        // both slots at once: column col of slot 0 and of slot 1 at the same
+        // element, so each source word is loaded once
         static_assert(Gm::NJ == 2 && 2 * Gm::NC * Gm::SZ == 16 * T, "paired column unit");
         paired = nvalid >= 2 && io.same_src(sts[0], sts[1]);  // uniform in the CTA
         if (paired) {
-#pragma unroll PAIRED_UNROLL
-            for (int k = 0; k < 8; k++) {
-                const int r = tid + k * T;
-                u64 v0, v1;
-                io.load2(sts[0], sts[1], (Gm::elem(r) << N2) + lo0 + Gm::col(r), v0, v1);
-                sm[C::at(Gm::col(r), Gm::elem(r))] = v0;
-                sm[C::at(Gm::NC + Gm::col(r), Gm::elem(r))] = v1;
+            constexpr int ES = T / Gm::NC;  // elements between a thread's words
+            const int col = tid % Gm::NC, e0 = tid / Gm::NC;
+#pragma unroll 1
+            for (int k = 0; k < 8; k += CONV_P) {
+                u64 v0[CONV_P], v1[CONV_P];
+                conv_pair<CONV_P, (ES << N2), Gm::NN>(sts[0].cv, sts[1].cv, m0, m1, ((e0 + k * ES) << N2) + lo0 + col,
+                                                      v0, v1);
+#pragma unroll
+                for (int p = 0; p < CONV_P; p++) {
+                    sm[Gm::Lay::at(col, e0 + (k + p) * ES)] = v0[p];
+                    sm[Gm::Lay::at(Gm::NC + col, e0 + (k + p) * ES)] = v1[p];
+                }
             }
         }
     }
     if (!paired) {
-        if constexpr (Gm::PAIRED && FHE_NTT_PAIRED_FALLBACK_ROLLED) {
-            // the rare unit whose jobs read different sources: a rolled loop
-            // (small code beside the paired path)
+        // a unit whose jobs read different sources (or with one job left): a
+        // rolled loop, small code beside the paired path
 #pragma unroll 1
-            for (int k = 0; k < 16; k++) {
-                const int r = tid + k * T, j = Gm::jslot(r);
-                sm[C::at(j * Gm::NC + Gm::col(r), Gm::elem(r))] =
-                    j < nvalid ? io.load(sts[j], (Gm::elem(r) << N2) + lo0 + Gm::col(r)) : 0;
-            }
-        } else {
-            tile_in<IO::LDCH>(
-                tid,
-                [&](int r) {
-                    const int j = Gm::jslot(r);
-                    return j < nvalid ? io.load(sts[j], (Gm::elem(r) << N2) + lo0 + Gm::col(r)) : 0;
-                },
-                [&](int r, u64 v) { sm[C::at(Gm::jslot(r) * Gm::NC + Gm::col(r), Gm::elem(r))] = v; });
+        for (int k = 0; k < 16; k++) {
+            const int r = tid + k * T, j = Gm::jslot(r);
+            sm[Gm::Lay::at(j * Gm::NC + Gm::col(r), Gm::elem(r))] =
+                j < nvalid ? col_load<Gm::NN>(io, sg, sts[j], (Gm::elem(r) << N2) + lo0 + Gm::col(r)) : 0;
         }
     }
-    tws.store(W);
+    async_wait();
     __syncthreads();
-    subtx<N1, true>(sm, tid, ColTw<N1, N2, IO::XJ>{W, q0, q1});
+    const ColTw<N1, N2, IO::XJ> geo{W, m0.q, m1.q, &m0, &m1};
+    u64 x[16];
+    u64 *b = sm + Gm::Lay::base(c);
+    get1<C::G>(b + g, x);
+    round1<N1, true>(x, geo, c);
+    put1<C::G>(b + g, x);
     __syncthreads();
-#pragma unroll 4
-    for (int k = 0; k < 16; k++) {
-        const int r = tid + k * T, j = Gm::jslot(r);
-        if (j < nvalid)
-            io.inter(sts[j])[(Gm::elem(r) << N2) + lo0 + Gm::col(r)] =
-                sm[C::at(j * Gm::NC + Gm::col(r), Gm::elem(r))];
+    get2(b + 17 * g, x);
+    round2<N1, true>(x, geo, c, g);
+    const int j = c / Gm::NC;
+    if (j < nvalid) {
+        u64 *mid = io.inter(sts[j]) + (g << (N2 + 4)) + lo0 + c % Gm::NC;
+#pragma unroll
+        for (int k = 0; k < 16; k++) mid[k << N2] = x[k];
     }
 }
 
@@ -666,7 +809,7 @@ __device__ __forceinline__ void fwd_cols_unit(const IO &io, int sg, int lu, u64 
 // job's constant) and stores.
 template <int N1, int N2, class IO>
 __device__ __forceinline__ void inv_cols_unit(const IO &io, int sg, int lu, u64 *sm, ulonglong2 *W,
-                                              typename IO::St *sts)
+                                              typename IO::CSt *sts)
 {
     using Gm = ColGeo<N1, N2, IO::XJ>;
     using C = typename Gm::C;
@@ -674,33 +817,33 @@ __device__ __forceinline__ void inv_cols_unit(const IO &io, int sg, int lu, u64 
         inv_cols_unit1<N1, N2>(io, sg, lu, sm, W);
         return;
     }
-    const int tid = threadIdx.x;
+    const int c = threadIdx.x % C::NS, g = threadIdx.x / C::NS;
     int lo0;
     const int nvalid = col_jobs<N1, N2>(io, sg, lu, sts, &lo0);
     const SegHdr &H = io.h[sg];
-    ColTwStage<N1, N2, IO::XJ> tws;
-    tws.load(H, sts, nvalid);
-    const u64 q0 = H.mq[sts[0].prime].q, q1 = nvalid > 1 ? H.mq[sts[Gm::NJ - 1].prime].q : q0;
-    tile_in<16>(
-        tid,
-        [&](int r) {
-            const int j = Gm::jslot(r);
-            return j < nvalid ? io.inter(sts[j])[(Gm::elem(r) << N2) + lo0 + Gm::col(r)] : 0;
-        },
-        [&](int r, u64 v) { sm[C::at(Gm::jslot(r) * Gm::NC + Gm::col(r), Gm::elem(r))] = v; });
-    tws.store(W);
+    const ModQ &m0 = H.mq[sts[0].prime], &m1 = H.mq[sts[nvalid > 1 ? Gm::NJ - 1 : 0].prime];
+    for (int j = 0; j < Gm::NJ && j < nvalid; j++)
+        col_twiddles<N1>(W + j * Gm::TWC, H.tw + (size_t)sts[j].prime * Gm::NN);
+    const ColTw<N1, N2, IO::XJ> geo{W, m0.q, m1.q, &m0, &m1};
+    // a slot without a job transforms the first job's words and stores nothing
+    const int j = c / Gm::NC, lo = lo0 + c % Gm::NC, jv = j < nvalid ? j : 0;
+    u64 x[16];
+    const u64 *mid = io.inter(sts[jv]) + (g << (N2 + 4)) + lo;
+#pragma unroll
+    for (int k = 0; k < 16; k++) x[k] = mid[k << N2];
+    async_wait();
     __syncthreads();
-    subtx<N1, false>(sm, tid, ColTw<N1, N2, IO::XJ>{W, q0, q1});
+    round2<N1, false>(x, geo, c, g);
+    u64 *b = sm + Gm::Lay::base(c);
+    put2(b + 17 * g, x);
     __syncthreads();
-#pragma unroll 4
-    for (int k = 0; k < 16; k++) {
-        const int r = tid + k * T, j = Gm::jslot(r);
-        if (j < nvalid) {
-            const ulonglong2 ni = io.final_scale(sts[j]);
-            const u64 q = j == 0 ? q0 : q1;
-            io.store(sts[j], (Gm::elem(r) << N2) + lo0 + Gm::col(r),
-                     shoup(sm[C::at(j * Gm::NC + Gm::col(r), Gm::elem(r))], ni.x, ni.y, q));
-        }
+    get1<C::G>(b + g, x);
+    round1<N1, false>(x, geo, c);
+    if (j < nvalid) {
+        const ulonglong2 ni = io.final_scale(sts[j]);
+        const ModQ &m = j == 0 ? m0 : m1;
+#pragma unroll
+        for (int k = 0; k < 16; k++) io.store(sts[j], ((k * C::G + g) << N2) + lo, inv_scaled(x[k], ni, m));
     }
 }
 
@@ -708,7 +851,7 @@ __device__ __forceinline__ void inv_cols_unit(const IO &io, int sg, int lu, u64 
 // + l, rows hi0 .. hi0+R-1; single: slot 0 holds the job, rows hi0 ..
 // hi0+NS-1.  Returns the number of valid slots.
 template <int N1, int N2, bool GRP, class IO>
-__device__ __forceinline__ int row_jobs(const IO &io, int sg, int lu, typename IO::St *sts, int *hi0)
+__device__ __forceinline__ int row_jobs(const IO &io, int sg, int lu, typename IO::RSt *sts, int *hi0)
 {
     using Gm = RowGeo<N1, N2>;
     const SegHdr &H = io.h[sg];
@@ -719,11 +862,11 @@ __device__ __forceinline__ int row_jobs(const IO &io, int sg, int lu, typename I
         const int oc = t % OC, l = t / OC;
         *hi0 = hc * Gm::R;
         nvalid = min(ROW_J, H.outer - oc * ROW_J);
-        if ((int)threadIdx.x < nvalid) io.begin(sg, (oc * ROW_J + threadIdx.x) * H.nl + l, sts[threadIdx.x]);
+        if ((int)threadIdx.x < nvalid) io.begin_r(sg, (oc * ROW_J + threadIdx.x) * H.nl + l, sts[threadIdx.x]);
     } else {
         *hi0 = (lu % Gm::CHS) * Gm::NS;
         nvalid = 1;
-        if (threadIdx.x == 0) io.begin(sg, lu / Gm::CHS, sts[0]);
+        if (threadIdx.x == 0) io.begin_r(sg, lu / Gm::CHS, sts[0]);
     }
     __syncthreads();
     return nvalid;
@@ -732,33 +875,17 @@ __device__ __forceinline__ int row_jobs(const IO &io, int sg, int lu, typename I
 // Grouped rows stage the R rows' twiddles: entry k of row r is the stage
 // u = floor(log2(k+1)) twiddle with in-stage index (hi0 + r) 2^u + k+1-2^u.
 template <int N1, int N2>
-struct RowTwStage {
+__device__ __forceinline__ void row_twiddles(ulonglong2 *W, const ulonglong2 *tw, int hi0)
+{
     using Gm = RowGeo<N1, N2>;
-    static constexpr int NW = Gm::R * (Gm::SZ - 1);
-    static constexpr int PER = (NW + T - 1) / T;
-    ulonglong2 v[PER];
-    __device__ void load(const ulonglong2 *tw, int hi0)
-    {
+    constexpr int NW = Gm::R * (Gm::SZ - 1);
 #pragma unroll
-        for (int k = 0; k < PER; k++) {
-            const int i = threadIdx.x + k * T;
-            v[k] = make_ulonglong2(0, 0);
-            if (i < NW) {
-                const int r = i / (Gm::SZ - 1), e = i % (Gm::SZ - 1);
-                const int u = 31 - __clz(e + 1);
-                v[k] = __ldg(tw + (1 << (N1 + u)) + ((hi0 + r) << u) + (e + 1 - (1 << u)));
-            }
-        }
+    for (int i = threadIdx.x; i < NW; i += T) {
+        const int r = i / (Gm::SZ - 1), e = i % (Gm::SZ - 1);
+        const int u = 31 - __clz(e + 1);
+        async16(W + r * Gm::TWR + twp(e), tw + (1 << (N1 + u)) + ((hi0 + r) << u) + (e + 1 - (1 << u)));
     }
-    __device__ void store(ulonglong2 *W) const
-    {
-#pragma unroll
-        for (int k = 0; k < PER; k++) {
-            const int i = threadIdx.x + k * T;
-            if (i < NW) W[(i / (Gm::SZ - 1)) * Gm::TWR + twp(i % (Gm::SZ - 1))] = v[k];
-        }
-    }
-};
+}
 
 // word r of a row unit -> (sub-transform c = r >> N2, element f); the job
 // slot and row of c
@@ -768,82 +895,116 @@ struct RowMap {
     int hi0;
     __device__ int c(int r) const { return r >> N2; }
     __device__ int f(int r) const { return r & (Gm::SZ - 1); }
-    __device__ int slot(int r) const { return GRP ? c(r) / Gm::R : 0; }
-    __device__ int row(int r) const { return hi0 + (GRP ? c(r) % Gm::R : c(r)); }
+    __device__ int cslot(int c) const { return GRP ? c / Gm::R : 0; }
+    __device__ int crow(int c) const { return hi0 + (GRP ? c % Gm::R : c); }
+    __device__ int slot(int r) const { return cslot(c(r)); }
+    __device__ int row(int r) const { return crow(c(r)); }
 };
 
-// Forward, rows: global stages N1..N1+N2-1, reduction to [0, q), store.
+// Forward, rows: global stages N1..N1+N2-1, then the functor's store.
 template <int N1, int N2, bool GRP, class IO>
 __device__ __forceinline__ void fwd_rows_unit(const IO &io, int sg, int lu, u64 *sm, ulonglong2 *W,
-                                          typename IO::St *sts)
+                                          typename IO::RSt *sts)
 {
     using Gm = RowGeo<N1, N2>;
     using C = typename Gm::C;
+    using Lay = typename Gm::Lay;
     const int tid = threadIdx.x;
     const SegHdr &H = io.h[sg];
     int hi0;
     const int nvalid = row_jobs<N1, N2, GRP>(io, sg, lu, sts, &hi0);
     const RowMap<N1, N2, GRP> mp{hi0};
     const int prime = sts[0].prime;
-    const ModQ mqp = H.mq[prime];
+    const ModQ &m = H.mq[prime];
     const ulonglong2 *tw = H.tw + (size_t)prime * Gm::NN;
-    RowTwStage<N1, N2> tws;
-    if (GRP) tws.load(tw, hi0);
-    tile_in<16>(
-        tid,
-        [&](int r) {
-            const int j = mp.slot(r);
-            return j < nvalid ? io.inter(sts[j])[(mp.row(r) << N2) + mp.f(r)] : 0;
-        },
-        [&](int r, u64 v) { sm[C::at(mp.c(r), mp.f(r))] = v; });
-    if (GRP) tws.store(W);
+    if (GRP) row_twiddles<N1, N2>(W, tw, hi0);
+    // thread (c, g) reads its first round's words: runs of G words
+    const int c = tid / C::G, g = tid % C::G;
+    u64 x[16];
+    {
+        const int j = mp.cslot(c);  // a slot without a job transforms the first job's words and stores nothing
+        const u64 *src = io.inter(sts[j < nvalid ? j : 0]) + (mp.crow(c) << N2) + g;
+#pragma unroll
+        for (int k = 0; k < 16; k++) x[k] = src[k * C::G];
+    }
+    if (GRP) {
+        async_wait();
+        __syncthreads();  // the twiddles
+    }
+    u64 *b = sm + Lay::base(c);
+    if (GRP) {
+        const RowGrpTw<N1, N2> geo{W, hi0, m, N1};
+        round1<N2, true>(x, geo, c);
+        put1<C::G>(b + g, x);
+        __syncthreads();
+        get2(b + 17 * g, x);
+        round2<N2, true>(x, geo, c, g);
+    } else {
+        const RowOneTw geo{GTw{tw}, hi0, m, N1};
+        round1<N2, true>(x, geo, c);
+        put1<C::G>(b + g, x);
+        __syncthreads();
+        get2(b + 17 * g, x);
+        round2<N2, true>(x, geo, c, g);
+    }
+    put2(b + 17 * g, x);
     __syncthreads();
-    if (GRP)
-        subtx<N2, true>(sm, tid, RowGrpTw<N1, N2>{W, hi0, mqp.q, N1});
-    else
-        subtx<N2, true>(sm, tid, RowOneTw{GTw{tw}, hi0, mqp.q, N1});
-    __syncthreads();
+    const typename IO::RowK rk = io.row_k(sg, prime);
     tile_out(
-        io, tid, [&](int r) -> const typename IO::St & { return sts[mp.slot(r)]; },
+        io, rk, m, tid, [&](int r) -> const typename IO::RSt & { return sts[mp.slot(r)]; },
         [&](int r) { return mp.slot(r) < nvalid; }, [&](int r) { return (mp.row(r) << N2) + mp.f(r); },
-        [&](int r) { return reduce64(sm[C::at(mp.c(r), mp.f(r))], mqp); });
+        [&](int r) { return sm[Lay::at(mp.c(r), mp.f(r))]; });
 }
 
 // Inverse, rows first: undoes global stages N1+N2-1..N1.
 template <int N1, int N2, bool GRP, class IO>
 __device__ __forceinline__ void inv_rows_unit(const IO &io, int sg, int lu, u64 *sm, ulonglong2 *W,
-                                          typename IO::St *sts)
+                                          typename IO::RSt *sts)
 {
     using Gm = RowGeo<N1, N2>;
     using C = typename Gm::C;
+    using Lay = typename Gm::Lay;
     const int tid = threadIdx.x;
     const SegHdr &H = io.h[sg];
     int hi0;
     const int nvalid = row_jobs<N1, N2, GRP>(io, sg, lu, sts, &hi0);
     const RowMap<N1, N2, GRP> mp{hi0};
     const int prime = sts[0].prime;
-    const u64 q = H.mq[prime].q;
+    const ModQ &m = H.mq[prime];
     const ulonglong2 *tw = H.tw + (size_t)prime * Gm::NN;
-    RowTwStage<N1, N2> tws;
-    if (GRP) tws.load(tw, hi0);
-    tile_in<IO::LDCH>(
-        tid,
-        [&](int r) {
-            const int j = mp.slot(r);
-            return j < nvalid ? io.load(sts[j], (mp.row(r) << N2) + mp.f(r)) : 0;
-        },
-        [&](int r, u64 v) { sm[C::at(mp.c(r), mp.f(r))] = v; });
-    if (GRP) tws.store(W);
-    __syncthreads();
-    if (GRP)
-        subtx<N2, false>(sm, tid, RowGrpTw<N1, N2>{W, hi0, q, N1});
-    else
-        subtx<N2, false>(sm, tid, RowOneTw{GTw{tw}, hi0, q, N1});
-    __syncthreads();
-#pragma unroll 4
+    if (GRP) row_twiddles<N1, N2>(W, tw, hi0);
+#pragma unroll
     for (int k = 0; k < 16; k++) {
         const int r = tid + k * T, j = mp.slot(r);
-        if (j < nvalid) io.inter(sts[j])[(mp.row(r) << N2) + mp.f(r)] = sm[C::at(mp.c(r), mp.f(r))];
+        if (j < nvalid) io.load_async(&sm[Lay::at(mp.c(r), mp.f(r))], sts[j], (mp.row(r) << N2) + mp.f(r));
+    }
+    async_wait();
+    __syncthreads();
+    const int c = tid / C::G, g = tid % C::G;
+    u64 *b = sm + Lay::base(c);
+    u64 x[16];
+    get2(b + 17 * g, x);  // a slot without a job transforms what is there and stores nothing
+    if (GRP) {
+        const RowGrpTw<N1, N2> geo{W, hi0, m, N1};
+        round2<N2, false>(x, geo, c, g);
+        put2(b + 17 * g, x);
+        __syncthreads();
+        get1<C::G>(b + g, x);
+        round1<N2, false>(x, geo, c);
+    } else {
+        const RowOneTw geo{GTw{tw}, hi0, m, N1};
+        round2<N2, false>(x, geo, c, g);
+        put2(b + 17 * g, x);
+        __syncthreads();
+        get1<C::G>(b + g, x);
+        round1<N2, false>(x, geo, c);
+    }
+    // the sums (below 4q 2^N2) come down to 2q for the column pass
+    const int j = mp.cslot(c);
+    if (j < nvalid) {
+        u64 *mid = io.inter(sts[j]) + (mp.crow(c) << N2) + g;
+#pragma unroll
+        for (int k = 0; k < 16; k++) mid[k * C::G] = k < 8 ? reduce_few(x[k], m) : x[k];
     }
 }
 
@@ -875,14 +1036,39 @@ __device__ __forceinline__ void by_degree(int logN, F f)
     }
 }
 
+// shared memory of a column kernel: twiddle entries and job states over its
+// range of ring degrees
+template <class IO, int LO, int HI>
+constexpr int col_tw_entries()
+{
+    using Gm = ColGeo<Deg<LO>::N1, Deg<LO>::N2, IO::XJ>;
+    constexpr int n = Gm::NJ * Gm::TWC;
+    if constexpr (LO == HI)
+        return n;
+    else
+        return n > col_tw_entries<IO, LO + 1, HI>() ? n : col_tw_entries<IO, LO + 1, HI>();
+}
+template <class IO, int LO, int HI>
+constexpr int col_words()
+{
+    constexpr int n = ColGeo<Deg<LO>::N1, Deg<LO>::N2, IO::XJ>::Lay::WORDS;
+    if constexpr (LO == HI)
+        return n;
+    else
+        return n > col_words<IO, LO + 1, HI>() ? n : col_words<IO, LO + 1, HI>();
+}
+constexpr int ROW_WORDS = RowLay<7>::WORDS;
+static_assert(RowLay<5>::WORDS <= ROW_WORDS && RowLay<6>::WORDS <= ROW_WORDS, "row units");
+constexpr int COL_J = 2;  // jobs per column unit, at most
+
 template <class IO, int LO, int HI>
 __global__ void __launch_bounds__(T, IO::XJ == 2 ? FHE_NTT_MINB_PAIRED : FHE_NTT_MINB)
     k_fwd_cols(const __grid_constant__ IO io)
 {
     pdl_begin();
-    __shared__ u64 sm[SM_WORDS];
-    __shared__ ulonglong2 W[TW_WORDS];
-    __shared__ typename IO::St sts[ROW_J];
+    __shared__ u64 sm[col_words<IO, LO, HI>()];
+    __shared__ ulonglong2 W[col_tw_entries<IO, LO, HI>()];
+    __shared__ typename IO::CSt sts[COL_J];
     for (int u = blockIdx.x; u < io.ucols; u += gridDim.x) {
         const int sg = seg_of(io, u, false), lu = u - io.h[sg].u_cols;
         by_degree<LO, HI>(io.h[sg].logN, [&](auto d) {
@@ -893,13 +1079,13 @@ __global__ void __launch_bounds__(T, IO::XJ == 2 ? FHE_NTT_MINB_PAIRED : FHE_NTT
 }
 
 template <class IO, int LO, int HI>
-__global__ void __launch_bounds__(T, IO::NPRE >= 2 ? FHE_NTT_MINB_ST2 : FHE_NTT_MINB)
+__global__ void __launch_bounds__(T, FHE_NTT_MINB)
     k_fwd_rows(const __grid_constant__ IO io)
 {
     pdl_begin();
-    __shared__ u64 sm[SM_WORDS];
-    __shared__ ulonglong2 W[TW_WORDS];
-    __shared__ typename IO::St sts[ROW_J];
+    __shared__ u64 sm[ROW_WORDS];
+    __shared__ ulonglong2 W[TW_ROWS];
+    __shared__ typename IO::RSt sts[ROW_J];
     for (int u = blockIdx.x; u < io.urows; u += gridDim.x) {
         const int sg = seg_of(io, u, true), lu = u - io.h[sg].u_rows;
         if (io.h[sg].grouped)
@@ -918,9 +1104,9 @@ template <class IO, int LO, int HI>
 __global__ void __launch_bounds__(T, FHE_NTT_MINB) k_inv_rows(const __grid_constant__ IO io)
 {
     pdl_begin();
-    __shared__ u64 sm[SM_WORDS];
-    __shared__ ulonglong2 W[TW_WORDS];
-    __shared__ typename IO::St sts[ROW_J];
+    __shared__ u64 sm[ROW_WORDS];
+    __shared__ ulonglong2 W[TW_ROWS];
+    __shared__ typename IO::RSt sts[ROW_J];
     for (int u = blockIdx.x; u < io.urows; u += gridDim.x) {
         const int sg = seg_of(io, u, true), lu = u - io.h[sg].u_rows;
         if (io.h[sg].grouped)
@@ -939,9 +1125,9 @@ template <class IO, int LO, int HI>
 __global__ void __launch_bounds__(T, FHE_NTT_MINB) k_inv_cols(const __grid_constant__ IO io)
 {
     pdl_begin();
-    __shared__ u64 sm[SM_WORDS];
-    __shared__ ulonglong2 W[TW_WORDS];
-    __shared__ typename IO::St sts[ROW_J];
+    __shared__ u64 sm[col_words<IO, LO, HI>()];
+    __shared__ ulonglong2 W[col_tw_entries<IO, LO, HI>()];
+    __shared__ typename IO::CSt sts[COL_J];
     for (int u = blockIdx.x; u < io.ucols; u += gridDim.x) {
         const int sg = seg_of(io, u, false), lu = u - io.h[sg].u_cols;
         by_degree<LO, HI>(io.h[sg].logN, [&](auto d) {
@@ -952,8 +1138,13 @@ __global__ void __launch_bounds__(T, FHE_NTT_MINB) k_inv_cols(const __grid_const
 }
 
 // ---------------------------------------------------------------------------
-// load/store functors (one payload per segment)
+// load/store functors (one payload per segment).  A column pass keeps its
+// jobs' states as CSt (begin_c), a row pass as RSt (begin_r); RowK holds the
+// constants a row unit's stores share (its jobs have one prime and level).
 // ---------------------------------------------------------------------------
+
+struct NoRowK {
+};
 
 // A limb map: job (o, l) reads limb in_limb[l] of outer item o and writes
 // limb out_limb[l]; prime[l]; the inverse's final scale is N^-1 times the
@@ -966,31 +1157,59 @@ struct MapSeg {
     uint8_t in_limb[FHE_MAXP], out_limb[FHE_MAXP], prime[FHE_MAXP];
 };
 
+struct MapSt {
+    const u64 *in;
+    u64 *out;
+    int prime;
+};
+
+struct MapCSt : MapSt {
+    ulonglong2 fs;
+};
+
+template <class Io>
+__device__ __forceinline__ void map_begin(const Io &io, int sg, int job, MapSt &t, int *o_, int *l_)
+{
+    const SegHdr &H = io.h[sg];
+    const MapSeg &S = io.s[sg];
+    const int N = 1 << H.logN, o = job / H.nl, l = job % H.nl;
+    t.in = S.in + o * S.in_outer + (long long)S.in_limb[l] * N;
+    t.out = S.out + o * S.out_outer + (long long)S.out_limb[l] * N;
+    t.prime = S.prime[l];
+    *o_ = o;
+    *l_ = l;
+}
+
 struct IOMap : SegIO<MapSeg> {
-    struct St {
-        const u64 *in;
-        u64 *out;
-        ulonglong2 fs;
-        int prime;
-    };
-    __device__ void begin(int sg, int job, St &t) const
+    static constexpr int DIRS = DIR_FWD | DIR_INV;
+    using CSt = MapCSt;
+    using RSt = MapSt;
+    using RowK = NoRowK;
+    __device__ void begin_c(int sg, int job, CSt &t) const
     {
-        const SegHdr &H = h[sg];
-        const MapSeg &S = s[sg];
-        const int N = 1 << H.logN, o = job / H.nl, l = job % H.nl;
-        t.in = S.in + o * S.in_outer + (long long)S.in_limb[l] * N;
-        t.out = S.out + o * S.out_outer + (long long)S.out_limb[l] * N;
-        t.prime = S.prime[l];
-        t.fs = S.scale ? S.scale[l] : H.ninv[t.prime];
+        int o, l;
+        map_begin(*this, sg, job, t, &o, &l);
+        t.fs = s[sg].scale ? s[sg].scale[l] : h[sg].ninv[t.prime];
     }
-    __device__ u64 load(const St &t, int i) const { return t.in[i]; }
-    __device__ void store(const St &t, int i, u64 v) const { t.out[i] = v; }
-    static constexpr int NPRE = 0;   // operands the store reads
-    static constexpr int LDCH = 16;  // loads staged per chunk (0: not staged)
-    __device__ u64 pre(const St &, int, int) const { return 0; }
-    __device__ void store_pre(const St &t, int i, u64 v, const u64 *) const { t.out[i] = v; }
-    __device__ u64 *inter(const St &t) const { return t.out; }
-    __device__ ulonglong2 final_scale(const St &t) const { return t.fs; }
+    __device__ void begin_r(int sg, int job, RSt &t) const
+    {
+        int o, l;
+        map_begin(*this, sg, job, t, &o, &l);
+    }
+    __device__ RowK row_k(int, int) const { return {}; }
+    static constexpr bool PLAIN = true;  // a column pass loads src's words as they are
+    __device__ const u64 *src(const CSt &t) const { return t.in; }
+    __device__ u64 load(const CSt &t, int i) const { return t.in[i]; }
+    __device__ void load_async(u64 *dst, const RSt &t, int i) const { async8(dst, t.in + i); }
+    __device__ void store(const CSt &t, int i, u64 v) const { t.out[i] = v; }
+    static constexpr int NPRE = 0;  // operands the store reads
+    __device__ u64 pre(const RSt &, int, int) const { return 0; }
+    __device__ void store_pre(const RowK &, const ModQ &m, const RSt &t, int i, u64 v, const u64 *) const
+    {
+        t.out[i] = reduce2q(reduce_few(v, m), m.q);
+    }
+    __device__ u64 *inter(const MapSt &t) const { return t.out; }
+    __device__ ulonglong2 final_scale(const CSt &t) const { return t.fs; }
 };
 
 // A scaled inverse whose last map entry (limb l-1 of the relinearisation
@@ -1003,41 +1222,58 @@ struct YSeg : MapSeg {
     u64 Pm, Pm_s, qm;
 };
 
+struct YRSt : MapSt {
+    const u64 *add;
+    u64 Pm, Pm_s, qm;
+};
+
 struct IOScaledY : SegIO<YSeg> {
-    struct St {
-        const u64 *in, *add;
-        u64 *out;
-        ulonglong2 fs;
-        u64 Pm, Pm_s, qm;
-        int prime;
-    };
-    __device__ void begin(int sg, int job, St &t) const
+    static constexpr int DIRS = DIR_INV;
+    using CSt = MapCSt;
+    using RSt = YRSt;
+    __device__ void begin_c(int sg, int job, CSt &t) const
     {
-        const SegHdr &H = h[sg];
+        int o, e;
+        map_begin(*this, sg, job, t, &o, &e);
+        t.fs = s[sg].scale[e];
+    }
+    __device__ void begin_r(int sg, int job, RSt &t) const
+    {
+        int o, e;
+        map_begin(*this, sg, job, t, &o, &e);
         const YSeg &S = s[sg];
-        const int N = 1 << H.logN, o = job / H.nl, e = job % H.nl, pi = o & 1;
+        const int N = 1 << h[sg].logN, pi = o & 1;
         const long long c = o >> 1;
-        t.in = S.in + o * S.in_outer + (long long)S.in_limb[e] * N;
-        t.out = S.out + o * S.out_outer + (long long)S.out_limb[e] * N;
-        t.prime = S.prime[e];
-        t.fs = S.scale[e];
-        t.add = (e == H.nl - 1 && ((S.amask >> pi) & 1)) ? S.abase + c * S.a_outer + pi * S.a_poly + (long long)S.alimb * N
-                                                          : nullptr;
+        t.add = (e == h[sg].nl - 1 && ((S.amask >> pi) & 1))
+                    ? S.abase + c * S.a_outer + pi * S.a_poly + (long long)S.alimb * N
+                    : nullptr;
         t.Pm = S.Pm;
         t.Pm_s = S.Pm_s;
         t.qm = S.qm;
     }
-    __device__ u64 load(const St &t, int i) const
+    // the y entry (a unit's jobs are all of one entry) is computed on the way
+    __device__ void load_async(u64 *dst, const RSt &t, int i) const
     {
-        return t.add ? addmod(t.in[i], shoup(t.add[i], t.Pm, t.Pm_s, t.qm), t.qm) : t.in[i];
+        if (t.add)  // an accumulator below 2q and a product below q
+            *dst = t.in[i] + shoup(t.add[i], t.Pm, t.Pm_s, t.qm);
+        else
+            async8(dst, t.in + i);
     }
-    __device__ void store(const St &t, int i, u64 v) const { t.out[i] = v; }
+    __device__ void store(const CSt &t, int i, u64 v) const { t.out[i] = v; }
     static constexpr int NPRE = 0;
-    static constexpr int LDCH = 16;
-    __device__ u64 pre(const St &, int, int) const { return 0; }
-    __device__ void store_pre(const St &t, int i, u64 v, const u64 *) const { t.out[i] = v; }
-    __device__ u64 *inter(const St &t) const { return t.out; }
-    __device__ ulonglong2 final_scale(const St &t) const { return t.fs; }
+    __device__ u64 *inter(const MapSt &t) const { return t.out; }
+    __device__ ulonglong2 final_scale(const CSt &t) const { return t.fs; }
+};
+
+struct ConvCSt {
+    Conv cv;
+    int prime;
+};
+
+// a row pass that reads and writes one limb
+struct DstRSt {
+    u64 *out;
+    int prime;
 };
 
 // ModUp: extended limb t of digit j of ct c:  y = sum_a t_a (Q_j/q_a) mod r,
@@ -1052,62 +1288,57 @@ struct ModUpSeg {
 };
 
 struct IOModUp : SegIO<ModUpSeg> {
-    struct St {
-        const u64 *src;
-        u64 *dst;
-        int nsrc, prime, N, pad;
-        ModQ mt;
-        u64 hat[FHE_MAXK];
-    };
-    __device__ void begin(int sg, int job, St &t) const
+    using CSt = ConvCSt;
+    using RSt = DstRSt;
+    using RowK = NoRowK;
+    __device__ u64 *target(int sg, int job, int *entry) const
     {
         const SegHdr &H = h[sg];
         const ModUpSeg &S = s[sg];
-        const int N = 1 << H.logN, c = job / H.nl, e = job % H.nl;
-        const ModUpParams *P = S.P;
-        const int j = P->job_digit[e], tg = P->job_tgt[e];
-        const int lo = P->digit_lo[j];
-        t.nsrc = P->digit_n[j];
-        t.N = N;
-        t.src = S.d2c + ((long long)c * S.l + lo) * N;
-        t.dst = S.ext + (((long long)c * S.dnum + j) * (S.l + S.K) + tg) * N;
-        t.prime = P->job_prime[e];
-        t.mt = H.mq[t.prime];
-#pragma unroll
-        for (int a = 0; a < FHE_MAXK; a++)
-            if (a < t.nsrc) t.hat[a] = P->hat[j][a][tg];
+        const int c = job / H.nl, e = job % H.nl;
+        *entry = e;
+        return S.ext + (((long long)c * S.dnum + S.P->job_digit[e]) * (S.l + S.K) + S.P->job_tgt[e] << H.logN);
     }
-    __device__ u64 load(const St &t, int n) const
+    __device__ void begin_c(int sg, int job, CSt &t) const
     {
-        u128 acc = 0;
+        const ModUpSeg &S = s[sg];
+        const ModUpParams *P = S.P;
+        int e;
+        t.cv.dst = target(sg, job, &e);
+        const int j = P->job_digit[e], tg = P->job_tgt[e];
+        t.cv.n = P->digit_n[j];
+        t.cv.src = S.d2c + ((long long)(job / h[sg].nl) * S.l + P->digit_lo[j] << h[sg].logN);
+        t.prime = t.cv.prime = P->job_prime[e];
 #pragma unroll
         for (int a = 0; a < FHE_MAXK; a++)
-            if (a < t.nsrc) acc += (u128)t.src[(long long)a * t.N + n] * t.hat[a];
-        return conv_reduce(acc, t.mt);
+            if (a < t.cv.n) t.cv.c[a] = P->hat[j][a][tg];
     }
+    __device__ void begin_r(int sg, int job, RSt &t) const
+    {
+        int e;
+        t.out = target(sg, job, &e);
+        t.prime = s[sg].P->job_prime[e];
+    }
+    __device__ RowK row_k(int, int) const { return {}; }
+    __device__ u64 load(int sg, const CSt &t, int N, int n) const { return conv_one(t.cv, h[sg].mq[t.prime], N, n); }
     // two targets of one digit (same sources): each source word loaded once
     static constexpr int XJ = 2;
-    __device__ bool same_src(const St &a, const St &b) const { return a.src == b.src && a.nsrc == b.nsrc; }
-    __device__ void load2(const St &a, const St &b, int n, u64 &v0, u64 &v1) const
-    {
-        u128 s0 = 0, s1 = 0;
-#pragma unroll
-        for (int i = 0; i < FHE_MAXK; i++)
-            if (i < a.nsrc) {
-                const u64 x = a.src[(long long)i * a.N + n];
-                s0 += (u128)x * a.hat[i];
-                s1 += (u128)x * b.hat[i];
-            }
-        v0 = conv_reduce(s0, a.mt);
-        v1 = conv_reduce(s1, b.mt);
-    }
-    __device__ void store(const St &t, int k, u64 v) const { t.dst[k] = v; }
+    __device__ bool same_src(const CSt &a, const CSt &b) const { return a.cv.src == b.cv.src && a.cv.n == b.cv.n; }
     static constexpr int NPRE = 0;
-    static constexpr int LDCH = FHE_NTT_MULTI_LDCH;  // each load reads several limbs
-    __device__ u64 pre(const St &, int, int) const { return 0; }
-    __device__ void store_pre(const St &t, int k, u64 v, const u64 *) const { t.dst[k] = v; }
-    __device__ u64 *inter(const St &t) const { return t.dst; }
-    __device__ ulonglong2 final_scale(const St &) const { return make_ulonglong2(0, 0); }
+    __device__ u64 pre(const RSt &, int, int) const { return 0; }
+    __device__ void store_pre(const RowK &, const ModQ &m, const RSt &t, int k, u64 v, const u64 *) const
+    {
+        t.out[k] = reduce2q(reduce_few(v, m), m.q);
+    }
+    __device__ u64 *inter(const CSt &t) const { return t.cv.dst; }
+    __device__ u64 *inter(const RSt &t) const { return t.out; }
+};
+
+// a row pass whose store combines the transform with an operand or two
+struct DownRSt {
+    const u64 *x, *add;
+    u64 *out;
+    int prime;
 };
 
 // ModDown of poly pi of ct c, data limb i:
@@ -1125,77 +1356,45 @@ struct ModDownSeg {
 };
 
 struct IOModDown : SegIO<ModDownSeg> {
-    struct St {
-        const u64 *w, *acc, *add;
-        u64 *out;
-        int prime, K, N, pad;
-        ModQ mi;
-        u64 pinv, pinv_s;
-        u64 phat[FHE_MAXK];
+    using CSt = ConvCSt;
+    using RSt = DownRSt;
+    struct RowK {
+        DotC pinv;
     };
-    __device__ void begin(int sg, int job, St &t) const
+    __device__ void begin_c(int sg, int job, CSt &t) const
     {
-        const SegHdr &H = h[sg];
         const ModDownSeg &S = s[sg];
-        const int N = 1 << H.logN, l = S.l, K = S.K;
-        const int c = job / (2 * l), pi = (job / l) % 2, i = job % l;
-        t.w = S.accP + ((long long)c * 2 + pi) * K * N;
-        t.acc = S.acc + (((long long)c * 2 + pi) * (l + K) + i) * N;
-        t.add = ((S.amask >> pi) & 1) ? S.abase + c * S.a_outer + pi * S.a_poly + (long long)i * N : nullptr;
-        t.out = S.out + (((long long)c * 2 + pi) * l + i) * N;
-        t.prime = i;
-        t.K = K;
-        t.N = N;
-        t.mi = H.mq[i];
-        t.pinv = S.P->pinv[i];
-        t.pinv_s = S.P->pinv_s[i];
+        const int logN = h[sg].logN, o = job / S.l, i = job % S.l;
+        t.cv.src = S.accP + ((long long)o * S.K << logN);
+        t.cv.dst = S.out + ((long long)job << logN);
+        t.cv.n = S.K;
+        t.prime = t.cv.prime = i;
 #pragma unroll
         for (int k = 0; k < FHE_MAXK; k++)
-            if (k < K) t.phat[k] = S.P->phat[k][i];
+            if (k < S.K) t.cv.c[k] = S.P->phat[k][i];
     }
-    __device__ u64 load(const St &t, int n) const
+    __device__ void begin_r(int sg, int job, RSt &t) const
     {
-        u128 a = 0;
-#pragma unroll
-        for (int k = 0; k < FHE_MAXK; k++)
-            if (k < t.K) a += (u128)t.w[(long long)k * t.N + n] * t.phat[k];
-        return conv_reduce(a, t.mi);
+        const ModDownSeg &S = s[sg];
+        const int logN = h[sg].logN, o = job / S.l, i = job % S.l, c = o >> 1, pi = o & 1;
+        t.x = S.acc + ((long long)o * (S.l + S.K) + i << logN);
+        t.add = ((S.amask >> pi) & 1) ? S.abase + c * S.a_outer + pi * S.a_poly + ((long long)i << logN) : nullptr;
+        t.out = S.out + ((long long)job << logN);
+        t.prime = i;
     }
+    __device__ RowK row_k(int sg, int i) const { return RowK{s[sg].P->pinv[i]}; }
+    __device__ u64 load(int sg, const CSt &t, int N, int n) const { return conv_one(t.cv, h[sg].mq[t.prime], N, n); }
     // two data limbs of one (ct, poly): the special limbs loaded once
     static constexpr int XJ = 2;
-    __device__ bool same_src(const St &a, const St &b) const { return a.w == b.w && a.K == b.K; }
-    __device__ void load2(const St &a, const St &b, int n, u64 &v0, u64 &v1) const
-    {
-        u128 s0 = 0, s1 = 0;
-#pragma unroll
-        for (int k = 0; k < FHE_MAXK; k++)
-            if (k < a.K) {
-                const u64 x = a.w[(long long)k * a.N + n];
-                s0 += (u128)x * a.phat[k];
-                s1 += (u128)x * b.phat[k];
-            }
-        v0 = conv_reduce(s0, a.mi);
-        v1 = conv_reduce(s1, b.mi);
-    }
-    __device__ void store(const St &t, int k, u64 v) const
-    {
-        const u64 q = t.mi.q;
-        u64 r = shoup(submod(t.acc[k], v, q), t.pinv, t.pinv_s, q);
-        if (t.add) r = addmod(r, t.add[k], q);
-        t.out[k] = r;
-    }
+    __device__ bool same_src(const CSt &a, const CSt &b) const { return a.cv.src == b.cv.src && a.cv.n == b.cv.n; }
     static constexpr int NPRE = 2;  // accumulator, addend
-    static constexpr int LDCH = 16;
-    __device__ u64 pre(const St &t, int k, int w) const { return w == 0 ? t.acc[k] : (t.add ? t.add[k] : 0); }
-    __device__ void store_pre(const St &t, int k, u64 v, const u64 *pv) const
+    __device__ u64 pre(const RSt &t, int k, int w) const { return w == 0 ? t.x[k] : (t.add ? t.add[k] : 0); }
+    __device__ void store_pre(const RowK &K, const ModQ &m, const RSt &t, int k, u64 v, const u64 *pv) const
     {
-        const u64 q = t.mi.q;
-        u64 r = shoup(submod(pv[0], v, q), t.pinv, t.pinv_s, q);
-        if (t.add) r = addmod(r, pv[1], q);
-        t.out[k] = r;
+        t.out[k] = addmod(scaled1(lazy_diff(pv[0], v, m), K.pinv, m), pv[1], m.q);
     }
-    __device__ u64 *inter(const St &t) const { return t.out; }
-    __device__ ulonglong2 final_scale(const St &) const { return make_ulonglong2(0, 0); }
+    __device__ u64 *inter(const CSt &t) const { return t.cv.dst; }
+    __device__ u64 *inter(const RSt &t) const { return t.out; }
 };
 
 // Modulus switch l -> l-1 of poly pi of ct c, limb i < l-1:
@@ -1211,41 +1410,53 @@ struct SwitchSeg {
     int l, npoly;
 };
 
+struct SwitchRowK {
+    DotC inv;
+};
+
 struct IOModSwitch : SegIO<SwitchSeg> {
-    struct St {
-        const u64 *last, *in;
+    struct CSt {
+        const u64 *last;
         u64 *out;
-        int prime, pad;
-        u64 q, pi, pis, qi, qis;
+        u64 nq, pi, pis;
+        int prime;
     };
-    __device__ void begin(int sg, int job, St &t) const
+    using RSt = DownRSt;
+    using RowK = SwitchRowK;
+    __device__ void begin_c(int sg, int job, CSt &t) const
     {
-        const SegHdr &H = h[sg];
         const SwitchSeg &S = s[sg];
-        const int N = 1 << H.logN, l = S.l, np = S.npoly;
-        const int c = job / (np * (l - 1)), pi = (job / (l - 1)) % np, i = job % (l - 1);
-        t.last = S.last + ((long long)c * np + pi) * N;
-        t.in = S.in + (((long long)c * np + pi) * l + i) * N;
-        t.out = S.out + (((long long)c * np + pi) * (l - 1) + i) * N;
+        const int logN = h[sg].logN, o = job / (S.l - 1), i = job % (S.l - 1);
+        t.last = S.last + ((long long)o << logN);
+        t.out = S.out + ((long long)job << logN);
         t.prime = i;
-        t.q = H.mq[i].q;
+        t.nq = 0 - h[sg].mq[i].q;
         t.pi = S.P->p_i[i];
         t.pis = S.P->p_i_s[i];
-        t.qi = S.P->qinv[i];
-        t.qis = S.P->qinv_s[i];
     }
-    // [0, 4q): feeds the forward transform
-    __device__ u64 load(const St &t, int n) const { return shoup_lazy4_chain(t.last[n], t.pi, t.pis, 0 - t.q); }
-    __device__ void store(const St &t, int k, u64 v) const { t.out[k] = shoup(submod(t.in[k], v, t.q), t.qi, t.qis, t.q); }
-    static constexpr int NPRE = 1;  // the limb being switched
-    static constexpr int LDCH = 16;
-    __device__ u64 pre(const St &t, int k, int) const { return t.in[k]; }
-    __device__ void store_pre(const St &t, int k, u64 v, const u64 *pv) const
+    __device__ void begin_r(int sg, int job, RSt &t) const
     {
-        t.out[k] = shoup(submod(pv[0], v, t.q), t.qi, t.qis, t.q);
+        const SwitchSeg &S = s[sg];
+        const int logN = h[sg].logN, o = job / (S.l - 1), i = job % (S.l - 1);
+        t.x = S.in + ((long long)o * S.l + i << logN);
+        t.add = nullptr;
+        t.out = S.out + ((long long)job << logN);
+        t.prime = i;
     }
-    __device__ u64 *inter(const St &t) const { return t.out; }
-    __device__ ulonglong2 final_scale(const St &) const { return make_ulonglong2(0, 0); }
+    __device__ RowK row_k(int sg, int i) const { return RowK{s[sg].P->qinv[i]}; }
+    // a column pass's word is p w, in [0, 4q)
+    static constexpr bool PLAIN = false;
+    __device__ const u64 *src(const CSt &t) const { return t.last; }
+    __device__ u64 conv(const CSt &t, u64 v) const { return shoup_lazy4_chain(v, t.pi, t.pis, t.nq); }
+    __device__ u64 load(const CSt &t, int n) const { return conv(t, t.last[n]); }
+    static constexpr int NPRE = 1;  // the limb being switched
+    __device__ u64 pre(const RSt &t, int k, int) const { return t.x[k]; }
+    __device__ void store_pre(const RowK &K, const ModQ &m, const RSt &t, int k, u64 v, const u64 *pv) const
+    {
+        t.out[k] = scaled1(lazy_diff(pv[0], v, m), K.inv, m);
+    }
+    __device__ u64 *inter(const CSt &t) const { return t.out; }
+    __device__ u64 *inter(const RSt &t) const { return t.out; }
 };
 
 // Relinearisation fused with the modulus switch that follows it (l -> l-1)
@@ -1253,7 +1464,8 @@ struct IOModSwitch : SegIO<SwitchSeg> {
 //   correction_i = sum_{k<K} t_k h[k][i] + w h[K][i] (coefficient domain),
 //   out_i = (acc_i P^-1 + add_i - NTT(correction)_i) q_{l-1}^-1,
 // where src holds t_0..t_{K-1} (the special limbs, already scaled) and w.
-// Job = (c, pi) * (l-1) + i.
+// The store is one two-term sum: acc_i (P q_{l-1})^-1 + (add_i -
+// NTT(correction)_i) q_{l-1}^-1.  Job = (c, pi) * (l-1) + i.
 struct RelinMSSeg {
     const u64 *src;  // [count][2][K+1][N] coefficient domain
     const u64 *acc;  // [count][2][l+K][N] NTT domain
@@ -1265,75 +1477,45 @@ struct RelinMSSeg {
 };
 
 struct IORelinMS : SegIO<RelinMSSeg> {
-    struct St {
-        const u64 *w, *acc, *add;
-        u64 *out;
-        int prime, K, N, pad;
-        ModQ mi;
-        u64 pinv, pinv_s, qminv, qminv_s;
-        u64 h[FHE_MAXK];
+    using CSt = ConvCSt;
+    using RSt = DownRSt;
+    struct RowK {
+        DotC a, d;
     };
-    __device__ void begin(int sg, int job, St &t) const
+    __device__ void begin_c(int sg, int job, CSt &t) const
     {
-        const SegHdr &H = h[sg];
         const RelinMSSeg &S = s[sg];
-        const int N = 1 << H.logN, l = S.l, K = S.K, m = l - 1;
-        const int c = job / (2 * m), pi = (job / m) % 2, i = job % m;
-        t.w = S.src + ((long long)c * 2 + pi) * (K + 1) * N;
-        t.acc = S.acc + (((long long)c * 2 + pi) * (l + K) + i) * N;
-        t.add = ((S.amask >> pi) & 1) ? S.abase + c * S.a_outer + pi * S.a_poly + (long long)i * N : nullptr;
-        t.out = S.out + (((long long)c * 2 + pi) * m + i) * N;
-        t.prime = i;
-        t.K = K;
-        t.N = N;
-        t.mi = H.mq[i];
-        t.pinv = S.P->pinv[i];
-        t.pinv_s = S.P->pinv_s[i];
-        t.qminv = S.P->qminv[i];
-        t.qminv_s = S.P->qminv_s[i];
+        const int logN = h[sg].logN, m = S.l - 1, o = job / m, i = job % m;
+        t.cv.src = S.src + ((long long)o * (S.K + 1) << logN);
+        t.cv.dst = S.out + ((long long)job << logN);
+        t.cv.n = S.K + 1;
+        t.prime = t.cv.prime = i;
 #pragma unroll
         for (int k = 0; k < FHE_MAXK; k++)
-            if (k <= K) t.h[k] = S.P->h[k][i];
+            if (k <= S.K) t.cv.c[k] = S.P->h[k][i];
     }
-    // K + 1 <= FHE_MAXK products of canonical residues: below 2^(2b+3)
-    __device__ u64 load(const St &t, int n) const
+    __device__ void begin_r(int sg, int job, RSt &t) const
     {
-        u128 a = 0;
-#pragma unroll
-        for (int k = 0; k < FHE_MAXK; k++)
-            if (k <= t.K) a += (u128)t.w[(long long)k * t.N + n] * t.h[k];
-        return conv_reduce(a, t.mi);
+        const RelinMSSeg &S = s[sg];
+        const int logN = h[sg].logN, m = S.l - 1, o = job / m, i = job % m, c = o >> 1, pi = o & 1;
+        t.x = S.acc + ((long long)o * (S.l + S.K) + i << logN);
+        t.add = ((S.amask >> pi) & 1) ? S.abase + c * S.a_outer + pi * S.a_poly + ((long long)i << logN) : nullptr;
+        t.out = S.out + ((long long)job << logN);
+        t.prime = i;
     }
+    __device__ RowK row_k(int sg, int i) const { return RowK{s[sg].P->pqinv[i], s[sg].P->qminv[i]}; }
+    __device__ u64 load(int sg, const CSt &t, int N, int n) const { return conv_one(t.cv, h[sg].mq[t.prime], N, n); }
     // two data limbs of one (ct, poly): the K + 1 sources loaded once
     static constexpr int XJ = 2;
-    __device__ bool same_src(const St &a, const St &b) const { return a.w == b.w && a.K == b.K; }
-    __device__ void load2(const St &a, const St &b, int n, u64 &v0, u64 &v1) const
-    {
-        u128 s0 = 0, s1 = 0;
-#pragma unroll
-        for (int k = 0; k < FHE_MAXK; k++)
-            if (k <= a.K) {
-                const u64 x = a.w[(long long)k * a.N + n];
-                s0 += (u128)x * a.h[k];
-                s1 += (u128)x * b.h[k];
-            }
-        v0 = conv_reduce(s0, a.mi);
-        v1 = conv_reduce(s1, b.mi);
-    }
-    __device__ u64 combine(const St &t, u64 accv, u64 addv, u64 v) const
-    {
-        const u64 q = t.mi.q;
-        u64 r = shoup(accv, t.pinv, t.pinv_s, q);
-        if (t.add) r = addmod(r, addv, q);
-        return shoup(submod(r, v, q), t.qminv, t.qminv_s, q);
-    }
-    __device__ void store(const St &t, int k, u64 v) const { t.out[k] = combine(t, t.acc[k], t.add ? t.add[k] : 0, v); }
+    __device__ bool same_src(const CSt &a, const CSt &b) const { return a.cv.src == b.cv.src && a.cv.n == b.cv.n; }
     static constexpr int NPRE = 2;  // accumulator, addend
-    static constexpr int LDCH = FHE_NTT_MULTI_LDCH;  // each load reads several limbs
-    __device__ u64 pre(const St &t, int k, int w) const { return w == 0 ? t.acc[k] : (t.add ? t.add[k] : 0); }
-    __device__ void store_pre(const St &t, int k, u64 v, const u64 *pv) const { t.out[k] = combine(t, pv[0], pv[1], v); }
-    __device__ u64 *inter(const St &t) const { return t.out; }
-    __device__ ulonglong2 final_scale(const St &) const { return make_ulonglong2(0, 0); }
+    __device__ u64 pre(const RSt &t, int k, int w) const { return w == 0 ? t.x[k] : (t.add ? t.add[k] : 0); }
+    __device__ void store_pre(const RowK &K, const ModQ &m, const RSt &t, int k, u64 v, const u64 *pv) const
+    {
+        t.out[k] = scaled2(pv[0], K.a, lazy_diff(pv[1], v, m), K.d, m);
+    }
+    __device__ u64 *inter(const CSt &t) const { return t.cv.dst; }
+    __device__ u64 *inter(const RSt &t) const { return t.out; }
 };
 
 // k modulus switches at once (l -> l-k), poly pi of ct c, kept limb i < l-k:
@@ -1348,70 +1530,43 @@ struct MultiSeg {
 };
 
 struct IOMultiSwitch : SegIO<MultiSeg> {
-    struct St {
-        const u64 *w, *in;
-        u64 *out;
-        int prime, k, N, pad;
-        ModQ mi;
-        u64 dinv, dinv_s;
-        u64 g[FHE_MAXK];
-    };
-    __device__ void begin(int sg, int job, St &t) const
+    using CSt = ConvCSt;
+    using RSt = DownRSt;
+    using RowK = SwitchRowK;
+    __device__ void begin_c(int sg, int job, CSt &t) const
     {
-        const SegHdr &H = h[sg];
         const MultiSeg &S = s[sg];
-        const int N = 1 << H.logN, kept = S.l - S.k, np = S.npoly;
-        const int c = job / (np * kept), pi = (job / kept) % np, i = job % kept;
-        t.w = S.src + ((long long)c * np + pi) * S.k * N;
-        t.in = S.in + (((long long)c * np + pi) * S.l + i) * N;
-        t.out = S.out + (((long long)c * np + pi) * kept + i) * N;
-        t.prime = i;
-        t.k = S.k;
-        t.N = N;
-        t.mi = H.mq[i];
-        t.dinv = S.P->Dinv[i];
-        t.dinv_s = S.P->Dinv_s[i];
+        const int logN = h[sg].logN, kept = S.l - S.k, o = job / kept, i = job % kept;
+        t.cv.src = S.src + ((long long)o * S.k << logN);
+        t.cv.dst = S.out + ((long long)job << logN);
+        t.cv.n = S.k;
+        t.prime = t.cv.prime = i;
 #pragma unroll
         for (int j = 0; j < FHE_MAXK; j++)
-            if (j < S.k) t.g[j] = S.P->G[j][i];
+            if (j < S.k) t.cv.c[j] = S.P->G[j][i];
     }
-    __device__ u64 load(const St &t, int n) const
+    __device__ void begin_r(int sg, int job, RSt &t) const
     {
-        u128 a = 0;
-#pragma unroll
-        for (int j = 0; j < FHE_MAXK; j++)
-            if (j < t.k) a += (u128)t.w[(long long)j * t.N + n] * t.g[j];
-        return conv_reduce(a, t.mi);
+        const MultiSeg &S = s[sg];
+        const int logN = h[sg].logN, kept = S.l - S.k, o = job / kept, i = job % kept;
+        t.x = S.in + ((long long)o * S.l + i << logN);
+        t.add = nullptr;
+        t.out = S.out + ((long long)job << logN);
+        t.prime = i;
     }
+    __device__ RowK row_k(int sg, int i) const { return RowK{s[sg].P->Dinv[i]}; }
+    __device__ u64 load(int sg, const CSt &t, int N, int n) const { return conv_one(t.cv, h[sg].mq[t.prime], N, n); }
     // two kept limbs of one (ct, poly): the k switch values loaded once
     static constexpr int XJ = 2;
-    __device__ bool same_src(const St &a, const St &b) const { return a.w == b.w && a.k == b.k; }
-    __device__ void load2(const St &a, const St &b, int n, u64 &v0, u64 &v1) const
-    {
-        u128 s0 = 0, s1 = 0;
-#pragma unroll
-        for (int j = 0; j < FHE_MAXK; j++)
-            if (j < a.k) {
-                const u64 x = a.w[(long long)j * a.N + n];
-                s0 += (u128)x * a.g[j];
-                s1 += (u128)x * b.g[j];
-            }
-        v0 = conv_reduce(s0, a.mi);
-        v1 = conv_reduce(s1, b.mi);
-    }
-    __device__ void store(const St &t, int j, u64 v) const
-    {
-        t.out[j] = shoup(submod(t.in[j], v, t.mi.q), t.dinv, t.dinv_s, t.mi.q);
-    }
+    __device__ bool same_src(const CSt &a, const CSt &b) const { return a.cv.src == b.cv.src && a.cv.n == b.cv.n; }
     static constexpr int NPRE = 1;
-    static constexpr int LDCH = FHE_NTT_MULTI_LDCH;  // each load reads several limbs
-    __device__ u64 pre(const St &t, int j, int) const { return t.in[j]; }
-    __device__ void store_pre(const St &t, int j, u64 v, const u64 *pv) const
+    __device__ u64 pre(const RSt &t, int j, int) const { return t.x[j]; }
+    __device__ void store_pre(const RowK &K, const ModQ &m, const RSt &t, int j, u64 v, const u64 *pv) const
     {
-        t.out[j] = shoup(submod(pv[0], v, t.mi.q), t.dinv, t.dinv_s, t.mi.q);
+        t.out[j] = scaled1(lazy_diff(pv[0], v, m), K.inv, m);
     }
-    __device__ u64 *inter(const St &t) const { return t.out; }
-    __device__ ulonglong2 final_scale(const St &) const { return make_ulonglong2(0, 0); }
+    __device__ u64 *inter(const CSt &t) const { return t.cv.dst; }
+    __device__ u64 *inter(const RSt &t) const { return t.out; }
 };
 
 // ---------------------------------------------------------------------------
@@ -1442,7 +1597,7 @@ void unit_counts(SegHdr &H)
     const Split sp = split_of(H.logN);
     const int njobs = H.outer * H.nl;
     int nc = std::min(sp.ns1, 1 << sp.n2);
-    if (col_paired(H.xj, sp.n1, sp.ns1, nc)) nc /= 2;  // ColGeo's paired units
+    if (col_paired(H.xj, sp.ns1, nc)) nc /= 2;  // ColGeo's paired units
     const int nj = sp.ns1 / nc, blk = (1 << sp.n2) / nc;
     H.u_cols = ((njobs + nj - 1) / nj) * blk;
     H.u_rows = H.grouped ? H.nl * ((H.outer + ROW_J - 1) / ROW_J) * ((1 << sp.n1) / (sp.ns2 / ROW_J))
@@ -1502,13 +1657,16 @@ void recount(IO &io)
 template <class IO, int LO, int HI>
 void launch_passes(fhe_ctx *c, const IO &io, bool fwd)
 {
-    if (fwd) {
-        launch_pdl(k_fwd_cols<IO, LO, HI>, grid_of(c, io.ucols), T, c->stream, io);
-        launch_pdl(k_fwd_rows<IO, LO, HI>, grid_of(c, io.urows), T, c->stream, io);
-    } else {
-        launch_pdl(k_inv_rows<IO, LO, HI>, grid_of(c, io.urows), T, c->stream, io);
-        launch_pdl(k_inv_cols<IO, LO, HI>, grid_of(c, io.ucols), T, c->stream, io);
-    }
+    if constexpr ((IO::DIRS & DIR_FWD) != 0)
+        if (fwd) {
+            launch_pdl(k_fwd_cols<IO, LO, HI>, grid_of(c, io.ucols), T, c->stream, io);
+            launch_pdl(k_fwd_rows<IO, LO, HI>, grid_of(c, io.urows), T, c->stream, io);
+        }
+    if constexpr ((IO::DIRS & DIR_INV) != 0)
+        if (!fwd) {
+            launch_pdl(k_inv_rows<IO, LO, HI>, grid_of(c, io.urows), T, c->stream, io);
+            launch_pdl(k_inv_cols<IO, LO, HI>, grid_of(c, io.ucols), T, c->stream, io);
+        }
     c->launches += 2;
 }
 

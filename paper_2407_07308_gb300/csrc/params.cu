@@ -210,6 +210,7 @@ int build_tables(fhe_ctx *c)
     c->modup.assign(L + 1, ModUpParams());
     c->moddown.assign(L + 1, ModDownParams());
     c->modswitch.assign(L + 1, ModSwitchParams());
+    std::vector<u64> pinv((size_t)(L + 1) * FHE_MAXP, 0);  // [l][i]: P^-1 mod q_i
     for (int l = 1; l <= L; l++) {
         ModUpParams &U = c->modup[l];
         memset(&U, 0, sizeof(U));
@@ -231,7 +232,7 @@ int build_tables(fhe_ctx *c)
                     u64 tq = c->q[eprime(r)], h = 1;
                     for (int b = 0; b < n; b++)
                         if (b != a) h = host_mulmod(h, c->q[lo + b] % tq, tq);
-                    U.hat[j][a][r] = h;
+                    U.hat[j][a][r] = dot_const(h, c->mq[eprime(r)]);
                 }
             }
             for (int r = 0; r < l + K; r++) {
@@ -258,14 +259,14 @@ int build_tables(fhe_ctx *c)
                 u64 qi = c->q[i], h = c->p % qi;
                 for (int m = 0; m < K; m++)
                     if (m != k) h = host_mulmod(h, c->q[L + m] % qi, qi);
-                D.phat[k][i] = h;
+                D.phat[k][i] = dot_const(h, c->mq[i]);
             }
         }
         for (int i = 0; i < l; i++) {
             u64 qi = c->q[i], P = 1;
             for (int k = 0; k < K; k++) P = host_mulmod(P, c->q[L + k] % qi, qi);
-            D.pinv[i] = host_invmod(P, qi);
-            D.pinv_s[i] = shoup_const(D.pinv[i], qi);
+            pinv[(size_t)l * FHE_MAXP + i] = host_invmod(P, qi);
+            D.pinv[i] = dot_const(pinv[(size_t)l * FHE_MAXP + i], c->mq[i]);
         }
 
         ModSwitchParams &S = c->modswitch[l];
@@ -279,8 +280,7 @@ int build_tables(fhe_ctx *c)
                 u64 qi = c->q[i];
                 S.p_i[i] = c->p % qi;
                 S.p_i_s[i] = shoup_const(S.p_i[i], qi);
-                S.qinv[i] = host_invmod(ql % qi, qi);
-                S.qinv_s[i] = shoup_const(S.qinv[i], qi);
+                S.qinv[i] = dot_const(host_invmod(ql % qi, qi), c->mq[i]);
             }
         }
     }
@@ -302,12 +302,12 @@ int build_tables(fhe_ctx *c)
         R.Pm_s = shoup_const(Pm, qm);
         for (int i = 0; i < l - 1; i++) {
             const u64 qi = c->q[i], pi = c->p % qi;
-            for (int k = 0; k < K; k++) R.h[k][i] = host_mulmod(pi, host_invmod(c->q[L + k] % qi, qi), qi);
-            R.h[K][i] = pi;
-            R.pinv[i] = c->moddown[l].pinv[i];
-            R.pinv_s[i] = c->moddown[l].pinv_s[i];
-            R.qminv[i] = c->modswitch[l].qinv[i];
-            R.qminv_s[i] = c->modswitch[l].qinv_s[i];
+            for (int k = 0; k < K; k++) 
+                R.h[k][i] = dot_const(host_mulmod(pi, host_invmod(c->q[L + k] % qi, qi), qi), c->mq[i]);
+            R.h[K][i] = dot_const(pi, c->mq[i]);
+            const u64 qminv = host_invmod(qm % qi, qi);
+            R.pqinv[i] = dot_const(host_mulmod(pinv[(size_t)l * FHE_MAXP + i], qminv, qi), c->mq[i]);
+            R.qminv[i] = dot_const(qminv, c->mq[i]);
         }
     }
     if ((e = upload(c, (void **)&c->d_rms, c->rms.data(), sizeof(RelinMSParams) * (L + 1)))) return e;
@@ -325,11 +325,10 @@ int build_tables(fhe_ctx *c)
                 const u64 qi = c->q[i];
                 u64 D = 1;
                 for (int t = 0; t < k; t++) {
-                    S.G[t][i] = host_mulmod(c->p % qi, D, qi);
+                    S.G[t][i] = dot_const(host_mulmod(c->p % qi, D, qi), c->mq[i]);
                     D = host_mulmod(D, c->q[l - 1 - t] % qi, qi);
                 }
-                S.Dinv[i] = host_invmod(D, qi);
-                S.Dinv_s[i] = shoup_const(S.Dinv[i], qi);
+                S.Dinv[i] = dot_const(host_invmod(D, qi), c->mq[i]);
             }
             for (int j = 0; j < k; j++) {
                 const u64 qj = c->q[l - 1 - j];
