@@ -86,59 +86,6 @@ __global__ void k_tensor(const u64 *__restrict__ a, const u64 *__restrict__ b, u
     }
 }
 
-// Key-switching inner product.  Extended limb r = blockIdx.y of Q_l P
-// (r < l: data prime r; else special prime L + r - l); ciphertexts
-// blockIdx.z * CB .. + CB - 1 of the batch.  Every thread loads its 2*dnum
-// key words once and reuses them for its CB ciphertexts, whose input words
-// are all loaded before the first product so that the loads overlap.
-template <int CB>
-__global__ void __launch_bounds__(256, 3)
-    k_ks_inner(const u64 *__restrict__ ext, const u64 *__restrict__ xbase, long long x_outer,
-               const u64 *__restrict__ ksk, u64 *__restrict__ acc, int count, int l, int K, int L, int dnum,
-               int logN, const ModQ *__restrict__ mq)
-{
-    const int N = 1 << logN;
-    const int r = blockIdx.y;
-    const int prime = r < l ? r : L + (r - l);
-    const ModQ m = mq[prime];
-    const int LK = L + K, lK = l + K;
-    const int rdig = r < l ? r / K : -1;
-    const int c0 = blockIdx.z * CB;
-    const int ncb = min(CB, count - c0);
-    for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
-        u128 a0[CB], a1[CB];
-#pragma unroll
-        for (int cc = 0; cc < CB; cc++) a0[cc] = a1[cc] = 0;
-        for (int j = 0; j < dnum; j++) {
-            const u64 k0 = ksk[(((long long)j * 2 + 0) * LK + prime) * N + n];
-            const u64 k1 = ksk[(((long long)j * 2 + 1) * LK + prime) * N + n];
-            u64 y[CB];
-#pragma unroll
-            for (int cc = 0; cc < CB; cc++) {
-                const int c = c0 + cc;
-                if (cc < ncb)
-                    y[cc] = (j == rdig) ? xbase[c * x_outer + (long long)r * N + n]
-                                        : ext[(((long long)c * dnum + j) * lK + r) * N + n];
-            }
-#pragma unroll
-            for (int cc = 0; cc < CB; cc++) {
-                if (cc < ncb) {
-                    a0[cc] += (u128)y[cc] * k0;
-                    a1[cc] += (u128)y[cc] * k1;
-                }
-            }
-        }
-#pragma unroll
-        for (int cc = 0; cc < CB; cc++) {
-            const int c = c0 + cc;
-            if (cc < ncb) {
-                acc[(((long long)c * 2 + 0) * lK + r) * N + n] = barrett128(a0[cc], m);
-                acc[(((long long)c * 2 + 1) * lK + r) * N + n] = barrett128(a1[cc], m);
-            }
-        }
-    }
-}
-
 // Relinearisation fused with the modulus switch (the inverse NTT that
 // precedes this step formed y = acc_m + (P mod q_m) add_m while loading):
 // after the scaled inverse NTT of the special limbs and of y, in
@@ -277,10 +224,13 @@ __global__ void k_muladd(const u64 *__restrict__ a, const u64 *__restrict__ b, c
 }
 
 // One digit of a switching key over the L+K primes (NTT domain):
-//   k0 = e - a s + [i in D_j] (P mod q_i) s',  k1 = a.
+//   k0 = e - a s + [i in D_j] (P mod q_i) s',  k1 = a,
+// both stored as the inner product reads them: times 2^(2h) (R) mod q_i, as
+// packed half words (half_const).
 __global__ void k_ksk_digit(const u64 *__restrict__ a, const u64 *__restrict__ e, const u64 *__restrict__ s,
                             const u64 *__restrict__ sp, u64 *__restrict__ k0, u64 *__restrict__ k1, long long total,
-                            int logN, int dlo, int dhi, const LimbConsts Pm, const ModQ *__restrict__ mq)
+                            int logN, int dlo, int dhi, const LimbConsts Pm, const LimbConsts R,
+                            const ModQ *__restrict__ mq)
 {
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -288,8 +238,8 @@ __global__ void k_ksk_digit(const u64 *__restrict__ a, const u64 *__restrict__ e
         const ModQ m = mq[i];
         u64 v = submod(e[idx], barrett128((u128)a[idx] * s[idx], m), m.q);
         if (i >= dlo && i < dhi) v = addmod(v, shoup(sp[idx], Pm.w[i], Pm.ws[i], m.q), m.q);
-        k0[idx] = v;
-        k1[idx] = a[idx];
+        k0[idx] = half_pack(shoup(v, R.w[i], R.ws[i], m.q), m.half);
+        k1[idx] = half_pack(shoup(a[idx], R.w[i], R.ws[i], m.q), m.half);
     }
 }
 
@@ -377,20 +327,6 @@ void launch_tensor(fhe_ctx *c, const u64 *a, const u64 *b, u64 *out, int count, 
            c->d_mq);
 }
 
-void launch_ks_inner(fhe_ctx *c, const u64 *ext, const u64 *xbase, long long x_outer, const u64 *ksk, u64 *acc,
-                     int count, int level)
-{
-    const int dnum = c->modup[level].dnum;
-    constexpr int CB = 4;  // ciphertexts per thread
-    dim3 grid((c->N + TPB - 1) / TPB, level + c->K, (count + CB - 1) / CB);
-    // per (r, n): 2 dnum key words once, dnum inputs and 2 outputs per ciphertext
-    prof_begin(c, FHE_K_KS_INNER, 8.0 * (double)(level + c->K) * c->N * (2.0 * dnum + count * (dnum + 2.0)));
-    k_ks_inner<CB><<<grid, TPB, 0, c->stream>>>(ext, xbase, x_outer, ksk, acc, count, level, c->K, c->L, dnum, c->logN,
-                                            c->d_mq);
-    prof_end(c);
-    c->launches++;
-}
-
 void launch_automorphism(fhe_ctx *c, const u64 *in, u64 *out, int outer, int level, const int *perm)
 {
     LAUNCH_CLS(FHE_K_AUTOMORPHISM, k_automorphism, (long long)outer * level * c->N, in, out, (long long)outer * level * c->N, c->logN, perm);
@@ -449,10 +385,14 @@ void launch_muladd(fhe_ctx *c, const u64 *a, const u64 *b, const u64 *cc, u64 *o
 void launch_ksk_digit(fhe_ctx *c, const u64 *a, const u64 *e, const u64 *s, const u64 *sp, u64 *k0, u64 *k1, int dlo,
                       int dhi, const u64 *Pw, const u64 *Pws)
 {
-    LimbConsts Pm;
-    for (int i = 0; i < c->np; i++) Pm.w[i] = Pw[i], Pm.ws[i] = Pws[i];
+    LimbConsts Pm, R;
+    for (int i = 0; i < c->np; i++) {
+        Pm.w[i] = Pw[i], Pm.ws[i] = Pws[i];
+        R.w[i] = (u64)(((u128)1 << (2 * c->mq[i].half)) % c->q[i]);
+        R.ws[i] = shoup_const(R.w[i], c->q[i]);
+    }
     LAUNCH(k_ksk_digit, (long long)c->np * c->N, a, e, s, sp, k0, k1, (long long)c->np * c->N, c->logN, dlo, dhi, Pm,
-           c->d_mq);
+           R, c->d_mq);
 }
 
 // ---------------------------------------------------------------------------

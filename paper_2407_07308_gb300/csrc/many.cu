@@ -9,6 +9,8 @@
 // single-batch kernels in kernels.cu; only the addressing differs.
 #include <string.h>
 
+#include <algorithm>
+
 #include "fhe_internal.h"
 
 namespace {
@@ -239,6 +241,24 @@ __global__ void k_tensor_many(const __grid_constant__ TensorTable t)
 // digit j, else the ModUp limb.  A block covers TPB coefficients of one
 // extended limb r for CB ciphertexts; each thread loads its 2 dnum key words
 // once for its CB ciphertexts.
+//
+// Bound by the multiplier pipe, and by the loads' round trips where few
+// ciphertexts share a launch.  The key words are stored as packed half words
+// times 2^(2h) (see HalfAcc): a product is three wide multiplications, a sum
+// is reduced by two half-word Montgomery steps.  All of a thread's words come
+// by asynchronous copies into shared memory before its first product.
+// Ciphertexts of items that use the same key at the same level (the products
+// of a wave, the requests of an uneven batch) form one run: their key words
+// are loaded once for CB of them, and a thread multiplies only for the
+// ciphertexts it has (single requests used to multiply for four).
+//
+// Measured per pass (before: 128-bit multiply-adds, one run per item, one
+// digit's words ahead in registers): tournament of 8 ciphertexts, N = 2^15,
+// 36.5 -> 17.7 ms; 7 pairs at N = 2^15 5.80 -> 5.24 ms; 16 pairs at N = 2^14
+// equal (1.53, 1.55 ms).  With the words ahead in registers as before the new
+// arithmetic took 23.6 / 7.6 / 1.84 ms.  Ciphertexts a thread and blocks an
+// SM (16 pairs / 7 pairs / tournament, ms): 4 and 3 as here; 2 and 4 1.81 /
+// 6.14 / 19.2; 3 and 3 1.62 / 5.46 / 18.7; 5 and 2 1.68 / 5.58 / 20.5.
 
 #ifndef FHE_KS_CB
 #define FHE_KS_CB 4
@@ -254,6 +274,7 @@ struct KsSeg {
     const ModQ *mq;
     long long x_outer;
     int count, l, K, L, dnum, logN, b0, nbx;  // nbx: blocks along n
+    int run;  // ciphertexts of the run this item opens (0: the item belongs to an earlier one's)
 };
 
 struct KsTable {
@@ -261,62 +282,129 @@ struct KsTable {
     KsSeg s[FHE_SEGS];
 };
 
+// Digit group g of this thread's copies has arrived once at most `left` later
+// groups are in flight.
+__device__ __forceinline__ void async_wait_left(int left)
+{
+    switch (left) {
+    case 0: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;
+    case 1: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
+    case 2: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
+    case 3: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
+    case 4: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
+    case 5: asm volatile("cp.async.wait_group 5;" ::: "memory"); break;
+    case 6: asm volatile("cp.async.wait_group 6;" ::: "memory"); break;
+    default: asm volatile("cp.async.wait_group 7;" ::: "memory"); break;
+    }
+}
+
+__device__ __forceinline__ void async8(u64 *dst, const u64 *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+// The sums of a thread's ciphertexts (FULL: all KS_CB of them, so that no
+// branch stands between the copies).  own(cc): the ciphertext's word of the
+// digit that holds limb r itself; ep: its ModUp words, advanced digit by
+// digit; out(cc): its two sums.  w: the thread's words in shared memory, TPB
+// apart: the two key words, then the ciphertexts', digit by digit.  Every
+// digit's words are under way before the first product, in registers they
+// would take 12 dnum (one digit ahead, in registers: four round trips to L2
+// one after the other for dnum = 4, which bounded the kernel).
+template <bool FULL, class Own, class Out>
+__device__ __forceinline__ void ks_sum(u64 *w, const u64 *(&ep)[KS_CB], const u64 *kp, long long kstride,
+                                       long long dstride, int rdig, int dnum, int ncb, const ModQ &m, Own own, Out out)
+{
+    const int h = m.half;
+    const uint32_t mask = ((uint32_t)1 << h) - 1;
+    {
+        u64 *d = w;
+        for (int j = 0; j < dnum; j++) {
+            async8(d, kp);
+            async8(d + TPB, kp + kstride);
+#pragma unroll
+            for (int cc = 0; cc < KS_CB; cc++) {
+                if (FULL || cc < ncb) async8(d + (2 + cc) * TPB, j == rdig ? own(cc) : ep[cc]);
+                ep[cc] += dstride;
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            kp += 2 * kstride;
+            d += (2 + KS_CB) * TPB;
+        }
+    }
+    HalfAcc a0[KS_CB], a1[KS_CB];
+#pragma unroll
+    for (int cc = 0; cc < KS_CB; cc++) a0[cc] = a1[cc] = HalfAcc{0, 0, 0};
+    for (int j = 0; j < dnum; j++) {
+        async_wait_left(dnum - 1 - j);
+        const u64 c0 = w[0], c1 = w[TPB];
+        const uint32_t c0l = (uint32_t)c0, c0h = (uint32_t)(c0 >> 32), c0s = c0l + c0h;
+        const uint32_t c1l = (uint32_t)c1, c1h = (uint32_t)(c1 >> 32), c1s = c1l + c1h;
+#pragma unroll
+        for (int cc = 0; cc < KS_CB; cc++)
+            if (FULL || cc < ncb) {
+                const u64 z = w[(2 + cc) * TPB];
+                const uint32_t zl = (uint32_t)z & mask, zh = (uint32_t)(z >> h), zs = zl + zh;
+                half_mac(a0[cc], zl, zh, zs, c0l, c0h, c0s);
+                half_mac(a1[cc], zl, zh, zs, c1l, c1h, c1s);
+            }
+        w += (2 + KS_CB) * TPB;
+    }
+    // in [0, 2q): what reads the sums (the inverse transforms and the stores
+    // of ModDown and of relinearise + switch) takes them
+#pragma unroll
+    for (int cc = 0; cc < KS_CB; cc++)
+        if (FULL || cc < ncb) {
+            u64 *o = out(cc);
+            o[0] = reduce_few(half_mont(a0[cc], m), m);
+            o[dstride] = reduce_few(half_mont(a1[cc], m), m);
+        }
+}
+
 __global__ void __launch_bounds__(TPB, FHE_KS_MINB) k_ks_inner_many(const __grid_constant__ KsTable t)
 {
     pdl_begin();
-    const KsSeg &S = t.s[block_seg(t.s, t.nseg)];
+    extern __shared__ u64 ks_words[];  // [dnum][2 + KS_CB][TPB]
+    const int sg = block_seg(t.s, t.nseg);
+    const KsSeg &S = t.s[sg];
     const int lb = blockIdx.x - S.b0;
     const int lK = S.l + S.K, N = 1 << S.logN;
     const int bx = lb % S.nbx, r = (lb / S.nbx) % lK, cz = lb / (S.nbx * lK);
     const int n = bx * TPB + threadIdx.x;
     if (n >= N) return;
     const int prime = r < S.l ? r : S.L + (r - S.l);
-    const ModQ m = S.mq[prime];
-    const int LK = S.L + S.K;
+    const ModQ &m = S.mq[prime];
     const int rdig = r < S.l ? r / S.K : -1;
-    const int c0 = cz * KS_CB;
-    const int ncb = min(KS_CB, S.count - c0);
-    u128 a0[KS_CB], a1[KS_CB];
-#pragma unroll
-    for (int cc = 0; cc < KS_CB; cc++) a0[cc] = a1[cc] = 0;
-    // digit j's two key words and CB inputs; the next digit's are loaded
-    // before this digit's products (two digits' loads in flight)
-    auto load = [&](int j, u64 &k0, u64 &k1, u64 (&y)[KS_CB]) {
-        k0 = S.ksk[(((long long)j * 2 + 0) * LK + prime) * N + n];
-        k1 = S.ksk[(((long long)j * 2 + 1) * LK + prime) * N + n];
+    const int ncb = min(KS_CB, S.run - cz * KS_CB);
+    // the block's ciphertexts: item and place in it (the run's ciphertexts in
+    // order, over the items from sg on)
+    int it[KS_CB], pl[KS_CB];
+    {
+        int i = sg, c = cz * KS_CB;
 #pragma unroll
         for (int cc = 0; cc < KS_CB; cc++) {
-            const int c = c0 + cc;
-            y[cc] = cc >= ncb ? 0
-                    : (j == rdig) ? S.xbase[c * S.x_outer + (long long)r * N + n]
-                                  : S.ext[(((long long)c * S.dnum + j) * lK + r) * N + n];
-        }
-    };
-    u64 k0, k1, y[KS_CB];
-    load(0, k0, k1, y);
-    for (int j = 0; j < S.dnum; j++) {
-        u64 nk0 = 0, nk1 = 0, ny[KS_CB];
-#pragma unroll
-        for (int cc = 0; cc < KS_CB; cc++) ny[cc] = 0;
-        if (j + 1 < S.dnum) load(j + 1, nk0, nk1, ny);
-#pragma unroll
-        for (int cc = 0; cc < KS_CB; cc++) {
-            a0[cc] += (u128)y[cc] * k0;
-            a1[cc] += (u128)y[cc] * k1;
-        }
-        k0 = nk0;
-        k1 = nk1;
-#pragma unroll
-        for (int cc = 0; cc < KS_CB; cc++) y[cc] = ny[cc];
-    }
-#pragma unroll
-    for (int cc = 0; cc < KS_CB; cc++) {
-        const int c = c0 + cc;
-        if (cc < ncb) {
-            S.acc[(((long long)c * 2 + 0) * lK + r) * N + n] = barrett128(a0[cc], m);
-            S.acc[(((long long)c * 2 + 1) * lK + r) * N + n] = barrett128(a1[cc], m);
+            it[cc] = sg;
+            pl[cc] = 0;
+            if (cc < ncb) {
+                while (c >= t.s[i].count) c -= t.s[i].count, i++;
+                it[cc] = i;
+                pl[cc] = c++;
+            }
         }
     }
+    const u64 *ep[KS_CB];
+#pragma unroll
+    for (int cc = 0; cc < KS_CB; cc++)
+        ep[cc] = t.s[it[cc]].ext + ((long long)pl[cc] * S.dnum * lK + r) * N + n;
+    auto own = [&](int cc) { return t.s[it[cc]].xbase + pl[cc] * t.s[it[cc]].x_outer + (long long)r * N + n; };
+    auto out = [&](int cc) { return t.s[it[cc]].acc + ((long long)pl[cc] * 2 * lK + r) * N + n; };
+    const u64 *kp = S.ksk + (long long)prime * N + n;
+    const long long kstride = (long long)(S.L + S.K) * N, dstride = (long long)lK * N;
+    if (ncb == KS_CB)
+        ks_sum<true>(ks_words + threadIdx.x, ep, kp, kstride, dstride, rdig, S.dnum, ncb, m, own, out);
+    else
+        ks_sum<false>(ks_words + threadIdx.x, ep, kp, kstride, dstride, rdig, S.dnum, ncb, m, own, out);
 }
 
 // ---- folds of the fused relinearise + switch and of the multi-prime switch
@@ -500,31 +588,82 @@ void launch_tensor_many(const std::vector<TensorArgs> &items)
         [](const TensorTable &t, int blocks, cudaStream_t s) { launch_pdl(k_tensor_many, blocks, TPB, s, t); });
 }
 
+// shared memory of a block for dnum digits
+static int ks_bytes(int dnum) { return (int)sizeof(u64) * dnum * (2 + KS_CB) * TPB; }
+
 void launch_ks_inner_many(const std::vector<KsInnerArgs> &items)
 {
-    launch_tables<KsTable>(
-        items, FHE_K_KS_INNER,
-        [](KsSeg &S, const KsInnerArgs &a, double *bytes) {
-            fhe_ctx *c = a.c;
-            if (a.count <= 0) return 0;
-            S.ext = a.ext;
-            S.xbase = a.xbase;
-            S.ksk = a.ksk;
-            S.acc = a.acc;
-            S.mq = c->d_mq;
-            S.x_outer = a.x_outer;
-            S.count = a.count;
-            S.l = a.level;
-            S.K = c->K;
-            S.L = c->L;
-            S.dnum = c->modup[a.level].dnum;
-            S.logN = c->logN;
-            S.nbx = (c->N + TPB - 1) / TPB;
+    // items of one key and level side by side (a run); an item keeps its
+    // place otherwise
+    std::vector<KsInnerArgs> a;
+    std::vector<char> taken(items.size(), 0);
+    for (size_t i = 0; i < items.size(); i++) {
+        if (taken[i] || items[i].count <= 0) continue;
+        for (size_t j = i; j < items.size(); j++)
+            if (!taken[j] && items[j].count > 0 && items[j].c == items[i].c && items[j].ksk == items[i].ksk &&
+                items[j].level == items[i].level) {
+                a.push_back(items[j]);
+                taken[j] = 1;
+            }
+    }
+    for (size_t i = 0; i < a.size();) {
+        KsTable t;
+        memset(&t, 0, sizeof(t));
+        fhe_ctx *c0 = a[i].c;
+        int blocks = 0, dmax = 0;
+        double bytes = 0;
+        while (i < a.size() && t.nseg < FHE_SEGS) {
+            fhe_ctx *c = a[i].c;
+            const int level = a[i].level, dnum = c->modup[level].dnum, lead = t.nseg;
+            const u64 *key = a[i].ksk;
+            dmax = std::max(dmax, dnum);
+            const int b0 = blocks;
+            int run = 0;
+            for (; i < a.size() && t.nseg < FHE_SEGS && a[i].c == c && a[i].ksk == key && a[i].level == level; i++) {
+                KsSeg &S = t.s[t.nseg++];
+                S.ext = a[i].ext;
+                S.xbase = a[i].xbase;
+                S.ksk = key;
+                S.acc = a[i].acc;
+                S.mq = c->d_mq;
+                S.x_outer = a[i].x_outer;
+                S.count = a[i].count;
+                S.l = level;
+                S.K = c->K;
+                S.L = c->L;
+                S.dnum = dnum;
+                S.logN = c->logN;
+                S.nbx = (c->N + TPB - 1) / TPB;
+                run += a[i].count;
+            }
+            blocks += t.s[lead].nbx * (level + c->K) * ((run + KS_CB - 1) / KS_CB);
+            // the items behind the leader own no blocks
+            for (int s = lead; s < t.nseg; s++) t.s[s].b0 = s == lead ? b0 : blocks;
+            t.s[lead].run = run;
             // per (r, n): 2 dnum key words once per CB ciphertexts, dnum inputs and 2 outputs per ciphertext
-            *bytes = 8.0 * (double)(a.level + c->K) * c->N * (2.0 * S.dnum + a.count * (S.dnum + 2.0));
-            return S.nbx * (a.level + c->K) * ((a.count + KS_CB - 1) / KS_CB);
-        },
-        [](const KsTable &t, int blocks, cudaStream_t s) { launch_pdl(k_ks_inner_many, blocks, TPB, s, t); });
+            bytes += 8.0 * (double)(level + c->K) * c->N * (2.0 * dnum + run * (dnum + 2.0));
+        }
+        prof_begin(c0, FHE_K_KS_INNER, bytes);
+        // per device, once: more than 48 KB of dynamic shared memory
+        static std::mutex mu;
+        static bool allowed[64] = {false};
+        {
+            std::lock_guard<std::mutex> g(mu);
+            const int dev = c0->device >= 0 && c0->device < 64 ? c0->device : 0;
+            if (!allowed[dev])
+                allowed[dev] = cudaFuncSetAttribute(k_ks_inner_many, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    ks_bytes(FHE_MAXD)) == cudaSuccess;
+        }
+        launch_pdl_smem(k_ks_inner_many, blocks, TPB, ks_bytes(dmax), c0->stream, t);
+        prof_end(c0);
+        c0->launches++;
+    }
+}
+
+void launch_ks_inner(fhe_ctx *c, const u64 *ext, const u64 *xbase, long long x_outer, const u64 *ksk, u64 *acc,
+                     int count, int level)
+{
+    launch_ks_inner_many({KsInnerArgs{c, ext, xbase, x_outer, ksk, acc, count, level}});
 }
 
 void launch_rms_fold_many(const std::vector<FoldArgs> &items)

@@ -30,13 +30,13 @@ __device__ __forceinline__ void pdl_begin()
 }
 
 template <class... KArgs, class... Args>
-inline void launch_pdl(void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args &&...args)
+inline void launch_pdl_smem(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, Args &&...args)
 {
 #if FHE_PDL
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -45,6 +45,12 @@ inline void launch_pdl(void (*kernel)(KArgs...), int grid, int block, cudaStream
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);  // errors surface in cudaGetLastError
 #else
-    kernel<<<grid, block, 0, s>>>(std::forward<Args>(args)...);
+    kernel<<<grid, block, smem, s>>>(std::forward<Args>(args)...);
 #endif
+}
+
+template <class... KArgs, class... Args>
+inline void launch_pdl(void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args &&...args)
+{
+    launch_pdl_smem(kernel, grid, block, 0, s, std::forward<Args>(args)...);
 }
