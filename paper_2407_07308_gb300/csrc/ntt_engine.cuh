@@ -49,7 +49,7 @@
 // degree, twiddle and constant tables), pointers and level.  One launch can
 // therefore serve ciphertexts of different ring degree, level and origin:
 // the units of all segments are numbered in order and every CTA walks them
-// with a grid stride, dispatching each unit on its segment's ring degree.
+// with a grid stride (segments of different ring degree: one launch each).
 // The grid is either one CTA per unit or a fixed number of resident CTAs per
 // SM (the autotuner's choice per context).
 //
@@ -172,11 +172,6 @@ constexpr int T = 128;  // threads per CTA, 16 residues each
 // The same for the column kernels of paired units (two targets per load).
 #ifndef FHE_NTT_MINB_PAIRED
 #define FHE_NTT_MINB_PAIRED 7
-#endif
-// Launches that mix ring degrees 2^13..2^15 take the kernel that dispatches
-// every unit on its degree (1), or one launch per degree in turn (0).
-#ifndef FHE_NTT_MIXED_KERNEL
-#define FHE_NTT_MIXED_KERNEL 1
 #endif
 // Shared-memory twiddle tables: entry k at k + k / 8 (one 16-byte pad per 8
 // entries), so that the second round's strided twiddle reads (stride up to 8
@@ -355,6 +350,7 @@ struct ColGeo {
     static constexpr int NJ = NS / NC;                                 // jobs per unit
     static constexpr int BLK = (1 << N2) / NC;                         // column blocks per job
     static constexpr int TWC = twp_size(1 << N1);                      // staged twiddles per job
+    static constexpr int TW = NJ * TWC;
     static_assert(NJ <= 2, "jobs per column unit");
     // word r of the unit: job slot, column in job, element
     __device__ static int jslot(int r) { return NJ == 1 ? 0 : r / (NC * SZ); }
@@ -424,10 +420,15 @@ struct RowOneTw {
 // ---------------------------------------------------------------------------
 
 // Per segment: jobs = outer * nl, job = o * nl + l, and the prime of a job
-// depends on l only (so the jobs l, nl + l, 2 nl + l ... can share a CTA).
+// depends on l only (so the jobs l, nl + l, 2 nl + l ... can share a CTA).  A
+// segment joins the batches of one context, level and count (the products of
+// a wave): outer item o belongs to payload first + o / per, as its item o %
+// per, so that small batches fill the grouped row units together.  Row units
+// of 16 jobs serve the first gouter outer items, units of one job the rest.
 struct SegHdr {
-    int logN, outer, nl, grouped;  // grouped: row units of 16 jobs
-    int u_cols, u_rows, xj, pad1;  // xj: the functor's XJ (0 read as 1)
+    int logN, outer, nl, gouter;
+    int u_cols, u_rows, xj, g_units;  // xj: the functor's XJ (0 read as 1); g_units: grouped row units
+    int first, per;
     const ModQ *mq;
     const ulonglong2 *tw;    // forward or inverse table of the segment's context
     const ulonglong2 *ninv;  // N^-1 per prime (Shoup pairs)
@@ -437,9 +438,18 @@ constexpr int DIR_FWD = 1, DIR_INV = 2;
 
 template <class S>
 struct SegIO {
-    int nseg, ucols, urows, pad;
+    using Payload = S;
+    int nseg, ucols, urows, pad;  // segments (headers); payloads may be more
     SegHdr h[FHE_SEGS];
     S s[FHE_SEGS];
+    // the payload of a job, with the job's place in it
+    __device__ const S &payload(int sg, int &job) const
+    {
+        const SegHdr &H = h[sg];
+        const int k = H.outer == H.per ? 0 : job / (H.nl * H.per);
+        job -= k * H.nl * H.per;
+        return s[H.first + k];
+    }
     // jobs per column unit asked for (2: functors whose loads convert, with same_src)
     static constexpr int XJ = 1;
     static constexpr bool PLAIN = false;
@@ -530,16 +540,37 @@ __device__ __forceinline__ void conv_pair(const Conv &a, const Conv &b, const Mo
     }
 }
 
-// one target
-__device__ __forceinline__ u64 conv_one(const Conv &a, const ModQ &m, int N, int n)
+// One target at P positions.
+template <int P, int STEP, int NN>
+__device__ __forceinline__ void conv_one(const Conv &a, const ModQ &m, int n, u64 (&v)[P])
 {
-    DotAcc s{0, (int64_t)(2 * m.q2)};
+    DotAcc s[P];
+#pragma unroll
+    for (int p = 0; p < P; p++) s[p] = DotAcc{0, (int64_t)(2 * m.q2)};
+    const int h = m.half, ns = a.n;
+    const u64 *src = a.src + n;
 #pragma unroll 1
-    for (int i = 0; i < a.n; i++) {
-        dot_mac(s, a.src[(size_t)i * N + n], a.c[i], m.half);
-        if (m.half > 27 && (i & 1)) s = DotAcc{0, dot_fold(s, m)};
+    for (int i0 = 0; i0 < ns; i0 += 4) {
+        u64 x[4][P];
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+            if (i0 + i < ns) {
+#pragma unroll
+                for (int p = 0; p < P; p++) x[i][p] = src[(size_t)i * NN + p * STEP];
+            }
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+            if (i0 + i < ns) {
+#pragma unroll
+                for (int p = 0; p < P; p++) {
+                    dot_mac(s[p], x[i][p], a.c[i0 + i], h);
+                    if (h > 27 && (i & 1)) s[p] = DotAcc{0, dot_fold(s[p], m)};
+                }
+            }
+        src += (size_t)4 * NN;
     }
-    return (u64)dot_fold(s, m);
+#pragma unroll
+    for (int p = 0; p < P; p++) v[p] = (u64)dot_fold(s[p], m);
 }
 
 // ---------------------------------------------------------------------------
@@ -730,10 +761,13 @@ __device__ __forceinline__ void inv_cols_unit1(const IO &io, int sg, int lu, u64
 template <int NN, class IO>
 __device__ __forceinline__ u64 col_load(const IO &io, int sg, const typename IO::CSt &st, int n)
 {
-    if constexpr (IO::XJ == 2)
-        return io.load(sg, st, NN, n);
-    else
+    if constexpr (IO::XJ == 2) {
+        u64 v[1];
+        conv_one<1, 0, NN>(st.cv, io.h[sg].mq[st.prime], n, v);
+        return v[0];
+    } else {
         return io.load(st, n);
+    }
 }
 
 // Forward, columns: global stages 0..N1-1.
@@ -776,14 +810,30 @@ __device__ __forceinline__ void fwd_cols_unit(const IO &io, int sg, int lu, u64 
             }
         }
     }
-    if (!paired) {
-        // a unit whose jobs read different sources (or with one job left): a
-        // rolled loop, small code beside the paired path
+    if constexpr (Gm::PAIRED) {
+        // a unit whose jobs read different sources, or with one job left (a
+        // slot without a job transforms what is there and stores nothing):
+        // rolled loops, small code beside the paired path
+        if (!paired) {
+            constexpr int ES = T / Gm::NC;
+            const int col = tid % Gm::NC, e0 = tid / Gm::NC;
+#pragma unroll 1
+            for (int j = 0; j < 2 && j < nvalid; j++)
+#pragma unroll 1
+                for (int k = 0; k < 8; k += CONV_P) {
+                    u64 v[CONV_P];
+                    conv_one<CONV_P, (ES << N2), Gm::NN>(sts[j].cv, j == 0 ? m0 : m1, ((e0 + k * ES) << N2) + lo0 + col, v);
+#pragma unroll
+                    for (int p = 0; p < CONV_P; p++) sm[Gm::Lay::at(j * Gm::NC + col, e0 + (k + p) * ES)] = v[p];
+                }
+        }
+    } else {
 #pragma unroll 1
         for (int k = 0; k < 16; k++) {
             const int r = tid + k * T, j = Gm::jslot(r);
-            sm[Gm::Lay::at(j * Gm::NC + Gm::col(r), Gm::elem(r))] =
-                j < nvalid ? col_load<Gm::NN>(io, sg, sts[j], (Gm::elem(r) << N2) + lo0 + Gm::col(r)) : 0;
+            if (j < nvalid)
+                sm[Gm::Lay::at(j * Gm::NC + Gm::col(r), Gm::elem(r))] =
+                    col_load<Gm::NN>(io, sg, sts[j], (Gm::elem(r) << N2) + lo0 + Gm::col(r));
         }
     }
     async_wait();
@@ -857,16 +907,17 @@ __device__ __forceinline__ int row_jobs(const IO &io, int sg, int lu, typename I
     const SegHdr &H = io.h[sg];
     int nvalid;
     if (GRP) {
-        const int OC = (H.outer + ROW_J - 1) / ROW_J;
+        const int OC = (H.gouter + ROW_J - 1) / ROW_J;
         const int hc = lu % Gm::CH, t = lu / Gm::CH;
         const int oc = t % OC, l = t / OC;
         *hi0 = hc * Gm::R;
-        nvalid = min(ROW_J, H.outer - oc * ROW_J);
+        nvalid = min(ROW_J, H.gouter - oc * ROW_J);
         if ((int)threadIdx.x < nvalid) io.begin_r(sg, (oc * ROW_J + threadIdx.x) * H.nl + l, sts[threadIdx.x]);
     } else {
-        *hi0 = (lu % Gm::CHS) * Gm::NS;
+        const int v = lu - H.g_units;
+        *hi0 = (v % Gm::CHS) * Gm::NS;
         nvalid = 1;
-        if (threadIdx.x == 0) io.begin_r(sg, lu / Gm::CHS, sts[0]);
+        if (threadIdx.x == 0) io.begin_r(sg, H.gouter * H.nl + v / Gm::CHS, sts[0]);
     }
     __syncthreads();
     return nvalid;
@@ -1009,11 +1060,11 @@ __device__ __forceinline__ void inv_rows_unit(const IO &io, int sg, int lu, u64 
 }
 
 // ---------------------------------------------------------------------------
-// kernels: one per (functor, direction, pass, range of ring degrees).  A
-// launch whose segments share one ring degree takes the kernel of that
-// degree alone (the smallest code, the best instruction-fetch behaviour);
-// only a launch that mixes ring degrees takes the 2^13..2^15 kernel, which
-// dispatches every unit on its segment's degree.
+// kernels: one per (functor, direction, pass, ring degree).  A launch whose
+// segments mix ring degrees runs one kernel per degree: a kernel that
+// dispatched every unit on its segment's degree halved the launches of an
+// uneven batch but spilled and fetched more instructions (32 requests over
+// 2^13..2^15: 55.6 ms a pass with it, 50.8 without; 4 requests 5.13 and 4.33).
 // ---------------------------------------------------------------------------
 
 template <int L>
@@ -1021,64 +1072,25 @@ struct Deg {
     static constexpr int N1 = (L + 1) / 2, N2 = L / 2;
 };
 
-// f(Deg<logN>) for logN in [L, HI]; with L == HI no test (the host sends only
-// that degree), otherwise the last degree is the fall-through.
-template <int L, int HI, class F>
-__device__ __forceinline__ void by_degree(int logN, F f)
-{
-    if constexpr (L == HI) {
-        f(Deg<L>{});
-    } else {
-        if (logN == L)
-            f(Deg<L>{});
-        else
-            by_degree<L + 1, HI>(logN, f);
-    }
-}
-
-// shared memory of a column kernel: twiddle entries and job states over its
-// range of ring degrees
-template <class IO, int LO, int HI>
-constexpr int col_tw_entries()
-{
-    using Gm = ColGeo<Deg<LO>::N1, Deg<LO>::N2, IO::XJ>;
-    constexpr int n = Gm::NJ * Gm::TWC;
-    if constexpr (LO == HI)
-        return n;
-    else
-        return n > col_tw_entries<IO, LO + 1, HI>() ? n : col_tw_entries<IO, LO + 1, HI>();
-}
-template <class IO, int LO, int HI>
-constexpr int col_words()
-{
-    constexpr int n = ColGeo<Deg<LO>::N1, Deg<LO>::N2, IO::XJ>::Lay::WORDS;
-    if constexpr (LO == HI)
-        return n;
-    else
-        return n > col_words<IO, LO + 1, HI>() ? n : col_words<IO, LO + 1, HI>();
-}
 constexpr int ROW_WORDS = RowLay<7>::WORDS;
 static_assert(RowLay<5>::WORDS <= ROW_WORDS && RowLay<6>::WORDS <= ROW_WORDS, "row units");
-constexpr int COL_J = 2;  // jobs per column unit, at most
 
-template <class IO, int LO, int HI>
+template <class IO, int L>
 __global__ void __launch_bounds__(T, IO::XJ == 2 ? FHE_NTT_MINB_PAIRED : FHE_NTT_MINB)
     k_fwd_cols(const __grid_constant__ IO io)
 {
     pdl_begin();
-    __shared__ u64 sm[col_words<IO, LO, HI>()];
-    __shared__ ulonglong2 W[col_tw_entries<IO, LO, HI>()];
-    __shared__ typename IO::CSt sts[COL_J];
+    __shared__ u64 sm[ColGeo<Deg<L>::N1, Deg<L>::N2, IO::XJ>::Lay::WORDS];
+    __shared__ ulonglong2 W[ColGeo<Deg<L>::N1, Deg<L>::N2, IO::XJ>::TW];
+    __shared__ typename IO::CSt sts[ColGeo<Deg<L>::N1, Deg<L>::N2, IO::XJ>::NJ];
     for (int u = blockIdx.x; u < io.ucols; u += gridDim.x) {
         const int sg = seg_of(io, u, false), lu = u - io.h[sg].u_cols;
-        by_degree<LO, HI>(io.h[sg].logN, [&](auto d) {
-            fwd_cols_unit<decltype(d)::N1, decltype(d)::N2>(io, sg, lu, sm, W, sts);
-        });
+        fwd_cols_unit<Deg<L>::N1, Deg<L>::N2>(io, sg, lu, sm, W, sts);
         __syncthreads();
     }
 }
 
-template <class IO, int LO, int HI>
+template <class IO, int L>
 __global__ void __launch_bounds__(T, FHE_NTT_MINB)
     k_fwd_rows(const __grid_constant__ IO io)
 {
@@ -1088,19 +1100,15 @@ __global__ void __launch_bounds__(T, FHE_NTT_MINB)
     __shared__ typename IO::RSt sts[ROW_J];
     for (int u = blockIdx.x; u < io.urows; u += gridDim.x) {
         const int sg = seg_of(io, u, true), lu = u - io.h[sg].u_rows;
-        if (io.h[sg].grouped)
-            by_degree<LO, HI>(io.h[sg].logN, [&](auto d) {
-                fwd_rows_unit<decltype(d)::N1, decltype(d)::N2, true>(io, sg, lu, sm, W, sts);
-            });
+        if (lu < io.h[sg].g_units)
+            fwd_rows_unit<Deg<L>::N1, Deg<L>::N2, true>(io, sg, lu, sm, W, sts);
         else
-            by_degree<LO, HI>(io.h[sg].logN, [&](auto d) {
-                fwd_rows_unit<decltype(d)::N1, decltype(d)::N2, false>(io, sg, lu, sm, W, sts);
-            });
+            fwd_rows_unit<Deg<L>::N1, Deg<L>::N2, false>(io, sg, lu, sm, W, sts);
         __syncthreads();
     }
 }
 
-template <class IO, int LO, int HI>
+template <class IO, int L>
 __global__ void __launch_bounds__(T, FHE_NTT_MINB) k_inv_rows(const __grid_constant__ IO io)
 {
     pdl_begin();
@@ -1109,30 +1117,24 @@ __global__ void __launch_bounds__(T, FHE_NTT_MINB) k_inv_rows(const __grid_const
     __shared__ typename IO::RSt sts[ROW_J];
     for (int u = blockIdx.x; u < io.urows; u += gridDim.x) {
         const int sg = seg_of(io, u, true), lu = u - io.h[sg].u_rows;
-        if (io.h[sg].grouped)
-            by_degree<LO, HI>(io.h[sg].logN, [&](auto d) {
-                inv_rows_unit<decltype(d)::N1, decltype(d)::N2, true>(io, sg, lu, sm, W, sts);
-            });
+        if (lu < io.h[sg].g_units)
+            inv_rows_unit<Deg<L>::N1, Deg<L>::N2, true>(io, sg, lu, sm, W, sts);
         else
-            by_degree<LO, HI>(io.h[sg].logN, [&](auto d) {
-                inv_rows_unit<decltype(d)::N1, decltype(d)::N2, false>(io, sg, lu, sm, W, sts);
-            });
+            inv_rows_unit<Deg<L>::N1, Deg<L>::N2, false>(io, sg, lu, sm, W, sts);
         __syncthreads();
     }
 }
 
-template <class IO, int LO, int HI>
+template <class IO, int L>
 __global__ void __launch_bounds__(T, FHE_NTT_MINB) k_inv_cols(const __grid_constant__ IO io)
 {
     pdl_begin();
-    __shared__ u64 sm[col_words<IO, LO, HI>()];
-    __shared__ ulonglong2 W[col_tw_entries<IO, LO, HI>()];
-    __shared__ typename IO::CSt sts[COL_J];
+    __shared__ u64 sm[ColGeo<Deg<L>::N1, Deg<L>::N2, IO::XJ>::Lay::WORDS];
+    __shared__ ulonglong2 W[ColGeo<Deg<L>::N1, Deg<L>::N2, IO::XJ>::TW];
+    __shared__ typename IO::CSt sts[ColGeo<Deg<L>::N1, Deg<L>::N2, IO::XJ>::NJ];
     for (int u = blockIdx.x; u < io.ucols; u += gridDim.x) {
         const int sg = seg_of(io, u, false), lu = u - io.h[sg].u_cols;
-        by_degree<LO, HI>(io.h[sg].logN, [&](auto d) {
-            inv_cols_unit<decltype(d)::N1, decltype(d)::N2>(io, sg, lu, sm, W, sts);
-        });
+        inv_cols_unit<Deg<L>::N1, Deg<L>::N2>(io, sg, lu, sm, W, sts);
         __syncthreads();
     }
 }
@@ -1157,6 +1159,15 @@ struct MapSeg {
     uint8_t in_limb[FHE_MAXP], out_limb[FHE_MAXP], prime[FHE_MAXP];
 };
 
+// Whether two payloads' jobs l, nl + l, .. share primes and constants, so that
+// one segment may hold both.
+inline bool joins(const MapSeg &a, const MapSeg &b) { return !memcmp(a.prime, b.prime, sizeof(a.prime)); }
+template <class S>
+inline bool joins(const S &a, const S &b)
+{
+    return a.P == b.P;
+}
+
 struct MapSt {
     const u64 *in;
     u64 *out;
@@ -1168,16 +1179,18 @@ struct MapCSt : MapSt {
 };
 
 template <class Io>
-__device__ __forceinline__ void map_begin(const Io &io, int sg, int job, MapSt &t, int *o_, int *l_)
+__device__ __forceinline__ const typename Io::Payload &map_begin(const Io &io, int sg, int job, MapSt &t, int *o_,
+                                                                 int *l_)
 {
     const SegHdr &H = io.h[sg];
-    const MapSeg &S = io.s[sg];
+    const typename Io::Payload &S = io.payload(sg, job);
     const int N = 1 << H.logN, o = job / H.nl, l = job % H.nl;
     t.in = S.in + o * S.in_outer + (long long)S.in_limb[l] * N;
     t.out = S.out + o * S.out_outer + (long long)S.out_limb[l] * N;
     t.prime = S.prime[l];
     *o_ = o;
     *l_ = l;
+    return S;
 }
 
 struct IOMap : SegIO<MapSeg> {
@@ -1188,8 +1201,8 @@ struct IOMap : SegIO<MapSeg> {
     __device__ void begin_c(int sg, int job, CSt &t) const
     {
         int o, l;
-        map_begin(*this, sg, job, t, &o, &l);
-        t.fs = s[sg].scale ? s[sg].scale[l] : h[sg].ninv[t.prime];
+        const MapSeg &S = map_begin(*this, sg, job, t, &o, &l);
+        t.fs = S.scale ? S.scale[l] : h[sg].ninv[t.prime];
     }
     __device__ void begin_r(int sg, int job, RSt &t) const
     {
@@ -1222,6 +1235,11 @@ struct YSeg : MapSeg {
     u64 Pm, Pm_s, qm;
 };
 
+inline bool joins(const YSeg &a, const YSeg &b)
+{
+    return joins(static_cast<const MapSeg &>(a), static_cast<const MapSeg &>(b)) && a.Pm == b.Pm && a.qm == b.qm;
+}
+
 struct YRSt : MapSt {
     const u64 *add;
     u64 Pm, Pm_s, qm;
@@ -1234,14 +1252,13 @@ struct IOScaledY : SegIO<YSeg> {
     __device__ void begin_c(int sg, int job, CSt &t) const
     {
         int o, e;
-        map_begin(*this, sg, job, t, &o, &e);
-        t.fs = s[sg].scale[e];
+        const YSeg &S = map_begin(*this, sg, job, t, &o, &e);
+        t.fs = S.scale[e];
     }
     __device__ void begin_r(int sg, int job, RSt &t) const
     {
         int o, e;
-        map_begin(*this, sg, job, t, &o, &e);
-        const YSeg &S = s[sg];
+        const YSeg &S = map_begin(*this, sg, job, t, &o, &e);
         const int N = 1 << h[sg].logN, pi = o & 1;
         const long long c = o >> 1;
         t.add = (e == h[sg].nl - 1 && ((S.amask >> pi) & 1))
@@ -1294,17 +1311,17 @@ struct IOModUp : SegIO<ModUpSeg> {
     __device__ u64 *target(int sg, int job, int *entry) const
     {
         const SegHdr &H = h[sg];
-        const ModUpSeg &S = s[sg];
+        const ModUpSeg &S = payload(sg, job);
         const int c = job / H.nl, e = job % H.nl;
         *entry = e;
         return S.ext + (((long long)c * S.dnum + S.P->job_digit[e]) * (S.l + S.K) + S.P->job_tgt[e] << H.logN);
     }
     __device__ void begin_c(int sg, int job, CSt &t) const
     {
-        const ModUpSeg &S = s[sg];
-        const ModUpParams *P = S.P;
         int e;
         t.cv.dst = target(sg, job, &e);
+        const ModUpSeg &S = payload(sg, job);
+        const ModUpParams *P = S.P;
         const int j = P->job_digit[e], tg = P->job_tgt[e];
         t.cv.n = P->digit_n[j];
         t.cv.src = S.d2c + ((long long)(job / h[sg].nl) * S.l + P->digit_lo[j] << h[sg].logN);
@@ -1317,10 +1334,9 @@ struct IOModUp : SegIO<ModUpSeg> {
     {
         int e;
         t.out = target(sg, job, &e);
-        t.prime = s[sg].P->job_prime[e];
+        t.prime = s[h[sg].first].P->job_prime[e];
     }
     __device__ RowK row_k(int, int) const { return {}; }
-    __device__ u64 load(int sg, const CSt &t, int N, int n) const { return conv_one(t.cv, h[sg].mq[t.prime], N, n); }
     // two targets of one digit (same sources): each source word loaded once
     static constexpr int XJ = 2;
     __device__ bool same_src(const CSt &a, const CSt &b) const { return a.cv.src == b.cv.src && a.cv.n == b.cv.n; }
@@ -1363,7 +1379,7 @@ struct IOModDown : SegIO<ModDownSeg> {
     };
     __device__ void begin_c(int sg, int job, CSt &t) const
     {
-        const ModDownSeg &S = s[sg];
+        const ModDownSeg &S = payload(sg, job);
         const int logN = h[sg].logN, o = job / S.l, i = job % S.l;
         t.cv.src = S.accP + ((long long)o * S.K << logN);
         t.cv.dst = S.out + ((long long)job << logN);
@@ -1375,15 +1391,14 @@ struct IOModDown : SegIO<ModDownSeg> {
     }
     __device__ void begin_r(int sg, int job, RSt &t) const
     {
-        const ModDownSeg &S = s[sg];
+        const ModDownSeg &S = payload(sg, job);
         const int logN = h[sg].logN, o = job / S.l, i = job % S.l, c = o >> 1, pi = o & 1;
         t.x = S.acc + ((long long)o * (S.l + S.K) + i << logN);
         t.add = ((S.amask >> pi) & 1) ? S.abase + c * S.a_outer + pi * S.a_poly + ((long long)i << logN) : nullptr;
         t.out = S.out + ((long long)job << logN);
         t.prime = i;
     }
-    __device__ RowK row_k(int sg, int i) const { return RowK{s[sg].P->pinv[i]}; }
-    __device__ u64 load(int sg, const CSt &t, int N, int n) const { return conv_one(t.cv, h[sg].mq[t.prime], N, n); }
+    __device__ RowK row_k(int sg, int i) const { return RowK{s[h[sg].first].P->pinv[i]}; }
     // two data limbs of one (ct, poly): the special limbs loaded once
     static constexpr int XJ = 2;
     __device__ bool same_src(const CSt &a, const CSt &b) const { return a.cv.src == b.cv.src && a.cv.n == b.cv.n; }
@@ -1425,7 +1440,7 @@ struct IOModSwitch : SegIO<SwitchSeg> {
     using RowK = SwitchRowK;
     __device__ void begin_c(int sg, int job, CSt &t) const
     {
-        const SwitchSeg &S = s[sg];
+        const SwitchSeg &S = payload(sg, job);
         const int logN = h[sg].logN, o = job / (S.l - 1), i = job % (S.l - 1);
         t.last = S.last + ((long long)o << logN);
         t.out = S.out + ((long long)job << logN);
@@ -1436,14 +1451,14 @@ struct IOModSwitch : SegIO<SwitchSeg> {
     }
     __device__ void begin_r(int sg, int job, RSt &t) const
     {
-        const SwitchSeg &S = s[sg];
+        const SwitchSeg &S = payload(sg, job);
         const int logN = h[sg].logN, o = job / (S.l - 1), i = job % (S.l - 1);
         t.x = S.in + ((long long)o * S.l + i << logN);
         t.add = nullptr;
         t.out = S.out + ((long long)job << logN);
         t.prime = i;
     }
-    __device__ RowK row_k(int sg, int i) const { return RowK{s[sg].P->qinv[i]}; }
+    __device__ RowK row_k(int sg, int i) const { return RowK{s[h[sg].first].P->qinv[i]}; }
     // a column pass's word is p w, in [0, 4q)
     static constexpr bool PLAIN = false;
     __device__ const u64 *src(const CSt &t) const { return t.last; }
@@ -1484,7 +1499,7 @@ struct IORelinMS : SegIO<RelinMSSeg> {
     };
     __device__ void begin_c(int sg, int job, CSt &t) const
     {
-        const RelinMSSeg &S = s[sg];
+        const RelinMSSeg &S = payload(sg, job);
         const int logN = h[sg].logN, m = S.l - 1, o = job / m, i = job % m;
         t.cv.src = S.src + ((long long)o * (S.K + 1) << logN);
         t.cv.dst = S.out + ((long long)job << logN);
@@ -1496,15 +1511,14 @@ struct IORelinMS : SegIO<RelinMSSeg> {
     }
     __device__ void begin_r(int sg, int job, RSt &t) const
     {
-        const RelinMSSeg &S = s[sg];
+        const RelinMSSeg &S = payload(sg, job);
         const int logN = h[sg].logN, m = S.l - 1, o = job / m, i = job % m, c = o >> 1, pi = o & 1;
         t.x = S.acc + ((long long)o * (S.l + S.K) + i << logN);
         t.add = ((S.amask >> pi) & 1) ? S.abase + c * S.a_outer + pi * S.a_poly + ((long long)i << logN) : nullptr;
         t.out = S.out + ((long long)job << logN);
         t.prime = i;
     }
-    __device__ RowK row_k(int sg, int i) const { return RowK{s[sg].P->pqinv[i], s[sg].P->qminv[i]}; }
-    __device__ u64 load(int sg, const CSt &t, int N, int n) const { return conv_one(t.cv, h[sg].mq[t.prime], N, n); }
+    __device__ RowK row_k(int sg, int i) const { return RowK{s[h[sg].first].P->pqinv[i], s[h[sg].first].P->qminv[i]}; }
     // two data limbs of one (ct, poly): the K + 1 sources loaded once
     static constexpr int XJ = 2;
     __device__ bool same_src(const CSt &a, const CSt &b) const { return a.cv.src == b.cv.src && a.cv.n == b.cv.n; }
@@ -1535,7 +1549,7 @@ struct IOMultiSwitch : SegIO<MultiSeg> {
     using RowK = SwitchRowK;
     __device__ void begin_c(int sg, int job, CSt &t) const
     {
-        const MultiSeg &S = s[sg];
+        const MultiSeg &S = payload(sg, job);
         const int logN = h[sg].logN, kept = S.l - S.k, o = job / kept, i = job % kept;
         t.cv.src = S.src + ((long long)o * S.k << logN);
         t.cv.dst = S.out + ((long long)job << logN);
@@ -1547,15 +1561,14 @@ struct IOMultiSwitch : SegIO<MultiSeg> {
     }
     __device__ void begin_r(int sg, int job, RSt &t) const
     {
-        const MultiSeg &S = s[sg];
+        const MultiSeg &S = payload(sg, job);
         const int logN = h[sg].logN, kept = S.l - S.k, o = job / kept, i = job % kept;
         t.x = S.in + ((long long)o * S.l + i << logN);
         t.add = nullptr;
         t.out = S.out + ((long long)job << logN);
         t.prime = i;
     }
-    __device__ RowK row_k(int sg, int i) const { return RowK{s[sg].P->Dinv[i]}; }
-    __device__ u64 load(int sg, const CSt &t, int N, int n) const { return conv_one(t.cv, h[sg].mq[t.prime], N, n); }
+    __device__ RowK row_k(int sg, int i) const { return RowK{s[h[sg].first].P->Dinv[i]}; }
     // two kept limbs of one (ct, poly): the k switch values loaded once
     static constexpr int XJ = 2;
     __device__ bool same_src(const CSt &a, const CSt &b) const { return a.cv.src == b.cv.src && a.cv.n == b.cv.n; }
@@ -1587,8 +1600,10 @@ Split split_of(int logN)
     return s;
 }
 
-// Row units are grouped (16 jobs of one prime) once a segment has at least
-// this many outer items; below it a unit holds adjacent rows of one job.
+// Row units are grouped (16 jobs of one prime) as far as the outer items fill
+// them; a rest of fewer than GROUP_MIN_OUTER items takes units of adjacent
+// rows of one job, whose twiddles are read through the cache (twice the data's
+// bytes at N2 = 7).
 constexpr int GROUP_MIN_OUTER = 12;
 
 // Unit counts of a segment (column and row passes) from its geometry.
@@ -1600,8 +1615,11 @@ void unit_counts(SegHdr &H)
     if (col_paired(H.xj, sp.ns1, nc)) nc /= 2;  // ColGeo's paired units
     const int nj = sp.ns1 / nc, blk = (1 << sp.n2) / nc;
     H.u_cols = ((njobs + nj - 1) / nj) * blk;
-    H.u_rows = H.grouped ? H.nl * ((H.outer + ROW_J - 1) / ROW_J) * ((1 << sp.n1) / (sp.ns2 / ROW_J))
-                         : njobs * ((1 << sp.n1) / sp.ns2);
+    const bool always = (1 << sp.n1) < sp.ns2;  // a limb has fewer rows than a unit
+    const int rest = H.outer % ROW_J;
+    H.gouter = always || rest >= GROUP_MIN_OUTER ? H.outer : H.outer - rest;
+    H.g_units = H.nl * ((H.gouter + ROW_J - 1) / ROW_J) * ((1 << sp.n1) / (sp.ns2 / ROW_J));
+    H.u_rows = H.g_units + (H.outer - H.gouter) * H.nl * ((1 << sp.n1) / sp.ns2);
 }
 
 // Fills the header of a segment (jobs = outer * nl) with its unit counts
@@ -1609,14 +1627,13 @@ void unit_counts(SegHdr &H)
 void seg_header(SegHdr &H, const fhe_ctx *c, bool fwd, int outer, int nl)
 {
     memset(&H, 0, sizeof(H));
-    const Split sp = split_of(c->logN);
     H.logN = c->logN;
     H.outer = outer;
     H.nl = nl;
     H.mq = c->d_mq;
     H.tw = fwd ? c->d_fwd : c->d_inv;
     H.ninv = c->d_ninv;
-    H.grouped = outer >= GROUP_MIN_OUTER || (1 << sp.n1) < sp.ns2;
+    H.per = outer;
     unit_counts(H);
 }
 
@@ -1654,24 +1671,23 @@ void recount(IO &io)
     for (int s = 0; s < io.nseg; s++) unit_counts(io.h[s]);
 }
 
-template <class IO, int LO, int HI>
+template <class IO, int L>
 void launch_passes(fhe_ctx *c, const IO &io, bool fwd)
 {
     if constexpr ((IO::DIRS & DIR_FWD) != 0)
         if (fwd) {
-            launch_pdl(k_fwd_cols<IO, LO, HI>, grid_of(c, io.ucols), T, c->stream, io);
-            launch_pdl(k_fwd_rows<IO, LO, HI>, grid_of(c, io.urows), T, c->stream, io);
+            launch_pdl(k_fwd_cols<IO, L>, grid_of(c, io.ucols), T, c->stream, io);
+            launch_pdl(k_fwd_rows<IO, L>, grid_of(c, io.urows), T, c->stream, io);
         }
     if constexpr ((IO::DIRS & DIR_INV) != 0)
         if (!fwd) {
-            launch_pdl(k_inv_rows<IO, LO, HI>, grid_of(c, io.urows), T, c->stream, io);
-            launch_pdl(k_inv_cols<IO, LO, HI>, grid_of(c, io.ucols), T, c->stream, io);
+            launch_pdl(k_inv_rows<IO, L>, grid_of(c, io.urows), T, c->stream, io);
+            launch_pdl(k_inv_cols<IO, L>, grid_of(c, io.ucols), T, c->stream, io);
         }
     c->launches += 2;
 }
 
-// Segments of one degree take that degree's kernels; a mix within
-// 2^13..2^15 takes the mixed kernels; any other mix is split by degree.
+// Segments of one degree take that degree's kernels; a mix is split by degree.
 template <class IO>
 void launch_segments(fhe_ctx *c, IO &io, bool fwd)
 {
@@ -1681,25 +1697,26 @@ void launch_segments(fhe_ctx *c, IO &io, bool fwd)
     if (io.ucols == 0) return;
     if (lo == hi) {
         switch (lo) {
-        case 10: launch_passes<IO, 10, 10>(c, io, fwd); break;
-        case 11: launch_passes<IO, 11, 11>(c, io, fwd); break;
-        case 12: launch_passes<IO, 12, 12>(c, io, fwd); break;
-        case 13: launch_passes<IO, 13, 13>(c, io, fwd); break;
-        case 14: launch_passes<IO, 14, 14>(c, io, fwd); break;
-        case 15: launch_passes<IO, 15, 15>(c, io, fwd); break;
+        case 10: launch_passes<IO, 10>(c, io, fwd); break;
+        case 11: launch_passes<IO, 11>(c, io, fwd); break;
+        case 12: launch_passes<IO, 12>(c, io, fwd); break;
+        case 13: launch_passes<IO, 13>(c, io, fwd); break;
+        case 14: launch_passes<IO, 14>(c, io, fwd); break;
+        case 15: launch_passes<IO, 15>(c, io, fwd); break;
         default: break;
         }
-    } else if (FHE_NTT_MIXED_KERNEL && lo >= 13 && hi <= 15) {
-        launch_passes<IO, 13, 15>(c, io, fwd);
     } else {
         for (int n = lo; n <= hi; n++) {
             IO sub;
             memset(&sub, 0, sizeof(sub));
+            int np = 0;
             for (int s = 0; s < io.nseg; s++)
                 if (io.h[s].logN == n) {
-                    sub.h[sub.nseg] = io.h[s];
-                    sub.s[sub.nseg] = io.s[s];
-                    sub.nseg++;
+                    SegHdr &H = sub.h[sub.nseg++];
+                    H = io.h[s];
+                    for (int k = 0; k < H.outer / H.per; k++) sub.s[np + k] = io.s[io.h[s].first + k];
+                    H.first = np;
+                    np += H.outer / H.per;
                 }
             if (sub.nseg) {
                 recount(sub);
@@ -1738,27 +1755,63 @@ void map_seg(MapSeg &S, const u64 *in, u64 *out, const LimbMap &m, const ulonglo
     }
 }
 
-// Runs `fill(io, item)` over items in launches of at most FHE_SEGS segments.
+// Runs `fill(io, 0, item, ..)` over items: the payloads of one context and
+// geometry that join side by side as one segment, in launches of at most
+// FHE_SEGS payloads.
 template <class IO, class Item, class Fill>
 void run_many(const std::vector<Item> &items, bool fwd, int cls, Fill fill)
 {
-    size_t i = 0;
-    while (i < items.size()) {
-        IO io;
-        memset(&io, 0, sizeof(io));
-        fhe_ctx *c0 = items[i].c;
-        double bytes = 0, bfly = 0;
-        for (; i < items.size() && io.nseg < FHE_SEGS; i++) {
-            double b = 0, f = 0;
-            if (fill(io, io.nseg, items[i], &b, &f)) {
-                if (IO::XJ != 1) {
-                    io.h[io.nseg].xj = IO::XJ;
-                    unit_counts(io.h[io.nseg]);
-                }
-                io.nseg++;
+    struct One {
+        fhe_ctx *c;
+        SegHdr h;
+        typename IO::Payload s;
+        double bytes, bfly;
+        bool taken;
+    };
+    std::vector<One> all;
+    all.reserve(items.size());
+    std::unique_ptr<IO> tmp(new IO);
+    for (const Item &it : items) {
+        One o;
+        memset(&o, 0, sizeof(o));
+        memset(&tmp->h[0], 0, sizeof(tmp->h[0]));
+        memset(&tmp->s[0], 0, sizeof(tmp->s[0]));
+        if (!fill(*tmp, 0, it, &o.bytes, &o.bfly)) continue;
+        o.c = it.c;
+        o.h = tmp->h[0];
+        o.s = tmp->s[0];
+        all.push_back(o);
+    }
+    std::vector<One *> order;
+    for (size_t i = 0; i < all.size(); i++)
+        for (size_t j = i; j < all.size(); j++)
+            if (!all[j].taken && (j == i || (!all[i].taken && all[j].c == all[i].c && all[j].h.nl == all[i].h.nl &&
+                                             all[j].h.per == all[i].h.per && joins(all[j].s, all[i].s)))) {
+                if (j != i) all[j].taken = true;
+                order.push_back(&all[j]);
+            } else if (j == i) {
+                break;
             }
-            bytes += b;
-            bfly += f;
+    for (size_t i = 0; i < order.size();) {
+        memset(tmp.get(), 0, sizeof(IO));
+        IO &io = *tmp;
+        fhe_ctx *c0 = order[i]->c;
+        double bytes = 0, bfly = 0;
+        for (int np = 0; i < order.size() && np < FHE_SEGS; i++, np++) {
+            const One &o = *order[i];
+            SegHdr *H = io.nseg ? &io.h[io.nseg - 1] : nullptr;
+            if (H && o.c == order[i - 1]->c && H->nl == o.h.nl && H->per == o.h.per && joins(io.s[H->first], o.s)) {
+                H->outer += o.h.outer;
+            } else {
+                H = &io.h[io.nseg++];
+                *H = o.h;
+                H->first = np;
+                if (IO::XJ != 1) H->xj = IO::XJ;
+            }
+            io.s[np] = o.s;
+            unit_counts(*H);
+            bytes += o.bytes;
+            bfly += o.bfly;
         }
         run(c0, io, fwd, cls, bytes, bfly);
     }
