@@ -1626,13 +1626,18 @@ extern "C" int fhe_selftest_modarith(uint64_t prime_mod, uint64_t prime_lo, uint
             HalfAcc ha{0, 0, 0};
             u128 hs = 0;
             for (int k = 0; k < 8; k++) {
-                half_mac(ha, half_pack(a[k], m.half), half_const(b[k], m));
+                half_mac(ha, halves_of(half_pack(a[k], m.half)), halves_of(half_const(b[k], m)));
                 hs = (hs + (u128)a[k] * b[k]) % q;
                 const u64 r = half_mont(ha, m);
                 if (r > (u64)(k + 2) * q || r % q != (u64)hs) bad++;
                 const u64 f = reduce_few(r, m);
                 if (f >= 2 * q || f % q != (u64)hs) bad++;
             }
+            HalfAcc h2{0, 0, 0};
+            for (int k = 0; k < 8; k += 2)
+                half_mac2(h2, halves_of(half_pack(a[k], m.half)), halves_of(half_const(b[k], m)),
+                          halves_of(half_pack(a[k + 1], m.half)), halves_of(half_const(b[k + 1], m)));
+            if (half_mont(h2, m) != half_mont(ha, m)) bad++;
             // sums of constant products, folded after each even count as the
             // kernels do for the largest primes
             DotAcc da{0, 0};

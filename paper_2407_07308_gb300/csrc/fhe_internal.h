@@ -96,7 +96,7 @@ struct RelinMSParams {
     DotC h[FHE_MAXK + 1][FHE_MAXP];         // h[k][i] = p p_k^-1 mod q_i, h[K][i] = p mod q_i
     DotC pqinv[FHE_MAXP];                    // (P q_m)^-1 mod q_i
     DotC qminv[FHE_MAXP];                    // q_m^-1 mod q_i
-    u64 pkinv[FHE_MAXK];                     // p_k^-1 mod q_m
+    DotC pkinv[FHE_MAXK];                    // p_k^-1 mod q_m
     u64 Pm, Pm_s;                            // P mod q_m
 };
 
@@ -110,7 +110,7 @@ struct MultiSwitchParams {
     int l, k;
     DotC G[FHE_MAXK][FHE_MAXP];          // p D_t mod q_i
     DotC Dinv[FHE_MAXP];                 // D_k^-1 mod q_i
-    u64 F[FHE_MAXK][FHE_MAXK];           // D_t D_j^-1 mod q_{l-1-j}
+    DotC F[FHE_MAXK][FHE_MAXK];          // D_t D_j^-1 mod q_{l-1-j}
 };
 
 // ---------------------------------------------------------------------------

@@ -1,7 +1,8 @@
-// kernels.cu -- streaming (HBM-bound) kernels on NTT-domain limbs: add, sub,
-// neg, scalar and constant terms, the ciphertext tensor product, the
-// key-switching inner product, Galois automorphisms as index permutations, and
-// small helpers for key generation, encryption and decryption.
+// kernels.cu -- streaming (HBM-bound) kernels on NTT-domain limbs of one batch:
+// neg, scalar and constant terms, plaintext operands, Galois automorphisms as
+// index permutations (sums, tensor products, inner products and switch folds
+// run through many.cu's kernels, as a table of one batch), and small helpers
+// for key generation, encryption and decryption.
 //
 // Layout: a batch of ciphertexts is u64 [count][npoly][level][N]; an "outer"
 // index runs over count*npoly polys, and the limb of element idx is
@@ -20,16 +21,6 @@ inline int grid_for(long long n, int per_thread = 1)
     long long b = (n + (long long)TPB * per_thread - 1) / ((long long)TPB * per_thread);
     if (b > (1 << 30)) b = 1 << 30;
     return (int)(b > 0 ? b : 1);
-}
-
-__global__ void k_add(const u64 *__restrict__ a, const u64 *__restrict__ b, u64 *__restrict__ out,
-                      long long total, int logN, int level, const ModQ *__restrict__ mq, int sub)
-{
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const u64 q = mq[(int)((idx >> logN) % level)].q;
-        out[idx] = sub ? submod(a[idx], b[idx], q) : addmod(a[idx], b[idx], q);
-    }
 }
 
 __global__ void k_neg(const u64 *__restrict__ a, u64 *__restrict__ out, long long total, int logN, int level,
@@ -66,72 +57,6 @@ __global__ void k_add_const(const u64 *__restrict__ a, u64 *__restrict__ out, lo
         const int i = (int)(li % level);
         const int poly = (int)((li / level) % 2);
         out[idx] = poly == 0 ? addmod(a[idx], k.w[i], mq[i].q) : a[idx];
-    }
-}
-
-// (a0,a1) x (b0,b1) -> (a0 b0, a0 b1 + a1 b0, a1 b1), all NTT domain.
-__global__ void k_tensor(const u64 *__restrict__ a, const u64 *__restrict__ b, u64 *__restrict__ out,
-                         long long total, int logN, int level, const ModQ *__restrict__ mq)
-{
-    const long long LN = (long long)level << logN;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const long long c = idx / LN, r = idx % LN;
-        const ModQ m = mq[(int)(r >> logN)];
-        const u64 a0 = a[2 * c * LN + r], a1 = a[(2 * c + 1) * LN + r];
-        const u64 b0 = b[2 * c * LN + r], b1 = b[(2 * c + 1) * LN + r];
-        out[3 * c * LN + r] = barrett128((u128)a0 * b0, m);
-        out[(3 * c + 1) * LN + r] = barrett128((u128)a0 * b1 + (u128)a1 * b0, m);
-        out[(3 * c + 2) * LN + r] = barrett128((u128)a1 * b1, m);
-    }
-}
-
-// Relinearisation fused with the modulus switch (the inverse NTT that
-// precedes this step formed y = acc_m + (P mod q_m) add_m while loading):
-// after the scaled inverse NTT of the special limbs and of y, in
-// src[c][pi] = (t_0 .. t_{K-1}, Y'), Y' = INTT(y) (p P)^-1, replace Y' by
-// w = Y' - sum_k t_k p_k^-1 mod q_m, i.e. [x_m p^-1]_{q_m} of the
-// relinearised x.
-__global__ void k_rms_fold(u64 *__restrict__ src, long long total, int logN, int l, int K,
-                           const RelinMSParams *__restrict__ P, const ModQ *__restrict__ mq)
-{
-    const int N = 1 << logN;
-    const ModQ mm = mq[l - 1];
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const long long cp = idx >> logN;
-        const int n = (int)(idx & (N - 1));
-        u64 *base = src + cp * (K + 1) * N + n;
-        u128 a = 0;
-        for (int k = 0; k < K; k++) a += (u128)base[(long long)k * N] * P->pkinv[k];
-        base[(long long)K * N] = submod(base[(long long)K * N], barrett128(a, mm), mm.q);
-    }
-}
-
-// k modulus switches at once: src[o] = (X'_0 .. X'_{k-1}) becomes
-// (w_0 .. w_{k-1}), w_j = X'_j - sum_{t<j} w_t F[j][t] mod q_{l-1-j}.
-__global__ void k_ms_fold(u64 *__restrict__ src, long long total, int logN, int l, int k,
-                          const MultiSwitchParams *__restrict__ P, const ModQ *__restrict__ mq)
-{
-    const int N = 1 << logN;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const long long o = idx >> logN;
-        const int n = (int)(idx & (N - 1));
-        u64 *base = src + o * k * N + n;
-        u64 w[FHE_MAXK];
-#pragma unroll
-        for (int j = 0; j < FHE_MAXK; j++) {
-            if (j < k) {
-                const ModQ mj = mq[l - 1 - j];
-                u128 a = 0;
-#pragma unroll
-                for (int t = 0; t < FHE_MAXK; t++)
-                    if (t < j) a += (u128)w[t] * P->F[j][t];
-                w[j] = submod(base[(long long)j * N], barrett128(a, mj), mj.q);
-                base[(long long)j * N] = w[j];
-            }
-        }
     }
 }
 
@@ -294,12 +219,6 @@ __global__ void k_lincomb(const LinComb lc, u64 *__restrict__ out, long long tot
 #define LAUNCH_CLS(cls, kern, total, ...) LAUNCH_CLS_W(cls, 2, kern, total, __VA_ARGS__)
 #define LAUNCH(kern, total, ...) LAUNCH_CLS_W(FHE_K_ELEMWISE, 2, kern, total, __VA_ARGS__)
 
-void launch_add(fhe_ctx *c, const u64 *a, const u64 *b, u64 *out, int outer, int level, int sub)
-{
-    LAUNCH_CLS_W(FHE_K_ELEMWISE, 3, k_add, (long long)outer * level * c->N, a, b, out, (long long)outer * level * c->N, c->logN, level,
-           c->d_mq, sub);
-}
-
 void launch_neg(fhe_ctx *c, const u64 *a, u64 *out, int outer, int level)
 {
     LAUNCH(k_neg, (long long)outer * level * c->N, a, out, (long long)outer * level * c->N, c->logN, level, c->d_mq);
@@ -321,29 +240,9 @@ void launch_add_const(fhe_ctx *c, const u64 *a, u64 *out, int count, int level, 
            level, c->d_mq, k);
 }
 
-void launch_tensor(fhe_ctx *c, const u64 *a, const u64 *b, u64 *out, int count, int level)
-{
-    LAUNCH_CLS_W(FHE_K_TENSOR, 7, k_tensor, (long long)count * level * c->N, a, b, out, (long long)count * level * c->N, c->logN, level,
-           c->d_mq);
-}
-
 void launch_automorphism(fhe_ctx *c, const u64 *in, u64 *out, int outer, int level, const int *perm)
 {
     LAUNCH_CLS(FHE_K_AUTOMORPHISM, k_automorphism, (long long)outer * level * c->N, in, out, (long long)outer * level * c->N, c->logN, perm);
-}
-
-void launch_ms_fold(fhe_ctx *c, u64 *src, int outer, int level, int k)
-{
-    const long long total = (long long)outer * c->N;
-    LAUNCH_CLS_W(FHE_K_ELEMWISE, 2.0 * k, k_ms_fold, total, src, total, c->logN, level, k,
-                 c->d_mss + (size_t)level * (FHE_MAXK + 1) + k, c->d_mq);
-}
-
-void launch_rms_fold(fhe_ctx *c, u64 *src, int count, int level)
-{
-    const long long total = (long long)count * 2 * c->N;
-    LAUNCH_CLS_W(FHE_K_ELEMWISE, c->K + 2.0, k_rms_fold, total, src, total, c->logN, level, c->K, c->d_rms + level,
-                 c->d_mq);
 }
 
 void launch_add_plain(fhe_ctx *c, const u64 *a, const u64 *m, u64 *out, int count, int npoly, int level, int sub)

@@ -5,8 +5,7 @@
 // A launch carries a table of up to FHE_SEGS segments (one batch each, of any
 // context, level and size on one device); segment s owns a contiguous range
 // of blocks, so a block never straddles two segments and every warp still
-// reads 256 contiguous bytes.  The arithmetic per element is the one of the
-// single-batch kernels in kernels.cu; only the addressing differs.
+// reads 256 contiguous bytes.  Single batches run through the same kernels.
 #include <string.h>
 
 #include <algorithm>
@@ -183,6 +182,80 @@ __global__ void k_ew_many(const __grid_constant__ EwTable t)
         ew_block<1>(S);
 }
 
+// ---- linear combinations of shared operands ---------------------------------
+// out[o] = sum_t k[o][t] x[t] for up to eight outputs over the same (up to
+// eight) operands: the leaves of a Paterson-Stockmeyer evaluation combine the
+// same baby powers with different coefficients.  Bound by HBM: each operand
+// word is read once for all outputs, where a launch of single combinations
+// read it once per output (the leaves' operands of a batch exceed L2: p = 257
+// has 16 leaves over eight powers).  Measured per pass, all element-wise
+// launches: 7 pairs at N = 2^15 4.59 -> 2.19 ms, 16 pairs at N = 2^14 0.96 ->
+// 0.49 ms.  Scalars as in FHE_EW_LINCOMB's 64-bit
+// form: with a negative scalar's q |k| added, every sum is non-negative and
+// below q sum |k| < 2^64.
+
+constexpr int LC_N = 8;
+
+struct LcSeg {
+    const u64 *x[LC_N];
+    u64 *out[LC_N];
+    const ModQ *mq;
+    long long total;  // elements: outer * level * N
+    int logN, level, n, nout, b0, vec;
+    int32_t k[LC_N][LC_N];  // [output][operand]
+    uint32_t neg[LC_N];     // sum of |k| over an output's negative scalars
+};
+
+struct LcTable {
+    int nseg, pad;
+    LcSeg s[FHE_SEGS];
+};
+
+template <int V>
+__device__ __forceinline__ void lc_block(const LcSeg &S)
+{
+    const long long base = (long long)(blockIdx.x - S.b0) * EW_ELEMS;
+    const int i = (int)((base >> S.logN) % S.level);  // a block's elements lie in one limb
+    const ModQ &m = S.mq[i];
+    const u64 q = m.q;
+#pragma unroll 1
+    for (int e = threadIdx.x * V; e < EW_ELEMS; e += TPB * V) {
+        const long long idx = base + e;
+        if (idx >= S.total) break;
+        Vec<V> a[LC_N];
+#pragma unroll
+        for (int t = 0; t < LC_N; t++)
+            if (t < S.n) a[t] = ld_vec<V>(S.x[t] + idx);
+#pragma unroll 1
+        for (int o = 0; o < S.nout; o++) {
+            u64 acc[V];
+#pragma unroll
+            for (int u = 0; u < V; u++) acc[u] = q * S.neg[o];
+#pragma unroll
+            for (int t = 0; t < LC_N; t++)
+                if (t < S.n) {
+                    const u64 k = (u64)(int64_t)S.k[o][t];
+#pragma unroll
+                    for (int u = 0; u < V; u++) acc[u] += a[t].v[u] * k;
+                }
+            Vec<V> r;
+#pragma unroll
+            for (int u = 0; u < V; u++) r.v[u] = reduce64(acc[u], m);
+            st_vec<V>(S.out[o] + idx, r);
+        }
+    }
+}
+
+__global__ void k_lincomb_many(const __grid_constant__ LcTable t)
+{
+    pdl_begin();
+    const LcSeg &S = t.s[block_seg(t.s, t.nseg)];
+    if (S.vec)
+        lc_block<2>(S);
+    else
+        lc_block<1>(S);
+}
+
 // ---- tensor: (a0,a1) x (b0,b1) -> (a0 b0, a0 b1 + a1 b0, a1 b1) -----------
 
 struct TensorSeg {
@@ -254,11 +327,12 @@ __global__ void k_tensor_many(const __grid_constant__ TensorTable t)
 //
 // Measured per pass (before: 128-bit multiply-adds, one run per item, one
 // digit's words ahead in registers): tournament of 8 ciphertexts, N = 2^15,
-// 36.5 -> 17.7 ms; 7 pairs at N = 2^15 5.80 -> 5.24 ms; 16 pairs at N = 2^14
-// equal (1.53, 1.55 ms).  With the words ahead in registers as before the new
-// arithmetic took 23.6 / 7.6 / 1.84 ms.  Ciphertexts a thread and blocks an
-// SM (16 pairs / 7 pairs / tournament, ms): 4 and 3 as here; 2 and 4 1.81 /
-// 6.14 / 19.2; 3 and 3 1.62 / 5.46 / 18.7; 5 and 2 1.68 / 5.58 / 20.5.
+// 36.5 -> 15.5 ms; 7 pairs at N = 2^15 5.80 -> 4.58 ms; 16 pairs at N = 2^14
+// 1.53 -> 1.38 ms (17.7 / 5.24 / 1.55 with one product a statement instead of
+// the digits in pairs; 23.6 / 7.6 / 1.84 with the words ahead in registers).
+// Ciphertexts a thread and blocks an SM, one product a statement (16 pairs /
+// 7 pairs / tournament, ms): 4 and 3 as here; 2 and 4 1.81 / 6.14 / 19.2; 3
+// and 3 1.62 / 5.46 / 18.7; 5 and 2 1.68 / 5.58 / 20.5.
 
 #ifndef FHE_KS_CB
 #define FHE_KS_CB 4
@@ -336,20 +410,30 @@ __device__ __forceinline__ void ks_sum(u64 *w, const u64 *(&ep)[KS_CB], const u6
     HalfAcc a0[KS_CB], a1[KS_CB];
 #pragma unroll
     for (int cc = 0; cc < KS_CB; cc++) a0[cc] = a1[cc] = HalfAcc{0, 0, 0};
-    for (int j = 0; j < dnum; j++) {
-        async_wait_left(dnum - 1 - j);
-        const u64 c0 = w[0], c1 = w[TPB];
-        const uint32_t c0l = (uint32_t)c0, c0h = (uint32_t)(c0 >> 32), c0s = c0l + c0h;
-        const uint32_t c1l = (uint32_t)c1, c1h = (uint32_t)(c1 >> 32), c1s = c1l + c1h;
+    auto split = [&](u64 z) { return halves((uint32_t)z & mask, (uint32_t)(z >> h)); };
+    constexpr int DW = (2 + KS_CB) * TPB;  // a digit's words
+    int j = 0;
+    for (; j + 2 <= dnum; j += 2, w += 2 * DW) {
+        async_wait_left(dnum - 2 - j);
+        const Halves c0 = halves_of(w[0]), c1 = halves_of(w[TPB]), d0 = halves_of(w[DW]), d1 = halves_of(w[DW + TPB]);
 #pragma unroll
         for (int cc = 0; cc < KS_CB; cc++)
             if (FULL || cc < ncb) {
-                const u64 z = w[(2 + cc) * TPB];
-                const uint32_t zl = (uint32_t)z & mask, zh = (uint32_t)(z >> h), zs = zl + zh;
-                half_mac(a0[cc], zl, zh, zs, c0l, c0h, c0s);
-                half_mac(a1[cc], zl, zh, zs, c1l, c1h, c1s);
+                const Halves z = split(w[(2 + cc) * TPB]), y = split(w[DW + (2 + cc) * TPB]);
+                half_mac2(a0[cc], z, c0, y, d0);
+                half_mac2(a1[cc], z, c1, y, d1);
             }
-        w += (2 + KS_CB) * TPB;
+    }
+    if (j < dnum) {
+        async_wait_left(0);
+        const Halves c0 = halves_of(w[0]), c1 = halves_of(w[TPB]);
+#pragma unroll
+        for (int cc = 0; cc < KS_CB; cc++)
+            if (FULL || cc < ncb) {
+                const Halves z = split(w[(2 + cc) * TPB]);
+                half_mac(a0[cc], z, c0);
+                half_mac(a1[cc], z, c1);
+            }
     }
     // in [0, 2q): what reads the sums (the inverse transforms and the stores
     // of ModDown and of relinearise + switch) takes them
@@ -417,88 +501,99 @@ struct FoldSeg {
     int logN, l, k, K, b0, vec;  // vec: src 16-byte aligned
 };
 
+// y - s for the folded sum s (within 3q of 0) of constant products
+__device__ __forceinline__ u64 fold_sub(u64 y, int64_t s, const ModQ &m)
+{
+    return reduce2q(reduce_few(y + 2 * m.q2 - (u64)s, m), m.q);
+}
+
 struct FoldTable {
     int nseg, rms;
     FoldSeg s[FHE_SEGS];
 };
 
-// The relinearise + switch fold with its block's polynomial and constants
-// found once (a block's EW_ELEMS words lie in one polynomial: EW_ELEMS
-// divides N) and two adjacent words per 16-byte access (measured: the
-// element-wise class 1.356 -> 1.308 ms per step on the 16-pair comparison at
-// N = 2^14).
+// The relinearise + switch fold: src[c][pi] = (t_0 .. t_{K-1}, Y') -> Y' -
+// sum_k t_k p_k^-1 mod q_{l-1}.  A block's FOLD_ELEMS words lie in one
+// polynomial (FOLD_ELEMS divides N), so polynomial and constants are found
+// once; a thread has one pair of adjacent words, all its 16-byte loads in
+// flight together (with two pairs in turn, the second's loads behind the
+// first's store, the kernel waited on loads 13 of 18 cycles an instruction
+// at 46% of HBM; folds of 12 max/min pairs at N = 2^15 0.80 -> 0.68 ms).
+constexpr int FOLD_ELEMS = TPB * 2;
+
 __device__ __forceinline__ void fold_rms_block(const FoldSeg &S)
 {
     const int N = 1 << S.logN;
-    const long long base = (long long)(blockIdx.x - S.b0) * EW_ELEMS;
+    const long long base = (long long)(blockIdx.x - S.b0) * FOLD_ELEMS;
     if (base >= S.total) return;
     const long long o = base >> S.logN;
-    const int n0 = (int)(base & (N - 1));
     const RelinMSParams *P = (const RelinMSParams *)S.P;
-    const ModQ mm = S.mq[S.l - 1];
-    u64 pk[FHE_MAXK];
+    const ModQ &m = S.mq[S.l - 1];
+    const int h = m.half;
+    u64 *b = S.src + o * (S.K + 1) * N + (base & (N - 1)) + threadIdx.x * 2;
+    auto pair = [&](const u64 *p) {
+        return S.vec ? *reinterpret_cast<const ulonglong2 *>(p) : make_ulonglong2(p[0], p[1]);
+    };
+    ulonglong2 v[FHE_MAXK];
+    u64 *y = b + (long long)S.K * N;
 #pragma unroll
-    for (int k = 0; k < FHE_MAXK; k++) pk[k] = k < S.K ? P->pkinv[k] : 0;
-    u64 *b = S.src + o * (S.K + 1) * N + n0;
+    for (int k = 0; k < FHE_MAXK; k++)
+        if (k < S.K) v[k] = pair(b + (long long)k * N);
+    const ulonglong2 yv = pair(y);
+    DotAcc a0{0, 0}, a1{0, 0};
 #pragma unroll
-    for (int e = threadIdx.x * 2; e < EW_ELEMS; e += TPB * 2) {
-        u128 a0 = 0, a1 = 0;
-#pragma unroll
-        for (int k = 0; k < FHE_MAXK; k++)
-            if (k < S.K) {
-                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(b + (long long)k * N + e);
-                a0 += (u128)v.x * pk[k];
-                a1 += (u128)v.y * pk[k];
-            }
-        u64 *y = b + (long long)S.K * N + e;
-        const ulonglong2 yv = *reinterpret_cast<const ulonglong2 *>(y);
-        *reinterpret_cast<ulonglong2 *>(y) =
-            make_ulonglong2(submod(yv.x, barrett128(a0, mm), mm.q), submod(yv.y, barrett128(a1, mm), mm.q));
-    }
+    for (int k = 0; k < FHE_MAXK; k++)
+        if (k < S.K) {
+            const DotC c = P->pkinv[k];
+            dot_mac(a0, v[k].x, c, h);
+            dot_mac(a1, v[k].y, c, h);
+            if (h > 27 && (k & 1)) a0 = DotAcc{0, dot_fold(a0, m)}, a1 = DotAcc{0, dot_fold(a1, m)};
+        }
+    const ulonglong2 w = make_ulonglong2(fold_sub(yv.x, dot_fold(a0, m), m), fold_sub(yv.y, dot_fold(a1, m), m));
+    if (S.vec)
+        *reinterpret_cast<ulonglong2 *>(y) = w;
+    else
+        y[0] = w.x, y[1] = w.y;
 }
 
-// rms: src[c][pi] = (t_0 .. t_{K-1}, Y') -> Y' - sum_k t_k p_k^-1 mod q_{l-1}.
-// multi-switch: src[o] = (X'_0 .. X'_{k-1}) -> w_j = X'_j - sum_{t<j} w_t F[j][t].
-__global__ void k_fold_many(const __grid_constant__ FoldTable t)
+// multi-switch: src[o] = (X'_0 .. X'_{k-1}) -> w_j = X'_j - sum_{t<j} w_t F[j][t],
+// one word a thread: its words of all k limbs loaded first, then the
+// recurrence in registers.
+__device__ __forceinline__ void fold_multi_block(const FoldSeg &S)
+{
+    const int N = 1 << S.logN;
+    const MultiSwitchParams *P = (const MultiSwitchParams *)S.P;
+    const long long idx = (long long)(blockIdx.x - S.b0) * TPB + threadIdx.x;
+    if (idx >= S.total) return;
+    u64 *b = S.src + (idx >> S.logN) * S.k * N + (idx & (N - 1));
+    u64 w[FHE_MAXK];
+#pragma unroll
+    for (int j = 0; j < FHE_MAXK; j++)
+        if (j < S.k) w[j] = b[(long long)j * N];
+#pragma unroll
+    for (int j = 1; j < FHE_MAXK; j++)
+        if (j < S.k) {
+            const ModQ &m = S.mq[S.l - 1 - j];
+            DotAcc a{0, 0};
+#pragma unroll
+            for (int t = 0; t < FHE_MAXK; t++)
+                if (t < j) {
+                    dot_mac(a, w[t], P->F[j][t], m.half);
+                    if (m.half > 27 && (t & 1)) a = DotAcc{0, dot_fold(a, m)};
+                }
+            w[j] = fold_sub(w[j], dot_fold(a, m), m);
+            b[(long long)j * N] = w[j];
+        }
+}
+
+__global__ void __launch_bounds__(TPB) k_fold_many(const __grid_constant__ FoldTable t)
 {
     pdl_begin();
     const FoldSeg &S = t.s[block_seg(t.s, t.nseg)];
-    if (t.rms && S.vec) {
+    if (t.rms)
         fold_rms_block(S);
-        return;
-    }
-    const int N = 1 << S.logN;
-    const long long base = (long long)(blockIdx.x - S.b0) * EW_ELEMS;
-    for (int e = threadIdx.x; e < EW_ELEMS; e += TPB) {
-        const long long idx = base + e;
-        if (idx >= S.total) break;
-        const long long o = idx >> S.logN;
-        const int n = (int)(idx & (N - 1));
-        if (t.rms) {
-            const RelinMSParams *P = (const RelinMSParams *)S.P;
-            const ModQ mm = S.mq[S.l - 1];
-            u64 *b = S.src + o * (S.K + 1) * N + n;
-            u128 a = 0;
-            for (int k = 0; k < S.K; k++) a += (u128)b[(long long)k * N] * P->pkinv[k];
-            b[(long long)S.K * N] = submod(b[(long long)S.K * N], barrett128(a, mm), mm.q);
-        } else {
-            const MultiSwitchParams *P = (const MultiSwitchParams *)S.P;
-            u64 *b = S.src + o * S.k * N + n;
-            u64 w[FHE_MAXK];
-#pragma unroll
-            for (int j = 0; j < FHE_MAXK; j++) {
-                if (j < S.k) {
-                    const ModQ mj = S.mq[S.l - 1 - j];
-                    u128 a = 0;
-#pragma unroll
-                    for (int q = 0; q < FHE_MAXK; q++)
-                        if (q < j) a += (u128)w[q] * P->F[j][q];
-                    w[j] = submod(b[(long long)j * N], barrett128(a, mj), mj.q);
-                    b[(long long)j * N] = w[j];
-                }
-            }
-        }
-    }
+    else
+        fold_multi_block(S);
 }
 
 int ew_blocks(long long total) { return (int)((total + EW_ELEMS - 1) / EW_ELEMS); }
@@ -535,8 +630,98 @@ void launch_tables(const std::vector<Item> &items, int cls, Fill fill, Launch la
 
 }  // namespace
 
-void launch_ew_many(const std::vector<EwArgs> &items)
+// q_max sum |k_j| < 2^64 over the item's scalars: its combination fits 64 bits
+static bool fits64(const EwArgs &a)
 {
+    u64 qmax = 0;
+    for (u64 q : a.c->q) qmax = q > qmax ? q : qmax;
+    const int nk = a.op == FHE_EW_LINCOMB ? a.n : 1;
+    unsigned __int128 ksum = 0;
+    for (int j = 0; j < nk && j < 8; j++) ksum += (u64)(a.k[j] < 0 ? -a.k[j] : a.k[j]);
+    return ksum * qmax < ((unsigned __int128)1 << 64);
+}
+
+// Linear combinations over the same operands, as many as fit one segment
+// (LC_N operands in all, LC_N outputs): at least two items.
+struct LcItem {
+    fhe_ctx *c;
+    std::vector<const EwArgs *> of;
+    std::vector<const u64 *> x;
+};
+
+// Takes the combinations that share operands out of `items`.
+static std::vector<LcItem> shared_lincombs(const std::vector<EwArgs> &items, std::vector<EwArgs> &rest)
+{
+    std::vector<LcItem> open;
+    for (const EwArgs &a : items) {
+        if (a.op != FHE_EW_LINCOMB || a.n < 1 || !fits64(a)) {
+            rest.push_back(a);
+            continue;
+        }
+        LcItem *to = nullptr;
+        for (LcItem &g : open) {
+            const EwArgs &b = *g.of[0];
+            if (g.c != a.c || b.level != a.level || b.outer != a.outer || (int)g.of.size() == LC_N) continue;
+            int fresh = 0;
+            for (int j = 0; j < a.n; j++) fresh += std::find(g.x.begin(), g.x.end(), a.x[j]) == g.x.end();
+            if (fresh < a.n && (int)g.x.size() + fresh <= LC_N) {
+                to = &g;
+                break;
+            }
+        }
+        if (!to) {
+            open.push_back(LcItem{a.c, {}, {}});
+            to = &open.back();
+        }
+        for (int j = 0; j < a.n; j++)
+            if (std::find(to->x.begin(), to->x.end(), a.x[j]) == to->x.end()) to->x.push_back(a.x[j]);
+        to->of.push_back(&a);
+    }
+    std::vector<LcItem> got;
+    for (LcItem &g : open)
+        if (g.of.size() > 1)
+            got.push_back(g);
+        else
+            rest.push_back(*g.of[0]);
+    return got;
+}
+
+void launch_ew_many(const std::vector<EwArgs> &all)
+{
+    std::vector<EwArgs> items;
+    const std::vector<LcItem> shared = shared_lincombs(all, items);
+    launch_tables<LcTable>(
+        shared, FHE_K_ELEMWISE,
+        [](LcSeg &S, const LcItem &g, double *bytes) {
+            const EwArgs &a = *g.of[0];
+            S.total = (long long)a.outer * a.level * a.c->N;
+            if (S.total <= 0) return 0;
+            bool vec = true;
+            S.n = (int)g.x.size();
+            for (int t = 0; t < S.n; t++) {
+                S.x[t] = g.x[t];
+                vec = vec && ((uintptr_t)g.x[t] & 15) == 0;
+            }
+            S.nout = (int)g.of.size();
+            for (int o = 0; o < S.nout; o++) {
+                const EwArgs &b = *g.of[o];
+                S.out[o] = b.out;
+                vec = vec && ((uintptr_t)b.out & 15) == 0;
+                for (int j = 0; j < b.n; j++) {  // an operand may occur more than once
+                    const int t = (int)(std::find(g.x.begin(), g.x.end(), b.x[j]) - g.x.begin());
+                    S.k[o][t] += (int32_t)b.k[j];
+                }
+                for (int t = 0; t < S.n; t++)
+                    if (S.k[o][t] < 0) S.neg[o] += (uint32_t)-S.k[o][t];
+            }
+            S.mq = a.c->d_mq;
+            S.logN = a.c->logN;
+            S.level = a.level;
+            S.vec = vec;
+            *bytes = 8.0 * (S.n + S.nout) * S.total;
+            return ew_blocks(S.total);
+        },
+        [](const LcTable &t, int blocks, cudaStream_t s) { launch_pdl(k_lincomb_many, blocks, TPB, s, t); });
     launch_tables<EwTable>(
         items, FHE_K_ELEMWISE,
         [](EwSeg &S, const EwArgs &a, double *bytes) {
@@ -552,15 +737,7 @@ void launch_ew_many(const std::vector<EwArgs> &items)
             bool vec = ((uintptr_t)a.out & 15) == 0;
             for (int j = 0; j < 8; j++) vec = vec && ((uintptr_t)a.x[j] & 15) == 0;
             S.vec = vec;
-            // the 64-bit form applies when q_max * sum |k_j| < 2^64
-            {
-                u64 qmax = 0;
-                for (u64 q : a.c->q) qmax = q > qmax ? q : qmax;
-                const int nk = a.op == FHE_EW_LINCOMB ? a.n : 1;
-                unsigned __int128 ksum = 0;
-                for (int j = 0; j < nk && j < 8; j++) ksum += (u64)(a.k[j] < 0 ? -a.k[j] : a.k[j]);
-                S.small = (a.op == FHE_EW_LINCOMB || a.op == FHE_EW_CMUL) && ksum * qmax < ((unsigned __int128)1 << 64);
-            }
+            S.small = (a.op == FHE_EW_LINCOMB || a.op == FHE_EW_CMUL) && fits64(a);
             const int reads = a.op == FHE_EW_LINCOMB ? a.n : (a.op == FHE_EW_ADD || a.op == FHE_EW_SUB) ? 2 : 1;
             *bytes = 8.0 * (reads + 1) * S.total;
             return ew_blocks(S.total);
@@ -682,12 +859,32 @@ void launch_rms_fold_many(const std::vector<FoldArgs> &items)
             S.K = c->K;
             S.vec = ((uintptr_t)a.src & 15) == 0;
             *bytes = 8.0 * (c->K + 2.0) * S.total;
-            return ew_blocks(S.total);
+            return (int)(S.total / FOLD_ELEMS);
         },
         [](FoldTable &t, int blocks, cudaStream_t s) {
             t.rms = 1;
             launch_pdl(k_fold_many, blocks, TPB, s, t);
         });
+}
+
+void launch_rms_fold(fhe_ctx *c, u64 *src, int count, int level)
+{
+    launch_rms_fold_many({FoldArgs{c, src, count, level, 0}});
+}
+
+void launch_ms_fold(fhe_ctx *c, u64 *src, int outer, int level, int k)
+{
+    launch_ms_fold_many({FoldArgs{c, src, outer, level, k}});
+}
+
+void launch_tensor(fhe_ctx *c, const u64 *a, const u64 *b, u64 *out, int count, int level)
+{
+    launch_tensor_many({TensorArgs{c, a, b, out, count, level}});
+}
+
+void launch_add(fhe_ctx *c, const u64 *a, const u64 *b, u64 *out, int outer, int level, int sub)
+{
+    launch_ew_many({EwArgs{c, sub ? FHE_EW_SUB : FHE_EW_ADD, 2, {a, b}, {}, out, outer, level}});
 }
 
 void launch_ms_fold_many(const std::vector<FoldArgs> &items)
@@ -705,7 +902,7 @@ void launch_ms_fold_many(const std::vector<FoldArgs> &items)
             S.l = a.level;
             S.k = a.k;
             *bytes = 8.0 * 2.0 * a.k * S.total;
-            return ew_blocks(S.total);
+            return (int)((S.total + TPB - 1) / TPB);
         },
         [](FoldTable &t, int blocks, cudaStream_t s) {
             t.rms = 0;

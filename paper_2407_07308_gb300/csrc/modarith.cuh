@@ -34,6 +34,33 @@ FHE_HD u64 fhe_mulhi(u64 a, u64 b)
 #endif
 }
 
+// 32 x 32 -> 64 products as single wide multiplications.  Sums of them are
+// written with two products a statement, which become three-input additions
+// on the addition pipe; a C product added to one accumulator at a time puts
+// half of its 64-bit addition on the multiplier pipe (register-resident
+// probes: conversions 531 -> 814 G residues/s, half-word products 6.3 -> 8.5
+// T/s).
+FHE_HD u64 wide_mul(uint32_t a, uint32_t b)
+{
+#ifdef __CUDA_ARCH__
+    u64 p;
+    asm("mul.wide.u32 %0, %1, %2;" : "=l"(p) : "r"(a), "r"(b));
+    return p;
+#else
+    return (u64)a * b;
+#endif
+}
+FHE_HD int64_t wide_mul_s(int32_t a, int32_t b)
+{
+#ifdef __CUDA_ARCH__
+    int64_t p;
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(p) : "r"(a), "r"(b));
+    return p;
+#else
+    return (int64_t)a * b;
+#endif
+}
+
 // Per-prime constants used by the kernels.
 struct ModQ {
     u64 q;       // the prime
@@ -198,19 +225,27 @@ struct HalfAcc {
 // the two halves of x in the two 32-bit words of the result
 FHE_HD u64 half_pack(u64 x, int h) { return ((x >> h) << 32) | (x & (((u64)1 << h) - 1)); }
 
-// acc += x y; xs, ys: the sums of the halves
-FHE_HD void half_mac(HalfAcc &a, uint32_t xl, uint32_t xh, uint32_t xs, uint32_t yl, uint32_t yh, uint32_t ys)
+// one factor's halves and their sum
+struct Halves {
+    uint32_t l, h, s;
+};
+FHE_HD Halves halves(uint32_t l, uint32_t h) { return Halves{l, h, l + h}; }
+FHE_HD Halves halves_of(u64 packed) { return halves((uint32_t)packed, (uint32_t)(packed >> 32)); }
+
+// acc += x y
+FHE_HD void half_mac(HalfAcc &a, const Halves &x, const Halves &y)
 {
-    a.lo += (u64)xl * yl;
-    a.hi += (u64)xh * yh;
-    a.mid += (u64)xs * ys;
+    a.lo += wide_mul(x.l, y.l);
+    a.hi += wide_mul(x.h, y.h);
+    a.mid += wide_mul(x.s, y.s);
 }
 
-// acc += x y, x and y packed halves
-FHE_HD void half_mac(HalfAcc &a, u64 x, u64 y)
+// acc += x y + u v
+FHE_HD void half_mac2(HalfAcc &a, const Halves &x, const Halves &y, const Halves &u, const Halves &v)
 {
-    const uint32_t xl = (uint32_t)x, xh = (uint32_t)(x >> 32), yl = (uint32_t)y, yh = (uint32_t)(y >> 32);
-    half_mac(a, xl, xh, xl + xh, yl, yh, yl + yh);
+    a.lo = a.lo + wide_mul(x.l, y.l) + wide_mul(u.l, v.l);
+    a.hi = a.hi + wide_mul(x.h, y.h) + wide_mul(u.h, v.h);
+    a.mid = a.mid + wide_mul(x.s, y.s) + wide_mul(u.s, v.s);
 }
 
 // The sum S of n <= 8 products of canonical residues, divided by 2^(2h):
@@ -255,10 +290,8 @@ struct DotAcc {
 // x in half words: xl = x mod 2^h, xh = x >> h, below 2^31 each
 FHE_HD void dot_mac(DotAcc &a, uint32_t xl, uint32_t xh, const DotC &c)
 {
-    a.l += (int64_t)(int32_t)xl * c.wl;
-    a.h += (int64_t)(int32_t)xl * c.wh;
-    a.l += (int64_t)(int32_t)xh * c.vl;
-    a.h += (int64_t)(int32_t)xh * c.vh;
+    a.l = a.l + wide_mul_s((int32_t)xl, c.wl) + wide_mul_s((int32_t)xh, c.vl);
+    a.h = a.h + wide_mul_s((int32_t)xl, c.wh) + wide_mul_s((int32_t)xh, c.vh);
 }
 
 FHE_HD void dot_mac(DotAcc &a, u64 x, const DotC &c, int h)

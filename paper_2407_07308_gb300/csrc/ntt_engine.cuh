@@ -42,7 +42,8 @@
 // replay) and on 7 pairs at N = 2^15 (p = 257, 3 digits, level 17): 12.0 and
 // 59.8 ms with conversions in 128-bit arithmetic, normalised inverse
 // butterflies and three conflicting exchanges a pass; 12.1 and 57.6 ms with
-// the arithmetic below alone; 11.2 and 50.0 ms with the layouts too.
+// the arithmetic below alone; 11.2 and 50.0 ms with the layouts too; 9.7 and
+// 41.1 ms with joined segments and sums of two products a statement.
 //
 // Segments and persistence.  A launch carries a table of up to FHE_SEGS
 // segments; a segment is one batch of limb jobs with its own context (ring
@@ -540,37 +541,25 @@ __device__ __forceinline__ void conv_pair(const Conv &a, const Conv &b, const Mo
     }
 }
 
-// One target at P positions.
-template <int P, int STEP, int NN>
-__device__ __forceinline__ void conv_one(const Conv &a, const ModQ &m, int n, u64 (&v)[P])
+// One target at position n.
+template <int NN>
+__device__ __forceinline__ u64 conv_one(const Conv &a, const ModQ &m, int n)
 {
-    DotAcc s[P];
-#pragma unroll
-    for (int p = 0; p < P; p++) s[p] = DotAcc{0, (int64_t)(2 * m.q2)};
-    const int h = m.half, ns = a.n;
+    DotAcc s{0, (int64_t)(2 * m.q2)};
     const u64 *src = a.src + n;
 #pragma unroll 1
-    for (int i0 = 0; i0 < ns; i0 += 4) {
-        u64 x[4][P];
+    for (int i0 = 0; i0 < a.n; i0 += 4) {
+        u64 x[4];
 #pragma unroll
-        for (int i = 0; i < 4; i++)
-            if (i0 + i < ns) {
+        for (int i = 0; i < 4; i++) x[i] = i0 + i < a.n ? src[(size_t)i * NN] : 0;
 #pragma unroll
-                for (int p = 0; p < P; p++) x[i][p] = src[(size_t)i * NN + p * STEP];
-            }
-#pragma unroll
-        for (int i = 0; i < 4; i++)
-            if (i0 + i < ns) {
-#pragma unroll
-                for (int p = 0; p < P; p++) {
-                    dot_mac(s[p], x[i][p], a.c[i0 + i], h);
-                    if (h > 27 && (i & 1)) s[p] = DotAcc{0, dot_fold(s[p], m)};
-                }
-            }
+        for (int i = 0; i < 4; i++) {
+            if (i0 + i < a.n) dot_mac(s, x[i], a.c[i0 + i], m.half);
+            if (m.half > 27 && (i & 1)) s = DotAcc{0, dot_fold(s, m)};
+        }
         src += (size_t)4 * NN;
     }
-#pragma unroll
-    for (int p = 0; p < P; p++) v[p] = (u64)dot_fold(s[p], m);
+    return (u64)dot_fold(s, m);
 }
 
 // ---------------------------------------------------------------------------
@@ -761,13 +750,10 @@ __device__ __forceinline__ void inv_cols_unit1(const IO &io, int sg, int lu, u64
 template <int NN, class IO>
 __device__ __forceinline__ u64 col_load(const IO &io, int sg, const typename IO::CSt &st, int n)
 {
-    if constexpr (IO::XJ == 2) {
-        u64 v[1];
-        conv_one<1, 0, NN>(st.cv, io.h[sg].mq[st.prime], n, v);
-        return v[0];
-    } else {
+    if constexpr (IO::XJ == 2)
+        return conv_one<NN>(st.cv, io.h[sg].mq[st.prime], n);
+    else
         return io.load(st, n);
-    }
 }
 
 // Forward, columns: global stages 0..N1-1.
@@ -820,12 +806,9 @@ __device__ __forceinline__ void fwd_cols_unit(const IO &io, int sg, int lu, u64 
 #pragma unroll 1
             for (int j = 0; j < 2 && j < nvalid; j++)
 #pragma unroll 1
-                for (int k = 0; k < 8; k += CONV_P) {
-                    u64 v[CONV_P];
-                    conv_one<CONV_P, (ES << N2), Gm::NN>(sts[j].cv, j == 0 ? m0 : m1, ((e0 + k * ES) << N2) + lo0 + col, v);
-#pragma unroll
-                    for (int p = 0; p < CONV_P; p++) sm[Gm::Lay::at(j * Gm::NC + col, e0 + (k + p) * ES)] = v[p];
-                }
+                for (int k = 0; k < 8; k++)
+                    sm[Gm::Lay::at(j * Gm::NC + col, e0 + k * ES)] =
+                        conv_one<Gm::NN>(sts[j].cv, j == 0 ? m0 : m1, ((e0 + k * ES) << N2) + lo0 + col);
         }
     } else {
 #pragma unroll 1
@@ -1024,10 +1007,32 @@ __device__ __forceinline__ void inv_rows_unit(const IO &io, int sg, int lu, u64 
     const ModQ &m = H.mq[prime];
     const ulonglong2 *tw = H.tw + (size_t)prime * Gm::NN;
     if (GRP) row_twiddles<N1, N2>(W, tw, hi0);
+    // a unit's jobs are of one map entry, so either all or none have an addend
+    // per polynomial; its words are computed on the way, eight at a time with
+    // all loads before the first store (one at a time, each store held the
+    // next loads back: 16 pairs at N = 2^14 1.04 -> 0.83 ms of these passes)
+    if (io.adds(sts[0]) || io.adds(sts[nvalid > 1 ? 1 : 0])) {
+#pragma unroll 1
+        for (int k0 = 0; k0 < 16; k0 += 8) {
+            u64 v[8], w[8];
 #pragma unroll
-    for (int k = 0; k < 16; k++) {
-        const int r = tid + k * T, j = mp.slot(r);
-        if (j < nvalid) io.load_async(&sm[Lay::at(mp.c(r), mp.f(r))], sts[j], (mp.row(r) << N2) + mp.f(r));
+            for (int k = 0; k < 8; k++) {
+                const int r = tid + (k0 + k) * T, j = mp.slot(r), i = (mp.row(r) << N2) + mp.f(r);
+                v[k] = j < nvalid ? sts[j].in[i] : 0;
+                w[k] = j < nvalid ? io.addend(sts[j], i) : 0;
+            }
+#pragma unroll
+            for (int k = 0; k < 8; k++) {
+                const int r = tid + (k0 + k) * T, j = mp.slot(r);
+                if (j < nvalid) sm[Lay::at(mp.c(r), mp.f(r))] = io.sum(sts[j], v[k], w[k]);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 16; k++) {
+            const int r = tid + k * T, j = mp.slot(r);
+            if (j < nvalid) async8(&sm[Lay::at(mp.c(r), mp.f(r))], sts[j].in + (mp.row(r) << N2) + mp.f(r));
+        }
     }
     async_wait();
     __syncthreads();
@@ -1213,7 +1218,10 @@ struct IOMap : SegIO<MapSeg> {
     static constexpr bool PLAIN = true;  // a column pass loads src's words as they are
     __device__ const u64 *src(const CSt &t) const { return t.in; }
     __device__ u64 load(const CSt &t, int i) const { return t.in[i]; }
-    __device__ void load_async(u64 *dst, const RSt &t, int i) const { async8(dst, t.in + i); }
+    // the inverse row pass's word: the limb's alone
+    __device__ static constexpr bool adds(const RSt &) { return false; }
+    __device__ u64 addend(const RSt &, int) const { return 0; }
+    __device__ u64 sum(const RSt &, u64 v, u64) const { return v; }
     __device__ void store(const CSt &t, int i, u64 v) const { t.out[i] = v; }
     static constexpr int NPRE = 0;  // operands the store reads
     __device__ u64 pre(const RSt &, int, int) const { return 0; }
@@ -1268,14 +1276,10 @@ struct IOScaledY : SegIO<YSeg> {
         t.Pm_s = S.Pm_s;
         t.qm = S.qm;
     }
-    // the y entry (a unit's jobs are all of one entry) is computed on the way
-    __device__ void load_async(u64 *dst, const RSt &t, int i) const
-    {
-        if (t.add)  // an accumulator below 2q and a product below q
-            *dst = t.in[i] + shoup(t.add[i], t.Pm, t.Pm_s, t.qm);
-        else
-            async8(dst, t.in + i);
-    }
+    // the y entry's word: an accumulator below 2q and a product below q
+    __device__ static bool adds(const RSt &t) { return t.add != nullptr; }
+    __device__ u64 addend(const RSt &t, int i) const { return t.add ? t.add[i] : 0; }
+    __device__ u64 sum(const RSt &t, u64 v, u64 w) const { return t.add ? v + shoup(w, t.Pm, t.Pm_s, t.qm) : v; }
     __device__ void store(const CSt &t, int i, u64 v) const { t.out[i] = v; }
     static constexpr int NPRE = 0;
     __device__ u64 *inter(const MapSt &t) const { return t.out; }

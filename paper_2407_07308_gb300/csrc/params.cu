@@ -296,7 +296,7 @@ int build_tables(fhe_ctx *c)
         for (int k = 0; k < K; k++) {
             const u64 pk = c->q[L + k];
             Pm = host_mulmod(Pm, pk % qm, qm);
-            R.pkinv[k] = host_invmod(pk % qm, qm);
+            R.pkinv[k] = dot_const(host_invmod(pk % qm, qm), c->mq[l - 1]);
         }
         R.Pm = Pm;
         R.Pm_s = shoup_const(Pm, qm);
@@ -335,7 +335,7 @@ int build_tables(fhe_ctx *c)
                 std::vector<u64> D(j + 1, 1);  // D_t mod q_j, t <= j
                 for (int t = 1; t <= j; t++) D[t] = host_mulmod(D[t - 1], c->q[l - t] % qj, qj);
                 const u64 Djinv = host_invmod(D[j], qj);
-                for (int t = 0; t < j; t++) S.F[j][t] = host_mulmod(D[t], Djinv, qj);
+                for (int t = 0; t < j; t++) S.F[j][t] = dot_const(host_mulmod(D[t], Djinv, qj), c->mq[l - 1 - j]);
                 const u64 ni = host_invmod((u64)N % qj, qj);
                 const u64 v = host_mulmod(host_mulmod(ni, host_invmod(c->p % qj, qj), qj), Djinv, qj);
                 c->mss_scale[((size_t)l * (FHE_MAXK + 1) + k) * FHE_MAXK + j] = make_ulonglong2(v, shoup_const(v, qj));
