@@ -755,6 +755,7 @@ struct Dag {
         cudaStream_t s = c->branch_streams[k];
         for (size_t m = 0; m < mem.size(); m++) {
             mem[m]->stream = s;
+            mem[m]->on_branch = true;
             mem[m]->pool.stream = s;
             mem[m]->pool.cap_free = &frees[m][k];
         }
@@ -815,6 +816,7 @@ struct Dag {
         for (size_t m = 0; m < mem.size(); m++) {
             fhe_ctx *x = mem[m];
             x->stream = main;
+            x->on_branch = false;
             x->pool.stream = main;
             x->pool.cap_free = main_free[m];
             for (auto &f : frees[m])

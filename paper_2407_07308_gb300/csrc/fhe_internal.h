@@ -230,6 +230,7 @@ struct fhe_ctx {
     // them concurrently.  Each branch has its own capture-private free list.
     bool capturing = false;
     bool multistream = false;  // the same scheduling without capture (batch execution)
+    bool on_branch = false;    // launches go to one of the scheduler's streams (see pdl.cuh)
     int wave_split = 2;        // a circuit's product wave runs as this many merged operations (streams)
     std::vector<cudaStream_t> branch_streams;
     std::vector<cudaEvent_t> branch_events;  // reused by every capture
@@ -243,6 +244,12 @@ struct fhe_ctx {
     BatchPlan *bplan_active = nullptr;  // the graph being replayed (kept when memory runs out)
     long long launches = 0;       // kernels launched since creation
 };
+
+// whether a launch of grid x block threads overlaps its predecessor (pdl.cuh)
+inline bool pdl_on(const fhe_ctx *c, int grid, int block)
+{
+    return !c->on_branch || (long long)grid * block <= (long long)FHE_PDL_THREADS * c->sms;
+}
 
 struct fhe_batch;
 int batch_job_done(fhe_batch *B, int job);  // 1 once job `job` of the batch has its results

@@ -394,17 +394,19 @@ __device__ __forceinline__ void ks_sum(u64 *w, const u64 *(&ep)[KS_CB], const u6
     const uint32_t mask = ((uint32_t)1 << h) - 1;
     {
         u64 *d = w;
-        for (int j = 0; j < dnum; j++) {
+        for (int j = 0; j < dnum; j++, kp += 2 * kstride, d += (2 + KS_CB) * TPB) {
             async8(d, kp);
             async8(d + TPB, kp + kstride);
+        }
+        pdl_wait();
+        d = w;
+        for (int j = 0; j < dnum; j++, d += (2 + KS_CB) * TPB) {
 #pragma unroll
             for (int cc = 0; cc < KS_CB; cc++) {
                 if (FULL || cc < ncb) async8(d + (2 + cc) * TPB, j == rdig ? own(cc) : ep[cc]);
                 ep[cc] += dstride;
             }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            kp += 2 * kstride;
-            d += (2 + KS_CB) * TPB;
+            asm volatile("cp.async.commit_group;" ::: "memory");  // the first also holds the key words
         }
     }
     HalfAcc a0[KS_CB], a1[KS_CB];
@@ -448,7 +450,7 @@ __device__ __forceinline__ void ks_sum(u64 *w, const u64 *(&ep)[KS_CB], const u6
 
 __global__ void __launch_bounds__(TPB, FHE_KS_MINB) k_ks_inner_many(const __grid_constant__ KsTable t)
 {
-    pdl_begin();
+    pdl_trigger();
     extern __shared__ u64 ks_words[];  // [dnum][2 + KS_CB][TPB]
     const int sg = block_seg(t.s, t.nseg);
     const KsSeg &S = t.s[sg];
@@ -622,7 +624,7 @@ void launch_tables(const std::vector<Item> &items, int cls, Fill fill, Launch la
         }
         if (!t.nseg) continue;
         prof_begin(c, cls, bytes);
-        launch(t, blocks, c->stream);
+        launch(t, pdl_on(c, blocks, TPB), blocks, c->stream);
         prof_end(c);
         c->launches++;
     }
@@ -721,7 +723,7 @@ void launch_ew_many(const std::vector<EwArgs> &all)
             *bytes = 8.0 * (S.n + S.nout) * S.total;
             return ew_blocks(S.total);
         },
-        [](const LcTable &t, int blocks, cudaStream_t s) { launch_pdl(k_lincomb_many, blocks, TPB, s, t); });
+        [](const LcTable &t, bool pdl, int blocks, cudaStream_t s) { launch_pdl(k_lincomb_many, pdl, blocks, TPB, s, t); });
     launch_tables<EwTable>(
         items, FHE_K_ELEMWISE,
         [](EwSeg &S, const EwArgs &a, double *bytes) {
@@ -742,7 +744,7 @@ void launch_ew_many(const std::vector<EwArgs> &all)
             *bytes = 8.0 * (reads + 1) * S.total;
             return ew_blocks(S.total);
         },
-        [](const EwTable &t, int blocks, cudaStream_t s) { launch_pdl(k_ew_many, blocks, TPB, s, t); });
+        [](const EwTable &t, bool pdl, int blocks, cudaStream_t s) { launch_pdl(k_ew_many, pdl, blocks, TPB, s, t); });
 }
 
 void launch_tensor_many(const std::vector<TensorArgs> &items)
@@ -762,7 +764,7 @@ void launch_tensor_many(const std::vector<TensorArgs> &items)
             *bytes = 8.0 * 7 * S.total;
             return ew_blocks(S.total);
         },
-        [](const TensorTable &t, int blocks, cudaStream_t s) { launch_pdl(k_tensor_many, blocks, TPB, s, t); });
+        [](const TensorTable &t, bool pdl, int blocks, cudaStream_t s) { launch_pdl(k_tensor_many, pdl, blocks, TPB, s, t); });
 }
 
 // shared memory of a block for dnum digits
@@ -831,7 +833,7 @@ void launch_ks_inner_many(const std::vector<KsInnerArgs> &items)
                 allowed[dev] = cudaFuncSetAttribute(k_ks_inner_many, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                     ks_bytes(FHE_MAXD)) == cudaSuccess;
         }
-        launch_pdl_smem(k_ks_inner_many, blocks, TPB, ks_bytes(dmax), c0->stream, t);
+        launch_pdl_smem(k_ks_inner_many, pdl_on(c0, blocks, TPB), blocks, TPB, ks_bytes(dmax), c0->stream, t);
         prof_end(c0);
         c0->launches++;
     }
@@ -861,9 +863,9 @@ void launch_rms_fold_many(const std::vector<FoldArgs> &items)
             *bytes = 8.0 * (c->K + 2.0) * S.total;
             return (int)(S.total / FOLD_ELEMS);
         },
-        [](FoldTable &t, int blocks, cudaStream_t s) {
+        [](FoldTable &t, bool pdl, int blocks, cudaStream_t s) {
             t.rms = 1;
-            launch_pdl(k_fold_many, blocks, TPB, s, t);
+            launch_pdl(k_fold_many, pdl, blocks, TPB, s, t);
         });
 }
 
@@ -904,8 +906,8 @@ void launch_ms_fold_many(const std::vector<FoldArgs> &items)
             *bytes = 8.0 * 2.0 * a.k * S.total;
             return (int)((S.total + TPB - 1) / TPB);
         },
-        [](FoldTable &t, int blocks, cudaStream_t s) {
+        [](FoldTable &t, bool pdl, int blocks, cudaStream_t s) {
             t.rms = 0;
-            launch_pdl(k_fold_many, blocks, TPB, s, t);
+            launch_pdl(k_fold_many, pdl, blocks, TPB, s, t);
         });
 }

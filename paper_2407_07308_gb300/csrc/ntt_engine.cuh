@@ -688,6 +688,7 @@ __device__ __forceinline__ void fwd_cols_unit1(const IO &io, int sg, int lu, u64
     col_twiddles<N1>(W, H.tw + (size_t)st.prime * Gm::NN);
     const ModQ &m = H.mq[st.prime];
     const ColTw<N1, N2, IO::XJ> geo{W, m.q, m.q, &m, &m};
+    pdl_wait();
     u64 x[16];
     const u64 *src = io.src(st) + (g << N2) + lo;
 #pragma unroll
@@ -729,6 +730,7 @@ __device__ __forceinline__ void inv_cols_unit1(const IO &io, int sg, int lu, u64
     col_twiddles<N1>(W, H.tw + (size_t)st.prime * Gm::NN);
     const ModQ &m = H.mq[st.prime];
     const ColTw<N1, N2, IO::XJ> geo{W, m.q, m.q, &m, &m};
+    pdl_wait();
     u64 x[16];
     const u64 *mid = io.inter(st) + (g << (N2 + 4)) + lo;
 #pragma unroll
@@ -774,6 +776,7 @@ __device__ __forceinline__ void fwd_cols_unit(const IO &io, int sg, int lu, u64 
     const ModQ &m0 = H.mq[sts[0].prime], &m1 = H.mq[sts[nvalid > 1 ? Gm::NJ - 1 : 0].prime];
     for (int j = 0; j < Gm::NJ && j < nvalid; j++)
         col_twiddles<N1>(W + j * Gm::TWC, H.tw + (size_t)sts[j].prime * Gm::NN);
+    pdl_wait();
     bool paired = false;
     if constexpr (Gm::PAIRED) {
         // both slots at once: column col of slot 0 and of slot 1 at the same
@@ -860,6 +863,7 @@ __device__ __forceinline__ void inv_cols_unit(const IO &io, int sg, int lu, u64 
     const ColTw<N1, N2, IO::XJ> geo{W, m0.q, m1.q, &m0, &m1};
     // a slot without a job transforms the first job's words and stores nothing
     const int j = c / Gm::NC, lo = lo0 + c % Gm::NC, jv = j < nvalid ? j : 0;
+    pdl_wait();
     u64 x[16];
     const u64 *mid = io.inter(sts[jv]) + (g << (N2 + 4)) + lo;
 #pragma unroll
@@ -952,6 +956,7 @@ __device__ __forceinline__ void fwd_rows_unit(const IO &io, int sg, int lu, u64 
     const ModQ &m = H.mq[prime];
     const ulonglong2 *tw = H.tw + (size_t)prime * Gm::NN;
     if (GRP) row_twiddles<N1, N2>(W, tw, hi0);
+    pdl_wait();
     // thread (c, g) reads its first round's words: runs of G words
     const int c = tid / C::G, g = tid % C::G;
     u64 x[16];
@@ -1007,6 +1012,7 @@ __device__ __forceinline__ void inv_rows_unit(const IO &io, int sg, int lu, u64 
     const ModQ &m = H.mq[prime];
     const ulonglong2 *tw = H.tw + (size_t)prime * Gm::NN;
     if (GRP) row_twiddles<N1, N2>(W, tw, hi0);
+    pdl_wait();
     // a unit's jobs are of one map entry, so either all or none have an addend
     // per polynomial; its words are computed on the way, eight at a time with
     // all loads before the first store (one at a time, each store held the
@@ -1084,7 +1090,7 @@ template <class IO, int L>
 __global__ void __launch_bounds__(T, IO::XJ == 2 ? FHE_NTT_MINB_PAIRED : FHE_NTT_MINB)
     k_fwd_cols(const __grid_constant__ IO io)
 {
-    pdl_begin();
+    pdl_trigger();
     __shared__ u64 sm[ColGeo<Deg<L>::N1, Deg<L>::N2, IO::XJ>::Lay::WORDS];
     __shared__ ulonglong2 W[ColGeo<Deg<L>::N1, Deg<L>::N2, IO::XJ>::TW];
     __shared__ typename IO::CSt sts[ColGeo<Deg<L>::N1, Deg<L>::N2, IO::XJ>::NJ];
@@ -1099,7 +1105,7 @@ template <class IO, int L>
 __global__ void __launch_bounds__(T, FHE_NTT_MINB)
     k_fwd_rows(const __grid_constant__ IO io)
 {
-    pdl_begin();
+    pdl_trigger();
     __shared__ u64 sm[ROW_WORDS];
     __shared__ ulonglong2 W[TW_ROWS];
     __shared__ typename IO::RSt sts[ROW_J];
@@ -1116,7 +1122,7 @@ __global__ void __launch_bounds__(T, FHE_NTT_MINB)
 template <class IO, int L>
 __global__ void __launch_bounds__(T, FHE_NTT_MINB) k_inv_rows(const __grid_constant__ IO io)
 {
-    pdl_begin();
+    pdl_trigger();
     __shared__ u64 sm[ROW_WORDS];
     __shared__ ulonglong2 W[TW_ROWS];
     __shared__ typename IO::RSt sts[ROW_J];
@@ -1133,7 +1139,7 @@ __global__ void __launch_bounds__(T, FHE_NTT_MINB) k_inv_rows(const __grid_const
 template <class IO, int L>
 __global__ void __launch_bounds__(T, FHE_NTT_MINB) k_inv_cols(const __grid_constant__ IO io)
 {
-    pdl_begin();
+    pdl_trigger();
     __shared__ u64 sm[ColGeo<Deg<L>::N1, Deg<L>::N2, IO::XJ>::Lay::WORDS];
     __shared__ ulonglong2 W[ColGeo<Deg<L>::N1, Deg<L>::N2, IO::XJ>::TW];
     __shared__ typename IO::CSt sts[ColGeo<Deg<L>::N1, Deg<L>::N2, IO::XJ>::NJ];
@@ -1680,13 +1686,13 @@ void launch_passes(fhe_ctx *c, const IO &io, bool fwd)
 {
     if constexpr ((IO::DIRS & DIR_FWD) != 0)
         if (fwd) {
-            launch_pdl(k_fwd_cols<IO, L>, grid_of(c, io.ucols), T, c->stream, io);
-            launch_pdl(k_fwd_rows<IO, L>, grid_of(c, io.urows), T, c->stream, io);
+            launch_pdl(k_fwd_cols<IO, L>, pdl_on(c, grid_of(c, io.ucols), T), grid_of(c, io.ucols), T, c->stream, io);
+            launch_pdl(k_fwd_rows<IO, L>, pdl_on(c, grid_of(c, io.urows), T), grid_of(c, io.urows), T, c->stream, io);
         }
     if constexpr ((IO::DIRS & DIR_INV) != 0)
         if (!fwd) {
-            launch_pdl(k_inv_rows<IO, L>, grid_of(c, io.urows), T, c->stream, io);
-            launch_pdl(k_inv_cols<IO, L>, grid_of(c, io.ucols), T, c->stream, io);
+            launch_pdl(k_inv_rows<IO, L>, pdl_on(c, grid_of(c, io.urows), T), grid_of(c, io.urows), T, c->stream, io);
+            launch_pdl(k_inv_cols<IO, L>, pdl_on(c, grid_of(c, io.ucols), T), grid_of(c, io.ucols), T, c->stream, io);
         }
     c->launches += 2;
 }

@@ -1,38 +1,50 @@
 // pdl.cuh -- programmatic dependent launch for the hot kernels.
 //
-// A kernel launched with launch_pdl may have its CTAs made resident while
+// A kernel launched with the attribute may have its CTAs made resident while
 // the previous kernel on its stream is still finishing (that kernel lets its
-// dependents launch once all of its CTAs have started); every such kernel
-// first calls pdl_begin(), which lets its own dependents launch and then
-// waits until all prerequisite grids have completed and their memory
-// operations are visible -- before it reads or writes any global memory.
-// In a captured graph the launches become programmatic edges.  A kernel
-// launched without the attribute passes pdl_begin() at once.
+// dependents launch once all of its CTAs have started, pdl_trigger); it finds
+// its unit and fetches tables that no kernel writes (twiddles, level
+// constants, key words) and then waits until all prerequisite grids have
+// completed and their memory operations are visible (pdl_wait) -- before it
+// reads or writes anything another kernel touches.  Every kernel of this kind
+// waits in every CTA, so completion carries over from launch to launch.  In a
+// captured graph the launches become programmatic edges.  A kernel launched
+// without the attribute passes both at once.
 //
-// Off by default (FHE_PDL 0: plain launches): measured on the 16-pair
-// comparison, the waiting CTAs hold SM slots that the concurrent stream's
-// kernels would use, 2415 against 2454 slot-comparisons/s.
+// Where it is used: always on a context's own stream, where every launch
+// follows the one before (launch and prologue are then hidden: one less-than
+// on the small ring 668 -> 508 us, one LT + EQ at N = 2^14 2249 -> 2116 us,
+// tournament of 8 ciphertexts 171.8 -> 164.3 ms); under the dependency
+// scheduler, whose streams run side by side, only for launches of at most
+// FHE_PDL_THREADS threads per SM, since waiting CTAs hold slots that another
+// stream's kernels would use (16 pairs as a graph: 9.62 ms without, 9.63 at
+// 256, 9.69 at 512, 9.84 with all; 32 uneven requests 46.8, 46.5, 46.5, 46.3).
 #pragma once
 #include <cuda_runtime.h>
 
 #include <utility>
 
-#ifndef FHE_PDL
-#define FHE_PDL 0
+#ifndef FHE_PDL_THREADS
+#define FHE_PDL_THREADS 256
 #endif
+
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ void pdl_begin()
 {
-#if FHE_PDL
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-#endif
+    pdl_trigger();
+    pdl_wait();
 }
 
 template <class... KArgs, class... Args>
-inline void launch_pdl_smem(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, Args &&...args)
+inline void launch_pdl_smem(void (*kernel)(KArgs...), bool overlap, int grid, int block, size_t smem, cudaStream_t s,
+                            Args &&...args)
 {
-#if FHE_PDL
+    if (!overlap) {
+        kernel<<<grid, block, smem, s>>>(std::forward<Args>(args)...);
+        return;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)block);
@@ -44,13 +56,10 @@ inline void launch_pdl_smem(void (*kernel)(KArgs...), int grid, int block, size_
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);  // errors surface in cudaGetLastError
-#else
-    kernel<<<grid, block, smem, s>>>(std::forward<Args>(args)...);
-#endif
 }
 
 template <class... KArgs, class... Args>
-inline void launch_pdl(void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args &&...args)
+inline void launch_pdl(void (*kernel)(KArgs...), bool overlap, int grid, int block, cudaStream_t s, Args &&...args)
 {
-    launch_pdl_smem(kernel, grid, block, 0, s, std::forward<Args>(args)...);
+    launch_pdl_smem(kernel, overlap, grid, block, 0, s, std::forward<Args>(args)...);
 }
