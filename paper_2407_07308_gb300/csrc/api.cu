@@ -247,22 +247,23 @@ void primes_range(int *pr, int n, int off)
     for (int i = 0; i < n; i++) pr[i] = off + i;
 }
 
-// slot values (n_s) -> plaintext coefficients (N), values in [0, p)
-void encode_slots(const fhe_ctx *c, const uint64_t *v, int64_t *m)
+// slot values (n_s) -> the M plaintext coefficients of the subring, in [0, p)
+// (coefficient j belongs to X^(j N / M))
+void encode_sub(const fhe_ctx *c, const uint64_t *v, int64_t *m)
 {
     const u64 p = c->p;
-    const int M = c->M, stride = c->N / M;
-    memset(m, 0, sizeof(int64_t) * c->N);
+    const int M = c->M;
     if (c->slots_linear) {
-        // m_j = M^-1 sum_s v_s zeta^(-e_s j)
+        // m_j = M^-1 sum_s v_s zeta^(-e_s j), powers of zeta from a table
+        std::vector<u64> pw(2 * M);
+        pw[0] = 1;
+        for (int k = 1; k < 2 * M; k++) pw[k] = pw[k - 1] * c->zeta % p;
         const u64 Minv = host_invmod(M % p, p);
         for (int j = 0; j < M; j++) {
             u64 acc = 0;
-            for (int s = 0; s < c->ns; s++) {
-                const u64 e = (u64)((2 * M - (int64_t)c->slot_exp[s] * j % (2 * M)) % (2 * M));
-                acc = (acc + (v[s] % p) * host_powmod(c->zeta, e, p)) % p;
-            }
-            m[(size_t)j * stride] = (int64_t)host_mulmod(acc, Minv, p);
+            for (int s = 0; s < c->ns; s++)
+                acc = (acc + (v[s] % p) * pw[(2 * M - (int64_t)c->slot_exp[s] * j % (2 * M)) % (2 * M)]) % p;
+            m[j] = (int64_t)host_mulmod(acc, Minv, p);
         }
     } else {
         // two slots: m = (v0+v1)/2 + (v0-v1)/2 h(Y), h = -(Y + Y^3)/gamma
@@ -270,25 +271,33 @@ void encode_slots(const fhe_ctx *c, const uint64_t *v, int64_t *m)
         const u64 a = (v[0] % p + v[1] % p) % p * inv2 % p;
         const u64 b = (v[0] % p + p - v[1] % p) % p * inv2 % p;
         const u64 h = (p - ig) % p;
+        for (int j = 0; j < M; j++) m[j] = 0;
         m[0] = (int64_t)a;
-        m[(size_t)1 * stride] = (int64_t)(b * h % p);
-        m[(size_t)3 * stride] = (int64_t)(b * h % p);
+        m[1] = m[3] = (int64_t)(b * h % p);
     }
 }
 
-// plaintext coefficients in [0, p) -> slots; false if not a slot encoding
-bool decode_slots(const fhe_ctx *c, const int64_t *m, uint64_t *v)
+// slot values (n_s) -> plaintext coefficients (N), values in [0, p)
+void encode_slots(const fhe_ctx *c, const uint64_t *v, int64_t *m)
+{
+    std::vector<int64_t> sub(c->M);
+    encode_sub(c, v, sub.data());
+    memset(m, 0, sizeof(int64_t) * c->N);
+    for (int j = 0; j < c->M; j++) m[(size_t)j * (c->N / c->M)] = sub[j];
+}
+
+// the subring's M plaintext coefficients in [0, p) -> slots; false if not a
+// slot encoding
+bool decode_sub(const fhe_ctx *c, const int64_t *m, uint64_t *v)
 {
     const u64 p = c->p;
-    const int M = c->M, stride = c->N / M;
-    for (int n = 0; n < c->N; n++)
-        if (n % stride && m[n]) return false;
+    const int M = c->M;
     if (c->slots_linear) {
         for (int s = 0; s < c->ns; s++) {
             const u64 z = host_powmod(c->zeta, (u64)c->slot_exp[s], p);
             u64 acc = 0, zz = 1;
             for (int j = 0; j < M; j++) {
-                acc = (acc + (u64)m[(size_t)j * stride] * zz) % p;
+                acc = (acc + (u64)m[j] * zz) % p;
                 zz = zz * z % p;
             }
             v[s] = acc;
@@ -299,7 +308,7 @@ bool decode_slots(const fhe_ctx *c, const int64_t *m, uint64_t *v)
         const u64 g = s == 0 ? c->gamma : p - c->gamma;  // factor Y^2 + g Y - 1
         u64 a0 = 0, a1 = 0, w0 = 1, w1 = 0;             // residue and Y^j mod factor
         for (int j = 0; j < M; j++) {
-            const u64 mj = (u64)m[(size_t)j * stride];
+            const u64 mj = (u64)m[j];
             a0 = (a0 + mj * w0) % p;
             a1 = (a1 + mj * w1) % p;
             const u64 n0 = w1, n1 = (w0 + p - g * w1 % p) % p;  // Y (w0 + w1 Y), Y^2 = 1 - gY
@@ -327,8 +336,6 @@ int sync_check(fhe_ctx *c, const char *where)
 
 void encode_slot_vector(const fhe_ctx *c, const uint64_t *v, int64_t *m) { encode_slots(c, v, m); }
 
-// Stream tags of the seeded samplers (see sample.cu).
-enum { TAG_S = 1, TAG_E_PK = 2, TAG_A_PK = 3, TAG_U = 16, TAG_E0 = 17, TAG_E1 = 18, TAG_KSK = 1024 };
 
 // ---------------------------------------------------------------------------
 // context
@@ -536,9 +543,9 @@ static int keygen_dev(fhe_ctx *c, const int64_t *ds, const u64 *da, const int64_
     cudaMemcpyAsync(ta.p, da, sizeof(u64) * L * N, cudaMemcpyDeviceToDevice, c->stream);
     int pr[FHE_MAXP];
     primes_range(pr, np, 0);
-    launch_rns_from_i64(c, ds, nullptr, 1, S->d_s, 1, np, pr);
+    launch_rns_from_i64(c, ds, 1, S->d_s, 1, np, pr);
     ntt_blocks(c, S->d_s, S->d_s, 1, np, 0, false);
-    launch_rns_from_i64(c, de, nullptr, (int64_t)c->p, te.u(), 1, L, pr);
+    launch_rns_from_i64(c, de, (int64_t)c->p, te.u(), 1, L, pr);
     ntt_blocks(c, te.u(), te.u(), 1, L, 0, false);
     u64 *pk1 = Pk->d + (size_t)L * N;
     ntt_blocks(c, ta.u(), pk1, 1, L, 0, false);
@@ -645,7 +652,7 @@ static int evk_create(fhe_ctx *c, const fhe_sk *sk, const int64_t *galois, int n
                 cudaMemcpyAsync(de.p, e + off * N, sizeof(int64_t) * N, cudaMemcpyHostToDevice, c->stream);
             }
             ntt_blocks(c, ta.u(), ta.u(), 1, np, 0, false);
-            launch_rns_from_i64(c, de.i(), nullptr, (int64_t)c->p, te.u(), 1, np, pr);
+            launch_rns_from_i64(c, de.i(), (int64_t)c->p, te.u(), 1, np, pr);
             ntt_blocks(c, te.u(), te.u(), 1, np, 0, false);
             u64 *k0 = k.d + (size_t)(j * 2 + 0) * np * N, *k1 = k.d + (size_t)(j * 2 + 1) * np * N;
             launch_ksk_digit(c, ta.u(), te.u(), sk->d_s, sp.u(), k0, k1, j * K, std::min((j + 1) * K, L), Pw, Pws);
@@ -691,41 +698,33 @@ extern "C" void fhe_evk_destroy(fhe_evk *evk)
 // encryption, decryption, import/export
 // ---------------------------------------------------------------------------
 
-// Encryption from device-resident inputs: m, u, e0, e1 are int64[count][N].
+// Encryption from device-resident inputs: u, e0, e1 are int64[count][N].
 // Enc(m) = (pk0 u + p e0 + m, pk1 u + p e1) at level L.
-static int encrypt_dev(fhe_ctx *c, const fhe_pk *pk, const int64_t *dm, const int64_t *du, const int64_t *d0,
+// dm: the plaintexts' coefficients, mn of each (mn = N, or the subring's M,
+// coefficient j of which belongs to X^(j N / M)).
+static int encrypt_dev(fhe_ctx *c, const fhe_pk *pk, const int64_t *dm, int mn, const int64_t *du, const int64_t *d0,
                        const int64_t *d1, int count, fhe_ct **out)
 {
     const int N = c->N, L = c->L;
     int err = 0;
-    DevBuf U(c, sizeof(u64) * count * L * N, &err), T0(c, sizeof(u64) * count * L * N, &err),
-        T1(c, sizeof(u64) * count * L * N, &err);
-    DevBuf C0(c, sizeof(u64) * count * L * N, &err), C1(c, sizeof(u64) * count * L * N, &err);
+    DevBuf t(c, sizeof(u64) * 3 * count * L * N, &err);  // u, p e0 + m, p e1
     if (err) return fhe_fail(c, err, "encrypt: out of memory");
     fhe_ct *ct = ct_new(c, count, 2, L, &err);
     if (!ct) return err;
-    int pr[FHE_MAXP];
-    primes_range(pr, L, 0);
-    launch_rns_from_i64(c, du, nullptr, 1, U.u(), count, L, pr);
-    launch_rns_from_i64(c, d0, dm, (int64_t)c->p, T0.u(), count, L, pr);
-    launch_rns_from_i64(c, d1, nullptr, (int64_t)c->p, T1.u(), count, L, pr);
-    ntt_blocks(c, U.u(), U.u(), count, L, 0, false);
-    ntt_blocks(c, T0.u(), T0.u(), count, L, 0, false);
-    ntt_blocks(c, T1.u(), T1.u(), count, L, 0, false);
-    launch_muladd(c, U.u(), pk->d, T0.u(), C0.u(), count, L, 0, 0);
-    launch_muladd(c, U.u(), pk->d + (size_t)L * N, T1.u(), C1.u(), count, L, 0, 0);
-    launch_copy_limbs(c, C0.u(), ct->d, count, L, (long long)L * N, 2LL * L * N);
-    launch_copy_limbs(c, C1.u(), ct->d + (size_t)L * N, count, L, (long long)L * N, 2LL * L * N);
+    launch_enc_rns(c, du, d0, d1, dm, mn, t.u(), count, L);
+    ntt_blocks(c, t.u(), t.u(), 3 * count, L, 0, false);
+    launch_enc_combine(c, t.u(), pk->d, ct->d, count, L);
     *out = ct;
     return 0;
 }
 
+// the M subring coefficients of every ciphertext's slots
 static int encode_batch(fhe_ctx *c, const uint64_t *slots, int count, std::vector<int64_t> &m)
 {
     for (long long i = 0; i < (long long)count * c->ns; i++)
         if (slots[i] >= c->p) return fhe_fail(c, FHE_EINVAL, "slot value out of [0, p)");
-    m.assign((size_t)count * c->N, 0);
-    for (int i = 0; i < count; i++) encode_slots(c, slots + (size_t)i * c->ns, m.data() + (size_t)i * c->N);
+    m.assign((size_t)count * c->M, 0);
+    for (int i = 0; i < count; i++) encode_sub(c, slots + (size_t)i * c->ns, m.data() + (size_t)i * c->M);
     return 0;
 }
 
@@ -753,15 +752,15 @@ extern "C" int fhe_encrypt_explicit(fhe_ctx *c, const fhe_pk *pk, const uint64_t
     std::vector<int64_t> m;
     int err = encode_batch(c, slots, count, m);
     if (err) return err;
-    const size_t vb = sizeof(int64_t) * count * c->N;
-    DevBuf du(c, vb, &err), d0(c, vb, &err), d1(c, vb, &err), dm(c, vb, &err);
+    const size_t vb = sizeof(int64_t) * count * c->N, mb = sizeof(int64_t) * m.size();
+    DevBuf du(c, vb, &err), d0(c, vb, &err), d1(c, vb, &err), dm(c, mb, &err);
     if (err) return fhe_fail(c, err, "encrypt: out of memory");
     cudaMemcpyAsync(du.p, u, vb, cudaMemcpyHostToDevice, c->stream);
     cudaMemcpyAsync(d0.p, e0, vb, cudaMemcpyHostToDevice, c->stream);
     cudaMemcpyAsync(d1.p, e1, vb, cudaMemcpyHostToDevice, c->stream);
-    cudaMemcpyAsync(dm.p, m.data(), vb, cudaMemcpyHostToDevice, c->stream);
+    cudaMemcpyAsync(dm.p, m.data(), mb, cudaMemcpyHostToDevice, c->stream);
     fhe_ct *ct = nullptr;
-    if ((err = encrypt_dev(c, pk, dm.i(), du.i(), d0.i(), d1.i(), count, &ct))) return err;
+    if ((err = encrypt_dev(c, pk, dm.i(), c->M, du.i(), d0.i(), d1.i(), count, &ct))) return err;
     int r = sync_check(c, "encrypt");
     if (r) {
         fhe_ct_destroy(ct);
@@ -782,14 +781,12 @@ extern "C" int fhe_encrypt(fhe_ctx *c, const fhe_pk *pk, const uint64_t *slots, 
     if (err) return err;
     const long long n = (long long)count * c->N;
     DevBuf du(c, sizeof(int64_t) * n, &err), d0(c, sizeof(int64_t) * n, &err), d1(c, sizeof(int64_t) * n, &err),
-        dm(c, sizeof(int64_t) * n, &err);
+        dm(c, sizeof(int64_t) * m.size(), &err);
     if (err) return fhe_fail(c, err, "encrypt: out of memory");
-    cudaMemcpyAsync(dm.p, m.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, c->stream);
-    sample_ternary(c, du.i(), n, seed, TAG_U);
-    sample_gaussian(c, d0.i(), n, seed, TAG_E0);
-    sample_gaussian(c, d1.i(), n, seed, TAG_E1);
+    cudaMemcpyAsync(dm.p, m.data(), sizeof(int64_t) * m.size(), cudaMemcpyHostToDevice, c->stream);
+    sample_encryption(c, du.i(), d0.i(), d1.i(), n, seed);
     fhe_ct *ct = nullptr;
-    if ((err = encrypt_dev(c, pk, dm.i(), du.i(), d0.i(), d1.i(), count, &ct))) return err;
+    if ((err = encrypt_dev(c, pk, dm.i(), c->M, du.i(), d0.i(), d1.i(), count, &ct))) return err;
     int r = sync_check(c, "encrypt");
     if (r) {
         fhe_ct_destroy(ct);
@@ -799,26 +796,27 @@ extern "C" int fhe_encrypt(fhe_ctx *c, const fhe_pk *pk, const uint64_t *slots, 
     return 0;
 }
 
-// Plaintext coefficients of a batch, on the device: modulus switch a copy to
-// one prime, t = c0 + c1 s (limb 0), INTT, centred mod q0, then mod p.
+// c0 + c1 s of a batch switched to one prime, coefficient domain: [count][N]
+static int decrypt_residues(fhe_ctx *c, const fhe_sk *sk, const fhe_ct *ct, u64 *t)
+{
+    fhe_ct *low = nullptr;
+    if (ct->level > 1)
+        if (int err = op_lower(c, ct, 1, &low)) return err;
+    launch_dec_dot(c, low ? low->d : ct->d, sk->d_s, t, ct->count);
+    ntt_blocks(c, t, t, ct->count, 1, 0, true);
+    if (low) fhe_ct_destroy(low);
+    return 0;
+}
+
+// Plaintext coefficients of a batch, on the device: the residues of
+// decrypt_residues centred mod q0, then mod p.
 static int decrypt_coeffs_dev(fhe_ctx *c, const fhe_sk *sk, const fhe_ct *ct, int64_t *dm)
 {
-    const int N = c->N, count = ct->count;
-    fhe_ct *one = nullptr;
-    int err = op_lower(c, ct, 1, &one);
-    if (err) return err;
-    DevBuf t(c, sizeof(u64) * count * N, &err), c0(c, sizeof(u64) * count * N, &err),
-        c1(c, sizeof(u64) * count * N, &err);
-    if (err) {
-        fhe_ct_destroy(one);
-        return fhe_fail(c, err, "decrypt: out of memory");
-    }
-    launch_copy_limbs(c, one->d, c0.u(), count, 1, 2LL * N, N);
-    launch_copy_limbs(c, one->d + N, c1.u(), count, 1, 2LL * N, N);
-    launch_muladd(c, c1.u(), sk->d_s, c0.u(), t.u(), count, 1, 0, 0);
-    ntt_blocks(c, t.u(), t.u(), count, 1, 0, true);
-    launch_centre_mod_p(c, t.u(), dm, (long long)count * N);
-    fhe_ct_destroy(one);
+    int err = 0;
+    DevBuf t(c, sizeof(u64) * ct->count * c->N, &err);
+    if (err) return fhe_fail(c, err, "decrypt: out of memory");
+    if ((err = decrypt_residues(c, sk, ct, t.u()))) return err;
+    launch_centre_mod_p(c, t.u(), dm, (long long)ct->count * c->N);
     return 0;
 }
 
@@ -828,17 +826,24 @@ extern "C" int fhe_decrypt(fhe_ctx *c, const fhe_sk *sk, const fhe_ct *ct, uint6
     CHECK_CTX(c);
     if (!sk || !ct || !slots || ct->npoly != 2) return FHE_EINVAL;
     LOCK(c);
-    const int N = c->N, count = ct->count;
+    const int count = ct->count, M = c->M, runs = centre_sub_runs(c);
     int err = 0;
-    DevBuf dm(c, sizeof(int64_t) * count * N, &err);
+    // per ciphertext the subring's coefficients, then a word a run of all
+    // coefficients for whether it holds another that is not zero
+    DevBuf t(c, sizeof(u64) * count * c->N, &err), dm(c, sizeof(int64_t) * count * (M + runs), &err);
     if (err) return fhe_fail(c, err, "decrypt: out of memory");
-    if ((err = decrypt_coeffs_dev(c, sk, ct, dm.i()))) return err;
-    std::vector<int64_t> m((size_t)count * N);
+    if ((err = decrypt_residues(c, sk, ct, t.u()))) return err;
+    launch_centre_sub(c, t.u(), dm.i(), count);
+    std::vector<int64_t> m((size_t)count * (M + runs));
     cudaMemcpyAsync(m.data(), dm.p, sizeof(int64_t) * m.size(), cudaMemcpyDeviceToHost, c->stream);
     if ((err = sync_check(c, "decrypt"))) return err;
-    for (int i = 0; i < count; i++)
-        if (!decode_slots(c, m.data() + (size_t)i * N, slots + (size_t)i * c->ns))
+    for (int i = 0; i < count; i++) {
+        const int64_t *mi = m.data() + (size_t)i * (M + runs);
+        bool other = false;
+        for (int b = 0; b < runs; b++) other |= mi[M + b] != 0;
+        if (other || !decode_sub(c, mi, slots + (size_t)i * c->ns))
             return fhe_fail(c, FHE_EINVAL, "decrypt: plaintext is not a slot encoding");
+    }
     return 0;
 }
 
@@ -869,11 +874,9 @@ extern "C" int fhe_encrypt_ext(fhe_ctx *c, const fhe_pk *pk, const uint64_t *dig
         dm(c, sizeof(int64_t) * n, &err);
     if (err) return fhe_fail(c, err, "encrypt: out of memory");
     cudaMemcpyAsync(dm.p, m.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, c->stream);
-    sample_ternary(c, du.i(), n, seed, TAG_U);
-    sample_gaussian(c, d0.i(), n, seed, TAG_E0);
-    sample_gaussian(c, d1.i(), n, seed, TAG_E1);
+    sample_encryption(c, du.i(), d0.i(), d1.i(), n, seed);
     fhe_ct *ct = nullptr;
-    if ((err = encrypt_dev(c, pk, dm.i(), du.i(), d0.i(), d1.i(), count, &ct))) return err;
+    if ((err = encrypt_dev(c, pk, dm.i(), c->N, du.i(), d0.i(), d1.i(), count, &ct))) return err;
     if ((err = sync_check(c, "encrypt"))) {
         fhe_ct_destroy(ct);
         return err;
@@ -899,7 +902,7 @@ extern "C" int fhe_encrypt_ext_explicit(fhe_ctx *c, const fhe_pk *pk, const uint
     cudaMemcpyAsync(d1.p, e1, vb, cudaMemcpyHostToDevice, c->stream);
     cudaMemcpyAsync(dm.p, m.data(), vb, cudaMemcpyHostToDevice, c->stream);
     fhe_ct *ct = nullptr;
-    if ((err = encrypt_dev(c, pk, dm.i(), du.i(), d0.i(), d1.i(), count, &ct))) return err;
+    if ((err = encrypt_dev(c, pk, dm.i(), c->N, du.i(), d0.i(), d1.i(), count, &ct))) return err;
     if ((err = sync_check(c, "encrypt"))) {
         fhe_ct_destroy(ct);
         return err;
@@ -940,7 +943,7 @@ static int refresh_dev(fhe_ctx *c, const fhe_sk *sk, const fhe_pk *pk, const fhe
     DevBuf dm(c, sizeof(int64_t) * ct->count * c->N, &err);
     if (err) return fhe_fail(c, err, "refresh: out of memory");
     if ((err = decrypt_coeffs_dev(c, sk, ct, dm.i()))) return err;
-    return encrypt_dev(c, pk, dm.i(), du, d0, d1, ct->count, out);
+    return encrypt_dev(c, pk, dm.i(), c->N, du, d0, d1, ct->count, out);
 }
 
 extern "C" int fhe_refresh_explicit(fhe_ctx *c, const fhe_sk *sk, const fhe_pk *pk, const fhe_ct *ct,
@@ -966,9 +969,7 @@ int refresh_seeded(fhe_ctx *c, const fhe_sk *sk, const fhe_pk *pk, const fhe_ct 
     int err = 0;
     DevBuf du(c, sizeof(int64_t) * n, &err), d0(c, sizeof(int64_t) * n, &err), d1(c, sizeof(int64_t) * n, &err);
     if (err) return fhe_fail(c, err, "refresh: out of memory");
-    sample_ternary(c, du.i(), n, seed, TAG_U);
-    sample_gaussian(c, d0.i(), n, seed, TAG_E0);
-    sample_gaussian(c, d1.i(), n, seed, TAG_E1);
+    sample_encryption(c, du.i(), d0.i(), d1.i(), n, seed);
     return refresh_dev(c, sk, pk, ct, du.i(), d0.i(), d1.i(), out);
 }
 

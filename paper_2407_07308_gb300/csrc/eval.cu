@@ -636,7 +636,7 @@ static int plain_ntt(fhe_ctx *c, const int64_t *m_in, int level, fhe_ct **out)
     cudaMemcpyAsync(t.p, m.data(), sizeof(int64_t) * N, cudaMemcpyHostToDevice, c->stream);
     std::vector<int> primes(level);
     for (int i = 0; i < level; i++) primes[i] = i;
-    launch_rns_from_i64(c, (const int64_t *)t.p, nullptr, 1, r->d, 1, level, primes.data());
+    launch_rns_from_i64(c, (const int64_t *)t.p, 1, r->d, 1, level, primes.data());
     LimbMap lm = identity_map(level, (long long)level * N, (long long)level * N, 0, 0, 0);
     launch_ntt_fwd_plain(c, r->d, r->d, lm, level);
     *out = r;

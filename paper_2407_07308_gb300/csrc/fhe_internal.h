@@ -473,8 +473,7 @@ void launch_ks_inner(fhe_ctx *c, const u64 *ext, const u64 *xbase, long long x_o
                      int count, int level);
 void launch_automorphism(fhe_ctx *c, const u64 *in, u64 *out, int outer, int level, const int *perm);
 void launch_mul_poly(fhe_ctx *c, const u64 *a, const u64 *b, u64 *out, int outer, int level, long long b_outer);
-void launch_rns_from_i64(fhe_ctx *c, const int64_t *x, const int64_t *y, int64_t scale, u64 *out, int outer, int nl,
-                         const int *primes);
+void launch_rns_from_i64(fhe_ctx *c, const int64_t *x, int64_t scale, u64 *out, int outer, int nl, const int *primes);
 void launch_muladd(fhe_ctx *c, const u64 *a, const u64 *b, const u64 *cc, u64 *out, int outer, int level,
                    long long b_outer, int neg);
 void launch_ksk_digit(fhe_ctx *c, const u64 *a, const u64 *e, const u64 *s, const u64 *sp, u64 *k0, u64 *k1, int dlo,
@@ -489,7 +488,10 @@ void launch_lincomb(fhe_ctx *c, const u64 *const *x, const u64 (*w)[FHE_MAXP], i
 int op_lincomb(fhe_ctx *c, const fhe_ct *const *x, const int64_t *k, int n, fhe_ct **out);
 
 // seeded samplers (sample.cu)
+// Stream tags of the seeded samplers (see sample.cu).
+enum { TAG_S = 1, TAG_E_PK = 2, TAG_A_PK = 3, TAG_U = 16, TAG_E0 = 17, TAG_E1 = 18, TAG_KSK = 1024 };
 void sample_ternary(fhe_ctx *c, int64_t *out, long long n, uint64_t seed, uint32_t tag);
+void sample_encryption(fhe_ctx *c, int64_t *u, int64_t *e0, int64_t *e1, long long n, uint64_t seed);
 void sample_gaussian(fhe_ctx *c, int64_t *out, long long n, uint64_t seed, uint32_t tag);
 void sample_uniform(fhe_ctx *c, u64 *out, int outer, int nl, uint64_t seed, uint32_t tag);
 // out[i] = centred(x[i] mod q0) mod p, as int64 in [0, p)
@@ -557,5 +559,10 @@ int batch_check_job(const fhe_job &j);
 int circuit_tournament(fhe_ctx *c, const fhe_evk *evk, const fhe_sk *sk, const fhe_pk *pk, const fhe_ct *const *x,
                        int d, bool want_max, bool want_min, uint64_t seed, fhe_ct **out_max, fhe_ct **out_min);
 
-void launch_copy_limbs(fhe_ctx *c, const u64 *in, u64 *out, int outer, int nl, long long in_outer,
-                       long long out_outer);
+// encryption and decryption (kernels.cu)
+void launch_enc_rns(fhe_ctx *c, const int64_t *u, const int64_t *e0, const int64_t *e1, const int64_t *m, int mn,
+                    u64 *out, int count, int level);
+void launch_enc_combine(fhe_ctx *c, const u64 *t, const u64 *pk, u64 *ct, int count, int level);
+void launch_dec_dot(fhe_ctx *c, const u64 *ct, const u64 *s, u64 *t, int count);
+int centre_sub_runs(const fhe_ctx *c);
+void launch_centre_sub(fhe_ctx *c, const u64 *x, int64_t *out, int count);

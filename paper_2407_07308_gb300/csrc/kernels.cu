@@ -101,21 +101,9 @@ __global__ void k_mul_poly(const u64 *__restrict__ a, const u64 *__restrict__ b,
     }
 }
 
-__global__ void k_copy_limbs(const u64 *__restrict__ in, u64 *__restrict__ out, long long total, int logN, int nl,
-                             long long in_outer, long long out_outer)
-{
-    const long long LN = (long long)nl << logN;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const long long o = idx / LN, r = idx % LN;
-        out[o * out_outer + r] = in[o * in_outer + r];
-    }
-}
-
-// out[o][i][n] = (scale * x[o][n] + y[o][n]) mod q_{prime[i]}  (y may be NULL)
-__global__ void k_rns_from_i64(const int64_t *__restrict__ x, const int64_t *__restrict__ y, int64_t scale,
-                               u64 *__restrict__ out, long long total, int logN, int nl, const LimbConsts pm,
-                               const ModQ *__restrict__ mq)
+// out[o][i][n] = scale * x[o][n] mod q_{prime[i]}
+__global__ void k_rns_from_i64(const int64_t *__restrict__ x, int64_t scale, u64 *__restrict__ out,
+                               long long total, int logN, int nl, const LimbConsts pm, const ModQ *__restrict__ mq)
 {
     const int N = 1 << logN;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
@@ -125,9 +113,74 @@ __global__ void k_rns_from_i64(const int64_t *__restrict__ x, const int64_t *__r
         const long long o = li / nl;
         const int n = (int)(idx & (N - 1));
         const u64 q = mq[(int)pm.w[i]].q;
-        const int64_t v = scale * x[o * N + n] + (y ? y[o * N + n] : 0);
+        const int64_t v = scale * x[o * N + n];
         const int64_t r = v % (int64_t)q;
         out[idx] = (u64)(r < 0 ? r + (int64_t)q : r);
+    }
+}
+
+// v mod q in [0, q); a sum and a comparison where |v| < q, which all but the
+// smallest primes make of p times an error's bound
+__device__ __forceinline__ u64 lift(int64_t v, u64 q)
+{
+    if (v < 0) v += (int64_t)q;
+    if ((u64)v < q) return (u64)v;
+    const int64_t r = v % (int64_t)q;
+    return (u64)(r < 0 ? r + (int64_t)q : r);
+}
+
+// The three polynomials of an encryption, out[3][count][L][N]: u, p e0 + m and
+// p e1 over the first L primes.  m holds mn coefficients a plaintext, N / mn
+// apart.  One launch, and one transform over all three, in place of three of
+// each: at one ciphertext every launch is a few microseconds of latency.  A
+// client's round trip (encryption of 2 ciphertexts, N = 2^14, 10 primes, in 5
+// launches in place of 16; a reply's decryption with M coefficients over the
+// bus in place of N) went from 334 to 150 us.
+__global__ void k_enc_rns(const int64_t *__restrict__ u, const int64_t *__restrict__ e0, const int64_t *__restrict__ e1,
+                          const int64_t *__restrict__ m, int mn, int64_t p, u64 *__restrict__ out, long long total,
+                          int logN, int L, const ModQ *__restrict__ mq)
+{
+    const int N = 1 << logN, gap = N / mn;
+    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
+         idx += (long long)gridDim.x * blockDim.x) {
+        const long long li = idx >> logN, o = li / L;
+        const int i = (int)(idx & (N - 1));
+        const u64 q = mq[(int)(li - o * L)].q;
+        const long long s = o * N + i;
+        out[idx] = lift(u[s], q);
+        out[total + idx] = lift(p * e0[s] + (i % gap == 0 ? m[o * mn + i / gap] : 0), q);
+        out[2 * total + idx] = lift(p * e1[s], q);
+    }
+}
+
+// ct[o][pi] = t[1 + pi][o] + t[0][o] pk[pi] (NTT domain; t[3][count][L][N]),
+// both polynomials written where they belong
+__global__ void k_enc_combine(const u64 *__restrict__ t, const u64 *__restrict__ pk, u64 *__restrict__ ct,
+                              long long total, int logN, int L, const ModQ *__restrict__ mq)
+{
+    const long long LN = (long long)L << logN;
+    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
+         idx += (long long)gridDim.x * blockDim.x) {
+        const long long o = idx / LN, r = idx - o * LN;
+        const ModQ m = mq[(int)(r >> logN)];
+        const u64 u = t[idx];
+        u64 *d = ct + 2 * o * LN + r;
+        d[0] = addmod(t[total + idx], barrett128((u128)u * pk[r], m), m.q);
+        d[LN] = addmod(t[2 * total + idx], barrett128((u128)u * pk[LN + r], m), m.q);
+    }
+}
+
+// t[o] = c0 + c1 s of two-poly ciphertexts of one limb (NTT domain)
+__global__ void k_dec_dot(const u64 *__restrict__ ct, const u64 *__restrict__ s, u64 *__restrict__ t, long long total,
+                          int logN, const ModQ *__restrict__ mq)
+{
+    const int N = 1 << logN;
+    const ModQ m = mq[0];
+    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
+         idx += (long long)gridDim.x * blockDim.x) {
+        const long long o = idx >> logN;
+        const int n = (int)(idx & (N - 1));
+        t[idx] = addmod(ct[2 * o * N + n], barrett128((u128)ct[(2 * o + 1) * N + n] * s[n], m), m.q);
     }
 }
 
@@ -178,6 +231,33 @@ __global__ void k_centre_mod_p(const u64 *__restrict__ x, int64_t *__restrict__ 
         int64_t r = cv % p;
         out[i] = r < 0 ? r + p : r;
     }
+}
+
+// The same for plaintexts of a subring (coefficients N / M apart), a block for
+// every SUB_RUN coefficients of a ciphertext: out[o][0 .. M) the subring's
+// coefficients, then a word a block for whether it met another that is not
+// zero.  M words a ciphertext cross the bus in place of N.
+constexpr int SUB_RUN = 1024;
+__global__ void __launch_bounds__(256)
+    k_centre_sub(const u64 *__restrict__ x, int64_t *__restrict__ out, int N, int M, int runs, u64 q0, int64_t p)
+{
+    const int o = blockIdx.x / runs, b = blockIdx.x % runs;
+    const u64 *xo = x + (long long)o * N;
+    int64_t *d = out + (long long)o * (M + runs);
+    const int gap = N / M, end = min(N, (b + 1) * SUB_RUN);
+    int other = 0;
+    for (int i = b * SUB_RUN + threadIdx.x; i < end; i += blockDim.x) {
+        const u64 v = xo[i];
+        const int64_t cv = v > q0 / 2 ? -(int64_t)(q0 - v) : (int64_t)v;
+        int64_t r = cv % p;
+        if (r < 0) r += p;
+        if (i % gap == 0)
+            d[i / gap] = r;
+        else
+            other |= r != 0;
+    }
+    other = __syncthreads_or(other);
+    if (threadIdx.x == 0) d[M + b] = other;
 }
 
 // out = sum_t w_t x_t (mod q_i), up to 8 ciphertext batches of one shape;
@@ -258,19 +338,11 @@ void launch_mul_poly(fhe_ctx *c, const u64 *a, const u64 *b, u64 *out, int outer
            b_outer, c->d_mq);
 }
 
-void launch_copy_limbs(fhe_ctx *c, const u64 *in, u64 *out, int outer, int nl, long long in_outer,
-                       long long out_outer)
-{
-    LAUNCH(k_copy_limbs, (long long)outer * nl * c->N, in, out, (long long)outer * nl * c->N, c->logN, nl, in_outer,
-           out_outer);
-}
-
-void launch_rns_from_i64(fhe_ctx *c, const int64_t *x, const int64_t *y, int64_t scale, u64 *out, int outer, int nl,
-                         const int *primes)
+void launch_rns_from_i64(fhe_ctx *c, const int64_t *x, int64_t scale, u64 *out, int outer, int nl, const int *primes)
 {
     LimbConsts pm;
     for (int i = 0; i < nl; i++) pm.w[i] = (u64)primes[i], pm.ws[i] = 0;
-    LAUNCH(k_rns_from_i64, (long long)outer * nl * c->N, x, y, scale, out, (long long)outer * nl * c->N, c->logN, nl,
+    LAUNCH(k_rns_from_i64, (long long)outer * nl * c->N, x, scale, out, (long long)outer * nl * c->N, c->logN, nl,
            pm, c->d_mq);
 }
 
@@ -393,4 +465,36 @@ void launch_lincomb(fhe_ctx *c, const u64 *const *x, const u64 (*w)[FHE_MAXP], i
 void launch_centre_mod_p(fhe_ctx *c, const u64 *x, int64_t *out, long long n)
 {
     LAUNCH(k_centre_mod_p, n, x, out, n, c->q[0], (int64_t)c->p);
+}
+
+void launch_enc_rns(fhe_ctx *c, const int64_t *u, const int64_t *e0, const int64_t *e1, const int64_t *m, int mn,
+                    u64 *out, int count, int level)
+{
+    const long long total = (long long)count * level * c->N;
+    LAUNCH_CLS_W(FHE_K_ELEMWISE, 3 + 3.0 / level, k_enc_rns, total, u, e0, e1, m, mn, (int64_t)c->p, out, total,
+                 c->logN, level, c->d_mq);
+}
+
+void launch_enc_combine(fhe_ctx *c, const u64 *t, const u64 *pk, u64 *ct, int count, int level)
+{
+    const long long total = (long long)count * level * c->N;
+    LAUNCH_CLS_W(FHE_K_ELEMWISE, 5 + 2.0 / count, k_enc_combine, total, t, pk, ct, total, c->logN, level, c->d_mq);
+}
+
+void launch_dec_dot(fhe_ctx *c, const u64 *ct, const u64 *s, u64 *t, int count)
+{
+    const long long total = (long long)count * c->N;
+    LAUNCH_CLS_W(FHE_K_ELEMWISE, 3 + 1.0 / count, k_dec_dot, total, ct, s, t, total, c->logN, c->d_mq);
+}
+
+int centre_sub_runs(const fhe_ctx *c) { return (c->N + SUB_RUN - 1) / SUB_RUN; }
+
+void launch_centre_sub(fhe_ctx *c, const u64 *x, int64_t *out, int count)
+{
+    if (count < 1) return;
+    const int runs = centre_sub_runs(c);
+    prof_begin(c, FHE_K_ELEMWISE, 8.0 * count * (c->N + c->M + runs));
+    k_centre_sub<<<count * runs, 256, 0, c->stream>>>(x, out, c->N, c->M, runs, c->q[0], (int64_t)c->p);
+    prof_end(c);
+    c->launches++;
 }

@@ -45,21 +45,32 @@ __device__ inline Philox draw(uint64_t seed, uint32_t tag, uint64_t n)
     return philox4x32_10((uint32_t)n, (uint32_t)(n >> 32), tag, 0, (uint32_t)seed, (uint32_t)(seed >> 32));
 }
 
+__device__ inline int64_t small_value(const Philox &r, bool gaussian)
+{
+    if (!gaussian) return (int64_t)(((uint64_t)r.v[0] * 3u) >> 32) - 1;
+    const float u1 = ((float)r.v[0] + 1.0f) * 2.3283064e-10f;  // (0, 1]
+    const float u2 = (float)r.v[1] * 2.3283064e-10f;           // [0, 1)
+    const float g = 3.2f * sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
+    const long long v = llrintf(g);
+    return v > 20 ? 20 : (v < -20 ? -20 : v);
+}
+
 // kind: 0 ternary, 1 gaussian  -> int64 out[n]
 __global__ void k_sample_small(int64_t *__restrict__ out, long long n, uint64_t seed, uint32_t tag, int kind)
 {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const Philox r = draw(seed, tag, (uint64_t)i);
-        if (kind == 0) {
-            out[i] = (int64_t)(((uint64_t)r.v[0] * 3u) >> 32) - 1;
-        } else {
-            const float u1 = ((float)r.v[0] + 1.0f) * 2.3283064e-10f;  // (0, 1]
-            const float u2 = (float)r.v[1] * 2.3283064e-10f;           // [0, 1)
-            const float g = 3.2f * sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
-            long long v = llrintf(g);
-            out[i] = v > 20 ? 20 : (v < -20 ? -20 : v);
-        }
-    }
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        out[i] = small_value(draw(seed, tag, (uint64_t)i), kind);
+}
+
+// The three vectors of an encryption, one grid row each: ternary u, gaussian
+// e0 and e1, of streams TAG_U, TAG_E0 and TAG_E1.
+__global__ void k_sample_encryption(int64_t *__restrict__ u, int64_t *__restrict__ e0, int64_t *__restrict__ e1,
+                                    long long n, uint64_t seed)
+{
+    const int k = blockIdx.y;
+    int64_t *out = k == 0 ? u : (k == 1 ? e0 : e1);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        out[i] = small_value(draw(seed, TAG_U + k, (uint64_t)i), k);
 }
 
 // uniform residues: out[o][i][n] in [0, q_i), o < outer, i < nl (primes 0..nl-1)
@@ -97,6 +108,12 @@ void sample_ternary(fhe_ctx *c, int64_t *out, long long n, uint64_t seed, uint32
 void sample_gaussian(fhe_ctx *c, int64_t *out, long long n, uint64_t seed, uint32_t tag)
 {
     k_sample_small<<<blocks_for(n), 256, 0, c->stream>>>(out, n, seed, tag, 1);
+    c->launches++;
+}
+
+void sample_encryption(fhe_ctx *c, int64_t *u, int64_t *e0, int64_t *e1, long long n, uint64_t seed)
+{
+    k_sample_encryption<<<dim3(blocks_for(n), 3), 256, 0, c->stream>>>(u, e0, e1, n, seed);
     c->launches++;
 }
 
