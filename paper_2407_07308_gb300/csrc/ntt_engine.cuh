@@ -52,7 +52,8 @@
 // the units of all segments are numbered in order and every CTA walks them
 // with a grid stride (segments of different ring degree: one launch each).
 // The grid is either one CTA per unit or a fixed number of resident CTAs per
-// SM (the autotuner's choice per context).
+// SM (the autotuner's choice per context).  Launches of a few units per SM run
+// both passes in one kernel, a cluster of CTAs per limb (k_fwd_small).
 //
 // Load/store functors let one kernel body serve the plain transform and the
 // fused variants: ModUp (basis conversion of a key-switching digit computed
@@ -562,6 +563,40 @@ __device__ __forceinline__ u64 conv_one(const Conv &a, const ModQ &m, int n)
     return (u64)dot_fold(s, m);
 }
 
+// One target at P positions n, n + STEP, ..
+template <int P, int STEP, int NN>
+__device__ __forceinline__ void conv_single(const Conv &a, const ModQ &m, int n, u64 *v)
+{
+    DotAcc s[P];
+#pragma unroll
+    for (int p = 0; p < P; p++) s[p] = DotAcc{0, (int64_t)(2 * m.q2)};
+    const int ns = a.n;
+    const u64 *src = a.src + n;
+#pragma unroll 1
+    for (int i0 = 0; i0 < ns; i0 += 4) {
+        u64 x[4][P];
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+            if (i0 + i < ns) {
+#pragma unroll
+                for (int p = 0; p < P; p++) x[i][p] = src[(size_t)i * NN + p * STEP];
+            }
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+            if (i0 + i < ns) {
+                const DotC c = a.c[i0 + i];
+#pragma unroll
+                for (int p = 0; p < P; p++) {
+                    dot_mac(s[p], x[i][p], c, m.half);
+                    if (m.half > 27 && (i & 1)) s[p] = DotAcc{0, dot_fold(s[p], m)};
+                }
+            }
+        src += (size_t)4 * NN;
+    }
+#pragma unroll
+    for (int p = 0; p < P; p++) v[p] = (u64)dot_fold(s[p], m);
+}
+
 // ---------------------------------------------------------------------------
 // kernels' stores: out = x A + d B mod q with constants, d = y - v for the
 // transform's lazy value v (below 71 q), x and y below 2q
@@ -670,32 +705,40 @@ __device__ __forceinline__ void col_twiddles(ulonglong2 *W, const ulonglong2 *tw
     for (int i = threadIdx.x; i < (1 << N1); i += T) async16(W + twp(i), tw + i);
 }
 
-// Column units of one job: the job's state is computed by every thread and
-// stays in registers.  Thread (c, g) reads and writes column lo0 + c in
+struct PdlWait {
+    __device__ void operator()() const { pdl_wait(); }
+};
+
+// Column units of one job.  Thread (c, g) reads and writes column lo0 + c in
 // global memory straight from its rounds' registers (neighbouring lanes,
 // neighbouring columns); shared memory carries the one exchange between the
 // rounds.
 template <int N1, int N2, class IO>
-__device__ __forceinline__ void fwd_cols_unit1(const IO &io, int sg, int lu, u64 *sm, ulonglong2 *W)
+__device__ __forceinline__ void fwd_cols_unit1(const IO &io, int sg, int lu, u64 *sm, ulonglong2 *W,
+                                               const typename IO::CSt &st)
 {
-    using Gm = ColGeo<N1, N2, IO::XJ>;
+    using Gm = ColGeo<N1, N2, 1>;
     using C = typename Gm::C;
     const int c = threadIdx.x % C::NS, g = threadIdx.x / C::NS;
     const SegHdr &H = io.h[sg];
     const int lo = (lu % Gm::BLK) * Gm::NC + c;
-    typename IO::CSt st;
-    io.begin_c(sg, lu / Gm::BLK, st);
     col_twiddles<N1>(W, H.tw + (size_t)st.prime * Gm::NN);
     const ModQ &m = H.mq[st.prime];
-    const ColTw<N1, N2, IO::XJ> geo{W, m.q, m.q, &m, &m};
+    const ColTw<N1, N2, 1> geo{W, m.q, m.q, &m, &m};
     pdl_wait();
     u64 x[16];
-    const u64 *src = io.src(st) + (g << N2) + lo;
+    if constexpr (IO::XJ == 2) {
 #pragma unroll
-    for (int k = 0; k < 16; k++) x[k] = src[(k * C::G) << N2];
-    if constexpr (!IO::PLAIN) {
+        for (int k = 0; k < 16; k += 4)
+            conv_single<4, (C::G << N2), Gm::NN>(st.cv, m, ((k * C::G + g) << N2) + lo, x + k);
+    } else {
+        const u64 *src = io.src(st) + (g << N2) + lo;
 #pragma unroll
-        for (int k = 0; k < 16; k++) x[k] = io.conv(st, x[k]);
+        for (int k = 0; k < 16; k++) x[k] = src[(k * C::G) << N2];
+        if constexpr (!IO::PLAIN) {
+#pragma unroll
+            for (int k = 0; k < 16; k++) x[k] = io.conv(st, x[k]);
+        }
     }
     async_wait();
     __syncthreads();  // the twiddles
@@ -717,10 +760,10 @@ __device__ __forceinline__ u64 inv_scaled(u64 v, const ulonglong2 ni, const ModQ
     return reduce4q(shoup_lazy4_chain(v, ni.x, ni.y, 0 - m.q), m.q2, m.q);
 }
 
-template <int N1, int N2, class IO>
-__device__ __forceinline__ void inv_cols_unit1(const IO &io, int sg, int lu, u64 *sm, ulonglong2 *W)
+template <int N1, int N2, class IO, class Wait = PdlWait>
+__device__ __forceinline__ void inv_cols_unit1(const IO &io, int sg, int lu, u64 *sm, ulonglong2 *W, Wait wait = {})
 {
-    using Gm = ColGeo<N1, N2, IO::XJ>;
+    using Gm = ColGeo<N1, N2, 1>;
     using C = typename Gm::C;
     const int c = threadIdx.x % C::NS, g = threadIdx.x / C::NS;
     const SegHdr &H = io.h[sg];
@@ -729,8 +772,8 @@ __device__ __forceinline__ void inv_cols_unit1(const IO &io, int sg, int lu, u64
     io.begin_c(sg, lu / Gm::BLK, st);
     col_twiddles<N1>(W, H.tw + (size_t)st.prime * Gm::NN);
     const ModQ &m = H.mq[st.prime];
-    const ColTw<N1, N2, IO::XJ> geo{W, m.q, m.q, &m, &m};
-    pdl_wait();
+    const ColTw<N1, N2, 1> geo{W, m.q, m.q, &m, &m};
+    wait();
     u64 x[16];
     const u64 *mid = io.inter(st) + (g << (N2 + 4)) + lo;
 #pragma unroll
@@ -766,7 +809,9 @@ __device__ __forceinline__ void fwd_cols_unit(const IO &io, int sg, int lu, u64 
     using Gm = ColGeo<N1, N2, IO::XJ>;
     using C = typename Gm::C;
     if constexpr (Gm::NJ == 1) {
-        fwd_cols_unit1<N1, N2>(io, sg, lu, sm, W);
+        typename IO::CSt st;  // computed by every thread, in registers
+        io.begin_c(sg, lu / Gm::BLK, st);
+        fwd_cols_unit1<N1, N2>(io, sg, lu, sm, W, st);
         return;
     }
     const int tid = threadIdx.x, c = tid % C::NS, g = tid / C::NS;
@@ -940,9 +985,9 @@ struct RowMap {
 };
 
 // Forward, rows: global stages N1..N1+N2-1, then the functor's store.
-template <int N1, int N2, bool GRP, class IO>
+template <int N1, int N2, bool GRP, class IO, class Wait = PdlWait>
 __device__ __forceinline__ void fwd_rows_unit(const IO &io, int sg, int lu, u64 *sm, ulonglong2 *W,
-                                          typename IO::RSt *sts)
+                                          typename IO::RSt *sts, Wait wait = {})
 {
     using Gm = RowGeo<N1, N2>;
     using C = typename Gm::C;
@@ -956,7 +1001,7 @@ __device__ __forceinline__ void fwd_rows_unit(const IO &io, int sg, int lu, u64 
     const ModQ &m = H.mq[prime];
     const ulonglong2 *tw = H.tw + (size_t)prime * Gm::NN;
     if (GRP) row_twiddles<N1, N2>(W, tw, hi0);
-    pdl_wait();
+    wait();
     // thread (c, g) reads its first round's words: runs of G words
     const int c = tid / C::G, g = tid % C::G;
     u64 x[16];
@@ -996,9 +1041,9 @@ __device__ __forceinline__ void fwd_rows_unit(const IO &io, int sg, int lu, u64 
 }
 
 // Inverse, rows first: undoes global stages N1+N2-1..N1.
-template <int N1, int N2, bool GRP, class IO>
+template <int N1, int N2, bool GRP, class IO, class Wait = PdlWait>
 __device__ __forceinline__ void inv_rows_unit(const IO &io, int sg, int lu, u64 *sm, ulonglong2 *W,
-                                          typename IO::RSt *sts)
+                                          typename IO::RSt *sts, Wait wait = {})
 {
     using Gm = RowGeo<N1, N2>;
     using C = typename Gm::C;
@@ -1012,7 +1057,7 @@ __device__ __forceinline__ void inv_rows_unit(const IO &io, int sg, int lu, u64 
     const ModQ &m = H.mq[prime];
     const ulonglong2 *tw = H.tw + (size_t)prime * Gm::NN;
     if (GRP) row_twiddles<N1, N2>(W, tw, hi0);
-    pdl_wait();
+    wait();
     // a unit's jobs are of one map entry, so either all or none have an addend
     // per polynomial; its words are computed on the way, eight at a time with
     // all loads before the first store (one at a time, each store held the
@@ -1148,6 +1193,67 @@ __global__ void __launch_bounds__(T, FHE_NTT_MINB) k_inv_cols(const __grid_const
         inv_cols_unit<Deg<L>::N1, Deg<L>::N2>(io, sg, lu, sm, W, sts);
         __syncthreads();
     }
+}
+
+// Both passes of a small launch in one kernel: a cluster of CTAs per job (a
+// limb's 1 .. 16 units), a column unit and a single-job row unit of it each,
+// with a cluster barrier (release / acquire) where the kernels' boundary would
+// be.  Such a launch is bound by latency: the second pass's state and twiddles
+// are fetched before the first pass runs (its wait), and a limb's rows start
+// when its own columns are done.  Four CTAs per SM, since six (80 registers) ran 5-7%
+// slower.  One LT + EQ at N = 2^14, 10 primes: 2078 -> 1718 us; one less-than
+// at N = 2^12 499 -> 425; one rotation at N = 2^15 (9 primes) 297 -> 250.
+template <int L>
+constexpr int SMALL_CTAS = 1 << (L - 11);  // units of a limb: the cluster
+constexpr int SMALL_LO = 11, SMALL_HI = 15;
+
+template <int L>
+__device__ __forceinline__ void job_barrier()
+{
+    if constexpr (SMALL_CTAS<L> == 1)
+        __syncthreads();
+    else
+        asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+template <int L>
+struct SmallGeo {
+    using Col = ColGeo<Deg<L>::N1, Deg<L>::N2, 1>;
+    using Row = RowGeo<Deg<L>::N1, Deg<L>::N2>;
+    static_assert(Col::NJ == 1 && Col::BLK == SMALL_CTAS<L> && Row::CHS == SMALL_CTAS<L>, "units of a limb");
+    static constexpr int WORDS = Col::Lay::WORDS > ROW_WORDS ? Col::Lay::WORDS : ROW_WORDS;
+};
+
+template <class IO, int L>
+__global__ void __launch_bounds__(T, 4) k_fwd_small(const __grid_constant__ IO io)
+{
+    pdl_trigger();
+    constexpr int N1 = Deg<L>::N1, N2 = Deg<L>::N2;
+    __shared__ u64 sm[SmallGeo<L>::WORDS];
+    __shared__ ulonglong2 W[SmallGeo<L>::Col::TW];
+    __shared__ typename IO::RSt rst[1];
+    __shared__ typename IO::CSt cst[1];
+    const int u = blockIdx.x, sg = seg_of(io, u, false), lu = u - io.h[sg].u_cols;
+    if (threadIdx.x == 32) io.begin_c(sg, lu / SMALL_CTAS<L>, cst[0]);  // published by row_jobs' barrier
+    fwd_rows_unit<N1, N2, false>(io, sg, lu, sm, W, rst, [&] {
+        fwd_cols_unit1<N1, N2>(io, sg, lu, sm, W, cst[0]);
+        job_barrier<L>();
+    });
+}
+
+template <class IO, int L>
+__global__ void __launch_bounds__(T, 4) k_inv_small(const __grid_constant__ IO io)
+{
+    pdl_trigger();
+    constexpr int N1 = Deg<L>::N1, N2 = Deg<L>::N2;
+    __shared__ u64 sm[SmallGeo<L>::WORDS];
+    __shared__ ulonglong2 W[SmallGeo<L>::Col::TW];
+    __shared__ typename IO::RSt rst[1];
+    const int u = blockIdx.x, sg = seg_of(io, u, false), lu = u - io.h[sg].u_cols;
+    inv_cols_unit1<N1, N2>(io, sg, lu, sm, W, [&] {
+        inv_rows_unit<N1, N2, false>(io, sg, lu, sm, W, rst);
+        job_barrier<L>();
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -1681,9 +1787,49 @@ void recount(IO &io)
     for (int s = 0; s < io.nseg; s++) unit_counts(io.h[s]);
 }
 
+// Where both passes run as one kernel: launches of at most this many units per
+// SM.  On a context's own stream the one kernel wins to about 6 (LT + EQ of 3
+// at N = 2^14: 3020 us without, 2785 at 6, 2798 at 8, 2846 at 12); at N = 2^15,
+// whose clusters of 16 take more of the chip at once, to one resident wave (one
+// LT + EQ of 12 primes: 2366 without, 2177 at 2, 2075 at 4, 2085 at 6; sixteen
+// products 2058 at 4, 2069 at 6).  Under the scheduler other streams fill the
+// chip and pairing targets is worth more (32 uneven requests: 46.1 ms without,
+// 45.6 at 1, 45.9 at 2, 46.7 at 4).
+#ifndef FHE_NTT_SMALL
+#define FHE_NTT_SMALL 6
+#endif
+#ifndef FHE_NTT_SMALL_15
+#define FHE_NTT_SMALL_15 4
+#endif
+#ifndef FHE_NTT_SMALL_BRANCH
+#define FHE_NTT_SMALL_BRANCH 1
+#endif
+
 template <class IO, int L>
-void launch_passes(fhe_ctx *c, const IO &io, bool fwd)
+void launch_passes(fhe_ctx *c, IO &io, bool fwd)
 {
+    if constexpr (L >= SMALL_LO && L <= SMALL_HI) {
+        constexpr int C = SMALL_CTAS<L>;
+        long long units = 0;
+        for (int s = 0; s < io.nseg; s++) units += (long long)C * io.h[s].outer * io.h[s].nl;
+        constexpr int own = L == 15 ? FHE_NTT_SMALL_15 : FHE_NTT_SMALL;
+        if (units <= (long long)(c->on_branch ? FHE_NTT_SMALL_BRANCH : own) * c->sms) {
+            int u = 0;
+            for (int s = 0; s < io.nseg; s++) {
+                SegHdr &H = io.h[s];
+                H.gouter = H.g_units = 0;
+                H.u_cols = H.u_rows = u;
+                u += C * H.outer * H.nl;
+            }
+            const bool pdl = pdl_on(c, u, T);
+            if constexpr ((IO::DIRS & DIR_FWD) != 0)
+                if (fwd) launch_pdl_cluster(k_fwd_small<IO, L>, pdl, u, T, C, c->stream, io);
+            if constexpr ((IO::DIRS & DIR_INV) != 0)
+                if (!fwd) launch_pdl_cluster(k_inv_small<IO, L>, pdl, u, T, C, c->stream, io);
+            c->launches++;
+            return;
+        }
+    }
     if constexpr ((IO::DIRS & DIR_FWD) != 0)
         if (fwd) {
             launch_pdl(k_fwd_cols<IO, L>, pdl_on(c, grid_of(c, io.ucols), T), grid_of(c, io.ucols), T, c->stream, io);

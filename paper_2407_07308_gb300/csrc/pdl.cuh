@@ -38,24 +38,48 @@ __device__ __forceinline__ void pdl_begin()
 }
 
 template <class... KArgs, class... Args>
-inline void launch_pdl_smem(void (*kernel)(KArgs...), bool overlap, int grid, int block, size_t smem, cudaStream_t s,
-                            Args &&...args)
+inline void launch_attrs(void (*kernel)(KArgs...), bool overlap, int cluster, int grid, int block, size_t smem,
+                         cudaStream_t s, Args &&...args)
 {
-    if (!overlap) {
-        kernel<<<grid, block, smem, s>>>(std::forward<Args>(args)...);
-        return;
-    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (overlap) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = (unsigned)cluster;
+        attr[n].val.clusterDim.y = 1;
+        attr[n++].val.clusterDim.z = 1;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = (unsigned)n;
     cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);  // errors surface in cudaGetLastError
+}
+
+template <class... KArgs, class... Args>
+inline void launch_pdl_smem(void (*kernel)(KArgs...), bool overlap, int grid, int block, size_t smem, cudaStream_t s,
+                            Args &&...args)
+{
+    if (!overlap)
+        kernel<<<grid, block, smem, s>>>(std::forward<Args>(args)...);
+    else
+        launch_attrs(kernel, true, 1, grid, block, smem, s, std::forward<Args>(args)...);
+}
+
+// grid a multiple of cluster (above 8, the portable size, the kernel opts in)
+template <class... KArgs, class... Args>
+inline void launch_pdl_cluster(void (*kernel)(KArgs...), bool overlap, int grid, int block, int cluster, cudaStream_t s,
+                               Args &&...args)
+{
+    if (cluster > 8) cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    launch_attrs(kernel, overlap, cluster, grid, block, 0, s, std::forward<Args>(args)...);
 }
 
 template <class... KArgs, class... Args>
