@@ -268,13 +268,13 @@ CLASS_SOURCES = {
     "elementwise": ("many.cu",),
 }
 DRAM_PER_ALGORITHMIC = {
-    "ntt_modup": (1.8, "62f98ef236093264"),
-    "ntt_moddown": (1.25, "62f98ef236093264"),
-    "ntt_inv": (1.1, "dfdb6d470d2fd9f3"),
-    "ntt_modswitch": (1.41, "6431ec87f0747706"),
-    "ks_inner": (0.8, "0ce32bc2efb401e2"),
-    "elementwise": (0.86, "0ce32bc2efb401e2"),
-    "tensor": (0.63, "0ce32bc2efb401e2"),
+    "ntt_modup": (1.98, "039d5a18ef76b8b8"),
+    "ntt_moddown": (1.33, "039d5a18ef76b8b8"),
+    "ntt_inv": (1.27, "75770092fe0d8ca6"),
+    "ntt_modswitch": (1.42, "41e4560f2460137e"),
+    "ks_inner": (0.89, "935c4c92edfb7dd5"),
+    "elementwise": (0.83, "935c4c92edfb7dd5"),
+    "tensor": (0.76, "935c4c92edfb7dd5"),
 }
 
 
@@ -819,7 +819,7 @@ def run_uneven(args):
 
     # same-level groups only (no alignment), the aligned form per context,
     # then the fused form (the value): the contexts of one plaintext prime in
-    # one circuit, every step one launch across ring degrees and levels
+    # one circuit, every step one launch across levels and digit counts
     unaligned = aligned = None
     if not args.quick:
         batched_step(check=True, flags=0)

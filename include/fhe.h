@@ -485,9 +485,10 @@ int fhe_batch_submit(const fhe_job *jobs, int n, fhe_batch **out);
  * run alone at its own level.
  * FHE_BATCH_FUSE_RINGS: the compare and max/min jobs of all contexts that
  * share a device and a plaintext prime (hence the digit polynomial) run in
- * one circuit, whose every step is one kernel launch over all their groups:
- * ring degrees, digit counts and levels mixed in one launch (the first such
- * context's stream carries the work; the others' streams wait for it).
+ * one circuit, whose every step is one kernel launch over all their groups'
+ * digit counts and levels: across ring degrees for the streaming steps, one
+ * launch per ring degree for the transforms (the first such context's stream
+ * carries the work; the others' streams wait for it).
  * A submission shape such a family has served before is captured (once)
  * into one CUDA graph for the family and replayed (up to 4 graphs per family;
  * they hold memory in every member's pool and are dropped when a member

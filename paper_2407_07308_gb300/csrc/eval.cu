@@ -1676,8 +1676,8 @@ int circuit_multi(fhe_ctx *c, const fhe_evk *evk, const std::vector<MultiItem> &
 }
 
 // The same over several contexts of one device and plaintext prime (one
-// circuit: every merged step is one launch across their ring degrees and
-// levels).  Item i uses keys evks[i]; evks[0]'s context leads.  The caller
+// circuit: every merged step is one launch across their levels, the
+// streaming steps across their ring degrees too).  Item i uses keys evks[i]; evks[0]'s context leads.  The caller
 // holds every context's lock and has pointed every context's stream (and
 // pool stream) at the leader's for the call.
 int circuit_multi_ctx(const std::vector<const fhe_evk *> &evks, const std::vector<MultiItem> &items)
