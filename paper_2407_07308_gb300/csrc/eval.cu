@@ -1141,8 +1141,14 @@ struct Circuit {
         if (err) return out;
         // the wave in `parts` merged operations (items dealt round robin),
         // each on a stream of its own under the scheduler, so that one
-        // part's streaming steps overlap another's transforms
-        const int parts = dag.on ? std::max(1, std::min((int)pr.size(), c->wave_split)) : 1;
+        // part's streaming steps overlap another's transforms (16 pairs at
+        // N = 2^14 9.71 ms in one part, 9.52 in two).  A wave over several
+        // ring degrees stays whole: its transforms are a launch per degree
+        // already, and halves of those leave the chip idle (32 uneven
+        // requests 45.8 ms in two parts, 44.3 in one; 4 requests 3.95, 3.79)
+        bool mixed = false;
+        for (const fhe_ct *x : low) mixed |= x && x->ctx->logN != low[0]->ctx->logN;
+        const int parts = dag.on && !mixed ? std::max(1, std::min((int)pr.size(), c->wave_split)) : 1;
         for (int part = 0; part < parts && !err; part++) {
             std::vector<MulItem> items;
             std::vector<size_t> at;
