@@ -683,6 +683,9 @@ int fhe_ctx_profile_read(fhe_ctx *ctx, double *ms, int64_t *count, double *bytes
  * pseudo-random and edge-case inputs per prime of the given chain.  Needs no
  * GPU.  Returns 0 if all agree, else the number of mismatches. */
 int fhe_selftest_modarith(uint64_t prime_mod, uint64_t prime_lo, uint64_t prime_hi, int nprimes, int iters);
+/* The NTT engine's rules on the host, without a GPU (each returns 0 or the
+ * number of mismatches): which batches may share a segment. */
+int fhe_selftest_ntt_joins(void);
 
 #ifdef __cplusplus
 }

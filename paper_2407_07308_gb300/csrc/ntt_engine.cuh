@@ -1058,7 +1058,7 @@ __device__ __forceinline__ void inv_rows_unit(const IO &io, int sg, int lu, u64 
     const ulonglong2 *tw = H.tw + (size_t)prime * Gm::NN;
     if (GRP) row_twiddles<N1, N2>(W, tw, hi0);
     wait();
-    // a unit's jobs are of one map entry, so either all or none have an addend
+    // a unit's jobs are of one map entry and one mask, so either all or none have an addend
     // per polynomial; its words are computed on the way, eight at a time with
     // all loads before the first store (one at a time, each store held the
     // next loads back: 16 pairs at N = 2^14 1.04 -> 0.83 ms of these passes)
@@ -1363,7 +1363,9 @@ struct YSeg : MapSeg {
 
 inline bool joins(const YSeg &a, const YSeg &b)
 {
-    return joins(static_cast<const MapSeg &>(a), static_cast<const MapSeg &>(b)) && a.Pm == b.Pm && a.qm == b.qm;
+    // a row unit asks its first two jobs whether there are addends
+    return joins(static_cast<const MapSeg &>(a), static_cast<const MapSeg &>(b)) && a.Pm == b.Pm && a.qm == b.qm &&
+           a.amask == b.amask;
 }
 
 struct YRSt : MapSt {

@@ -138,6 +138,7 @@ def lib() -> ctypes.CDLL:
             "fhe_ntt_inverse_batch": (ci, [vp, vp, ci, ci]),
             "fhe_ntt_inverse": (ci, [vp, vp, vp, ci]),
             "fhe_selftest_modarith": (ci, [u64, u64, u64, ci, ci]),
+            "fhe_selftest_ntt_joins": (ci, []),
             "fhe_ctx_profile": (ci, [vp, ci]),
             "fhe_ctx_autotune": (ci, [vp, ci]),
             "fhe_ctx_ntt_variant": (ci, [vp, ci, vp]),
@@ -944,3 +945,7 @@ def fhe_ctx_profile_read(ctx):
 
 def fhe_selftest_modarith(prime_mod, prime_lo, prime_hi, nprimes, iters) -> int:
     return int(lib().fhe_selftest_modarith(prime_mod, prime_lo, prime_hi, nprimes, iters))
+
+
+def fhe_selftest_ntt_joins() -> int:
+    return int(lib().fhe_selftest_ntt_joins())
