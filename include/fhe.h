@@ -657,7 +657,9 @@ int fhe_mod_switch_noalloc(fhe_ctx *ctx, const uint64_t *in, uint64_t *out, int 
  * contexts created afterwards, skipping the timing (for profiling runs,
  * whose timings would mislead the choice).
  * njobs counts limb transforms: polynomials of min(L+K, 10) limbs, rounded
- * to a multiple of 16 polynomials once there are 16 or more. */
+ * to a multiple of 16 polynomials once there are 16 or more, and raised to
+ * at least 12 units per SM in both passes (smaller launches run as one
+ * kernel, or get the same grid from several variants). */
 int fhe_ctx_autotune(fhe_ctx *ctx, int njobs);
 int fhe_ctx_ntt_variant(fhe_ctx *ctx, int set, float *ms);
 
@@ -683,9 +685,14 @@ int fhe_ctx_profile_read(fhe_ctx *ctx, double *ms, int64_t *count, double *bytes
  * pseudo-random and edge-case inputs per prime of the given chain.  Needs no
  * GPU.  Returns 0 if all agree, else the number of mismatches. */
 int fhe_selftest_modarith(uint64_t prime_mod, uint64_t prime_lo, uint64_t prime_hi, int nprimes, int iters);
-/* The NTT engine's rules on the host, without a GPU (each returns 0 or the
- * number of mismatches): which batches may share a segment. */
+/* The NTT engine's rules on the host, without a GPU (0, or the number of
+ * mismatches): which batches may share a segment. */
 int fhe_selftest_ntt_joins(void);
+/* What fhe_ctx_autotune(ctx, njobs) times for a context of `nprimes` primes on
+ * a device of `sms` SMs: out[0] limbs, out[1] whether they would run as one
+ * kernel (which has no grid policy), out[2..5] and out[6..9] the CTAs of the
+ * column and row pass under each of the four variants. */
+int fhe_selftest_ntt_tune(int log_n, int nprimes, int sms, int njobs, int32_t *out);
 
 #ifdef __cplusplus
 }

@@ -84,17 +84,14 @@ void launch_ntt_inv_scaled_y(fhe_ctx *c, const u64 *in, u64 *out, const LimbMap 
 
 bool ntt_variant_ok(int logN, int v) { return ntt_supported_logn(logN) && v >= 0 && v < FHE_NTT_VARIANTS; }
 
-// Times forward + inverse of `outer` x nl limbs (nl = min(primes, 10)),
-// `outer` rounded to a multiple of 16 when >= 16 so that the row units take
-// their grouped form as in batched use; keeps the faster variant.
+// Times forward + inverse of tune_outer() polynomials of nl = min(primes, 10)
+// limbs; keeps the faster variant.
 int ntt_autotune(fhe_ctx *c, int njobs, float *ms_out)
 {
     LimbMap m;
     memset(&m, 0, sizeof(m));
     m.nl = std::min(c->np, 10);
-    int outer = std::max(1, njobs / m.nl);
-    if (outer >= 16) outer -= outer % 16;
-    const int jobs = outer * m.nl;
+    const int outer = tune_outer(c->logN, m.nl, c->sms, njobs), jobs = outer * m.nl;
     m.in_outer = m.out_outer = (long long)m.nl * c->N;
     for (int i = 0; i < m.nl; i++) m.in_limb[i] = m.out_limb[i] = i, m.prime[i] = i;
     u64 *buf = nullptr;

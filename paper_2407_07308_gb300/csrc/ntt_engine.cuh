@@ -1763,13 +1763,13 @@ void seg_header(SegHdr &H, const fhe_ctx *c, bool fwd, int outer, int nl)
 
 // Grid of a pass: one CTA per unit (variant 0) or a fixed number of resident
 // CTAs per SM that walk the units (variants 1..3: 6, 4 and 2 per SM).
-int grid_of(const fhe_ctx *c, int units)
+int grid_of(int variant, int sms, int units)
 {
     static const int per_sm[FHE_NTT_VARIANTS] = {0, 6, 4, 2};
-    const int v = c->ntt_variant;
-    if (v <= 0 || v >= FHE_NTT_VARIANTS || c->sms <= 0) return units;
-    return std::min(units, per_sm[v] * c->sms);
+    if (variant <= 0 || variant >= FHE_NTT_VARIANTS || sms <= 0) return units;
+    return std::min(units, per_sm[variant] * sms);
 }
+int grid_of(const fhe_ctx *c, int units) { return grid_of(c->ntt_variant, c->sms, units); }
 
 // Unit counts per segment (seg_header) -> first unit of each segment.
 template <class IO>
@@ -1813,15 +1813,49 @@ void recount(IO &io)
 #define FHE_NTT_SMALL_BRANCH 1
 #endif
 
+// Whether a launch of `limbs` limbs of ring degree 2^logN runs as one kernel.
+bool one_kernel(int logN, int sms, bool on_branch, long long limbs)
+{
+    if (logN < SMALL_LO || logN > SMALL_HI) return false;
+    const int own = logN == 15 ? FHE_NTT_SMALL_15 : FHE_NTT_SMALL;
+    return (limbs << (logN - 11)) <= (long long)(on_branch ? FHE_NTT_SMALL_BRANCH : own) * sms;
+}
+
+// Polynomials of nl limbs that the autotuner times for a request of njobs
+// limbs: a multiple of 16 from 16 on, so that the row units take their grouped
+// form as in batched use, and raised until both passes have TUNE_UNITS units
+// per SM.  Below, the choice would rest on noise: launches of up to 6 units per
+// SM run as one kernel, which has no grid policy, and a pass of fewer units
+// than a policy's resident CTAs gets the grid of every other (six per SM is the
+// most; twice that, so that a CTA walks at least two units).
+constexpr int TUNE_UNITS = 12;
+static_assert(TUNE_UNITS > FHE_NTT_SMALL && TUNE_UNITS > FHE_NTT_SMALL_15, "timed in two passes");
+
+int tune_outer(int logN, int nl, int sms, int njobs)
+{
+    int outer = std::max(1, njobs / nl);
+    if (outer >= 16) outer -= outer % 16;
+    const int need = TUNE_UNITS * sms;
+    SegHdr H;
+    memset(&H, 0, sizeof(H));
+    H.logN = logN;
+    H.nl = nl;
+    for (; (long long)outer * nl < 2LL * need; outer = outer / 16 * 16 + 16) {  // a limb is half a unit or more
+        H.outer = outer;
+        unit_counts(H);
+        if (std::min(H.u_cols, H.u_rows) >= need) break;
+    }
+    return outer;
+}
+
 template <class IO, int L>
 void launch_passes(fhe_ctx *c, IO &io, bool fwd)
 {
     if constexpr (L >= SMALL_LO && L <= SMALL_HI) {
         constexpr int C = SMALL_CTAS<L>;
-        long long units = 0;
-        for (int s = 0; s < io.nseg; s++) units += (long long)C * io.h[s].outer * io.h[s].nl;
-        constexpr int own = L == 15 ? FHE_NTT_SMALL_15 : FHE_NTT_SMALL;
-        if (units <= (long long)(c->on_branch ? FHE_NTT_SMALL_BRANCH : own) * c->sms) {
+        long long limbs = 0;
+        for (int s = 0; s < io.nseg; s++) limbs += (long long)io.h[s].outer * io.h[s].nl;
+        if (one_kernel(L, c->sms, c->on_branch, limbs)) {
             int u = 0;
             for (int s = 0; s < io.nseg; s++) {
                 SegHdr &H = io.h[s];

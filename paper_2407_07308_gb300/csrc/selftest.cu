@@ -36,3 +36,23 @@ extern "C" int fhe_selftest_ntt_joins(void)
     bad += joins(x, y);
     return bad;
 }
+
+// The batch the autotuner times and what each grid policy makes of it.
+extern "C" int fhe_selftest_ntt_tune(int log_n, int nprimes, int sms, int njobs, int32_t *out)
+{
+    if (!ntt_supported_logn(log_n) || nprimes < 1 || nprimes > FHE_MAXP || sms < 1 || njobs < 1 || !out)
+        return FHE_EINVAL;
+    SegHdr H;
+    memset(&H, 0, sizeof(H));
+    H.logN = log_n;
+    H.nl = std::min(nprimes, 10);
+    H.outer = tune_outer(log_n, H.nl, sms, njobs);
+    unit_counts(H);
+    out[0] = H.outer * H.nl;
+    out[1] = one_kernel(log_n, sms, false, out[0]);
+    for (int v = 0; v < FHE_NTT_VARIANTS; v++) {
+        out[2 + v] = grid_of(v, sms, H.u_cols);
+        out[2 + FHE_NTT_VARIANTS + v] = grid_of(v, sms, H.u_rows);
+    }
+    return 0;
+}

@@ -139,6 +139,7 @@ def lib() -> ctypes.CDLL:
             "fhe_ntt_inverse": (ci, [vp, vp, vp, ci]),
             "fhe_selftest_modarith": (ci, [u64, u64, u64, ci, ci]),
             "fhe_selftest_ntt_joins": (ci, []),
+            "fhe_selftest_ntt_tune": (ci, [ci, ci, ci, ci, vp]),
             "fhe_ctx_profile": (ci, [vp, ci]),
             "fhe_ctx_autotune": (ci, [vp, ci]),
             "fhe_ctx_ntt_variant": (ci, [vp, ci, vp]),
@@ -949,3 +950,10 @@ def fhe_selftest_modarith(prime_mod, prime_lo, prime_hi, nprimes, iters) -> int:
 
 def fhe_selftest_ntt_joins() -> int:
     return int(lib().fhe_selftest_ntt_joins())
+
+
+def fhe_selftest_ntt_tune(log_n: int, nprimes: int, sms: int, njobs: int):
+    """(limbs timed, as one kernel, column CTAs per variant, row CTAs per variant)."""
+    out = np.zeros(10, dtype=np.int32)
+    _check(lib().fhe_selftest_ntt_tune(log_n, nprimes, sms, njobs, _ptr(out)))
+    return int(out[0]), bool(out[1]), out[2:6].tolist(), out[6:10].tolist()

@@ -18,3 +18,21 @@ def test_segments_join_only_what_shares_a_unit(fhe):
     only: a batch with an addend and one without (or with it on another
     polynomial) stay apart, as do other primes and constants."""
     assert fhe.fhe_selftest_ntt_joins() == 0
+
+
+@pytest.mark.parametrize("sms", [148, 152])
+@pytest.mark.parametrize("nprimes", [2, 5, 13, 24])
+@pytest.mark.parametrize("logN", [10, 11, 12, 13, 14, 15])
+def test_autotuner_times_batches_that_tell_the_policies_apart(fhe, logN, nprimes, sms):
+    """Whatever is asked for, the timed batch runs in two passes (launches in
+    one kernel have no grid policy) and every policy gives it a grid of its
+    own; from the default request up, a batch that does so already stays."""
+    nl = min(nprimes, 10)
+    for njobs in (1, 64, 320, 5000):
+        limbs, one, cols, rows = fhe.fhe_selftest_ntt_tune(logN, nprimes, sms, njobs)
+        assert not one and limbs % nl == 0
+        for grids in (cols, rows):
+            assert sorted(set(grids), reverse=True) == grids, (njobs, grids)
+            assert grids[1:] == [6 * sms, 4 * sms, 2 * sms]
+    if logN >= 14:  # 320 limbs are 2560 units and more
+        assert fhe.fhe_selftest_ntt_tune(logN, nprimes, sms, 320)[0] == 320 // nl // 16 * 16 * nl
