@@ -693,6 +693,13 @@ int fhe_selftest_ntt_joins(void);
  * kernel (which has no grid policy), out[2..5] and out[6..9] the CTAs of the
  * column and row pass under each of the four variants. */
 int fhe_selftest_ntt_tune(int log_n, int nprimes, int sms, int njobs, int32_t *out);
+/* The units of `outer` x nl limbs in every form of a launch, walked with the
+ * kernels' own maps: residues not touched exactly once, units that mix primes,
+ * clusters that mix limbs.  And the shared-memory layouts: elements that
+ * collide or lie outside, exchanges that miss an element, jobs of a joined
+ * segment that miss their batch. */
+int fhe_selftest_ntt_units(int log_n, int outer, int nl);
+int fhe_selftest_ntt_layouts(void);
 
 #ifdef __cplusplus
 }

@@ -175,6 +175,9 @@ constexpr int T = 128;  // threads per CTA, 16 residues each
 #ifndef FHE_NTT_MINB_PAIRED
 #define FHE_NTT_MINB_PAIRED 7
 #endif
+// The maps and layouts below also run on the host (selftest.cu).  Their inlining
+// is left to the compiler: forced, it cost the fused row kernels 16 bytes of
+// spills at N = 2^14 and 2^15.
 // Shared-memory twiddle tables: entry k at k + k / 8 (one 16-byte pad per 8
 // entries), so that the second round's strided twiddle reads (stride up to 8
 // entries across threads) hit distinct banks.
@@ -215,8 +218,8 @@ struct ColLay {
                              : M == 7 && PAIRED ? at_least_mod16(BASE, 2) : at_least_mod16(BASE, 1 + 2 * (BASE % 16 / 2));
     static constexpr int SLOT = !PAIRED ? 0 : M == 8 ? 2 : M == 7 ? 1 : 0;  // the second job's shift
     static constexpr int WORDS = C::NS * P + SLOT;
-    __device__ static int base(int c) { return c * P + (SLOT && c >= C::NS / 2 ? SLOT : 0); }
-    __device__ static int at(int c, int e) { return base(c) + e + (e >> 4); }
+    __host__ __device__ static int base(int c) { return c * P + (SLOT && c >= C::NS / 2 ? SLOT : 0); }
+    __host__ __device__ static int at(int c, int e) { return base(c) + e + (e >> 4); }
 };
 
 template <int M>
@@ -224,8 +227,8 @@ struct RowLay {
     using C = Sub<M>;
     static constexpr int P = at_least_mod16(C::SZ + C::SZ / 16, C::G % 16);
     static constexpr int WORDS = C::NS * P;
-    __device__ static int base(int c) { return c * P; }
-    __device__ static int at(int c, int e) { return c * P + e + (e >> 4); }
+    __host__ __device__ static int base(int c) { return c * P; }
+    __host__ __device__ static int at(int c, int e) { return c * P + e + (e >> 4); }
 };
 
 // staged twiddles (ulonglong2) of a row unit: one table of up to 255 entries,
@@ -311,23 +314,23 @@ __device__ __forceinline__ void round2(u64 (&x)[16], const Geo &geo, int c, int 
 // A thread's residues in shared memory: at the first round's elements (base
 // b + g, elements k G apart) or the second's (base b + 17 g', contiguous).
 template <int G>
-__device__ __forceinline__ void put1(u64 *b, const u64 (&x)[16])
+FHE_HD void put1(u64 *b, const u64 (&x)[16])
 {
 #pragma unroll
     for (int k = 0; k < 16; k++) b[k * G + ((k * G) >> 4)] = x[k];
 }
 template <int G>
-__device__ __forceinline__ void get1(const u64 *b, u64 (&x)[16])
+FHE_HD void get1(const u64 *b, u64 (&x)[16])
 {
 #pragma unroll
     for (int k = 0; k < 16; k++) x[k] = b[k * G + ((k * G) >> 4)];
 }
-__device__ __forceinline__ void put2(u64 *b, const u64 (&x)[16])
+FHE_HD void put2(u64 *b, const u64 (&x)[16])
 {
 #pragma unroll
     for (int k = 0; k < 16; k++) b[k] = x[k];
 }
-__device__ __forceinline__ void get2(const u64 *b, u64 (&x)[16])
+FHE_HD void get2(const u64 *b, u64 (&x)[16])
 {
 #pragma unroll
     for (int k = 0; k < 16; k++) x[k] = b[k];
@@ -354,6 +357,9 @@ struct ColGeo {
     static constexpr int TWC = twp_size(1 << N1);                      // staged twiddles per job
     static constexpr int TW = NJ * TWC;
     static_assert(NJ <= 2, "jobs per column unit");
+    // a unit's first job and its first column
+    __host__ __device__ static int job0(int lu) { return lu / BLK * NJ; }
+    __host__ __device__ static int lo0(int lu) { return lu % BLK * NC; }
     // word r of the unit: job slot, column in job, element
     __device__ static int jslot(int r) { return NJ == 1 ? 0 : r / (NC * SZ); }
     __device__ static int col(int r) { return r % NC; }
@@ -445,7 +451,7 @@ struct SegIO {
     SegHdr h[FHE_SEGS];
     S s[FHE_SEGS];
     // the payload of a job, with the job's place in it
-    __device__ const S &payload(int sg, int &job) const
+    __host__ __device__ const S &payload(int sg, int &job) const
     {
         const SegHdr &H = h[sg];
         const int k = H.outer == H.per ? 0 : job / (H.nl * H.per);
@@ -690,8 +696,8 @@ __device__ __forceinline__ int col_jobs(const IO &io, int sg, int lu, typename I
     using Gm = ColGeo<N1, N2, IO::XJ>;
     const SegHdr &H = io.h[sg];
     const int njobs = H.outer * H.nl;
-    const int job0 = (lu / Gm::BLK) * Gm::NJ;
-    *lo0 = (lu % Gm::BLK) * Gm::NC;
+    const int job0 = Gm::job0(lu);
+    *lo0 = Gm::lo0(lu);
     if (threadIdx.x < Gm::NJ && job0 + (int)threadIdx.x < njobs) io.begin_c(sg, job0 + threadIdx.x, sts[threadIdx.x]);
     __syncthreads();
     return njobs - job0;  // valid job slots (>= 1)
@@ -721,7 +727,7 @@ __device__ __forceinline__ void fwd_cols_unit1(const IO &io, int sg, int lu, u64
     using C = typename Gm::C;
     const int c = threadIdx.x % C::NS, g = threadIdx.x / C::NS;
     const SegHdr &H = io.h[sg];
-    const int lo = (lu % Gm::BLK) * Gm::NC + c;
+    const int lo = Gm::lo0(lu) + c;
     col_twiddles<N1>(W, H.tw + (size_t)st.prime * Gm::NN);
     const ModQ &m = H.mq[st.prime];
     const ColTw<N1, N2, 1> geo{W, m.q, m.q, &m, &m};
@@ -767,9 +773,9 @@ __device__ __forceinline__ void inv_cols_unit1(const IO &io, int sg, int lu, u64
     using C = typename Gm::C;
     const int c = threadIdx.x % C::NS, g = threadIdx.x / C::NS;
     const SegHdr &H = io.h[sg];
-    const int lo = (lu % Gm::BLK) * Gm::NC + c;
+    const int lo = Gm::lo0(lu) + c;
     typename IO::CSt st;
-    io.begin_c(sg, lu / Gm::BLK, st);
+    io.begin_c(sg, Gm::job0(lu), st);
     col_twiddles<N1>(W, H.tw + (size_t)st.prime * Gm::NN);
     const ModQ &m = H.mq[st.prime];
     const ColTw<N1, N2, 1> geo{W, m.q, m.q, &m, &m};
@@ -810,7 +816,7 @@ __device__ __forceinline__ void fwd_cols_unit(const IO &io, int sg, int lu, u64 
     using C = typename Gm::C;
     if constexpr (Gm::NJ == 1) {
         typename IO::CSt st;  // computed by every thread, in registers
-        io.begin_c(sg, lu / Gm::BLK, st);
+        io.begin_c(sg, Gm::job0(lu), st);
         fwd_cols_unit1<N1, N2>(io, sg, lu, sm, W, st);
         return;
     }
@@ -929,30 +935,42 @@ __device__ __forceinline__ void inv_cols_unit(const IO &io, int sg, int lu, u64 
     }
 }
 
-// The jobs of a row unit.  Grouped: slots jj < 16 hold jobs (oc 16 + jj) nl
-// + l, rows hi0 .. hi0+R-1; single: slot 0 holds the job, rows hi0 ..
-// hi0+NS-1.  Returns the number of valid slots.
+// The jobs of a row unit: slots jj < nvalid, rows hi0 on.  Grouped: jobs
+// (o0 + jj) nl + l, R rows; single: one job, l, NS rows.
+template <int N1, int N2, bool GRP>
+struct RowUnit {
+    using Gm = RowGeo<N1, N2>;
+    int hi0, nvalid, o0, l;
+    __host__ __device__ RowUnit(const SegHdr &H, int lu)
+    {
+        if (GRP) {
+            const int OC = (H.gouter + ROW_J - 1) / ROW_J;
+            const int hc = lu % Gm::CH, t = lu / Gm::CH;
+            const int oc = t % OC;
+            l = t / OC;
+            hi0 = hc * Gm::R;
+            o0 = oc * ROW_J;
+            nvalid = H.gouter - o0 < ROW_J ? H.gouter - o0 : ROW_J;
+        } else {
+            const int v = lu - H.g_units;
+            hi0 = (v % Gm::CHS) * Gm::NS;
+            nvalid = 1;
+            o0 = 0;
+            l = H.gouter * H.nl + v / Gm::CHS;
+        }
+    }
+    __host__ __device__ int job(const SegHdr &H, int jj) const { return GRP ? (o0 + jj) * H.nl + l : l; }
+};
+
+// The same, with the jobs' states begun; returns the number of valid slots.
 template <int N1, int N2, bool GRP, class IO>
 __device__ __forceinline__ int row_jobs(const IO &io, int sg, int lu, typename IO::RSt *sts, int *hi0)
 {
-    using Gm = RowGeo<N1, N2>;
-    const SegHdr &H = io.h[sg];
-    int nvalid;
-    if (GRP) {
-        const int OC = (H.gouter + ROW_J - 1) / ROW_J;
-        const int hc = lu % Gm::CH, t = lu / Gm::CH;
-        const int oc = t % OC, l = t / OC;
-        *hi0 = hc * Gm::R;
-        nvalid = min(ROW_J, H.gouter - oc * ROW_J);
-        if ((int)threadIdx.x < nvalid) io.begin_r(sg, (oc * ROW_J + threadIdx.x) * H.nl + l, sts[threadIdx.x]);
-    } else {
-        const int v = lu - H.g_units;
-        *hi0 = (v % Gm::CHS) * Gm::NS;
-        nvalid = 1;
-        if (threadIdx.x == 0) io.begin_r(sg, H.gouter * H.nl + v / Gm::CHS, sts[0]);
-    }
+    const RowUnit<N1, N2, GRP> u(io.h[sg], lu);
+    *hi0 = u.hi0;
+    if ((int)threadIdx.x < u.nvalid) io.begin_r(sg, u.job(io.h[sg], threadIdx.x), sts[threadIdx.x]);
     __syncthreads();
-    return nvalid;
+    return u.nvalid;
 }
 
 // Grouped rows stage the R rows' twiddles: entry k of row r is the stage
@@ -976,12 +994,12 @@ template <int N1, int N2, bool GRP>
 struct RowMap {
     using Gm = RowGeo<N1, N2>;
     int hi0;
-    __device__ int c(int r) const { return r >> N2; }
-    __device__ int f(int r) const { return r & (Gm::SZ - 1); }
-    __device__ int cslot(int c) const { return GRP ? c / Gm::R : 0; }
-    __device__ int crow(int c) const { return hi0 + (GRP ? c % Gm::R : c); }
-    __device__ int slot(int r) const { return cslot(c(r)); }
-    __device__ int row(int r) const { return crow(c(r)); }
+    __host__ __device__ int c(int r) const { return r >> N2; }
+    __host__ __device__ int f(int r) const { return r & (Gm::SZ - 1); }
+    __host__ __device__ int cslot(int c) const { return GRP ? c / Gm::R : 0; }
+    __host__ __device__ int crow(int c) const { return hi0 + (GRP ? c % Gm::R : c); }
+    __host__ __device__ int slot(int r) const { return cslot(c(r)); }
+    __host__ __device__ int row(int r) const { return crow(c(r)); }
 };
 
 // Forward, rows: global stages N1..N1+N2-1, then the functor's store.
@@ -1240,7 +1258,7 @@ __global__ void __launch_bounds__(T, 4) k_fwd_small(const __grid_constant__ IO i
     __shared__ typename IO::RSt rst[1];
     __shared__ typename IO::CSt cst[1];
     const int u = blockIdx.x, sg = seg_of(io, u, false), lu = u - io.h[sg].u_cols;
-    if (threadIdx.x == 32) io.begin_c(sg, lu / SMALL_CTAS<L>, cst[0]);  // published by row_jobs' barrier
+    if (threadIdx.x == 32) io.begin_c(sg, SmallGeo<L>::Col::job0(lu), cst[0]);  // published by row_jobs' barrier
     fwd_rows_unit<N1, N2, false>(io, sg, lu, sm, W, rst, [&] {
         fwd_cols_unit1<N1, N2>(io, sg, lu, sm, W, cst[0]);
         job_barrier<L>();
@@ -1848,6 +1866,15 @@ int tune_outer(int logN, int nl, int sms, int njobs)
     return outer;
 }
 
+// The segment's units of the one-kernel form from unit u on (a limb's units, one
+// limb after the other, in both passes); the unit after them.
+int one_kernel_units(SegHdr &H, int u)
+{
+    H.gouter = H.g_units = 0;
+    H.u_cols = H.u_rows = u;
+    return u + (H.outer * H.nl << (H.logN - SMALL_LO));
+}
+
 template <class IO, int L>
 void launch_passes(fhe_ctx *c, IO &io, bool fwd)
 {
@@ -1857,12 +1884,7 @@ void launch_passes(fhe_ctx *c, IO &io, bool fwd)
         for (int s = 0; s < io.nseg; s++) limbs += (long long)io.h[s].outer * io.h[s].nl;
         if (one_kernel(L, c->sms, c->on_branch, limbs)) {
             int u = 0;
-            for (int s = 0; s < io.nseg; s++) {
-                SegHdr &H = io.h[s];
-                H.gouter = H.g_units = 0;
-                H.u_cols = H.u_rows = u;
-                u += C * H.outer * H.nl;
-            }
+            for (int s = 0; s < io.nseg; s++) u = one_kernel_units(io.h[s], u);
             const bool pdl = pdl_on(c, u, T);
             if constexpr ((IO::DIRS & DIR_FWD) != 0)
                 if (fwd) launch_pdl_cluster(k_fwd_small<IO, L>, pdl, u, T, C, c->stream, io);

@@ -140,6 +140,8 @@ def lib() -> ctypes.CDLL:
             "fhe_selftest_modarith": (ci, [u64, u64, u64, ci, ci]),
             "fhe_selftest_ntt_joins": (ci, []),
             "fhe_selftest_ntt_tune": (ci, [ci, ci, ci, ci, vp]),
+            "fhe_selftest_ntt_units": (ci, [ci, ci, ci]),
+            "fhe_selftest_ntt_layouts": (ci, []),
             "fhe_ctx_profile": (ci, [vp, ci]),
             "fhe_ctx_autotune": (ci, [vp, ci]),
             "fhe_ctx_ntt_variant": (ci, [vp, ci, vp]),
@@ -957,3 +959,11 @@ def fhe_selftest_ntt_tune(log_n: int, nprimes: int, sms: int, njobs: int):
     out = np.zeros(10, dtype=np.int32)
     _check(lib().fhe_selftest_ntt_tune(log_n, nprimes, sms, njobs, _ptr(out)))
     return int(out[0]), bool(out[1]), out[2:6].tolist(), out[6:10].tolist()
+
+
+def fhe_selftest_ntt_units(log_n: int, outer: int, nl: int) -> int:
+    return _check(lib().fhe_selftest_ntt_units(log_n, outer, nl))
+
+
+def fhe_selftest_ntt_layouts() -> int:
+    return int(lib().fhe_selftest_ntt_layouts())

@@ -36,3 +36,16 @@ def test_autotuner_times_batches_that_tell_the_policies_apart(fhe, logN, nprimes
             assert grids[1:] == [6 * sms, 4 * sms, 2 * sms]
     if logN >= 14:  # 320 limbs are 2560 units and more
         assert fhe.fhe_selftest_ntt_tune(logN, nprimes, sms, 320)[0] == 320 // nl // 16 * 16 * nl
+
+
+@pytest.mark.parametrize("outer,nl", [(1, 3), (5, 2), (11, 1), (12, 2), (16, 3), (21, 2), (28, 1), (29, 1), (40, 2)])
+@pytest.mark.parametrize("logN", [10, 11, 12, 13, 14, 15])
+def test_units_cover_every_residue_once(fhe, logN, outer, nl):
+    """Column units of one job and of pairs (an odd number of jobs leaves a
+    slot empty), grouped row units with the rest as single ones (fewer than 12
+    outer items beyond a multiple of 16), and the one-kernel form."""
+    assert fhe.fhe_selftest_ntt_units(logN, outer, nl) == 0
+
+
+def test_layouts_keep_elements_apart(fhe):
+    assert fhe.fhe_selftest_ntt_layouts() == 0
