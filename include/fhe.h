@@ -700,6 +700,12 @@ int fhe_selftest_ntt_tune(int log_n, int nprimes, int sms, int njobs, int32_t *o
  * segment that miss their batch. */
 int fhe_selftest_ntt_units(int log_n, int outer, int nl);
 int fhe_selftest_ntt_layouts(void);
+/* One pass of a transform of one limb mod the prime q = 1 (mod 2N), in the
+ * kernels' own arithmetic, thread by thread: pass 0 forward columns (words
+ * below 7q), 1 forward rows (below (4 ceil(log_n / 2) + 7) q; canonical out),
+ * 2 inverse rows (below 4q), 3 inverse columns (below 4q; canonical out).
+ * Returns the number of residues that two unit forms disagree on or miss. */
+int fhe_selftest_ntt_pass(int log_n, uint64_t q, int pass, const uint64_t *in, uint64_t *out);
 
 #ifdef __cplusplus
 }

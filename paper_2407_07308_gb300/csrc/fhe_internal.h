@@ -332,6 +332,7 @@ int host_find_primes(u64 U, u64 lo, u64 hi, int count, u64 *out);
 u64 host_powmod(u64 a, u64 e, u64 q);
 u64 host_invmod(u64 a, u64 q);
 u64 host_mulmod(u64 a, u64 b, u64 q);
+u64 limb_tables(u64 q, int logN, ulonglong2 *fwd, ulonglong2 *inv, ulonglong2 *ninv);
 int build_tables(fhe_ctx *ctx);
 void lt_poly_coefficients(int p, std::vector<int> &out);
 void lt_bivariate_coefficients(int p, std::vector<int> &out);

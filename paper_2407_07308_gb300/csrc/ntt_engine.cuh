@@ -83,7 +83,7 @@ namespace {
 // chain).  Also measured and not kept: X + t by multiply-adds as well (2606,
 // no gain on its own: 2570), and the inverse's 4q reduction as an unsigned
 // minimum (2554).
-__device__ __forceinline__ u64 bfly_mul(u64 a, const ulonglong2 w, u64 q)
+FHE_HD u64 bfly_mul(u64 a, const ulonglong2 w, u64 q)
 {
     return shoup_lazy4_chain(a, w.x, w.y, 0 - q);
 }
@@ -94,7 +94,7 @@ __device__ __forceinline__ u64 bfly_mul(u64 a, const ulonglong2 w, u64 q)
 // the fused conversions) stay below (4s + 7) q <= 67 q < 2^64 after s <= 15
 // stages for primes below 2^57; one reduction at the end brings every value
 // to [0, q).  q4 = 4q.
-__device__ __forceinline__ void ct_bfly(u64 &X, u64 &Y, const ulonglong2 w, u64 q, u64 q4)
+FHE_HD void ct_bfly(u64 &X, u64 &Y, const ulonglong2 w, u64 q, u64 q4)
 {
     const u64 t = bfly_mul(Y, w, q);
     const u64 x = X;
@@ -108,7 +108,7 @@ __device__ __forceinline__ void ct_bfly(u64 &X, u64 &Y, const ulonglong2 w, u64 
 // stages' bounds are 4q 2^j; reduce_few brings the sums back at the end of a
 // row pass (and, for primes above 54 bits, between its two rounds), where a
 // compare and subtract in every butterfly took 5 of its 22 instructions.
-__device__ __forceinline__ void gs_bfly(u64 &X, u64 &Y, const ulonglong2 w, u64 q, u64 B)
+FHE_HD void gs_bfly(u64 &X, u64 &Y, const ulonglong2 w, u64 q, u64 B)
 {
     const u64 d = X - Y + B;
     X = X + Y;
@@ -118,7 +118,7 @@ __device__ __forceinline__ void gs_bfly(u64 &X, u64 &Y, const ulonglong2 w, u64 
 // Stages s0 .. s0+R-1 of the forward transform on one group x[0..2^R) whose
 // block index is hi.
 template <int R, class TW>
-__device__ __forceinline__ void fwd_round(u64 (&x)[1 << R], int s0, int hi, const TW &W, u64 q, u64 q4)
+FHE_HD void fwd_round(u64 (&x)[1 << R], int s0, int hi, const TW &W, u64 q, u64 q4)
 {
 #pragma unroll
     for (int u = 0; u < R; u++) {
@@ -139,7 +139,7 @@ __device__ __forceinline__ void fwd_round(u64 (&x)[1 << R], int s0, int hi, cons
 // half-distance 2^(R-1-U).  A template per stage keeps every index a
 // compile-time constant, so x stays in registers.
 template <int R, int U, class TW>
-__device__ __forceinline__ void inv_stage(u64 (&x)[1 << R], int s0, int hi, const TW &W, u64 q, u64 B)
+FHE_HD void inv_stage(u64 (&x)[1 << R], int s0, int hi, const TW &W, u64 q, u64 B)
 {
     constexpr int half = 1 << (R - 1 - U);
 #pragma unroll
@@ -153,7 +153,7 @@ __device__ __forceinline__ void inv_stage(u64 (&x)[1 << R], int s0, int hi, cons
 
 // Inputs below B; outputs below 2^R B, the upper half of x below 4q.
 template <int R, class TW>
-__device__ __forceinline__ void inv_round(u64 (&x)[1 << R], int s0, int hi, const TW &W, u64 q, u64 B)
+FHE_HD void inv_round(u64 (&x)[1 << R], int s0, int hi, const TW &W, u64 q, u64 B)
 {
     inv_stage<R, R - 1>(x, s0, hi, W, q, B);
 }
@@ -240,12 +240,19 @@ constexpr int ROW_J = 16;                    // jobs per grouped row unit
 // stage s with in-stage index j < 2^s.
 struct GTw {  // the full table in global memory, read-only path
     const ulonglong2 *__restrict__ p;
-    __device__ ulonglong2 get(int s, int j) const { return __ldg(p + (1 << s) + j); }
+    __host__ __device__ ulonglong2 get(int s, int j) const
+    {
+#ifdef __CUDA_ARCH__
+        return __ldg(p + (1 << s) + j);
+#else
+        return p[(1 << s) + j];
+#endif
+    }
 };
 
 struct PrefixTw {  // the first entries of the table, copied to shared memory
     const ulonglong2 *sm;
-    __device__ ulonglong2 get(int s, int j) const { return sm[twp((1 << s) + j)]; }
+    __host__ __device__ ulonglong2 get(int s, int j) const { return sm[twp((1 << s) + j)]; }
 };
 
 // Row twiddles of one row hi (stages N1.., in-stage index hi 2^u + t) staged
@@ -253,7 +260,7 @@ struct PrefixTw {  // the first entries of the table, copied to shared memory
 struct RowTw {
     const ulonglong2 *sm;
     int N1, hi;
-    __device__ ulonglong2 get(int s, int j) const
+    __host__ __device__ ulonglong2 get(int s, int j) const
     {
         const int u = s - N1;
         return sm[twp((1 << u) - 1 + j - (hi << u))];
@@ -273,7 +280,7 @@ struct RowTw {
 constexpr int INV_WIDE_BITS = 54;
 
 template <int M, bool FWD, class Geo>
-__device__ __forceinline__ void round1(u64 (&x)[16], const Geo &geo, int c)
+FHE_HD void round1(u64 (&x)[16], const Geo &geo, int c)
 {
     const auto W = geo.tw(c);
     const u64 q = geo.q(c), q4 = 4 * q;  // lazy bound of the butterflies
@@ -292,7 +299,7 @@ __device__ __forceinline__ void round1(u64 (&x)[16], const Geo &geo, int c)
 }
 
 template <int M, bool FWD, class Geo>
-__device__ __forceinline__ void round2(u64 (&x)[16], const Geo &geo, int c, int gp)
+FHE_HD void round2(u64 (&x)[16], const Geo &geo, int c, int gp)
 {
     constexpr int G = Sub<M>::G, R2 = Sub<M>::R2, NB = 16 / G;
     const auto W = geo.tw(c);
@@ -373,10 +380,10 @@ struct ColTw {
     u64 q0, q1;
     const ModQ *m0, *m1;
     static constexpr int S = 0;
-    __device__ PrefixTw tw(int c) const { return PrefixTw{W + (c / Gm::NC) * Gm::TWC}; }
-    __device__ int hi(int) const { return 0; }
-    __device__ u64 q(int c) const { return c / Gm::NC == 0 ? q0 : q1; }
-    __device__ const ModQ &mq(int c) const { return c / Gm::NC == 0 ? *m0 : *m1; }
+    __host__ __device__ PrefixTw tw(int c) const { return PrefixTw{W + (c / Gm::NC) * Gm::TWC}; }
+    __host__ __device__ int hi(int) const { return 0; }
+    __host__ __device__ u64 q(int c) const { return c / Gm::NC == 0 ? q0 : q1; }
+    __host__ __device__ const ModQ &mq(int c) const { return c / Gm::NC == 0 ? *m0 : *m1; }
 };
 
 // Row pass: grouped (16 jobs of one prime x R adjacent rows) or single (NS
@@ -402,14 +409,14 @@ struct RowGrpTw {
     int hi0;
     const ModQ &m;
     int S;
-    __device__ RowTw tw(int c) const
+    __host__ __device__ RowTw tw(int c) const
     {
         constexpr int R = RowGeo<N1, N2>::R;
         return RowTw{W + (c % R) * RowGeo<N1, N2>::TWR, N1, hi0 + c % R};
     }
-    __device__ int hi(int c) const { return hi0 + c % RowGeo<N1, N2>::R; }
-    __device__ u64 q(int) const { return m.q; }
-    __device__ const ModQ &mq(int) const { return m; }
+    __host__ __device__ int hi(int c) const { return hi0 + c % RowGeo<N1, N2>::R; }
+    __host__ __device__ u64 q(int) const { return m.q; }
+    __host__ __device__ const ModQ &mq(int) const { return m; }
 };
 
 struct RowOneTw {
@@ -417,10 +424,10 @@ struct RowOneTw {
     int hi0;
     const ModQ &m;
     int S;
-    __device__ GTw tw(int) const { return g; }
-    __device__ int hi(int c) const { return hi0 + c; }
-    __device__ u64 q(int) const { return m.q; }
-    __device__ const ModQ &mq(int) const { return m; }
+    __host__ __device__ GTw tw(int) const { return g; }
+    __host__ __device__ int hi(int c) const { return hi0 + c; }
+    __host__ __device__ u64 q(int) const { return m.q; }
+    __host__ __device__ const ModQ &mq(int) const { return m; }
 };
 
 // ---------------------------------------------------------------------------
@@ -761,7 +768,7 @@ __device__ __forceinline__ void fwd_cols_unit1(const IO &io, int sg, int lu, u64
 
 // The last product of an inverse transform: a value anywhere in 64 bits times
 // N^-1 (and the entry's constant), canonical.
-__device__ __forceinline__ u64 inv_scaled(u64 v, const ulonglong2 ni, const ModQ &m)
+FHE_HD u64 inv_scaled(u64 v, const ulonglong2 ni, const ModQ &m)
 {
     return reduce4q(shoup_lazy4_chain(v, ni.x, ni.y, 0 - m.q), m.q2, m.q);
 }

@@ -173,6 +173,29 @@ static int upload(fhe_ctx *c, void **dst, const void *src, size_t bytes)
     return 0;
 }
 
+// The transforms' tables of one prime (Shoup pairs): psi^brv(k) and psi^-brv(k)
+// for k < N, and N^-1.  Returns psi, a primitive 2N-th root of unity.
+u64 limb_tables(u64 q, int logN, ulonglong2 *fwd, ulonglong2 *inv, ulonglong2 *ninv)
+{
+    const int N = 1 << logN;
+    const u64 psi = host_powmod(smallest_primitive_root(q), (q - 1) / (2 * (u64)N), q), ipsi = host_invmod(psi, q);
+    // psi^k for k < N, then scatter to bit-reversed positions
+    std::vector<u64> pw(N), ipw(N);
+    pw[0] = ipw[0] = 1;
+    for (int k = 1; k < N; k++) {
+        pw[k] = host_mulmod(pw[k - 1], psi, q);
+        ipw[k] = host_mulmod(ipw[k - 1], ipsi, q);
+    }
+    for (int k = 0; k < N; k++) {
+        const u64 w = pw[bit_reverse(k, logN)], iw = ipw[bit_reverse(k, logN)];
+        fwd[k] = make_ulonglong2(w, shoup_const(w, q));
+        inv[k] = make_ulonglong2(iw, shoup_const(iw, q));
+    }
+    const u64 ni = host_invmod((u64)N % q, q);
+    *ninv = make_ulonglong2(ni, shoup_const(ni, q));
+    return psi;
+}
+
 int build_tables(fhe_ctx *c)
 {
     const int N = c->N, np = c->np, L = c->L, K = c->K;
@@ -180,25 +203,8 @@ int build_tables(fhe_ctx *c)
     c->psi.resize(np);
     std::vector<ulonglong2> fwd((size_t)np * N), inv((size_t)np * N), ninv(np);
     for (int i = 0; i < np; i++) {
-        u64 q = c->q[i];
-        c->mq[i] = make_modq(q);
-        u64 g = smallest_primitive_root(q);
-        u64 psi = host_powmod(g, (q - 1) / (2 * (u64)N), q), ipsi = host_invmod(psi, q);
-        c->psi[i] = psi;
-        // psi^k for k < N, then scatter to bit-reversed positions
-        std::vector<u64> pw(N), ipw(N);
-        pw[0] = ipw[0] = 1;
-        for (int k = 1; k < N; k++) {
-            pw[k] = host_mulmod(pw[k - 1], psi, q);
-            ipw[k] = host_mulmod(ipw[k - 1], ipsi, q);
-        }
-        for (int k = 0; k < N; k++) {
-            u64 w = pw[bit_reverse(k, c->logN)], iw = ipw[bit_reverse(k, c->logN)];
-            fwd[(size_t)i * N + k] = make_ulonglong2(w, shoup_const(w, q));
-            inv[(size_t)i * N + k] = make_ulonglong2(iw, shoup_const(iw, q));
-        }
-        u64 ni = host_invmod((u64)N % q, q);
-        ninv[i] = make_ulonglong2(ni, shoup_const(ni, q));
+        c->mq[i] = make_modq(c->q[i]);
+        c->psi[i] = limb_tables(c->q[i], c->logN, fwd.data() + (size_t)i * N, inv.data() + (size_t)i * N, &ninv[i]);
     }
     int e;
     if ((e = upload(c, (void **)&c->d_mq, c->mq.data(), sizeof(ModQ) * np))) return e;

@@ -238,3 +238,164 @@ extern "C" int fhe_selftest_ntt_layouts(void)
 {
     return check_layouts<5>() + check_layouts<6>() + check_layouts<7>() + check_layouts<8>() + check_payloads();
 }
+
+// ---------------------------------------------------------------------------
+// arithmetic: one pass over a limb, thread by thread, with the kernels' rounds,
+// twiddle accessors, layouts and closing reductions
+// ---------------------------------------------------------------------------
+
+namespace {
+
+struct Limb {
+    const u64 *in;
+    u64 *out;
+    std::vector<char> set;
+    int bad = 0;
+    Limb(const u64 *i, u64 *o, int N) : in(i), out(o), set(N, 0) {}
+    void put(int i, u64 v)  // several slots of a unit hold the same limb
+    {
+        bad += set[i] && out[i] != v;
+        out[i] = v;
+        set[i] = 1;
+    }
+};
+
+template <int L, bool FWD, int XJ>
+void pass_cols(Limb &io, const ModQ &m, const ulonglong2 *tw, ulonglong2 ninv)
+{
+    constexpr int N1 = Deg<L>::N1, N2 = Deg<L>::N2;
+    using Gm = ColGeo<N1, N2, XJ>;
+    using C = typename Gm::C;
+    std::vector<u64> sm(Gm::Lay::WORDS);
+    std::vector<ulonglong2> W(Gm::TW);
+    for (int j = 0; j < Gm::NJ; j++)
+        for (int i = 0; i < (1 << N1); i++) W[j * Gm::TWC + twp(i)] = tw[i];
+    const ColTw<N1, N2, XJ> geo{W.data(), m.q, m.q, &m, &m};
+    for (int lu = 0; lu < Gm::BLK; lu++)
+        for (int half = 0; half < 2; half++)  // before and after the exchange
+            for (int t = 0; t < T; t++) {
+                const int c = t % C::NS, g = t / C::NS, lo = Gm::lo0(lu) + c % Gm::NC;
+                u64 *b = sm.data() + Gm::Lay::base(c), x[16];
+                if (FWD && half == 0) {
+                    for (int k = 0; k < 16; k++) x[k] = io.in[((k * C::G + g) << N2) + lo];
+                    round1<N1, true>(x, geo, c);
+                    put1<C::G>(b + g, x);
+                } else if (FWD) {
+                    get2(b + 17 * g, x);
+                    round2<N1, true>(x, geo, c, g);
+                    for (int k = 0; k < 16; k++) io.put((((g << 4) + k) << N2) + lo, x[k]);
+                } else if (half == 0) {
+                    for (int k = 0; k < 16; k++) x[k] = io.in[(((g << 4) + k) << N2) + lo];
+                    round2<N1, false>(x, geo, c, g);
+                    put2(b + 17 * g, x);
+                } else {
+                    get1<C::G>(b + g, x);
+                    round1<N1, false>(x, geo, c);
+                    for (int k = 0; k < 16; k++) io.put(((k * C::G + g) << N2) + lo, inv_scaled(x[k], ninv, m));
+                }
+            }
+}
+
+template <int L, bool FWD, bool GRP>
+void pass_rows(Limb &io, const ModQ &m, const ulonglong2 *tw)
+{
+    constexpr int N1 = Deg<L>::N1, N2 = Deg<L>::N2;
+    using Gm = RowGeo<N1, N2>;
+    using C = typename Gm::C;
+    using Lay = typename Gm::Lay;
+    std::vector<u64> sm(Lay::WORDS);
+    std::vector<ulonglong2> W(TW_ROWS);
+    for (int lu = 0; lu < (GRP ? Gm::CH : Gm::CHS); lu++) {
+        const int hi0 = lu * (GRP ? Gm::R : Gm::NS);
+        const RowMap<N1, N2, GRP> mp{hi0};
+        for (int r = 0; r < (GRP ? Gm::R : 0); r++)
+            for (int e = 0; e < Gm::SZ - 1; e++) {
+                int u = 0;
+                while ((2 << u) <= e + 1) u++;
+                W[r * Gm::TWR + twp(e)] = tw[(1 << (N1 + u)) + ((hi0 + r) << u) + (e + 1 - (1 << u))];
+            }
+        const RowGrpTw<N1, N2> grp{W.data(), hi0, m, N1};
+        const RowOneTw one{GTw{tw}, hi0, m, N1};
+        auto first = [&](u64(&x)[16], int c) {
+            if constexpr (GRP)
+                round1<N2, FWD>(x, grp, c);
+            else
+                round1<N2, FWD>(x, one, c);
+        };
+        auto second = [&](u64(&x)[16], int c, int g) {
+            if constexpr (GRP)
+                round2<N2, FWD>(x, grp, c, g);
+            else
+                round2<N2, FWD>(x, one, c, g);
+        };
+        for (int half = 0; half < 2; half++)
+            for (int t = 0; t < T; t++) {
+                const int c = t / C::G, g = t % C::G, row = mp.crow(c) << N2;
+                u64 *b = sm.data() + Lay::base(c), x[16];
+                if (FWD && half == 0) {
+                    for (int k = 0; k < 16; k++) x[k] = io.in[row + k * C::G + g];
+                    first(x, c);
+                    put1<C::G>(b + g, x);
+                } else if (FWD) {
+                    get2(b + 17 * g, x);
+                    second(x, c, g);
+                    for (int k = 0; k < 16; k++) io.put(row + 16 * g + k, reduce2q(reduce_few(x[k], m), m.q));
+                } else if (half == 0) {
+                    for (int k = 0; k < 16; k++) x[k] = io.in[row + 16 * g + k];
+                    second(x, c, g);
+                    put2(b + 17 * g, x);
+                } else {
+                    get1<C::G>(b + g, x);
+                    first(x, c);
+                    for (int k = 0; k < 16; k++) io.put(row + k * C::G + g, k < 8 ? reduce_few(x[k], m) : x[k]);
+                }
+            }
+    }
+}
+
+template <int L>
+int run_pass(u64 q, int pass, const u64 *in, u64 *out)
+{
+    const int N = 1 << L;
+    std::vector<ulonglong2> fwd(N), inv(N);
+    ulonglong2 ninv;
+    limb_tables(q, L, fwd.data(), inv.data(), &ninv);
+    const ModQ m = make_modq(q);
+    Limb io(in, out, N);
+    switch (pass) {
+    case 0:
+        pass_cols<L, true, 1>(io, m, fwd.data(), ninv);
+        pass_cols<L, true, 2>(io, m, fwd.data(), ninv);
+        break;
+    case 1:
+        pass_rows<L, true, true>(io, m, fwd.data());
+        if (L > 10) pass_rows<L, true, false>(io, m, fwd.data());  // n = 10 has grouped units only
+        break;
+    case 2:
+        pass_rows<L, false, true>(io, m, inv.data());
+        if (L > 10) pass_rows<L, false, false>(io, m, inv.data());
+        break;
+    default:
+        pass_cols<L, false, 1>(io, m, inv.data(), ninv);
+        pass_cols<L, false, 2>(io, m, inv.data(), ninv);
+    }
+    for (char s : io.set) io.bad += !s;
+    return io.bad;
+}
+
+}  // namespace
+
+extern "C" int fhe_selftest_ntt_pass(int log_n, uint64_t q, int pass, const uint64_t *in, uint64_t *out)
+{
+    if (!in || !out || pass < 0 || pass > 3 || !ntt_supported_logn(log_n) || q >> 57 || (q - 1) % (2ull << log_n) ||
+        !host_is_prime(q))
+        return FHE_EINVAL;
+    switch (log_n) {
+    case 10: return run_pass<10>(q, pass, in, out);
+    case 11: return run_pass<11>(q, pass, in, out);
+    case 12: return run_pass<12>(q, pass, in, out);
+    case 13: return run_pass<13>(q, pass, in, out);
+    case 14: return run_pass<14>(q, pass, in, out);
+    default: return run_pass<15>(q, pass, in, out);
+    }
+}

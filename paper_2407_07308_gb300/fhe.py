@@ -142,6 +142,7 @@ def lib() -> ctypes.CDLL:
             "fhe_selftest_ntt_tune": (ci, [ci, ci, ci, ci, vp]),
             "fhe_selftest_ntt_units": (ci, [ci, ci, ci]),
             "fhe_selftest_ntt_layouts": (ci, []),
+            "fhe_selftest_ntt_pass": (ci, [ci, u64, ci, vp, vp]),
             "fhe_ctx_profile": (ci, [vp, ci]),
             "fhe_ctx_autotune": (ci, [vp, ci]),
             "fhe_ctx_ntt_variant": (ci, [vp, ci, vp]),
@@ -967,3 +968,11 @@ def fhe_selftest_ntt_units(log_n: int, outer: int, nl: int) -> int:
 
 def fhe_selftest_ntt_layouts() -> int:
     return int(lib().fhe_selftest_ntt_layouts())
+
+
+def fhe_selftest_ntt_pass(log_n: int, q: int, which: int, data):
+    """(mismatches, the pass's output) of one limb."""
+    a = np.ascontiguousarray(data, dtype=np.uint64)
+    assert a.shape == (1 << log_n,)
+    out = np.zeros_like(a)
+    return _check(lib().fhe_selftest_ntt_pass(log_n, q, which, _ptr(a), _ptr(out))), out
