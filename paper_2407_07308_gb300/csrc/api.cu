@@ -1662,6 +1662,31 @@ extern "C" int fhe_selftest_modarith(uint64_t prime_mod, uint64_t prime_lo, uint
                 if (r >= (int64_t)q || r <= -(int64_t)q ||
                     centred_mod(r, q) != (u64)(((u128)a[0] * b[1] + (u128)(z % q) * b[2]) % q)) bad++;
             }
+            // sums with small scalars: of the size of plaintext coefficients, and
+            // with the sum of their sizes as large as fits
+            for (int big = 0; big < 2; big++) {
+                const u64 most = std::min<u64>(~0ull / q, 0x7fffffff);  // sum |k| < 2^64 / q
+                const int n = edge ? 8 : 1 + (int)(rnd() % 8);
+                int32_t k[8];
+                u64 ksum = 0, s1 = 0;
+                uint32_t neg = 0;
+                for (int j = 0; j < n; j++) {
+                    const u64 size = big ? (j == n - 1 ? most - ksum : most / 8) : std::min<u64>(most / 8, 1 + rnd() % 128);
+                    k[j] = (edge ? (it >> j) & 1 : (int)(rnd() & 1)) ? -(int32_t)size : (int32_t)size;
+                    ksum += size;
+                    if (k[j] < 0) neg += (uint32_t)size;
+                }
+                if (!small_fits(q, ksum)) bad++;
+                u64 s2 = small_start(q, neg);
+                u128 want = 0;
+                for (int j = 0; j < n; j++) {
+                    const u64 v = it & 64 ? (it >> j & 1 ? q - 1 : 0) : a[j];
+                    s1 += small_scaled(v, k[j], q);
+                    s2 = small_add(s2, v, k[j]);
+                    want += (u128)v * (k[j] < 0 ? q - (u64)(-(int64_t)k[j]) % q : (u64)k[j]) % q;
+                }
+                if (s1 != s2 || reduce64(s1, m) != (u64)(want % q)) bad++;
+            }
             const u64 few = edge ? (u64)((((u128)q << 6) - 1 - it) & ~0ull) : x % (((u64)1 << 6) * q);
             if (reduce_few(few, m) >= 2 * q || reduce_few(few, m) % q != few % q) bad++;
         }

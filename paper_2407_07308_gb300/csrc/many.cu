@@ -37,15 +37,9 @@ struct EwSeg {
     const ModQ *mq;
     long long total;  // elements: outer * level * N
     int logN, level, n, op, b0, vec;  // vec: every pointer 16-byte aligned
-    int small, pad;   // small: q sum |k_j| < 2^64 for every prime (see ew_scaled)
+    int small, pad;   // small: q sum |k_j| < 2^64 for every prime (see small_scaled)
     int64_t k[8];     // centred scalars, |k| < p
 };
-
-// Scalar products with small centred scalars without 128-bit arithmetic:
-// a k = (q - a) |k| mod q for k < 0, and with a < q every term (q - a or a)
-// |k| is at most q |k|, so the terms sum to at most q sum |k_j|, which fits
-// 64 bits when small is set; reduce64 then gives [0, q).
-__device__ __forceinline__ u64 ew_scaled(u64 a, int64_t k, u64 q) { return (k < 0 ? q - a : a) * (u64)(k < 0 ? -k : k); }
 
 struct EwTable {
     int nseg, pad;
@@ -121,7 +115,7 @@ __device__ __forceinline__ void ew_block(const EwSeg &S)
             const Vec<V> a = ld_vec<V>(S.x[0] + idx);
             if (S.small) {
 #pragma unroll
-                for (int u = 0; u < V; u++) r.v[u] = reduce64(ew_scaled(a.v[u], S.k[0], q), S.mq[i]);
+                for (int u = 0; u < V; u++) r.v[u] = reduce64(small_scaled(a.v[u], S.k[0], q), S.mq[i]);
                 break;
             }
             const u64 k = small_mod(S.k[0], q);
@@ -147,7 +141,7 @@ __device__ __forceinline__ void ew_block(const EwSeg &S)
                     if (j < S.n) {
                         const Vec<V> a = ld_vec<V>(S.x[j] + idx);
 #pragma unroll
-                        for (int u = 0; u < V; u++) acc[u] += ew_scaled(a.v[u], S.k[j], q);
+                        for (int u = 0; u < V; u++) acc[u] += small_scaled(a.v[u], S.k[j], q);
                     }
 #pragma unroll
                 for (int u = 0; u < V; u++) r.v[u] = reduce64(acc[u], S.mq[i]);
@@ -190,9 +184,7 @@ __global__ void k_ew_many(const __grid_constant__ EwTable t)
 // read it once per output (the leaves' operands of a batch exceed L2: p = 257
 // has 16 leaves over eight powers).  Measured per pass, all element-wise
 // launches: 7 pairs at N = 2^15 4.59 -> 2.19 ms, 16 pairs at N = 2^14 0.96 ->
-// 0.49 ms.  Scalars as in FHE_EW_LINCOMB's 64-bit
-// form: with a negative scalar's q |k| added, every sum is non-negative and
-// below q sum |k| < 2^64.
+// 0.49 ms.  Sums in 64 bits (small_start, small_add).
 
 constexpr int LC_N = 8;
 
@@ -230,13 +222,13 @@ __device__ __forceinline__ void lc_block(const LcSeg &S)
         for (int o = 0; o < S.nout; o++) {
             u64 acc[V];
 #pragma unroll
-            for (int u = 0; u < V; u++) acc[u] = q * S.neg[o];
+            for (int u = 0; u < V; u++) acc[u] = small_start(q, S.neg[o]);
 #pragma unroll
             for (int t = 0; t < LC_N; t++)
                 if (t < S.n) {
-                    const u64 k = (u64)(int64_t)S.k[o][t];
+                    const int32_t k = S.k[o][t];
 #pragma unroll
-                    for (int u = 0; u < V; u++) acc[u] += a[t].v[u] * k;
+                    for (int u = 0; u < V; u++) acc[u] = small_add(acc[u], a[t].v[u], k);
                 }
             Vec<V> r;
 #pragma unroll
@@ -640,7 +632,7 @@ static bool fits64(const EwArgs &a)
     const int nk = a.op == FHE_EW_LINCOMB ? a.n : 1;
     unsigned __int128 ksum = 0;
     for (int j = 0; j < nk && j < 8; j++) ksum += (u64)(a.k[j] < 0 ? -a.k[j] : a.k[j]);
-    return ksum * qmax < ((unsigned __int128)1 << 64);
+    return small_fits(qmax, ksum);
 }
 
 // Linear combinations over the same operands, as many as fit one segment

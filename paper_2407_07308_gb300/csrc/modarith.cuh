@@ -190,6 +190,17 @@ FHE_HD u64 reduce64(u64 v, const ModQ &m)
     return r >= m.q ? r - m.q : r;
 }
 
+// ---- sums with small centred scalars, in 64 bits -----------------------------
+// sum_j k_j a_j mod q for canonical a_j without 128-bit arithmetic, where
+// q sum |k_j| < 2^64 (small_fits); reduce64 then gives [0, q).  Term by term:
+// a k = (q - a) |k| (mod q) for k < 0, and every term (q - a or a) |k| is at
+// most q |k|.  Or all products mod 2^64 on top of q times the negative
+// scalars' sum of |k|: the total is the same non-negative number.
+FHE_HD bool small_fits(u64 qmax, u128 ksum) { return ksum * qmax < ((u128)1 << 64); }
+FHE_HD u64 small_scaled(u64 a, int64_t k, u64 q) { return (k < 0 ? q - a : a) * (u64)(k < 0 ? -k : k); }
+FHE_HD u64 small_start(u64 q, uint32_t neg) { return q * neg; }
+FHE_HD u64 small_add(u64 acc, u64 a, int32_t k) { return acc + a * (u64)(int64_t)k; }
+
 // x < 2^11 q -> [0, (1 + 2^-12 x/q) q + 1], below 2q: the quotient estimate
 // qhat = floor(floor(x / 2^qsh) qmu / 2^32) never exceeds floor(x / q), and
 // qmu >= 2^12 keeps it above x/q (1 - 2^-12) - 2^-19 - 1.  One 32-bit high

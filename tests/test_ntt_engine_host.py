@@ -100,3 +100,11 @@ def test_passes_hold_at_the_top_of_their_ranges(fhe, logN, bits):
     top = np.full(N, q - 1, np.uint64)  # the same for the inverse columns alone: every word 4q - 1
     full = run(3, top + np.uint64(3 * q))
     assert np.array_equal(full, run(3, top)) and int(full.max()) < q
+
+
+@pytest.mark.parametrize("bits", [24, 36, 54, 55, 56, 57])
+def test_modarith_selftest_at_every_prime_size(fhe, bits):
+    """The modular arithmetic, among it the linear combinations' sums with the
+    largest scalars that fit 64 bits, for the largest primes of a size."""
+    lo = 2 ** bits - 2 ** (bits - (1 if bits < 30 else 6))
+    assert fhe.fhe_selftest_modarith(2 ** 12, lo, 2 ** bits, 4, 5000) == 0
