@@ -89,24 +89,13 @@ FHE_HD u64 shoup_lazy(u64 a, u64 w, u64 ws, u64 q) { return a * w - fhe_mulhi(a,
 // for any a < 2^64; the difference fits in 64 bits, so the arithmetic mod
 // 2^64 is exact.  One 32x32->64 and two 32x32->hi products instead of the
 // four 32x32->64 products (and their carries) of the exact high half.
-FHE_HD u64 shoup_lazy4(u64 a, u64 w, u64 ws, u64 q)
-{
-    const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32), wl = (uint32_t)ws, wh = (uint32_t)(ws >> 32);
-#ifdef __CUDA_ARCH__
-    const u64 qhat = (u64)ah * wh + ((u64)__umulhi(ah, wl) + __umulhi(al, wh));
-#else
-    const u64 qhat = (u64)ah * wh + ((((u64)ah * wl) >> 32) + (((u64)al * wh) >> 32));
-#endif
-    return a * w - qhat * q;
-}
-
-// shoup_lazy4 as one multiply-add chain: with nq = 2^64 - q, a w - qhat q =
-// a w + qhat nq (mod 2^64), so on the device the low words of a w and of
+//
+// On the device the product is one multiply-add chain: with nq = 2^64 - q,
+// a w - qhat q = a w + qhat nq (mod 2^64), so the low words of a w and of
 // qhat nq are summed by a wide multiply-add and the high word by four 32-bit
 // multiply-adds, with no separate 64-bit subtraction; the two high partial
 // products of the quotient are summed by a wide multiply-add too (t1 * 1 +
-// t2), so the whole product runs on the multiply-add pipe.  Same result as
-// shoup_lazy4 for every input (the host form is that expression in C).
+// t2), so the whole product runs on the multiply-add pipe.
 FHE_HD u64 shoup_lazy4_chain(u64 a, u64 w, u64 ws, u64 nq)
 {
 #ifdef __CUDA_ARCH__
@@ -160,15 +149,6 @@ FHE_HD u64 barrett128(u128 x, const ModQ &m)
     if (r >= m.q2) r -= m.q2;
     if (r >= m.q) r -= m.q;
     return r;
-}
-
-// The same reduction without its two corrections: a residue of x in [0, 3q).
-FHE_HD u64 barrett128_lazy(u128 x, const ModQ &m)
-{
-    u64 lo = (u64)x, hi = (u64)(x >> 64);
-    int s = m.bshift;
-    u64 t = (hi << (64 - s)) | (lo >> s);
-    return lo - fhe_mulhi(t, m.mu) * m.q;
 }
 
 FHE_HD u64 mulmod(u64 a, u64 b, const ModQ &m) { return barrett128((u128)a * b, m); }

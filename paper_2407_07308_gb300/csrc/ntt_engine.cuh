@@ -75,7 +75,7 @@
 
 namespace {
 
-// The butterflies' twiddle product: shoup_lazy4 as one multiply-add chain.
+// The butterflies' twiddle product: shoup_lazy4_chain.
 // Measured on the GB300 (16-pair comparison at N = 2^14, identical results):
 // the C form 2454 slot-comparisons/s, the chain with its quotient's two high
 // products summed by an add-with-carry 2563, by a wide multiply-add 2606
@@ -89,7 +89,7 @@ FHE_HD u64 bfly_mul(u64 a, const ulonglong2 w, u64 q)
 }
 
 // Forward butterfly without normalisation: t = [Y w] in [0, 4q) for any
-// 64-bit Y (shoup_lazy4), so if X, Y < B then X + t and X - t + 4q lie in
+// 64-bit Y (bfly_mul), so if X, Y < B then X + t and X - t + 4q lie in
 // [0, B + 4q).  Inputs below 7q (canonical residues, or the lazy results of
 // the fused conversions) stay below (4s + 7) q <= 67 q < 2^64 after s <= 15
 // stages for primes below 2^57; one reduction at the end brings every value
@@ -103,7 +103,7 @@ FHE_HD void ct_bfly(u64 &X, u64 &Y, const ulonglong2 w, u64 q, u64 q4)
 }
 
 // Inverse butterfly without normalisation: for X, Y < B, B a multiple of q,
-// X + Y < 2B and [(X - Y + B) w] in [0, 4q) (shoup_lazy4 takes any 64-bit
+// X + Y < 2B and [(X - Y + B) w] in [0, 4q) (bfly_mul takes any 64-bit
 // operand, and X - Y + B < 2B).  Sums double from stage to stage, so the
 // stages' bounds are 4q 2^j; reduce_few brings the sums back at the end of a
 // row pass (and, for primes above 54 bits, between its two rounds), where a
