@@ -367,10 +367,6 @@ struct ColGeo {
     // a unit's first job and its first column
     __host__ __device__ static int job0(int lu) { return lu / BLK * NJ; }
     __host__ __device__ static int lo0(int lu) { return lu % BLK * NC; }
-    // word r of the unit: job slot, column in job, element
-    __device__ static int jslot(int r) { return NJ == 1 ? 0 : r / (NC * SZ); }
-    __device__ static int col(int r) { return r % NC; }
-    __device__ static int elem(int r) { return (r % (NC * SZ)) / NC; }
 };
 
 template <int N1, int N2, int XJ = 1>
@@ -804,16 +800,6 @@ __device__ __forceinline__ void inv_cols_unit1(const IO &io, int sg, int lu, u64
     for (int k = 0; k < 16; k++) io.store(st, ((k * C::G + g) << N2) + lo, inv_scaled(x[k], ni, m));
 }
 
-// a column's input word: read from a limb, or converted from several
-template <int NN, class IO>
-__device__ __forceinline__ u64 col_load(const IO &io, int sg, const typename IO::CSt &st, int n)
-{
-    if constexpr (IO::XJ == 2)
-        return conv_one<NN>(st.cv, io.h[sg].mq[st.prime], n);
-    else
-        return io.load(st, n);
-}
-
 // Forward, columns: global stages 0..N1-1.
 template <int N1, int N2, class IO>
 __device__ __forceinline__ void fwd_cols_unit(const IO &io, int sg, int lu, u64 *sm, ulonglong2 *W,
@@ -834,16 +820,18 @@ __device__ __forceinline__ void fwd_cols_unit(const IO &io, int sg, int lu, u64 
     const ModQ &m0 = H.mq[sts[0].prime], &m1 = H.mq[sts[nvalid > 1 ? Gm::NJ - 1 : 0].prime];
     for (int j = 0; j < Gm::NJ && j < nvalid; j++)
         col_twiddles<N1>(W + j * Gm::TWC, H.tw + (size_t)sts[j].prime * Gm::NN);
+    const ColTw<N1, N2, IO::XJ> geo{W, m0.q, m1.q, &m0, &m1};
+    const int j = c / Gm::NC;
+    u64 x[16];
+    u64 *b = sm + Gm::Lay::base(c);
     pdl_wait();
-    bool paired = false;
     if constexpr (Gm::PAIRED) {
-        // both slots at once: column col of slot 0 and of slot 1 at the same
-        // element, so each source word is loaded once
         static_assert(Gm::NJ == 2 && 2 * Gm::NC * Gm::SZ == 16 * T, "paired column unit");
-        paired = nvalid >= 2 && io.same_src(sts[0], sts[1]);  // uniform in the CTA
-        if (paired) {
-            constexpr int ES = T / Gm::NC;  // elements between a thread's words
-            const int col = tid % Gm::NC, e0 = tid / Gm::NC;
+        constexpr int ES = T / Gm::NC;  // elements between a thread's words
+        const int col = tid % Gm::NC, e0 = tid / Gm::NC;
+        if (nvalid >= 2 && io.same_src(sts[0], sts[1])) {  // uniform in the CTA
+            // both slots at once: column col of slot 0 and of slot 1 at the
+            // same element, so each source word is loaded once
 #pragma unroll 1
             for (int k = 0; k < 8; k += CONV_P) {
                 u64 v0[CONV_P], v1[CONV_P];
@@ -855,43 +843,57 @@ __device__ __forceinline__ void fwd_cols_unit(const IO &io, int sg, int lu, u64 
                     sm[Gm::Lay::at(Gm::NC + col, e0 + (k + p) * ES)] = v1[p];
                 }
             }
-        }
-    }
-    if constexpr (Gm::PAIRED) {
-        // a unit whose jobs read different sources, or with one job left (a
-        // slot without a job transforms what is there and stores nothing):
-        // rolled loops, small code beside the paired path
-        if (!paired) {
-            constexpr int ES = T / Gm::NC;
-            const int col = tid % Gm::NC, e0 = tid / Gm::NC;
+        } else {
+            // a unit whose jobs read different sources, or with one job left
+            // (a slot without a job transforms what is there and stores
+            // nothing): rolled loops, small code beside the paired path
 #pragma unroll 1
-            for (int j = 0; j < 2 && j < nvalid; j++)
+            for (int i = 0; i < 2 && i < nvalid; i++)
 #pragma unroll 1
                 for (int k = 0; k < 8; k++)
-                    sm[Gm::Lay::at(j * Gm::NC + col, e0 + k * ES)] =
-                        conv_one<Gm::NN>(sts[j].cv, j == 0 ? m0 : m1, ((e0 + k * ES) << N2) + lo0 + col);
+                    sm[Gm::Lay::at(i * Gm::NC + col, e0 + k * ES)] =
+                        conv_one<Gm::NN>(sts[i].cv, i == 0 ? m0 : m1, ((e0 + k * ES) << N2) + lo0 + col);
         }
+        async_wait();
+        __syncthreads();
+        get1<C::G>(b + g, x);
     } else {
+        // n = 10: thread (c, g) takes its first round's words as in
+        // fwd_cols_unit1; a slot without a job transforms the first job's and
+        // stores nothing
+        const int jv = j < nvalid ? j : 0, lo = lo0 + c % Gm::NC;
+        const typename IO::CSt &st = sts[jv];
+        if constexpr (IO::XJ == 2) {
+            // conversions in a rolled loop, by way of the thread's own places
+            // in shared memory (unrolled into registers they spilled)
+            const ModQ &m = jv == 0 ? m0 : m1;
 #pragma unroll 1
-        for (int k = 0; k < 16; k++) {
-            const int r = tid + k * T, j = Gm::jslot(r);
-            if (j < nvalid)
-                sm[Gm::Lay::at(j * Gm::NC + Gm::col(r), Gm::elem(r))] =
-                    col_load<Gm::NN>(io, sg, sts[j], (Gm::elem(r) << N2) + lo0 + Gm::col(r));
+            for (int k = 0; k < 16; k += CONV_P) {
+                u64 v[CONV_P];
+                conv_single<CONV_P, (C::G << N2), Gm::NN>(st.cv, m, ((k * C::G + g) << N2) + lo, v);
+#pragma unroll
+                for (int p = 0; p < CONV_P; p++) sm[Gm::Lay::at(c, (k + p) * C::G + g)] = v[p];
+            }
+            get1<C::G>(b + g, x);
+        } else {
+            // all loads in flight (one after the other, a transform of 288
+            // plain limbs took 18.5 us among others and 30 alone; 15 and 19)
+            const u64 *src = io.src(st) + (g << N2) + lo;
+#pragma unroll
+            for (int k = 0; k < 16; k++) x[k] = src[(k * C::G) << N2];
+            if constexpr (!IO::PLAIN) {
+#pragma unroll
+                for (int k = 0; k < 16; k++) x[k] = io.conv(st, x[k]);
+            }
         }
+        async_wait();
+        __syncthreads();  // the twiddles
     }
-    async_wait();
-    __syncthreads();
-    const ColTw<N1, N2, IO::XJ> geo{W, m0.q, m1.q, &m0, &m1};
-    u64 x[16];
-    u64 *b = sm + Gm::Lay::base(c);
-    get1<C::G>(b + g, x);
     round1<N1, true>(x, geo, c);
     put1<C::G>(b + g, x);
     __syncthreads();
     get2(b + 17 * g, x);
     round2<N1, true>(x, geo, c, g);
-    const int j = c / Gm::NC;
     if (j < nvalid) {
         u64 *mid = io.inter(sts[j]) + (g << (N2 + 4)) + lo0 + c % Gm::NC;
 #pragma unroll
@@ -1360,7 +1362,6 @@ struct IOMap : SegIO<MapSeg> {
     __device__ RowK row_k(int, int) const { return {}; }
     static constexpr bool PLAIN = true;  // a column pass loads src's words as they are
     __device__ const u64 *src(const CSt &t) const { return t.in; }
-    __device__ u64 load(const CSt &t, int i) const { return t.in[i]; }
     // the inverse row pass's word: the limb's alone
     __device__ static constexpr bool adds(const RSt &) { return false; }
     __device__ u64 addend(const RSt &, int) const { return 0; }
@@ -1612,7 +1613,6 @@ struct IOModSwitch : SegIO<SwitchSeg> {
     static constexpr bool PLAIN = false;
     __device__ const u64 *src(const CSt &t) const { return t.last; }
     __device__ u64 conv(const CSt &t, u64 v) const { return shoup_lazy4_chain(v, t.pi, t.pis, t.nq); }
-    __device__ u64 load(const CSt &t, int n) const { return conv(t, t.last[n]); }
     static constexpr int NPRE = 1;  // the limb being switched
     __device__ u64 pre(const RSt &t, int k, int) const { return t.x[k]; }
     __device__ void store_pre(const RowK &K, const ModQ &m, const RSt &t, int k, u64 v, const u64 *pv) const
