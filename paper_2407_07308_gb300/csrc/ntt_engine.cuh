@@ -820,18 +820,16 @@ __device__ __forceinline__ void fwd_cols_unit(const IO &io, int sg, int lu, u64 
     const ModQ &m0 = H.mq[sts[0].prime], &m1 = H.mq[sts[nvalid > 1 ? Gm::NJ - 1 : 0].prime];
     for (int j = 0; j < Gm::NJ && j < nvalid; j++)
         col_twiddles<N1>(W + j * Gm::TWC, H.tw + (size_t)sts[j].prime * Gm::NN);
-    const ColTw<N1, N2, IO::XJ> geo{W, m0.q, m1.q, &m0, &m1};
-    const int j = c / Gm::NC;
-    u64 x[16];
-    u64 *b = sm + Gm::Lay::base(c);
     pdl_wait();
+    bool paired = false;
     if constexpr (Gm::PAIRED) {
+        // both slots at once: column col of slot 0 and of slot 1 at the same
+        // element, so each source word is loaded once
         static_assert(Gm::NJ == 2 && 2 * Gm::NC * Gm::SZ == 16 * T, "paired column unit");
-        constexpr int ES = T / Gm::NC;  // elements between a thread's words
-        const int col = tid % Gm::NC, e0 = tid / Gm::NC;
-        if (nvalid >= 2 && io.same_src(sts[0], sts[1])) {  // uniform in the CTA
-            // both slots at once: column col of slot 0 and of slot 1 at the
-            // same element, so each source word is loaded once
+        paired = nvalid >= 2 && io.same_src(sts[0], sts[1]);  // uniform in the CTA
+        if (paired) {
+            constexpr int ES = T / Gm::NC;  // elements between a thread's words
+            const int col = tid % Gm::NC, e0 = tid / Gm::NC;
 #pragma unroll 1
             for (int k = 0; k < 8; k += CONV_P) {
                 u64 v0[CONV_P], v1[CONV_P];
@@ -843,25 +841,31 @@ __device__ __forceinline__ void fwd_cols_unit(const IO &io, int sg, int lu, u64 
                     sm[Gm::Lay::at(Gm::NC + col, e0 + (k + p) * ES)] = v1[p];
                 }
             }
-        } else {
-            // a unit whose jobs read different sources, or with one job left
-            // (a slot without a job transforms what is there and stores
-            // nothing): rolled loops, small code beside the paired path
+        }
+    }
+    if constexpr (Gm::PAIRED) {
+        // a unit whose jobs read different sources, or with one job left (a
+        // slot without a job transforms what is there and stores nothing):
+        // rolled loops, small code beside the paired path.  (As an else-branch
+        // of that path it slowed the paired units: 7 pairs at N = 2^15 39.79
+        // -> 39.91 ms, 16 products 2042 -> 2051 us.)
+        if (!paired) {
+            constexpr int ES = T / Gm::NC;
+            const int col = tid % Gm::NC, e0 = tid / Gm::NC;
 #pragma unroll 1
-            for (int i = 0; i < 2 && i < nvalid; i++)
+            for (int j = 0; j < 2 && j < nvalid; j++)
 #pragma unroll 1
                 for (int k = 0; k < 8; k++)
-                    sm[Gm::Lay::at(i * Gm::NC + col, e0 + k * ES)] =
-                        conv_one<Gm::NN>(sts[i].cv, i == 0 ? m0 : m1, ((e0 + k * ES) << N2) + lo0 + col);
+                    sm[Gm::Lay::at(j * Gm::NC + col, e0 + k * ES)] =
+                        conv_one<Gm::NN>(sts[j].cv, j == 0 ? m0 : m1, ((e0 + k * ES) << N2) + lo0 + col);
         }
-        async_wait();
-        __syncthreads();
-        get1<C::G>(b + g, x);
-    } else {
+    }
+    u64 x[16];
+    if constexpr (!Gm::PAIRED) {
         // n = 10: thread (c, g) takes its first round's words as in
         // fwd_cols_unit1; a slot without a job transforms the first job's and
         // stores nothing
-        const int jv = j < nvalid ? j : 0, lo = lo0 + c % Gm::NC;
+        const int jv = c / Gm::NC < nvalid ? c / Gm::NC : 0, lo = lo0 + c % Gm::NC;
         const typename IO::CSt &st = sts[jv];
         if constexpr (IO::XJ == 2) {
             // conversions in a rolled loop, by way of the thread's own places
@@ -874,7 +878,6 @@ __device__ __forceinline__ void fwd_cols_unit(const IO &io, int sg, int lu, u64 
 #pragma unroll
                 for (int p = 0; p < CONV_P; p++) sm[Gm::Lay::at(c, (k + p) * C::G + g)] = v[p];
             }
-            get1<C::G>(b + g, x);
         } else {
             // all loads in flight (one after the other, a transform of 288
             // plain limbs took 18.5 us among others and 30 alone; 15 and 19)
@@ -886,14 +889,18 @@ __device__ __forceinline__ void fwd_cols_unit(const IO &io, int sg, int lu, u64 
                 for (int k = 0; k < 16; k++) x[k] = io.conv(st, x[k]);
             }
         }
-        async_wait();
-        __syncthreads();  // the twiddles
     }
+    async_wait();
+    __syncthreads();
+    const ColTw<N1, N2, IO::XJ> geo{W, m0.q, m1.q, &m0, &m1};
+    u64 *b = sm + Gm::Lay::base(c);
+    if constexpr (IO::XJ == 2) get1<C::G>(b + g, x);
     round1<N1, true>(x, geo, c);
     put1<C::G>(b + g, x);
     __syncthreads();
     get2(b + 17 * g, x);
     round2<N1, true>(x, geo, c, g);
+    const int j = c / Gm::NC;
     if (j < nvalid) {
         u64 *mid = io.inter(sts[j]) + (g << (N2 + 4)) + lo0 + c % Gm::NC;
 #pragma unroll
