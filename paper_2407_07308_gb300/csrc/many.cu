@@ -20,11 +20,23 @@ constexpr int EW_ELEMS = TPB * 4;  // elements per block of the element-wise ker
 // |k| < q: k mod q in [0, q)
 __device__ __forceinline__ u64 small_mod(int64_t k, u64 q) { return k >= 0 ? (u64)k : q - (u64)(-k); }
 
-template <class S>
-__device__ __forceinline__ int block_seg(const S *s, int n)
+// A launch's segments (kernel parameters) and the elements a block of the
+// element-wise kernels takes.  A call on one batch takes a table of one: with
+// room for FHE_SEGS the parameters of an addition are 4.4 KB, and a small
+// fhe_add took 3.7 us among others, 3.3 with one; fhe_mul 3.6 and 3.2.
+template <class Seg, int CAP, int ELEMS = EW_ELEMS>
+struct Table {
+    static constexpr int cap = CAP, elems = ELEMS;
+    int nseg, rms;  // rms: the folds' kind
+    Seg s[CAP];
+};
+
+template <class Seg, int CAP, int ELEMS>
+__device__ __forceinline__ int block_seg(const Table<Seg, CAP, ELEMS> &t)
 {
     int sg = 0;
-    while (sg + 1 < n && s[sg + 1].b0 <= (int)blockIdx.x) sg++;
+    if constexpr (CAP > 1)
+        while (sg + 1 < t.nseg && t.s[sg + 1].b0 <= (int)blockIdx.x) sg++;
     return sg;
 }
 
@@ -39,11 +51,6 @@ struct EwSeg {
     int logN, level, n, op, b0, vec;  // vec: every pointer 16-byte aligned
     int small, pad;   // small: q sum |k_j| < 2^64 for every prime (see small_scaled)
     int64_t k[8];     // centred scalars, |k| < p
-};
-
-struct EwTable {
-    int nseg, pad;
-    EwSeg s[FHE_SEGS];
 };
 
 // V adjacent elements (one limb: N is even) as one load per operand
@@ -166,10 +173,11 @@ __device__ __forceinline__ void ew_block(const EwSeg &S)
     }
 }
 
-__global__ void k_ew_many(const __grid_constant__ EwTable t)
+template <class Tb>
+__global__ void k_ew_many(const __grid_constant__ Tb t)
 {
     pdl_begin();
-    const EwSeg &S = t.s[block_seg(t.s, t.nseg)];
+    const EwSeg &S = t.s[block_seg(t)];
     if (S.vec)
         ew_block<2>(S);
     else
@@ -196,11 +204,6 @@ struct LcSeg {
     int logN, level, n, nout, b0, vec;
     int32_t k[LC_N][LC_N];  // [output][operand]
     uint32_t neg[LC_N];     // sum of |k| over an output's negative scalars
-};
-
-struct LcTable {
-    int nseg, pad;
-    LcSeg s[FHE_SEGS];
 };
 
 template <int V>
@@ -238,10 +241,11 @@ __device__ __forceinline__ void lc_block(const LcSeg &S)
     }
 }
 
-__global__ void k_lincomb_many(const __grid_constant__ LcTable t)
+template <class Tb>
+__global__ void k_lincomb_many(const __grid_constant__ Tb t)
 {
     pdl_begin();
-    const LcSeg &S = t.s[block_seg(t.s, t.nseg)];
+    const LcSeg &S = t.s[block_seg(t)];
     if (S.vec)
         lc_block<2>(S);
     else
@@ -258,17 +262,12 @@ struct TensorSeg {
     int logN, level, b0, vec;  // vec: every pointer 16-byte aligned
 };
 
-struct TensorTable {
-    int nseg, pad;
-    TensorSeg s[FHE_SEGS];
-};
-
-template <int V>
+template <int V, int ELEMS>
 __device__ __forceinline__ void tensor_block(const TensorSeg &S)
 {
-    // one limb of one ciphertext per block (EW_ELEMS divides N)
+    // one limb of one ciphertext per block (ELEMS divides N)
     const long long LN = (long long)S.level << S.logN;
-    const long long base = (long long)(blockIdx.x - S.b0) * EW_ELEMS;
+    const long long base = (long long)(blockIdx.x - S.b0) * ELEMS;
     if (base >= S.total) return;
     const long long c = base / LN, r0 = base % LN;
     const ModQ m = S.mq[(int)(r0 >> S.logN)];
@@ -276,7 +275,7 @@ __device__ __forceinline__ void tensor_block(const TensorSeg &S)
     const u64 *b0 = S.b + 2 * c * LN + r0, *b1 = b0 + LN;
     u64 *o0 = S.out + 3 * c * LN + r0, *o1 = o0 + LN, *o2 = o1 + LN;
 #pragma unroll
-    for (int e = threadIdx.x * V; e < EW_ELEMS; e += TPB * V) {
+    for (int e = threadIdx.x * V; e < ELEMS; e += TPB * V) {
         const Vec<V> x0 = ld_vec<V>(a0 + e), x1 = ld_vec<V>(a1 + e), y0 = ld_vec<V>(b0 + e), y1 = ld_vec<V>(b1 + e);
         Vec<V> r0v, r1v, r2v;
 #pragma unroll
@@ -291,14 +290,15 @@ __device__ __forceinline__ void tensor_block(const TensorSeg &S)
     }
 }
 
-__global__ void k_tensor_many(const __grid_constant__ TensorTable t)
+template <class Tb>
+__global__ void k_tensor_many(const __grid_constant__ Tb t)
 {
     pdl_begin();
-    const TensorSeg &S = t.s[block_seg(t.s, t.nseg)];
+    const TensorSeg &S = t.s[block_seg(t)];
     if (S.vec)
-        tensor_block<2>(S);
+        tensor_block<2, Tb::elems>(S);
     else
-        tensor_block<1>(S);
+        tensor_block<1, Tb::elems>(S);
 }
 
 // ---- key-switching inner product ------------------------------------------
@@ -343,10 +343,7 @@ struct KsSeg {
     int run;  // ciphertexts of the run this item opens (0: the item belongs to an earlier one's)
 };
 
-struct KsTable {
-    int nseg, pad;
-    KsSeg s[FHE_SEGS];
-};
+using KsTable = Table<KsSeg, FHE_SEGS>;
 
 // Digit group g of this thread's copies has arrived once at most `left` later
 // groups are in flight.
@@ -444,7 +441,7 @@ __global__ void __launch_bounds__(TPB, FHE_KS_MINB) k_ks_inner_many(const __grid
 {
     pdl_trigger();
     extern __shared__ u64 ks_words[];  // [dnum][2 + KS_CB][TPB]
-    const int sg = block_seg(t.s, t.nseg);
+    const int sg = block_seg(t);
     const KsSeg &S = t.s[sg];
     const int lb = blockIdx.x - S.b0;
     const int lK = S.l + S.K, N = 1 << S.logN;
@@ -500,11 +497,6 @@ __device__ __forceinline__ u64 fold_sub(u64 y, int64_t s, const ModQ &m)
 {
     return reduce2q(reduce_few(y + 2 * m.q2 - (u64)s, m), m.q);
 }
-
-struct FoldTable {
-    int nseg, rms;
-    FoldSeg s[FHE_SEGS];
-};
 
 // The relinearise + switch fold: src[c][pi] = (t_0 .. t_{K-1}, Y') -> Y' -
 // sum_k t_k p_k^-1 mod q_{l-1}.  A block's FOLD_ELEMS words lie in one
@@ -580,46 +572,51 @@ __device__ __forceinline__ void fold_multi_block(const FoldSeg &S)
         }
 }
 
-__global__ void __launch_bounds__(TPB) k_fold_many(const __grid_constant__ FoldTable t)
+template <class Tb>
+__global__ void __launch_bounds__(TPB) k_fold_many(const __grid_constant__ Tb t)
 {
     pdl_begin();
-    const FoldSeg &S = t.s[block_seg(t.s, t.nseg)];
+    const FoldSeg &S = t.s[block_seg(t)];
     if (t.rms)
         fold_rms_block(S);
     else
         fold_multi_block(S);
 }
 
-int ew_blocks(long long total) { return (int)((total + EW_ELEMS - 1) / EW_ELEMS); }
+int ew_blocks(long long total, int elems) { return (int)((total + elems - 1) / elems); }
 
-// Launches kern over `items` in tables of at most FHE_SEGS segments; fill
-// sets segment s from an item and returns its blocks (0 = nothing to do) and
-// its algorithmic bytes.
-template <class Table, class Item, class Fill, class Launch>
-void launch_tables(const std::vector<Item> &items, int cls, Fill fill, Launch launch)
+// Launches a kernel over items[i ..) as one table Tb; fill sets a segment from
+// an item and returns its blocks (0 = nothing to do) and its algorithmic
+// bytes.  Returns the first item behind the table.
+template <class Tb, class Item, class Fill, class Launch>
+size_t launch_table(const std::vector<Item> &items, size_t i, int cls, const Fill &fill, const Launch &launch)
 {
-    size_t i = 0;
-    while (i < items.size()) {
-        Table t;
-        memset(&t, 0, sizeof(t));
-        fhe_ctx *c = items[i].c;
-        int blocks = 0;
-        double bytes = 0;
-        for (; i < items.size() && t.nseg < FHE_SEGS; i++) {
-            double b = 0;
-            const int nb = fill(t.s[t.nseg], items[i], &b);
-            if (nb <= 0) continue;
-            t.s[t.nseg].b0 = blocks;
-            blocks += nb;
-            bytes += b;
-            t.nseg++;
-        }
-        if (!t.nseg) continue;
-        prof_begin(c, cls, bytes);
-        launch(t, pdl_on(c, blocks, TPB), blocks, c->stream);
-        prof_end(c);
-        c->launches++;
+    Tb t;
+    memset(&t, 0, sizeof(t));
+    fhe_ctx *c = items[i].c;
+    int blocks = 0;
+    double bytes = 0;
+    for (; i < items.size() && t.nseg < Tb::cap; i++) {
+        double b = 0;
+        const int nb = fill(t.s[t.nseg], items[i], Tb::elems, &b);
+        if (nb <= 0) continue;
+        t.s[t.nseg].b0 = blocks;
+        blocks += nb;
+        bytes += b;
+        t.nseg++;
     }
+    if (!t.nseg) return i;
+    prof_begin(c, cls, bytes);
+    launch(t, pdl_on(c, blocks, TPB), blocks, c->stream);
+    prof_end(c);
+    c->launches++;
+    return i;
+}
+
+template <class Seg, class Item, class Fill, class Launch>
+void launch_tables(const std::vector<Item> &items, int cls, const Fill &fill, const Launch &launch)
+{
+    for (size_t i = 0; i < items.size();) i = launch_table<Table<Seg, FHE_SEGS>>(items, i, cls, fill, launch);
 }
 
 }  // namespace
@@ -682,11 +679,13 @@ static std::vector<LcItem> shared_lincombs(const std::vector<EwArgs> &items, std
 
 void launch_ew_many(const std::vector<EwArgs> &all)
 {
-    std::vector<EwArgs> items;
-    const std::vector<LcItem> shared = shared_lincombs(all, items);
-    launch_tables<LcTable>(
+    std::vector<EwArgs> rest;
+    std::vector<LcItem> shared;
+    if (all.size() > 1) shared = shared_lincombs(all, rest);
+    const std::vector<EwArgs> &items = all.size() > 1 ? rest : all;
+    launch_tables<LcSeg>(
         shared, FHE_K_ELEMWISE,
-        [](LcSeg &S, const LcItem &g, double *bytes) {
+        [](LcSeg &S, const LcItem &g, int elems, double *bytes) {
             const EwArgs &a = *g.of[0];
             S.total = (long long)a.outer * a.level * a.c->N;
             if (S.total <= 0) return 0;
@@ -713,50 +712,65 @@ void launch_ew_many(const std::vector<EwArgs> &all)
             S.level = a.level;
             S.vec = vec;
             *bytes = 8.0 * (S.n + S.nout) * S.total;
-            return ew_blocks(S.total);
+            return ew_blocks(S.total, elems);
         },
-        [](const LcTable &t, bool pdl, int blocks, cudaStream_t s) { launch_pdl(k_lincomb_many, pdl, blocks, TPB, s, t); });
-    launch_tables<EwTable>(
-        items, FHE_K_ELEMWISE,
-        [](EwSeg &S, const EwArgs &a, double *bytes) {
-            S.total = (long long)a.outer * a.level * a.c->N;
-            if (S.total <= 0) return 0;
-            for (int j = 0; j < 8; j++) S.x[j] = a.x[j], S.k[j] = a.k[j];
-            S.out = a.out;
-            S.mq = a.c->d_mq;
-            S.logN = a.c->logN;
-            S.level = a.level;
-            S.n = a.n;
-            S.op = a.op;
-            bool vec = ((uintptr_t)a.out & 15) == 0;
-            for (int j = 0; j < 8; j++) vec = vec && ((uintptr_t)a.x[j] & 15) == 0;
-            S.vec = vec;
-            S.small = (a.op == FHE_EW_LINCOMB || a.op == FHE_EW_CMUL) && fits64(a);
-            const int reads = a.op == FHE_EW_LINCOMB ? a.n : (a.op == FHE_EW_ADD || a.op == FHE_EW_SUB) ? 2 : 1;
-            *bytes = 8.0 * (reads + 1) * S.total;
-            return ew_blocks(S.total);
-        },
-        [](const EwTable &t, bool pdl, int blocks, cudaStream_t s) { launch_pdl(k_ew_many, pdl, blocks, TPB, s, t); });
+        [](const auto &t, bool pdl, int blocks, cudaStream_t s) {
+            launch_pdl(k_lincomb_many<std::decay_t<decltype(t)>>, pdl, blocks, TPB, s, t);
+        });
+    auto fill = [](EwSeg &S, const EwArgs &a, int elems, double *bytes) {
+        S.total = (long long)a.outer * a.level * a.c->N;
+        if (S.total <= 0) return 0;
+        for (int j = 0; j < 8; j++) S.x[j] = a.x[j], S.k[j] = a.k[j];
+        S.out = a.out;
+        S.mq = a.c->d_mq;
+        S.logN = a.c->logN;
+        S.level = a.level;
+        S.n = a.n;
+        S.op = a.op;
+        bool vec = ((uintptr_t)a.out & 15) == 0;
+        for (int j = 0; j < 8; j++) vec = vec && ((uintptr_t)a.x[j] & 15) == 0;
+        S.vec = vec;
+        S.small = (a.op == FHE_EW_LINCOMB || a.op == FHE_EW_CMUL) && fits64(a);
+        const int reads = a.op == FHE_EW_LINCOMB ? a.n : (a.op == FHE_EW_ADD || a.op == FHE_EW_SUB) ? 2 : 1;
+        *bytes = 8.0 * (reads + 1) * S.total;
+        return ew_blocks(S.total, elems);
+    };
+    auto launch = [](const auto &t, bool pdl, int blocks, cudaStream_t s) {
+        launch_pdl(k_ew_many<std::decay_t<decltype(t)>>, pdl, blocks, TPB, s, t);
+    };
+    if (items.size() == 1)
+        launch_table<Table<EwSeg, 1>>(items, 0, FHE_K_ELEMWISE, fill, launch);
+    else
+        launch_tables<EwSeg>(items, FHE_K_ELEMWISE, fill, launch);
 }
 
 void launch_tensor_many(const std::vector<TensorArgs> &items)
 {
-    launch_tables<TensorTable>(
-        items, FHE_K_TENSOR,
-        [](TensorSeg &S, const TensorArgs &a, double *bytes) {
-            S.total = (long long)a.count * a.level * a.c->N;
-            if (S.total <= 0) return 0;
-            S.a = a.a;
-            S.b = a.b;
-            S.out = a.out;
-            S.mq = a.c->d_mq;
-            S.logN = a.c->logN;
-            S.level = a.level;
-            S.vec = (((uintptr_t)a.a | (uintptr_t)a.b | (uintptr_t)a.out) & 15) == 0;
-            *bytes = 8.0 * 7 * S.total;
-            return ew_blocks(S.total);
-        },
-        [](const TensorTable &t, bool pdl, int blocks, cudaStream_t s) { launch_pdl(k_tensor_many, pdl, blocks, TPB, s, t); });
+    auto fill = [](TensorSeg &S, const TensorArgs &a, int elems, double *bytes) {
+        S.total = (long long)a.count * a.level * a.c->N;
+        if (S.total <= 0) return 0;
+        S.a = a.a;
+        S.b = a.b;
+        S.out = a.out;
+        S.mq = a.c->d_mq;
+        S.logN = a.c->logN;
+        S.level = a.level;
+        S.vec = (((uintptr_t)a.a | (uintptr_t)a.b | (uintptr_t)a.out) & 15) == 0;
+        *bytes = 8.0 * 7 * S.total;
+        return ew_blocks(S.total, elems);
+    };
+    auto launch = [](const auto &t, bool pdl, int blocks, cudaStream_t s) {
+        launch_pdl(k_tensor_many<std::decay_t<decltype(t)>>, pdl, blocks, TPB, s, t);
+    };
+    // one batch of at most two blocks per SM: blocks of half the elements,
+    // whose second step would only wait for the first (one ciphertext at
+    // N = 2^10, alone: 12.5 us with whole blocks, 11.5 with halves; larger
+    // batches are better off with whole ones, 48 at N = 2^15 262 against 277)
+    if (items.size() == 1 &&
+        (long long)items[0].count * items[0].level * items[0].c->N <= 2LL * EW_ELEMS * items[0].c->sms)
+        launch_table<Table<TensorSeg, 1, EW_ELEMS / 2>>(items, 0, FHE_K_TENSOR, fill, launch);
+    else
+        launch_tables<TensorSeg>(items, FHE_K_TENSOR, fill, launch);
 }
 
 // shared memory of a block for dnum digits
@@ -839,9 +853,9 @@ void launch_ks_inner(fhe_ctx *c, const u64 *ext, const u64 *xbase, long long x_o
 
 void launch_rms_fold_many(const std::vector<FoldArgs> &items)
 {
-    launch_tables<FoldTable>(
+    launch_tables<FoldSeg>(
         items, FHE_K_ELEMWISE,
-        [](FoldSeg &S, const FoldArgs &a, double *bytes) {
+        [](FoldSeg &S, const FoldArgs &a, int, double *bytes) {
             fhe_ctx *c = a.c;
             S.total = (long long)a.outer * 2 * c->N;  // (ct, poly) pairs
             if (S.total <= 0) return 0;
@@ -855,9 +869,9 @@ void launch_rms_fold_many(const std::vector<FoldArgs> &items)
             *bytes = 8.0 * (c->K + 2.0) * S.total;
             return (int)(S.total / FOLD_ELEMS);
         },
-        [](FoldTable &t, bool pdl, int blocks, cudaStream_t s) {
+        [](auto &t, bool pdl, int blocks, cudaStream_t s) {
             t.rms = 1;
-            launch_pdl(k_fold_many, pdl, blocks, TPB, s, t);
+            launch_pdl(k_fold_many<std::decay_t<decltype(t)>>, pdl, blocks, TPB, s, t);
         });
 }
 
@@ -883,9 +897,9 @@ void launch_add(fhe_ctx *c, const u64 *a, const u64 *b, u64 *out, int outer, int
 
 void launch_ms_fold_many(const std::vector<FoldArgs> &items)
 {
-    launch_tables<FoldTable>(
+    launch_tables<FoldSeg>(
         items, FHE_K_ELEMWISE,
-        [](FoldSeg &S, const FoldArgs &a, double *bytes) {
+        [](FoldSeg &S, const FoldArgs &a, int, double *bytes) {
             fhe_ctx *c = a.c;
             S.total = (long long)a.outer * c->N;
             if (S.total <= 0 || a.k < 2) return 0;
@@ -898,8 +912,8 @@ void launch_ms_fold_many(const std::vector<FoldArgs> &items)
             *bytes = 8.0 * 2.0 * a.k * S.total;
             return (int)((S.total + TPB - 1) / TPB);
         },
-        [](FoldTable &t, bool pdl, int blocks, cudaStream_t s) {
+        [](auto &t, bool pdl, int blocks, cudaStream_t s) {
             t.rms = 0;
-            launch_pdl(k_fold_many, pdl, blocks, TPB, s, t);
+            launch_pdl(k_fold_many<std::decay_t<decltype(t)>>, pdl, blocks, TPB, s, t);
         });
 }
