@@ -268,13 +268,13 @@ CLASS_SOURCES = {
     "elementwise": ("many.cu",),
 }
 DRAM_PER_ALGORITHMIC = {
-    "ntt_modup": (1.98, "039d5a18ef76b8b8"),
-    "ntt_moddown": (1.33, "039d5a18ef76b8b8"),
-    "ntt_inv": (1.27, "75770092fe0d8ca6"),
-    "ntt_modswitch": (1.42, "41e4560f2460137e"),
-    "ks_inner": (0.89, "935c4c92edfb7dd5"),
-    "elementwise": (0.83, "935c4c92edfb7dd5"),
-    "tensor": (0.76, "935c4c92edfb7dd5"),
+    "ntt_modup": (1.71, "18da796d2795cbf6"),
+    "ntt_moddown": (1.22, "18da796d2795cbf6"),
+    "ntt_inv": (1.11, "d1567756784a2e5b"),
+    "ntt_modswitch": (1.42, "3be935ba656115f4"),
+    "ks_inner": (0.83, "7ddd821636d4496a"),
+    "elementwise": (0.82, "7ddd821636d4496a"),
+    "tensor": (0.63, "7ddd821636d4496a"),
 }
 
 

@@ -62,7 +62,7 @@ enum {
  * q = 1 (mod prime_mod) in [prime_lo, prime_hi): the first L carry data, the
  * last K (alpha) are the special primes of hybrid key switching.  prime_mod
  * must be a multiple of 2N and of p; all primes must have one bit length
- * below 58.  log_n in [10, 14]; p an odd prime, p = 1 (mod 4) or p = 3 (mod 8). */
+ * below 58.  log_n in [10, 15]; p an odd prime, p = 1 (mod 4) or p = 3 (mod 8). */
 typedef struct {
     int log_n;
     uint64_t p;
@@ -643,10 +643,11 @@ int fhe_mod_switch_noalloc(fhe_ctx *ctx, const uint64_t *in, uint64_t *out, int 
 
 /* The NTT splits N = 2^n1 x 2^n2 (n1 = ceil(n/2)) into a column pass and a
  * row pass, each one kernel whose CTAs (128 threads) work on units of 2048
- * residues; one launch serves batches of any ring degree 2^10..2^15 and
- * level.  The variant is the grid policy: variant 0 launches one CTA per
- * unit; variants 1, 2 and 3 launch 6, 4 and 2 resident CTAs per SM that walk
- * all units (persistent CTAs).  fhe_ctx_create times the variants on a
+ * residues; one launch serves batches of any level, batches of several ring
+ * degrees take one launch per degree.  Launches of a few units per SM run
+ * both passes in one kernel.  For the others the variant is the grid policy:
+ * variant 0 launches one CTA per unit; variants 1, 2 and 3 launch 6, 4 and 2
+ * resident CTAs per SM that walk all units (persistent CTAs).  fhe_ctx_create times the variants on a
  * representative batch and keeps variant 0 unless another is at least 3%
  * faster; fhe_ctx_autotune(ctx, njobs) re-times them on njobs limbs.  Both
  * return the chosen variant.

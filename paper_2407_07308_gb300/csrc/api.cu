@@ -380,8 +380,8 @@ extern "C" int fhe_ctx_create(const fhe_params *P, const fhe_allocator *alloc, v
     c->pool.owner = c;
     int e = build_tables(c);
     if (!e) e = fhe_cuda_check(c, cudaDeviceSynchronize(), "ctx_create");
-    // choose the NTT factorisation for this ring degree on 32 polynomials
-    // (16 ciphertexts) of up to 10 limbs, the scale of batched use
+    // choose the NTT grid policy on 32 polynomials (16 ciphertexts) of up to
+    // 10 limbs, the scale of batched use (more at small ring degrees).
     // FHE_NTT_VARIANT pins the variant (e.g. to profile the one a timed run
     // chose: timings under a profiler are not representative)
     const char *pin = getenv("FHE_NTT_VARIANT");

@@ -529,8 +529,9 @@ int replay_family(const std::vector<fhe_ctx *> &fam, const fhe_job *jobs, std::v
 }
 
 // The compare and max/min jobs of contexts that share a device and a
-// plaintext prime, in one circuit (fused launches across ring degrees,
-// digit counts and levels); their sort jobs afterwards, per context.  Every
+// plaintext prime, in one circuit (fused launches across digit counts and
+// levels, the streaming ones across ring degrees too); their sort jobs
+// afterwards, per context.  Every
 // member context works on the leader's stream meanwhile: the leader first
 // waits for what the others have queued, and they wait for the leader at
 // the end.  A submission shape the family has served before is captured

@@ -5,7 +5,8 @@
 // A launch carries a table of up to FHE_SEGS segments (one batch each, of any
 // context, level and size on one device); segment s owns a contiguous range
 // of blocks, so a block never straddles two segments and every warp still
-// reads 256 contiguous bytes.  Single batches run through the same kernels.
+// reads 256 contiguous bytes.  Single batches run through the same kernels,
+// sums and small products with a table of one.
 #include <string.h>
 
 #include <algorithm>

@@ -25,19 +25,23 @@
 // residues) and one round of the remaining M-4 stages (contiguous blocks).
 // Column passes read and write global memory straight from the rounds'
 // registers, with one exchange in shared memory between them (two where the
-// load converts several limbs); row passes exchange twice.  A column unit is NC adjacent
-// columns of each of NS/NC jobs (one job except at n = 10); a row unit is
-// either one row of each of 16 jobs that share a prime times NS/16 adjacent
-// rows (the batched case: the CTA stages those rows' twiddles once), or NS
-// adjacent rows of one job (small batches; twiddles read through the cache).
+// load converts several limbs); row passes exchange twice.  A column unit is
+// NC adjacent columns of each of NS/NC jobs (one job, but two at n = 10 and
+// where two targets share their sources); a row unit is either one row of each
+// of 16 jobs that share a prime times NS/16 adjacent rows (the batched case:
+// the CTA stages those rows' twiddles once), or NS adjacent rows of one job
+// (small batches; twiddles read through the cache).
 // Global memory is read and written in coalesced runs of at least 64 bytes
 // (32 in paired column units at N = 2^15).
 //
-// What bounds the passes: the multiplier pipe.  Register-resident probes: a
-// 32-bit multiply-add takes one slot of it, a 32 x 32 -> 64 or high product
-// two, and a 64-bit accumulation puts one of its two additions there, so a
-// butterfly's chained product takes about 15 slots; the other pipes and the
-// shared memory run beside it as long as they stay well below their peaks.
+// What bounds the passes: the multiplier pipe before all else (72 to 87% of
+// its slots in the row passes and in columns of one word; the columns that
+// convert several limbs are at 62 to 65% and wait on loads and barriers
+// besides).  Register-resident probes: a 32-bit multiply-add takes one slot of
+// it, a 32 x 32 -> 64 or high product two, and a 64-bit accumulation puts one
+// of its two additions there, so a butterfly's chained product takes about 15
+// slots; the other pipes and the shared memory run beside it as long as they
+// stay well below their peaks.
 // Measured on the comparison of 16 pairs (N = 2^14, 10 + 3 primes, one
 // replay) and on 7 pairs at N = 2^15 (p = 257, 3 digits, level 17): 12.0 and
 // 59.8 ms with conversions in 128-bit arithmetic, normalised inverse
@@ -46,11 +50,11 @@
 // 41.1 ms with joined segments and sums of two products a statement.
 //
 // Segments and persistence.  A launch carries a table of up to FHE_SEGS
-// segments; a segment is one batch of limb jobs with its own context (ring
-// degree, twiddle and constant tables), pointers and level.  One launch can
-// therefore serve ciphertexts of different ring degree, level and origin:
-// the units of all segments are numbered in order and every CTA walks them
-// with a grid stride (segments of different ring degree: one launch each).
+// segments; a segment is the limb jobs of one or more batches of a context and
+// level, with their ring degree, twiddle and constant tables.  One launch can
+// therefore serve ciphertexts of different level and origin: the units of all
+// segments are numbered in order and every CTA walks them with a grid stride
+// (segments of different ring degree: one launch each).
 // The grid is either one CTA per unit or a fixed number of resident CTAs per
 // SM (the autotuner's choice per context).  Launches of a few units per SM run
 // both passes in one kernel, a cluster of CTAs per limb (k_fwd_small).
